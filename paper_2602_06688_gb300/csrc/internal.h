@@ -285,6 +285,9 @@ int gemm_bf16_tn(specula_ctx *ctx, const void *A, const void *B, int M, int N, i
 int gemm_bf16_terms(specula_ctx *ctx, int n_terms, const void *const *A, const void *const *B,
                     int M, int N, int K, float *C, int splits, float *work, cudaStream_t st);
 
+// modes[b] = R slopes[b] in float32, b < nb (recon_f32.cu)
+int recon_f32_run(specula_ctx *ctx, const float *R, const float *s, float *m, int n_modes,
+                  int n_slopes, int nb, cudaStream_t st);
 int slopes_pyr_run(specula_ctx *ctx, const int32_t *idx, int n_sub, int n_valid,
                    const float *det, const float *ref, int n_batch, float *out, cudaStream_t st);
 

@@ -1,12 +1,13 @@
 // Modal reconstructor: modes[b] = R slopes[b] (Modalrec / Recmat, App. A,
 // Tabs. 3-4; Listing 2 `recmat_object`).
 //
-// At batch 1 the product is bound by reading R once from HBM (4 bytes per
-// element in float32, 2 in bfloat16).  One warp owns one row of R and streams
-// it with 16-byte loads that bypass L1 allocation; the slope vectors stay in
-// L1 through read-only loads.  NB slope vectors share each row load.  The
-// per-lane partial sums run in a fixed order and are combined by a fixed
-// shuffle tree: bit-reproducible.
+// The float32 products are in recon_f32.cu; this file has the bfloat16 ones
+// and the entry points.  At batch 1 a bf16 product is bound by reading R once
+// from HBM.  One warp owns one row of R and streams it with 16-byte loads
+// that bypass L1 allocation; the slope vectors stay in L1 through read-only
+// loads.  NB slope vectors share each row load.  The per-lane partial sums
+// run in a fixed order and are combined by a fixed shuffle tree:
+// bit-reproducible.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -17,13 +18,6 @@ namespace specula {
 
 constexpr int kReconWarps = 8;
 
-__device__ __forceinline__ float4 ld_stream(const float4 *p) {
-  float4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "l"(p));
-  return v;
-}
 __device__ __forceinline__ uint4 ld_stream_u4(const uint4 *p) {
   uint4 v;
   asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -38,106 +32,6 @@ __device__ __forceinline__ float warp_sum_r(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// FP32, vectorised (n_slopes % 4 == 0, 16-byte aligned rows).
-template <int NB>
-__global__ void __launch_bounds__(kReconWarps * 32) k_mvm_f32(
-    const float *__restrict__ R, const float *__restrict__ s, float *__restrict__ m, int n_modes,
-    int n_slopes, int n_batch, int b0) {
-  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= n_modes) return;
-  const float4 *r4 = reinterpret_cast<const float4 *>(R + (size_t)row * n_slopes);
-  const int n4 = n_slopes / 4;
-  float acc[NB];
-#pragma unroll
-  for (int q = 0; q < NB; ++q) acc[q] = 0.f;
-  // UL independent 16-byte row loads in flight per lane
-  constexpr int UL = NB == 1 ? 8 : 4;
-  for (int j0 = lane; j0 < n4; j0 += UL * 32) {
-    float4 a[UL];
-#pragma unroll
-    for (int u = 0; u < UL; ++u)
-      a[u] = (j0 + 32 * u < n4) ? ld_stream(r4 + j0 + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int u = 0; u < UL; ++u) {
-      const int j = j0 + 32 * u;
-      if (j < n4) {
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-          if (b0 + q < n_batch) {
-            const float4 x = __ldg(reinterpret_cast<const float4 *>(s + (size_t)(b0 + q) * n_slopes) + j);
-            acc[q] += a[u].x * x.x + a[u].y * x.y + a[u].z * x.z + a[u].w * x.w;
-          }
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < NB; ++q) {
-    const float v = warp_sum_r(acc[q]);
-    if (lane == 0 && b0 + q < n_batch) m[(size_t)(b0 + q) * n_modes + row] = v;
-  }
-}
-
-// FP32, one slope vector, one row per CTA of kSplitWarps warps: warp w streams
-// the w-th contiguous segment of the row (UL 16-byte loads in flight per
-// lane), then the warps' sums are added in warp order.  Four streams per row
-// keep more bytes in flight per row than one warp does.
-constexpr int kSplitWarps = 4;
-__global__ void __launch_bounds__(kSplitWarps * 32) k_mvm_f32_split(
-    const float *__restrict__ R, const float *__restrict__ s, float *__restrict__ m, int n_modes,
-    int n_slopes) {
-  __shared__ float s_w[kSplitWarps];
-  const int row = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const float4 *r4 = reinterpret_cast<const float4 *>(R + (size_t)row * n_slopes);
-  const float4 *s4 = reinterpret_cast<const float4 *>(s);
-  const int n4 = n_slopes / 4;
-  const int seg = (n4 + kSplitWarps - 1) / kSplitWarps;
-  const int lo = warp * seg, hi = min(n4, lo + seg);
-  constexpr int UL = 4;
-  float acc = 0.f;
-  for (int j0 = lo + lane; j0 < hi; j0 += UL * 32) {
-    float4 a[UL];
-#pragma unroll
-    for (int u = 0; u < UL; ++u)
-      a[u] = (j0 + 32 * u < hi) ? ld_stream(r4 + j0 + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int u = 0; u < UL; ++u) {
-      const int j = j0 + 32 * u;
-      if (j < hi) {
-        const float4 x = __ldg(s4 + j);
-        acc += a[u].x * x.x + a[u].y * x.y + a[u].z * x.z + a[u].w * x.w;
-      }
-    }
-  }
-  acc = warp_sum_r(acc);
-  if (lane == 0) s_w[warp] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float v = 0.f;
-#pragma unroll
-    for (int w = 0; w < kSplitWarps; ++w) v += s_w[w];
-    m[row] = v;
-  }
-}
-
-// FP32, scalar fallback for unaligned sizes.
-__global__ void __launch_bounds__(kReconWarps * 32) k_mvm_f32_scalar(
-    const float *__restrict__ R, const float *__restrict__ s, float *__restrict__ m, int n_modes,
-    int n_slopes, int n_batch) {
-  const int row = blockIdx.x * kReconWarps + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
-  if (row >= n_modes) return;
-  for (int b = 0; b < n_batch; ++b) {
-    float acc = 0.f;
-    for (int j = lane; j < n_slopes; j += 32)
-      acc += R[(size_t)row * n_slopes + j] * s[(size_t)b * n_slopes + j];
-    acc = warp_sum_r(acc);
-    if (lane == 0) m[(size_t)b * n_modes + row] = acc;
-  }
 }
 
 // BF16 (SPLIT = false) or BF16 hi + lo (SPLIT = true); n_slopes % 8 == 0.
@@ -291,25 +185,8 @@ extern "C" int specula_recon(specula_ctx *ctx, const specula_recon_desc *rec,
   constexpr int NB = 4;
   switch (rec->precision) {
     case SPECULA_PREC_FP32:
-      if (rec->n_slopes % 4 == 0 && al16) {
-        for (int b0 = 0; b0 < n_batch; b0 += NB) {
-          if (n_batch == 1)
-            SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st,
-                           k_mvm_f32_split<<<grid1, kSplitWarps * 32, 0, st>>>(
-                               (const float *)rec->R_dev, slopes_dev, modes_dev, rec->n_modes,
-                               rec->n_slopes));
-          else if (n_batch - b0 == 1)
-            SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st, k_mvm_f32<1><<<grid1, blk1, 0, st>>>((const float *)rec->R_dev, slopes_dev, modes_dev,
-                                               rec->n_modes, rec->n_slopes, n_batch, b0));
-          else
-            SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st, k_mvm_f32<NB><<<grid, blk, 0, st>>>((const float *)rec->R_dev, slopes_dev, modes_dev,
-                                                rec->n_modes, rec->n_slopes, n_batch, b0));
-        }
-      } else {
-        SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st, k_mvm_f32_scalar<<<grid, blk, 0, st>>>((const float *)rec->R_dev, slopes_dev, modes_dev,
-                                               rec->n_modes, rec->n_slopes, n_batch));
-      }
-      return SPECULA_OK;
+      return recon_f32_run(ctx, (const float *)rec->R_dev, slopes_dev, modes_dev, rec->n_modes,
+                           rec->n_slopes, n_batch, st);
     case SPECULA_PREC_BF16:
     case SPECULA_PREC_BF16X2: {
       const bool split = rec->precision == SPECULA_PREC_BF16X2;
