@@ -183,6 +183,9 @@ struct specula_ctx {
   // one wavelength's spots of the polychromatic Shack-Hartmann (grown on
   // demand outside stream capture)
   specula::DevBuf sh_poly_ws;
+  // batched screens: half spectra of one group, and the call's tables (grown
+  // on demand; at most 80 MB of spectra, or one screen's)
+  specula::DevBuf screen_ws;
 };
 
 namespace specula {

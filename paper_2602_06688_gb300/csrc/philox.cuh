@@ -40,11 +40,13 @@ __device__ __forceinline__ void philox_normals4(uint32_t c[4], uint64_t seed, do
 #pragma unroll
   for (int i = 0; i < 4; ++i) u[i] = philox_uniform(c[i]);
   const double r0 = sqrt(-2.0 * log(u[0])), r1 = sqrt(-2.0 * log(u[2]));
-  const double t0 = 2.0 * M_PI * u[1], t1 = 2.0 * M_PI * u[3];
-  g[0] = r0 * cos(t0);
-  g[1] = r0 * sin(t0);
-  g[2] = r1 * cos(t1);
-  g[3] = r1 * sin(t1);
+  double s0, c0, s1, c1;   // of 2 pi u, the multiple of pi exact
+  sincospi(2.0 * u[1], &s0, &c0);
+  sincospi(2.0 * u[3], &s1, &c1);
+  g[0] = r0 * c0;
+  g[1] = r0 * s0;
+  g[2] = r1 * c1;
+  g[3] = r1 * s1;
 }
 
 }  // namespace specula

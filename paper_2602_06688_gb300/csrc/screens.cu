@@ -5,12 +5,13 @@
 //   screen[y][x] = Re sum_k c_k sqrt(Phi(f_k)) df exp(2 pi i f_k . (x, y) pitch)
 //                + subharmonics - their spatial mean
 //
-// Everything runs in float64 on the device (a set-up cost, not per frame):
-// spectral weighting, a radix-2 Stockham FFT along rows in shared memory, a
+// Everything runs in float64 on the device (a set-up cost, not per frame).
+// The single screen from given noise: spectral weighting, a radix-2 Stockham FFT along rows in shared memory, a
 // tiled transpose, the second row pass, and a final kernel that adds the
 // separable subharmonic sum and rounds to float32 once.
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "internal.h"
@@ -121,94 +122,353 @@ __global__ void k_rng_complex(uint64_t seed, int sample0, int stream_id, long lo
   if (2 * pair + 1 < n) out[(size_t)b * n + 2 * pair + 1] = make_double2(g[2], g[3]);
 }
 
-// Philox screen noise (stream 0) times the spectral amplitude, per screen b
-__global__ void k_noise_psd_batch(double2 *__restrict__ A, int M, double Md, double coef,
-                                  double k0, uint64_t seed, int sample0) {
-  const long long pair = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const int b = blockIdx.y;
-  const long long n = (long long)M * M;
-  if (2 * pair >= n) return;
-  double g[4];
-  normals4((uint64_t)pair, (uint32_t)(sample0 + b), 0u, seed, g);
+// ---- batched screens ---------------------------------------------------------------
+// Everything is float64, whose rate bounds it (about 2 fused multiply-adds per
+// clock and SM): 256 screens of 256^2 took 6.5 ms for the noise (two pow per
+// pair of pixels), 2.0 ms for radix-2 transforms, 5.1 ms for the subharmonics
+// (24 complex products per pixel) before this form.
+//  * The spectral amplitude depends on (|kx|, |ky|) and not on the screen: one
+//    quadrant table per call.
+//  * Only the real part is wanted: Re IDFT(a) = IDFT(h), h the Hermitian part
+//    of a, so the row transforms run for ky = 0 .. M/2 only and the column
+//    transforms take two real columns at a time: half the transforms.
+//  * The subharmonics are separable: per column nine products, per pixel six
+//    fused multiply-adds.
+// 256 screens of 256^2 now: 2.79 ms (pass 1, of which the Box-Muller normals
+// are about 2.3) and 0.81 ms (pass 2).
+// Pass 1 (k_screen_rows) draws rows ky and -ky, combines and transforms them;
+// pass 2 (k_screen_cols) transforms the columns, adds the subharmonics and
+// rounds to float32 once.
+
+// Radix-4 Stockham pass of an M = 2^LOGM point inverse DFT (sign +), thread t
+// of M/4, in place in buf with the values held in registers between the two
+// barriers.  L: length transformed so far.  All threads of the CTA call it.
+__device__ __forceinline__ double2 dmul(double2 a, double2 w) {
+  return make_double2(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
+}
+__device__ __forceinline__ double2 dadd(double2 a, double2 b) {
+  return make_double2(a.x + b.x, a.y + b.y);
+}
+__device__ __forceinline__ double2 dsub(double2 a, double2 b) {
+  return make_double2(a.x - b.x, a.y - b.y);
+}
+__device__ __forceinline__ void dfft4(double2 (&x)[4]) {   // natural order, sign +
+  const double2 a = dadd(x[0], x[2]), b = dsub(x[0], x[2]);
+  const double2 c = dadd(x[1], x[3]), e = dsub(x[1], x[3]);
+  x[0] = dadd(a, c);
+  x[2] = dsub(a, c);
+  x[1] = make_double2(b.x - e.y, b.y + e.x);
+  x[3] = make_double2(b.x + e.y, b.y - e.x);
+}
+
+// M-point inverse DFT of one vector by M/4 threads.  load(i): input i of the
+// first pass, called before the first barrier; store(i, v): output i, called
+// after the last barrier (every load and exchange of the CTA is done).  tw[m]
+// = exp(2 pi i m / M).  Odd LOGM ends with a radix-2 pass.
+template <int LOGM, class Load, class Store>
+__device__ __forceinline__ void dfft(double2 *buf, int t, const double2 *__restrict__ tw,
+                                     Load load, Store store) {
+  constexpr int M = 1 << LOGM, P4 = LOGM / 2;
+  double2 x[4];
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const long long e = 2 * pair + q;
-    const int ky = (int)(e / M), kx = (int)(e % M);
-    const int sx = kx >= M / 2 ? kx - M : kx, sy = ky >= M / 2 ? ky - M : ky;
-    const double fx = (double)sx / Md, fy = (double)sy / Md;
+  for (int q = 0; q < 4; ++q) x[q] = load(t + q * (M / 4));
+#pragma unroll
+  for (int s = 0; s < P4; ++s) {
+    const int L = 1 << (2 * s);
+    const int k = t & (L - 1);
+    if (s > 0) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) x[q] = buf[t + q * (M / 4)];
+#pragma unroll
+      for (int q = 1; q < 4; ++q) x[q] = dmul(x[q], __ldg(tw + q * k * (M / (4 * L))));
+    }
+    dfft4(x);
+    __syncthreads();   // every input of this pass is in registers
+    if (s == P4 - 1 && LOGM % 2 == 0) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) store(t + q * (M / 4), x[q]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) buf[(t - k) * 4 + k + q * L] = x[q];
+      __syncthreads();
+    }
+  }
+  if constexpr (LOGM % 2 == 1) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // L = M/2: output i and i + M/2 from inputs i, i + M/2
+      const int i = t + h * (M / 4);
+      x[2 * h] = buf[i];
+      x[2 * h + 1] = dmul(buf[i + M / 2], __ldg(tw + i));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = t + h * (M / 4);
+      store(i, dadd(x[2 * h], x[2 * h + 1]));
+      store(i + M / 2, dsub(x[2 * h], x[2 * h + 1]));
+    }
+  }
+}
+
+constexpr int kScrThreads = 256;
+constexpr int kSubLevels = 3;
+
+// tw[m] = exp(2 pi i m / M), m < M; per level p: sub[p][x] = exp(2 pi i x /
+// (M 3^(p+1))); amp[j][i] = sqrt(Phi) df / 2 at |ky| = j, |kx| = i <= M/2 (the
+// half of the Hermitian part).
+__global__ void __launch_bounds__(256) k_screen_tables(double2 *__restrict__ tw,
+                                                       double2 *__restrict__ sub,
+                                                       double *__restrict__ amp, int M, double Md,
+                                                       double coef, double k0) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int H = M / 2 + 1;
+  if (e < M) {
+    double sn, cs;
+    sincospi(2.0 * (double)e / (double)M, &sn, &cs);
+    tw[e] = make_double2(cs, sn);
+    double w = 1.0;
+    for (int p = 0; p < kSubLevels; ++p) {
+      w *= 3.0;
+      sincospi(2.0 * (double)e / ((double)M * w), &sn, &cs);
+      sub[(size_t)p * M + e] = make_double2(cs, sn);
+    }
+  }
+  if (e < H * H) {
+    const double fx = (double)(e % H) / Md, fy = (double)(e / H) / Md;
     const double f2 = fx * fx + fy * fy;
-    double a = 0.0;
-    if (f2 > 0.0) a = sqrt(coef * pow(f2 + k0, -11.0 / 6.0)) / Md;
-    A[(size_t)b * n + e] = make_double2(g[2 * q] * a, g[2 * q + 1] * a);
+    amp[e] = f2 > 0.0 ? 0.5 * (sqrt(coef * pow(f2 + k0, -11.0 / 6.0)) / Md) : 0.0;
   }
 }
 
-__global__ void k_transpose_f64_batch(const double2 *__restrict__ in, double2 *__restrict__ out,
-                                      int M) {
-  __shared__ double2 tile[32][33];
-  const size_t off = (size_t)blockIdx.z * M * M;
-  const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y)
-    tile[r][threadIdx.x] = in[off + (size_t)(by + r) * M + bx + threadIdx.x];
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y)
-    out[off + (size_t)(bx + r) * M + by + threadIdx.x] = tile[threadIdx.x][r];
+// mean[p] = mean over x of sub[p][x]: one CTA per level, strided sums, then a
+// fixed tree.
+__global__ void __launch_bounds__(256) k_screen_sub_mean(const double2 *__restrict__ sub, int M,
+                                                         double2 *__restrict__ mean) {
+  __shared__ double2 s_v[256];
+  double2 v = make_double2(0.0, 0.0);
+  for (int x = threadIdx.x; x < M; x += 256) v = dadd(v, sub[(size_t)blockIdx.x * M + x]);
+  s_v[threadIdx.x] = v;
+  for (int o = 128; o > 0; o >>= 1) {
+    __syncthreads();
+    if (threadIdx.x < o) s_v[threadIdx.x] = dadd(s_v[threadIdx.x], s_v[threadIdx.x + o]);
+  }
+  if (threadIdx.x == 0) mean[blockIdx.x] = make_double2(s_v[0].x / M, s_v[0].y / M);
 }
 
-// per screen: subharmonic coefficients (Philox stream 1: 27 complex values,
-// element (p * 3 + b) * 3 + a) times the amplitudes, and the spatial mean of
-// the subharmonic sum (separable: sum Re(c mean(ex_a) mean(ey_b)))
-__global__ void k_sub_coef_batch(const double *__restrict__ amp27, const double2 *__restrict__ tmean,
-                                 uint64_t seed, int sample0, int n_screens,
-                                 double2 *__restrict__ coef, double *__restrict__ sub_mean) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= n_screens) return;
-  double2 c[28];
-  for (int pr = 0; pr < 14; ++pr) {
+// One warp per screen: its 27 subharmonic coefficients (Philox stream 1,
+// element e = (p * 3 + b) * 3 + a, frequencies (a - 1, b - 1) df / 3^(p+1))
+// and the spatial mean of their sum.
+__global__ void __launch_bounds__(256) k_screen_sub_coef(const double2 *__restrict__ mean,
+                                                         double Md, double psd, double k0,
+                                                         uint64_t seed, int sample0,
+                                                         int n_screens, double2 *__restrict__ coef,
+                                                         double *__restrict__ sub_mean) {
+  __shared__ double2 s_c[8][28];
+  const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int b = blockIdx.x * 8 + w;
+  if (b < n_screens && lane < 14) {
     double g[4];
-    normals4((uint64_t)pr, (uint32_t)(sample0 + b), 1u, seed, g);
-    c[2 * pr] = make_double2(g[0], g[1]);
-    c[2 * pr + 1] = make_double2(g[2], g[3]);
+    normals4((uint64_t)lane, (uint32_t)(sample0 + b), 1u, seed, g);
+    s_c[w][2 * lane] = make_double2(g[0], g[1]);
+    s_c[w][2 * lane + 1] = make_double2(g[2], g[3]);
   }
-  double mean = 0.0;
-  for (int e = 0; e < 27; ++e) {
-    const int p = e / 9, bb = (e / 3) % 3, a = e % 3;
-    const double2 v = make_double2(c[e].x * amp27[e], c[e].y * amp27[e]);
-    coef[(size_t)b * 27 + e] = v;
-    const double2 mx = tmean[p * 3 + a], my = tmean[p * 3 + bb];
-    const double2 m = make_double2(mx.x * my.x - mx.y * my.y, mx.x * my.y + mx.y * my.x);
-    mean += v.x * m.x - v.y * m.y;
+  __syncwarp();
+  double m = 0.0;
+  if (b < n_screens && lane < 27) {
+    const int p = lane / 9, bb = (lane / 3) % 3, a = lane % 3;
+    const double df = 1.0 / (Md * (p == 0 ? 3.0 : (p == 1 ? 9.0 : 27.0)));
+    const double fx = (a - 1) * df, fy = (bb - 1) * df, f2 = fx * fx + fy * fy;
+    const double amp = f2 > 0.0 ? sqrt(psd * pow(f2 + k0, -11.0 / 6.0)) * df : 0.0;
+    const double2 c = make_double2(s_c[w][lane].x * amp, s_c[w][lane].y * amp);
+    coef[(size_t)b * 27 + lane] = c;
+    const double2 e = mean[p];
+    const double2 mx = a == 1 ? make_double2(1.0, 0.0) : make_double2(e.x, a == 2 ? e.y : -e.y);
+    const double2 my = bb == 1 ? make_double2(1.0, 0.0) : make_double2(e.x, bb == 2 ? e.y : -e.y);
+    const double2 mm = dmul(mx, my);
+    m = c.x * mm.x - c.y * mm.y;
   }
-  sub_mean[b] = mean;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+  if (b < n_screens && lane == 0) sub_mean[b] = m;
 }
 
-__global__ void k_screen_final_batch(const double2 *__restrict__ T, const double2 *__restrict__ tab,
-                                     const double2 *__restrict__ coef,
-                                     const double *__restrict__ sub_mean, int M, int levels,
-                                     float *__restrict__ out) {
-  __shared__ double2 tile[32][33];
-  const int b = blockIdx.z;
-  const size_t off = (size_t)b * M * M;
-  const double2 *cf = coef + (size_t)b * 27;
-  const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y)
-    tile[r][threadIdx.x] = T[off + (size_t)(bx + r) * M + by + threadIdx.x];
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int y = by + r, x = bx + threadIdx.x;
-    double sub = 0.0;
-    for (int p = 0; p < levels; ++p)
-      for (int bb = 0; bb < 3; ++bb)
-        for (int aa = 0; aa < 3; ++aa) {
-          if (aa == 1 && bb == 1) continue;
-          const double2 ex = tab[((size_t)p * 3 + aa) * M + x];
-          const double2 ey = tab[((size_t)p * 3 + bb) * M + y];
-          const double2 e = make_double2(ex.x * ey.x - ex.y * ey.y, ex.x * ey.y + ex.y * ey.x);
-          const double2 c = cf[(p * 3 + bb) * 3 + aa];
-          sub += c.x * e.x - c.y * e.y;
-        }
-    out[off + (size_t)y * M + x] = (float)(tile[threadIdx.x][r].x + (sub - sub_mean[b]));
+template <int LOGM> struct ScrCfg {
+  static constexpr int M = 1 << LOGM, H = M / 2 + 1;
+  static constexpr int TPR = M / 4;                       // threads per transform
+  // rows per CTA of pass 1
+  static constexpr int RPB = TPR >= kScrThreads ? 1 : kScrThreads / TPR;
+  static constexpr size_t smem1 = (size_t)RPB * 2 * M * sizeof(double2);
+  // pass 2: TB transforms per CTA, two columns each (eight columns give the
+  // row tiles whole 128-byte lines; fewer where M/4 threads fill a CTA)
+  static constexpr int TB0 = TPR >= 1024 ? 1 : (TPR >= 512 ? 2 : (TPR >= 64 ? 4 : 256 / TPR));
+  static constexpr int TB = TB0 * 2 > M ? M / 2 : TB0;
+  static constexpr int W = 2 * TB, LD = H | 1;
+  static constexpr size_t smem2 =
+      ((size_t)W * LD > (size_t)TB * M ? (size_t)W * LD : (size_t)TB * M) * sizeof(double2) +
+      (size_t)W * 7 * sizeof(double);
+};
+
+// Pass 1: rows ky = 0 .. M/2 of the Hermitian part, transformed along kx.
+// grid (ceil(H / RPB), n_screens).
+template <int LOGM>
+__global__ void __launch_bounds__(ScrCfg<LOGM>::RPB *ScrCfg<LOGM>::TPR) k_screen_rows(
+    const double2 *__restrict__ tw, const double *__restrict__ amp, uint64_t seed, int sample0,
+    double2 *__restrict__ rows) {
+  using C = ScrCfg<LOGM>;
+  constexpr int M = C::M, TPR = C::TPR;
+  extern __shared__ __align__(16) double2 sm_d[];
+  const int v = threadIdx.x / TPR, t = threadIdx.x % TPR, b = blockIdx.y;
+  const int ky = blockIdx.x * C::RPB + v;
+  const bool ok = ky < C::H;
+  double2 *c1 = sm_d + (size_t)v * 2 * M, *c2 = c1 + M;   // noise rows ky and -ky
+  const int kyn = ky == 0 ? 0 : M - ky;
+  if (ok) {
+    for (int i = t; i < M; i += TPR) {   // M/2 counters per row, two rows
+      const bool second = i >= M / 2;
+      const int pr = second ? i - M / 2 : i;
+      double g[4];
+      normals4((uint64_t)(second ? kyn : ky) * (M / 2) + pr, (uint32_t)(sample0 + b), 0u, seed, g);
+      double2 *d = (second ? c2 : c1) + 2 * pr;
+      d[0] = make_double2(g[0], g[1]);
+      d[1] = make_double2(g[2], g[3]);
+    }
   }
+  __syncthreads();
+  const double *am = amp + (size_t)(ok ? ky : 0) * C::H;
+  double2 *dst = rows + ((size_t)b * C::H + (ok ? ky : 0)) * M;
+  dfft<LOGM>(
+      c1, t, tw,
+      [&](int i) {
+        const double a = __ldg(am + (i > M / 2 ? M - i : i));
+        const double2 p = c1[i], q = c2[i == 0 ? 0 : M - i];
+        return make_double2(a * (p.x + q.x), a * (p.y - q.y));
+      },
+      [&](int i, double2 z) {
+        if (ok) dst[i] = z;
+      });
+}
+
+// Pass 2: W columns of one screen, two at a time.  grid (M / W, n_screens).
+template <int LOGM>
+__global__ void __launch_bounds__(ScrCfg<LOGM>::TB *ScrCfg<LOGM>::TPR) k_screen_cols(
+    const double2 *__restrict__ rows, const double2 *__restrict__ tw,
+    const double2 *__restrict__ sub, const double2 *__restrict__ coef,
+    const double *__restrict__ sub_mean, float *__restrict__ out) {
+  using C = ScrCfg<LOGM>;
+  constexpr int M = C::M, TPR = C::TPR, W = C::W, LD = C::LD, NT = C::TB * TPR;
+  extern __shared__ __align__(16) double2 sm_d[];
+  const int v = threadIdx.x / TPR, t = threadIdx.x % TPR, b = blockIdx.y;
+  const int x0 = blockIdx.x * W;
+  double *s_sub = reinterpret_cast<double *>(
+      sm_d + ((size_t)W * LD > (size_t)C::TB * M ? (size_t)W * LD : (size_t)C::TB * M));
+  // the columns' half spectra, column-major
+  const double2 *src = rows + (size_t)b * C::H * M + x0;
+  for (int e = threadIdx.x; e < C::H * W; e += NT) {
+    const int c = e % W, ky = e / W;
+    sm_d[(size_t)c * LD + ky] = src[(size_t)ky * M + c];
+  }
+  // column x's subharmonics: s_sub[c][2p] cos + s_sub[c][2p + 1] sin of level
+  // p's row phase, plus s_sub[c][6]
+  for (int c = threadIdx.x; c < W; c += NT) {
+    double k = -sub_mean[b];
+    const double2 *cf = coef + (size_t)b * 27;
+#pragma unroll
+    for (int p = 0; p < kSubLevels; ++p) {
+      const double2 e = sub[(size_t)p * M + x0 + c], en = make_double2(e.x, -e.y);
+      double2 G[3];
+#pragma unroll
+      for (int bb = 0; bb < 3; ++bb) {
+        const double2 *q = cf + (p * 3 + bb) * 3;
+        G[bb] = dadd(dmul(q[0], en), dmul(q[2], e));
+        if (bb != 1) G[bb] = dadd(G[bb], q[1]);
+      }
+      s_sub[c * 7 + 2 * p] = G[2].x + G[0].x;
+      s_sub[c * 7 + 2 * p + 1] = G[0].y - G[2].y;
+      k += G[1].x;
+    }
+    s_sub[c * 7 + 6] = k;
+  }
+  __syncthreads();
+  const double2 *r1 = sm_d + (size_t)(2 * v) * LD, *r2 = r1 + LD;
+  const double *u1 = s_sub + (2 * v) * 7, *u2 = u1 + 7;
+  float *tile = reinterpret_cast<float *>(sm_d);
+  constexpr int TLD = M + 1;
+  dfft<LOGM>(
+      sm_d + (size_t)v * M, t, tw,
+      [&](int i) {
+        if (i == 0 || i == M / 2) return make_double2(r1[i].x, r2[i].x);
+        const int k = i < M / 2 ? i : M - i;
+        const double s = i < M / 2 ? 1.0 : -1.0;   // conjugates above M/2
+        const double2 a = r1[k], c = r2[k];
+        return make_double2(a.x - s * c.y, s * a.y + c.x);
+      },
+      [&](int y, double2 z) {
+        double v1 = u1[6], v2 = u2[6];
+#pragma unroll
+        for (int p = 0; p < kSubLevels; ++p) {
+          const double2 e = __ldg(sub + (size_t)p * M + y);
+          v1 += u1[2 * p] * e.x + u1[2 * p + 1] * e.y;
+          v2 += u2[2 * p] * e.x + u2[2 * p + 1] * e.y;
+        }
+        tile[(2 * v) * TLD + y] = (float)(z.x + v1);
+        tile[(2 * v + 1) * TLD + y] = (float)(z.y + v2);
+      });
+  __syncthreads();
+  float *dst = out + (size_t)b * M * M + x0;
+  for (int e = threadIdx.x; e < M * W; e += NT) {
+    const int c = e % W, y = e / W;
+    dst[(size_t)y * M + c] = tile[c * TLD + y];
+  }
+}
+
+// Bytes of the half spectra of one screen, and the most a group of screens
+// takes: a group stays in L2 between the two passes.
+static size_t screen_bytes(int M) { return (size_t)(M / 2 + 1) * M * sizeof(double2); }
+constexpr size_t kScreenGroupBytes = (size_t)80 << 20;
+
+template <int LOGM>
+static int screen_batch(specula_ctx *ctx, int n_screens, double pitch_m, double r0_m, double L0_m,
+                        uint64_t seed, int sample0, float *out, cudaStream_t st) {
+  using C = ScrCfg<LOGM>;
+  constexpr int M = C::M, H = C::H;
+  const double Md = (double)M * pitch_m;
+  const double coef = 0.023 * pow(r0_m, -5.0 / 3.0);
+  const double k0 = isinf(L0_m) ? 0.0 : 1.0 / (L0_m * L0_m);
+  const int groups = (int)(((size_t)n_screens * screen_bytes(M) + kScreenGroupBytes - 1) /
+                           kScreenGroupBytes);
+  const int G = std::min(n_screens, std::max(1, (n_screens + groups - 1) / groups));
+  // workspace, kept by the context: half spectra, twiddles, subharmonic row
+  // phases and their means, coefficients, amplitude quadrant
+  const size_t nd2 = (size_t)G * H * M + M + (size_t)kSubLevels * M + 4 + (size_t)G * 27;
+  const size_t need = nd2 * sizeof(double2) + ((size_t)G + (size_t)H * H) * sizeof(double);
+  int s;
+  if (ctx->screen_ws.bytes < need && (s = ctx->screen_ws.alloc(need))) return s;
+  double2 *rows = ctx->screen_ws.as<double2>(), *tw = rows + (size_t)G * H * M;
+  double2 *sub = tw + M, *mean = sub + (size_t)kSubLevels * M, *cf = mean + 4;
+  double *sm = reinterpret_cast<double *>(cf + (size_t)G * 27), *amp = sm + G;
+  if ((s = ensure_dynamic_smem((const void *)k_screen_rows<LOGM>, C::smem1)) ||
+      (s = ensure_dynamic_smem((const void *)k_screen_cols<LOGM>, C::smem2)))
+    return s;
+  SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
+                 k_screen_tables<<<(std::max(H * H, M) + 255) / 256, 256, 0, st>>>(
+                     tw, sub, amp, M, Md, coef, k0));
+  SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
+                 k_screen_sub_mean<<<kSubLevels, 256, 0, st>>>(sub, M, mean));
+  for (int g0 = 0; g0 < n_screens; g0 += G) {
+    const int ng = std::min(G, n_screens - g0);
+    SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
+                   k_screen_sub_coef<<<(ng + 7) / 8, 256, 0, st>>>(mean, Md, coef, k0, seed,
+                                                                   sample0 + g0, ng, cf, sm));
+    SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
+                   k_screen_rows<LOGM><<<dim3((H + C::RPB - 1) / C::RPB, ng), C::RPB * C::TPR,
+                                         C::smem1, st>>>(tw, amp, seed, sample0 + g0, rows));
+    SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
+                   k_screen_cols<LOGM><<<dim3(M / C::W, ng), C::TB * C::TPR, C::smem2, st>>>(
+                       rows, tw, sub, cf, sm, out + (size_t)g0 * M * M));
+  }
+  // the workspace is the context's, whatever stream its next call runs on
+  SPECULA_CK(cudaStreamSynchronize(st));
+  return SPECULA_OK;
 }
 
 // phase[b][j][i] = scale[b] * screen[b][j + o][i + o], o = (side - n) / 2
@@ -340,81 +600,22 @@ extern "C" int specula_screen_generate_batch(specula_ctx *ctx, int32_t n_screens
   if (!(pitch_m > 0) || !(r0_m > 0) || !(L0_m > 0)) return SPECULA_EINVAL;
   SPECULA_CK(cudaSetDevice(ctx->device));
   cudaStream_t st = (cudaStream_t)stream;
-  const int M = side;
-  int logM = 0;
-  while ((1 << logM) < M) ++logM;
-  const double Md = (double)M * pitch_m;
-  const double df = 1.0 / Md;
-  const double coef = 0.023 * pow(r0_m, -5.0 / 3.0);
-  const double k0 = isinf(L0_m) ? 0.0 : 1.0 / (L0_m * L0_m);
-  const int levels = 3;
-  std::vector<double2> tw(M / 2);
-  for (int k = 0; k < M / 2; ++k) {
-    const double a = 2.0 * M_PI * (double)k / (double)M;
-    tw[k] = make_double2(cos(a), sin(a));
+  switch (side) {
+#define SPECULA_SCREENS(LOGM_)                                                                 \
+  case 1 << LOGM_:                                                                             \
+    return screen_batch<LOGM_>(ctx, n_screens, pitch_m, r0_m, L0_m, seed, sample0, screens_dev, \
+                               st)
+    SPECULA_SCREENS(5);
+    SPECULA_SCREENS(6);
+    SPECULA_SCREENS(7);
+    SPECULA_SCREENS(8);
+    SPECULA_SCREENS(9);
+    SPECULA_SCREENS(10);
+    SPECULA_SCREENS(11);
+    SPECULA_SCREENS(12);
+#undef SPECULA_SCREENS
+    default: return SPECULA_EINVAL;
   }
-  std::vector<double2> tab((size_t)levels * 3 * M), tmean(levels * 3);
-  std::vector<double> amp27(27, 0.0);
-  for (int p = 0; p < levels; ++p) {
-    const double dfp = df / pow(3.0, p + 1);
-    for (int a = 0; a < 3; ++a) {
-      const double f = (a - 1) * dfp;
-      double sr = 0, si = 0;
-      for (int x = 0; x < M; ++x) {
-        const double ang = 2.0 * M_PI * f * ((double)x * pitch_m);
-        const double2 e = make_double2(cos(ang), sin(ang));
-        tab[((size_t)p * 3 + a) * M + x] = e;
-        sr += e.x;
-        si += e.y;
-      }
-      tmean[p * 3 + a] = make_double2(sr / M, si / M);
-    }
-    for (int b = 0; b < 3; ++b)
-      for (int a = 0; a < 3; ++a)
-        if (!(a == 1 && b == 1))
-          amp27[(p * 3 + b) * 3 + a] = sqrt(psd_host((a - 1) * dfp, (b - 1) * dfp, r0_m, L0_m)) * dfp;
-  }
-  DevBuf dtw, dtab, dtmean, damp;
-  int s;
-  if ((s = dtw.upload(tw.data(), tw.size() * sizeof(double2)))) return s;
-  if ((s = dtab.upload(tab.data(), tab.size() * sizeof(double2)))) return s;
-  if ((s = dtmean.upload(tmean.data(), tmean.size() * sizeof(double2)))) return s;
-  if ((s = damp.upload(amp27.data(), amp27.size() * sizeof(double)))) return s;
-  // screens per group: two complex float64 work arrays of at most 1 GiB in all
-  const size_t per = (size_t)M * M * sizeof(double2);
-  const int G = (int)std::max<size_t>(1, std::min<size_t>(n_screens, (1ull << 30) / (2 * per)));
-  DevBuf A, B, cf, sm;
-  if ((s = A.alloc(G * per)) || (s = B.alloc(G * per)) ||
-      (s = cf.alloc((size_t)G * 27 * sizeof(double2))) || (s = sm.alloc((size_t)G * sizeof(double))))
-    return s;
-  const size_t smem = 2 * (size_t)M * sizeof(double2);
-  if ((s = ensure_dynamic_smem((const void *)k_fft_rows_f64, smem))) return s;
-  for (int g0 = 0; g0 < n_screens; g0 += G) {
-    const int ng = std::min(G, n_screens - g0);
-    const long long pairs = (long long)M * M / 2;
-    SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
-                   k_noise_psd_batch<<<dim3((unsigned)((pairs + 255) / 256), ng), 256, 0, st>>>(
-                       A.as<double2>(), M, Md, coef, k0, seed, sample0 + g0));
-    SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
-                   k_fft_rows_f64<<<ng * M, 256, smem, st>>>(A.as<double2>(), dtw.as<double2>(), M,
-                                                             logM));
-    SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
-                   k_transpose_f64_batch<<<dim3(M / 32, M / 32, ng), dim3(32, 8), 0, st>>>(
-                       A.as<double2>(), B.as<double2>(), M));
-    SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
-                   k_fft_rows_f64<<<ng * M, 256, smem, st>>>(B.as<double2>(), dtw.as<double2>(), M,
-                                                             logM));
-    SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
-                   k_sub_coef_batch<<<(ng + 63) / 64, 64, 0, st>>>(
-                       damp.as<double>(), dtmean.as<double2>(), seed, sample0 + g0, ng,
-                       cf.as<double2>(), sm.as<double>()));
-    SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
-                   k_screen_final_batch<<<dim3(M / 32, M / 32, ng), dim3(32, 8), 0, st>>>(
-                       B.as<double2>(), dtab.as<double2>(), cf.as<double2>(), sm.as<double>(), M,
-                       levels, screens_dev + (size_t)g0 * M * M));
-  }
-  SPECULA_CK(cudaStreamSynchronize(st));   // the work arrays are freed on return
-  return SPECULA_OK;
 }
 
 extern "C" int specula_random_phase(specula_ctx *ctx, const float *screens_dev, int32_t n,
