@@ -1228,10 +1228,32 @@ int pwfs_plan_build(specula_ctx *ctx, const specula_pupil_desc *pupil,
   if ((s = p->twA.upload(ta.data(), ta.size() * sizeof(float2)))) return s;
   if ((s = p->twB.upload(tb.data(), tb.size() * sizeof(float2)))) return s;
 
-  // chunk: keep the two intermediates of a chunk near 48 MB (L2-resident)
-  const size_t per_item = ((size_t)Np * N + (size_t)N * N) * sizeof(float2);
-  int chunk = (int)std::max<size_t>(1, (48u << 20) / per_item);
-  chunk = std::min(chunk, 64);
+  // Default chunk.  Two-pass form: as many row-filter slots as keep the rows
+  // workspace within kRowsBytes, a size that L2 (129 MB) still holds between
+  // the passes, in whole batch elements where one fits (at most
+  // kChunkElements) and in equal parts of one where not.  Small chunks end
+  // each launch on a nearly empty last wave: 4 of the 39 m image's 25 slots
+  // per launch (120 row and 1536 column CTAs at a time) cost its frame 303 us
+  // against 253 us in one chunk; the ANDES image in 13 chunks 604 us, 402 us
+  // in one.
+  // Three-pass form: both intermediates near 48 MB.
+  constexpr size_t kRowsBytes = (size_t)100 << 20;
+  constexpr int kChunkElements = 32;
+  int chunk;
+  if (p->two_ok) {
+    const size_t slot = (size_t)Np * N * sizeof(float2);
+    const int fit = (int)std::max<size_t>(1, kRowsBytes / slot);
+    if (fit >= p->nc) {
+      chunk = std::min(fit / p->nc, kChunkElements) * p->nc;
+    } else {
+      const int parts = (p->nc + fit - 1) / fit;
+      chunk = (p->nc + parts - 1) / parts;
+    }
+    chunk = std::min(chunk, 4096);
+  } else {
+    const size_t per_item = ((size_t)Np * N + (size_t)N * N) * sizeof(float2);
+    chunk = (int)std::min<size_t>(64, std::max<size_t>(1, (48u << 20) / per_item));
+  }
   if ((s = pwfs_set_tiles(p.get(), chunk, 1, p->two_ok ? 2 : 3))) return s;
   *out = p.get();
   ctx->pwfs.push_back(std::move(p));
