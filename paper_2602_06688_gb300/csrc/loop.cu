@@ -6,47 +6,105 @@
 //   c_k = (1 - leak) c_{k-1} + gain m.
 // Every sum runs in a fixed order (no float atomics), so a loop is
 // bit-reproducible.
+#include <cooperative_groups.h>
+
 #include "internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace specula {
 
-constexpr int kDmThreads = 256;
+constexpr int kDmWarps = 8;
 constexpr int kDmUnroll = 8;
+constexpr int kDmMaxCluster = 8;
 constexpr int kLoopThreads = 256;
 
-// phase[p] = sum over j = 0 .. n_modes-1, in order, of cmd[j] B[j][p]: one
-// thread per pixel, the coefficients staged in shared memory, eight mode
-// rows' loads in flight (consecutive threads read consecutive pixels).
-__global__ void __launch_bounds__(kDmThreads) k_dm_shape(const float *__restrict__ B,
-                                                         const float *__restrict__ cmd,
-                                                         float *__restrict__ phase, int n_modes,
-                                                         int n_pix2) {
-  extern __shared__ float s_c[];
-  for (int j = threadIdx.x; j < n_modes; j += blockDim.x) s_c[j] = cmd[j];
-  __syncthreads();
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n_pix2) return;
-  const float *b = B + p;
-  float acc = 0.f;
-  int j = 0;
-  for (; j + kDmUnroll <= n_modes; j += kDmUnroll) {
-    float v[kDmUnroll];
+template <int V> struct DmVec;
+template <> struct DmVec<4> { using T = float4; };
+template <> struct DmVec<1> { using T = float; };
+__device__ __forceinline__ void dm_axpy(float4 &a, float c, float4 v) {
+  a.x += c * v.x;
+  a.y += c * v.y;
+  a.z += c * v.z;
+  a.w += c * v.w;
+}
+__device__ __forceinline__ void dm_axpy(float &a, float c, float v) { a += c * v; }
+
+// phase[p] = sum over j of cmd[j] B[j][p].  Bound by reading B once: one
+// thread per pixel over all modes kept 5 KB in flight per SM (500 modes of
+// 160^2 pixels: 33 us for 51 MB).  A CTA of eight warps takes 32 V pixels (V
+// = 4 floats per lane where the size and alignment allow, else 1), the modes
+// split over the warps and over a cluster of CTAs; eight rows' loads in
+// flight per lane.  Each warp adds its modes in order, then the warps' and
+// the CTAs' sums are added in order.
+template <int V>
+__global__ void __launch_bounds__(kDmWarps * 32, 4) k_dm_shape(const float *__restrict__ B,
+                                                            const float *__restrict__ cmd,
+                                                            float *__restrict__ phase,
+                                                            int n_modes, int n_pix2) {
+  using T = typename DmVec<V>::T;
+  __shared__ T s_p[kDmWarps][32];
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nv = n_pix2 / V;
+  const int p = blockIdx.x / cs * 32 + lane;
+  const int part = rank * kDmWarps + warp, parts = cs * kDmWarps;
+  int j = (int)((long long)n_modes * part / parts);
+  const int j1 = (int)((long long)n_modes * (part + 1) / parts);
+  const T *b = reinterpret_cast<const T *>(B) + min(p, nv - 1);
+  T acc = T{};
+  for (; j + kDmUnroll <= j1; j += kDmUnroll) {
+    T v[kDmUnroll];
 #pragma unroll
-    for (int u = 0; u < kDmUnroll; ++u) v[u] = __ldg(b + (size_t)(j + u) * n_pix2);
+    for (int u = 0; u < kDmUnroll; ++u) v[u] = __ldg(b + (size_t)(j + u) * nv);
 #pragma unroll
-    for (int u = 0; u < kDmUnroll; ++u) acc += s_c[j + u] * v[u];
+    for (int u = 0; u < kDmUnroll; ++u) dm_axpy(acc, __ldg(cmd + j + u), v[u]);
   }
-  for (; j < n_modes; ++j) acc += s_c[j] * __ldg(b + (size_t)j * n_pix2);
-  phase[p] = acc;
+  for (; j < j1; ++j) dm_axpy(acc, __ldg(cmd + j), __ldg(b + (size_t)j * nv));
+  s_p[warp][lane] = acc;
+  __syncthreads();
+  if (warp == 0) {
+    acc = s_p[0][lane];
+#pragma unroll
+    for (int w = 1; w < kDmWarps; ++w) dm_axpy(acc, 1.f, s_p[w][lane]);
+    s_p[0][lane] = acc;
+  }
+  if (cs > 1) {
+    cl.sync();
+    if (rank == 0 && warp == 0) {
+      for (int c = 1; c < cs; ++c) dm_axpy(acc, 1.f, cl.map_shared_rank(&s_p[0][0], c)[lane]);
+    }
+    cl.sync();   // no CTA leaves before its sums are read
+  }
+  if (rank == 0 && warp == 0 && p < nv) reinterpret_cast<T *>(phase)[p] = acc;
 }
 
-// residual = atm - dm over the grid; per-CTA float64 partial sums over the
-// pupil (weights amp): sum w, sum w r, sum w r^2, sum w cos(k r), sum w sin(k r)
-// (k = lambda_wfs / lambda_sci), block-strided so the order is fixed.
+// residual = atm - dm over the grid, and its statistics: float64 sums over
+// the pupil (weights amp) of w, w r, w r^2, w cos(k r), w sin(k r), k =
+// lambda_wfs / lambda_sci, per CTA in a fixed order; the CTA that finishes
+// last adds the CTAs' sums in a fixed order and writes
+//   stats[0] = sqrt(sum w r^2 / sum w - mean^2),
+//   stats[1] = |sum w e^{ikr}|^2 / (sum w)^2.
+// Up to kLoopMaxBlocks CTAs, one pixel per thread on the 8 m pupil: float64
+// runs at 2 operations per clock and SM, so 13 CTAs of 8 pixels per thread
+// took 13 us, and the statistics in a kernel of one thread 6.5 us.
+__device__ __forceinline__ void loop_block_sum(double (&a)[5], double (*s_p)[kLoopThreads / 32]) {
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a[q] += __shfl_xor_sync(0xffffffffu, a[q], o);
+    if ((threadIdx.x & 31) == 0) s_p[q][threadIdx.x >> 5] = a[q];
+  }
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(kLoopThreads) k_loop_residual(
     const float *__restrict__ amp, const float *__restrict__ atm, const float *__restrict__ dm,
-    float *__restrict__ resid, double *__restrict__ part, int n_pix2, float k) {
+    float *__restrict__ resid, double *__restrict__ part, unsigned *__restrict__ done,
+    double *__restrict__ stats, int n_pix2, float k) {
   __shared__ double s_p[5][kLoopThreads / 32];
+  __shared__ bool s_last;
   double a[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n_pix2; p += gridDim.x * blockDim.x) {
     const float r = atm[p] - dm[p];
@@ -60,29 +118,31 @@ __global__ void __launch_bounds__(kLoopThreads) k_loop_residual(
     a[3] += w * (double)cv;
     a[4] += w * (double)sv;
   }
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    double v = a[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) s_p[q][threadIdx.x >> 5] = v;
-  }
-  __syncthreads();
+  loop_block_sum(a, s_p);
   if (threadIdx.x < 5) {
     double v = 0.0;
     for (int w = 0; w < kLoopThreads / 32; ++w) v += s_p[threadIdx.x][w];
-    part[(size_t)blockIdx.x * 5 + threadIdx.x] = v;
+    __stcg(part + (size_t)blockIdx.x * 5 + threadIdx.x, v);
+    __threadfence();
   }
-}
-
-// stats[0] = sqrt(sum w r^2 / sum w - mean^2), stats[1] = |sum w e^{ikr}|^2 / (sum w)^2,
-// the CTA partials summed in CTA order.
-__global__ void k_loop_stats(const double *__restrict__ part, int n_part,
-                             double *__restrict__ stats) {
+  __syncthreads();
+  // atomicInc wraps to zero on the last CTA: ready for the next launch
+  if (threadIdx.x == 0) s_last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+#pragma unroll
+  for (int q = 0; q < 5; ++q) a[q] = 0.0;
+  for (int b = threadIdx.x; b < gridDim.x; b += blockDim.x)
+#pragma unroll
+    for (int q = 0; q < 5; ++q) a[q] += __ldcg(part + (size_t)b * 5 + q);
+  loop_block_sum(a, s_p);
   if (threadIdx.x != 0) return;
-  double a[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  for (int b = 0; b < n_part; ++b)
-    for (int q = 0; q < 5; ++q) a[q] += part[(size_t)b * 5 + q];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    a[q] = 0.0;
+    for (int w = 0; w < kLoopThreads / 32; ++w) a[q] += s_p[q][w];
+  }
   if (!(a[0] > 0.0)) {
     stats[0] = 0.0;
     stats[1] = 0.0;
@@ -102,8 +162,10 @@ __global__ void __launch_bounds__(256) k_loop_integrate(const float *__restrict_
 }
 
 int loop_alloc_workspace(specula_ctx *ctx) {
-  if (cudaMalloc(&ctx->loop_part, (size_t)kLoopMaxBlocks * 5 * sizeof(double)) != cudaSuccess)
-    return SPECULA_ENOMEM;
+  // the CTAs' sums, then the count of CTAs that are done (zero between calls)
+  const size_t n = (size_t)kLoopMaxBlocks * 5 * sizeof(double);
+  if (cudaMalloc(&ctx->loop_part, n + sizeof(double)) != cudaSuccess) return SPECULA_ENOMEM;
+  if (cudaMemset(ctx->loop_part, 0, n + sizeof(double)) != cudaSuccess) return SPECULA_ECUDA;
   return SPECULA_OK;
 }
 
@@ -116,12 +178,36 @@ extern "C" int specula_dm_shape(specula_ctx *ctx, int32_t n_modes, int32_t n_pix
                                 void *stream) {
   if (!ctx || !basis_dev || !cmd_dev || !phase_dev) return SPECULA_EINVAL;
   if (n_modes < 1 || n_pix2 < 1) return SPECULA_EINVAL;
-  if (n_modes > 12288) return SPECULA_EUNSUPPORTED;   // coefficients in 48 KB of shared memory
+  if (n_modes > 12288) return SPECULA_EUNSUPPORTED;
   cudaStream_t st = (cudaStream_t)stream;
-  SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
-                 k_dm_shape<<<(n_pix2 + kDmThreads - 1) / kDmThreads, kDmThreads,
-                              n_modes * sizeof(float), st>>>(basis_dev, cmd_dev, phase_dev,
-                                                             n_modes, n_pix2));
+  const bool v4 = n_pix2 % 4 == 0 && (((uintptr_t)basis_dev | (uintptr_t)phase_dev) % 16) == 0;
+  int sms = 0;
+  SPECULA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+  // modes over a cluster until there are two CTAs per SM, while every warp
+  // keeps a full unroll of modes
+  const int tiles = (n_pix2 / (v4 ? 4 : 1) + 31) / 32;
+  int cs = 1;
+  while (cs < kDmMaxCluster && tiles * cs < 2 * sms &&
+         n_modes / (kDmWarps * cs * 2) >= kDmUnroll)
+    cs *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)tiles * cs);
+  cfg.blockDim = dim3(kDmWarps * 32);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (v4)
+    SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
+                   SPECULA_CK(cudaLaunchKernelEx(&cfg, k_dm_shape<4>, basis_dev, cmd_dev,
+                                                 phase_dev, n_modes, n_pix2)));
+  else
+    SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
+                   SPECULA_CK(cudaLaunchKernelEx(&cfg, k_dm_shape<1>, basis_dev, cmd_dev,
+                                                 phase_dev, n_modes, n_pix2)));
   return SPECULA_OK;
 }
 
@@ -132,14 +218,13 @@ extern "C" int specula_loop_residual(specula_ctx *ctx, int32_t n_pix2, const flo
   if (!ctx || !amp_dev || !atm_dev || !dm_dev || !resid_dev || !stats_dev) return SPECULA_EINVAL;
   if (n_pix2 < 1 || !(wfs_over_sci > 0.0) || !isfinite(wfs_over_sci)) return SPECULA_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  int blocks = (n_pix2 + kLoopThreads * 8 - 1) / (kLoopThreads * 8);
-  blocks = blocks < 1 ? 1 : (blocks > kLoopMaxBlocks ? kLoopMaxBlocks : blocks);
+  int blocks = (n_pix2 + kLoopThreads - 1) / kLoopThreads;
+  blocks = blocks > kLoopMaxBlocks ? kLoopMaxBlocks : blocks;
+  unsigned *done = reinterpret_cast<unsigned *>(ctx->loop_part + (size_t)kLoopMaxBlocks * 5);
   SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
                  k_loop_residual<<<blocks, kLoopThreads, 0, st>>>(
-                     amp_dev, atm_dev, dm_dev, resid_dev, ctx->loop_part, n_pix2,
+                     amp_dev, atm_dev, dm_dev, resid_dev, ctx->loop_part, done, stats_dev, n_pix2,
                      (float)wfs_over_sci));
-  SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
-                 k_loop_stats<<<1, 32, 0, st>>>(ctx->loop_part, blocks, stats_dev));
   return SPECULA_OK;
 }
 
