@@ -17,6 +17,9 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <type_traits>
+#include <utility>
+
 namespace specula {
 
 // ---- small complex helpers ------------------------------------------------
@@ -113,6 +116,35 @@ static inline cudaError_t upload_codelet_twiddles() {
     }
   }
   return cudaMemcpyToSymbol(c_prime_pairs, pp, sizeof(pp));
+}
+
+// compile-time loop: f(integral_constant<int, I>) for I = B .. E-1
+template <int B, class F, int... I>
+__device__ __forceinline__ void static_for_impl(F &&f, std::integer_sequence<int, I...>) {
+  (f(std::integral_constant<int, B + I>{}), ...);
+}
+template <int B, int E, class F> __device__ __forceinline__ void static_for(F &&f) {
+  static_for_impl<B>(f, std::make_integer_sequence<int, E - B>{});
+}
+
+// cos, sin and -sin of 2 pi f / P as broadcast pairs, P a base prime
+template <int P> __device__ __forceinline__ float2 dft_cos(int f) {
+  if constexpr (P == 3) return c_bfly_pairs[0];
+  else if constexpr (P == 5) return c_bfly_pairs[1 + f];
+  else return c_prime_pairs[prime_off(P) + f - 1];
+}
+template <int P> __device__ __forceinline__ float2 dft_sin(int f) {
+  if constexpr (P == 3) return c_bfly_pairs[1];
+  else if constexpr (P == 5) return c_bfly_pairs[3 + f];
+  else return c_prime_pairs[prime_off(P) + (P - 1) / 2 + f - 1];
+}
+template <int P> __device__ __forceinline__ float2 dft_nsin(int f) {
+  if constexpr (P == 3 || P == 5) {
+    const float2 s = dft_sin<P>(f);
+    return make_float2(-s.x, -s.y);
+  } else {
+    return c_prime_pairs[prime_off(P) + (P - 1) + f - 1];
+  }
 }
 
 // W_N^J for the forward (exp(-2 pi i J/N)) or inverse (exp(+...)) sign.
@@ -308,6 +340,181 @@ template <bool INV> struct RegDFT<17, INV, 0> {
 };
 template <bool INV> struct RegDFT<5, INV, 0> {
   static __device__ __forceinline__ void run(float2 (&x)[5]) { bfly5<INV>(x[0], x[1], x[2], x[3], x[4]); }
+};
+
+// ---- DFT of inputs that are partly zero ------------------------------------------
+// RegDFTZ<N, INV, NZ>: as RegDFT, for x[j] that may be non-zero only where bit
+// j of NZ is set (the others are not read).  A zero-padded input leaves whole
+// operands of the first butterflies zero; the additions with them are left
+// out, which the compiler may not do by itself (x + 0 is not x for x = -0).
+template <bool A, bool B> __device__ __forceinline__ float2 cadd_z(float2 a, float2 b) {
+  if constexpr (A && B) return cadd(a, b);
+  else if constexpr (A) return a;
+  else return b;
+}
+template <bool A, bool B> __device__ __forceinline__ float2 csub_z(float2 a, float2 b) {
+  if constexpr (A && B) return csub(a, b);
+  else if constexpr (A) return a;
+  else return make_float2(-b.x, -b.y);
+}
+// b + s e and b - s e, s = -i (forward) or +i (inverse)
+template <bool INV, bool B, bool E> __device__ __forceinline__ float2 cadd_mi_z(float2 b, float2 e) {
+  if constexpr (B && E) return cadd_mi<INV>(b, e);
+  else if constexpr (B) return b;
+  else return mul_mi<INV>(e);
+}
+template <bool INV, bool B, bool E> __device__ __forceinline__ float2 csub_mi_z(float2 b, float2 e) {
+  if constexpr (B && E) return csub_mi<INV>(b, e);
+  else if constexpr (B) return b;
+  else return mul_mi<!INV>(e);
+}
+// c a + x
+template <bool A, bool X> __device__ __forceinline__ float2 cfma_z(float2 c, float2 a, float2 x) {
+  if constexpr (A && X) return __ffma2_rn(c, a, x);
+  else if constexpr (A) return __fmul2_rn(c, a);
+  else return x;
+}
+
+typedef unsigned long long nzmask;
+constexpr nzmask nz_full(int n) { return n >= 64 ? ~0ull : ((1ull << n) - 1ull); }
+constexpr bool nz_bit(nzmask m, int j) { return (m >> j) & 1ull; }
+constexpr nzmask nz_range(int lo, int hi) { return nz_full(hi) & ~nz_full(lo); }
+// masks of the sub-transforms: inputs n1 + P n2 (Cooley-Tukey), (a B + b A) mod N
+// (prime factor)
+constexpr nzmask nz_sub_ct(nzmask m, int P, int Q, int n1) {
+  nzmask r = 0;
+  for (int n2 = 0; n2 < Q; ++n2) r |= (nzmask)nz_bit(m, n1 + P * n2) << n2;
+  return r;
+}
+constexpr nzmask nz_sub_pfa(nzmask m, int A, int B, int a) {
+  nzmask r = 0;
+  for (int b = 0; b < B; ++b) r |= (nzmask)nz_bit(m, (a * B + b * A) % (A * B)) << b;
+  return r;
+}
+// which of the first-stage transforms have any non-zero input
+constexpr nzmask nz_outer(nzmask m, int P, int Q, bool pfa) {
+  nzmask r = 0;
+  for (int i = 0; i < P; ++i)
+    r |= (nzmask)((pfa ? nz_sub_pfa(m, P, Q, i) : nz_sub_ct(m, P, Q, i)) != 0) << i;
+  return r;
+}
+
+template <int N, bool INV, nzmask NZ> struct RegDFTZ;
+
+template <int N, bool INV, nzmask NZ> __device__ __forceinline__ void bfly_z(float2 (&x)[N]) {
+  constexpr bool n0 = nz_bit(NZ, 0);
+  if constexpr (N == 2) {
+    constexpr bool n1 = nz_bit(NZ, 1);
+    const float2 a = x[0], b = x[1];
+    x[0] = cadd_z<n0, n1>(a, b);
+    x[1] = csub_z<n0, n1>(a, b);
+  } else if constexpr (N == 4) {
+    constexpr bool n1 = nz_bit(NZ, 1), n2 = nz_bit(NZ, 2), n3 = nz_bit(NZ, 3);
+    constexpr bool nb = n0 || n2, ne = n1 || n3;
+    const float2 z = make_float2(0.f, 0.f);
+    const float2 a = nb ? cadd_z<n0, n2>(x[0], x[2]) : z, b = nb ? csub_z<n0, n2>(x[0], x[2]) : z;
+    const float2 c = ne ? cadd_z<n1, n3>(x[1], x[3]) : z, e = ne ? csub_z<n1, n3>(x[1], x[3]) : z;
+    x[0] = cadd_z<nb, ne>(a, c);
+    x[2] = csub_z<nb, ne>(a, c);
+    x[1] = cadd_mi_z<INV, nb, ne>(b, e);
+    x[3] = csub_mi_z<INV, nb, ne>(b, e);
+  } else {
+    // odd primes from the symmetric pairs (bfly3, bfly5, bfly_prime)
+    constexpr int H = (N - 1) / 2;
+    const float2 z = make_float2(0.f, 0.f);
+    float2 a[H + 1], b[H + 1], y[N];
+    const auto pair = [&](auto jc) {
+      constexpr int j = decltype(jc)::value;
+      constexpr bool u = nz_bit(NZ, j), v = nz_bit(NZ, N - j);
+      a[j] = (u || v) ? cadd_z<u, v>(x[j], x[N - j]) : z;
+      b[j] = (u || v) ? csub_z<u, v>(x[j], x[N - j]) : z;
+    };
+    static_for<1, H + 1>(pair);
+    constexpr auto has = [](int j) { return nz_bit(NZ, j) || nz_bit(NZ, N - j); };
+    y[0] = n0 ? x[0] : z;
+    static_for<1, H + 1>([&](auto jc) {
+      constexpr int j = decltype(jc)::value;
+      constexpr bool before = n0 || (NZ & nz_range(1, j)) || (NZ & nz_range(N - j + 1, N));
+      if constexpr (has(j)) y[0] = cadd_z<before, true>(y[0], a[j]);
+    });
+    static_for<1, H + 1>([&](auto kc) {
+      constexpr int k = decltype(kc)::value;
+      float2 p = n0 ? x[0] : z, q = z;
+      static_for<1, H + 1>([&](auto jc) {
+        constexpr int j = decltype(jc)::value;
+        constexpr int m = (j * k) % N, f = m <= H ? m : N - m;
+        constexpr bool q0 = (NZ & nz_range(1, j)) || (NZ & nz_range(N - j + 1, N));
+        if constexpr (has(j)) {
+          p = cfma_z<true, n0 || q0>(dft_cos<N>(f), a[j], p);
+          q = cfma_z<true, q0>(m <= H ? dft_sin<N>(f) : dft_nsin<N>(f), b[j], q);
+        }
+      });
+      constexpr bool anyp = NZ != 1ull;   // some pair is there
+      y[k] = cadd_mi_z<INV, true, anyp>(p, q);
+      y[N - k] = csub_mi_z<INV, true, anyp>(p, q);
+    });
+#pragma unroll
+    for (int k = 0; k < N; ++k) x[k] = y[k];
+  }
+}
+
+template <int N, bool INV, nzmask NZ> struct RegDFTZ {
+  static __device__ __forceinline__ void run(float2 (&x)[N]) {
+    constexpr int A = pfa_factor<N>::value;
+    if constexpr ((NZ & nz_full(N)) == nz_full(N)) {
+      RegDFT<N, INV>::run(x);
+    } else if constexpr (NZ == 0) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) x[k] = make_float2(0.f, 0.f);
+    } else if constexpr (N == 2 || N == 3 || N == 4 || N == 5 || N == 7 || N == 11 || N == 13 ||
+                         N == 17) {
+      bfly_z<N, INV, NZ>(x);
+    } else if constexpr (A > 0) {
+      constexpr int B = N / A;
+      constexpr int U = inverse_mod(B % A, A), V = inverse_mod(A % B, B);
+      constexpr nzmask OZ = nz_outer(NZ, A, B, true);
+      float2 y[A][B];
+      static_for<0, A>([&](auto ac) {
+        constexpr int a = decltype(ac)::value;
+#pragma unroll
+        for (int b = 0; b < B; ++b) y[a][b] = x[(a * B + b * A) % N];
+        if constexpr (nz_bit(OZ, a)) RegDFTZ<B, INV, nz_sub_pfa(NZ, A, B, a)>::run(y[a]);
+      });
+#pragma unroll
+      for (int kb = 0; kb < B; ++kb) {
+        float2 z[A];
+#pragma unroll
+        for (int a = 0; a < A; ++a) z[a] = y[a][kb];
+        RegDFTZ<A, INV, OZ>::run(z);
+#pragma unroll
+        for (int ka = 0; ka < A; ++ka) x[(ka * B * U + kb * A * V) % N] = z[ka];
+      }
+    } else {
+      constexpr int P = first_factor<N>::value, Q = N / P;
+      static_assert(P * Q == N && P > 1, "unsupported codelet size");
+      constexpr nzmask OZ = nz_outer(NZ, P, Q, false);
+      float2 y[P][Q];
+      static_for<0, P>([&](auto nc) {
+        constexpr int n1 = decltype(nc)::value;
+#pragma unroll
+        for (int n2 = 0; n2 < Q; ++n2) y[n1][n2] = x[n1 + P * n2];
+        if constexpr (nz_bit(OZ, n1)) {
+          RegDFTZ<Q, INV, nz_sub_ct(NZ, P, Q, n1)>::run(y[n1]);
+#pragma unroll
+          for (int k2 = 0; k2 < Q; ++k2) y[n1][k2] = apply_tw<N, INV>(y[n1][k2], n1 * k2);
+        }
+      });
+#pragma unroll
+      for (int k2 = 0; k2 < Q; ++k2) {
+        float2 z[P];
+#pragma unroll
+        for (int n1 = 0; n1 < P; ++n1) z[n1] = y[n1][k2];
+        RegDFTZ<P, INV, OZ>::run(z);
+#pragma unroll
+        for (int k1 = 0; k1 < P; ++k1) x[Q * k1 + k2] = z[k1];
+      }
+    }
+  }
 };
 
 }  // namespace specula

@@ -368,9 +368,11 @@ template <int N1, int N2> struct RowFiltCfg {
 // each item's own y factor gy[m][row] to its input.
 // R: grid (ceil(n_pix / VPC), ceil(n_slots / ka)); block VPC * G threads;
 // writes rows_out[slot][x][row].
-// GEN: any padding (the pupil at padded offset `off`, each lane loading the
-// registers whose padded index falls in the pupil); otherwise the pad-2
-// layout, where the pupil is exactly registers N2/4 .. 3 N2/4 of every lane.
+// PAD: the padding N / n_pix.  The pupil sits at padded offset PadRegs::OFF,
+// so only registers LO .. HI of a lane can be non-zero: the others are neither
+// loaded nor added (RegDFTZ).  With pad 2 and N2 % 4 == 0 the pupil is exactly
+// registers N2/4 .. 3 N2/4 of every lane; otherwise each lane checks its first
+// and last ones.
 // One-warp transforms (G = 32) run four warps per CTA, five CTAs per SM at
 // 96 registers (four rows per CTA: the transposed output goes out as whole
 // 32-byte sectors), and reload the field row for every slot (caching it
@@ -378,22 +380,31 @@ template <int N1, int N2> struct RowFiltCfg {
 // transforms run 256 threads, two CTAs per SM, with the cached row; wide
 // splits run 128-thread CTAs (bounded for up to 256 threads, one CTA per SM,
 // so that their 50-point transforms keep their registers).
+template <int N1, int N2, int PAD> struct PadRegs {
+  static constexpr int N = N1 * N2, NP = N / PAD, OFF = (N - NP) / 2;
+  static constexpr int LO = OFF / N1, HI = (OFF + NP - 1) / N1 + 1;
+  static constexpr bool ALIGNED = OFF % N1 == 0 && NP % N1 == 0;
+  static constexpr nzmask NZ = nz_range(LO, HI);
+  static_assert(N % PAD == 0, "whole pupil side");
+};
+
 template <int N1, int N2> struct RowFiltLaunch {
   using S = Split<N1, N2>;
   static constexpr int threads = S::WIDE ? 256 : (S::G == 32 ? 128 : 256);
   static constexpr int min_blocks = S::WIDE ? 1 : (S::G == 32 ? 5 : 2);
   static constexpr bool reload = S::G == 32;
 };
-template <int N1, int N2, bool GEN = false>
+template <int N1, int N2, int PAD>
 __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
                                   RowFiltLaunch<N1, N2>::min_blocks) k_rowfilt(
     const float2 *__restrict__ field, const float2 *__restrict__ gx,
     const float2 *__restrict__ twA, const float2 *__restrict__ twB,
     const float2 *__restrict__ mask, float2 *__restrict__ rows_out, int n_pix, int nc, int nbw,
-    int slot0, int n_slots, int ka, int off, int s0) {
+    int slot0, int n_slots, int ka, int s0) {
   using S = Split<N1, N2>;
+  using P = PadRegs<N1, N2, PAD>;
   constexpr int N = S::N, G = S::G, S1 = S::S1, S2 = S::S2;
-  constexpr int Q0 = N2 / 4, QH = N2 / 2;
+  constexpr int LO = P::LO, NR = P::HI - P::LO;
   extern __shared__ float2 smem[];
   const int vpc = blockDim.x / G;
   const int vec = threadIdx.x / G, lane = threadIdx.x % G;
@@ -406,7 +417,13 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
   const int j = blockIdx.x * vpc + vec;
   const bool row_ok = j < n_pix;
   const bool in_lane = row_ok && lane < N1;
-  float2 e[GEN ? 1 : QH];
+  // the pupil column of register LO + h is lane + N1 (LO + h) - OFF
+  const auto in_pupil = [&](int h) {
+    const int i = lane + N1 * (LO + h) - P::OFF;
+    return P::ALIGNED || ((h > 0 || i >= 0) && (h < NR - 1 || i < n_pix));
+  };
+  constexpr bool kReload = RowFiltLaunch<N1, N2>::reload || !P::ALIGNED;
+  float2 e[kReload ? 1 : NR];
   int cur_b = -1;
   const int it_begin = blockIdx.y * ka;
   for (int q = 0; q < ka; ++q) {
@@ -414,32 +431,32 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
     if (it >= n_slots) break;
     const int gi = slot0 + it;
     const int b = gi / nc, c = s0 + (gi - b * nc);   // nc slots per element from s0
-    if (!GEN && (RowFiltLaunch<N1, N2>::reload || b != cur_b)) {
-      cur_b = b;
-      const float2 *src = field + ((size_t)(b % nbw) * n_pix + (row_ok ? j : 0)) * n_pix + lane;
+    const float2 *src = field + ((size_t)(b % nbw) * n_pix + (row_ok ? j : 0)) * n_pix +
+                        (lane + N1 * LO - P::OFF);
+    if constexpr (!kReload) {
+      if (b != cur_b) {
+        cur_b = b;
 #pragma unroll
-      for (int h = 0; h < (GEN ? 1 : QH); ++h) e[h] = in_lane ? src[N1 * h] : make_float2(0.f, 0.f);
+        for (int h = 0; h < NR; ++h) e[h] = in_lane ? src[N1 * h] : make_float2(0.f, 0.f);
+      }
     }
     // forward row transform, pruned input (standard split)
     float2 r[N2];
+    {
+      const float2 *g = gx + (size_t)c * n_pix + (lane + N1 * LO - P::OFF);
+      float2 f[NR];
 #pragma unroll
-    for (int n2 = 0; n2 < N2; ++n2) r[n2] = make_float2(0.f, 0.f);
-    if (in_lane) {
-      if constexpr (GEN) {
-        const float2 *src = field + ((size_t)(b % nbw) * n_pix + j) * n_pix;
-        const float2 *g = gx + (size_t)c * n_pix;
-#pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) {
-          const int i = lane + N1 * n2 - off;                // pupil column
-          if (i >= 0 && i < n_pix) r[n2] = cmul(src[i], __ldg(g + i));
-        }
-      } else {
-        const float2 *g = gx + (size_t)c * n_pix + lane;
-#pragma unroll
-        for (int h = 0; h < QH; ++h) r[Q0 + h] = cmul(e[h], __ldg(g + N1 * h));
+      for (int h = 0; h < NR; ++h) {
+        if constexpr (kReload)
+          f[h] = in_lane && in_pupil(h) ? src[N1 * h] : make_float2(0.f, 0.f);
+        else
+          f[h] = e[h];
       }
+#pragma unroll
+      for (int h = 0; h < NR; ++h)
+        r[LO + h] = in_lane && in_pupil(h) ? cmul(f[h], __ldg(g + N1 * h)) : make_float2(0.f, 0.f);
     }
-    RegDFT<N2, false>::run(r);
+    RegDFTZ<N2, false, P::NZ>::run(r);
     __syncwarp();
     if (lane < N1) {
 #pragma unroll
@@ -549,7 +566,7 @@ template <int N1, int N2> struct ColFiltCfg {
 // 39 m pupil's bin side 5) take the variant bounded at 160 threads x 4 CTAs
 // per SM, the occupancy that 80 registers per thread gave them already:
 // 96 registers per thread, so the twiddle loads can be issued earlier.
-template <int N1, int N2, int MAXT = 256, bool GEN = false>
+template <int N1, int N2, int PAD, int MAXT>
 __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
                                               ? 1
                                               : (MAXT <= 160 ? 4 : (MAXT <= 256 ? 3 : 2)))
@@ -557,10 +574,11 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
     const float2 *__restrict__ rows_in, const float2 *__restrict__ gy,
     const float2 *__restrict__ twA, const float2 *__restrict__ twB,
     const float2 *__restrict__ mask, float *__restrict__ part, int n_pix, int fp, int fq,
-    float scale, int n_mod, int nc, int nbw, int slot0, int CS, int off, int s0) {
+    float scale, int n_mod, int nc, int nbw, int slot0, int CS, int s0) {
   using S = Split<N1, N2>;
+  using P = PadRegs<N1, N2, PAD>;
   constexpr int N = S::N, G = S::G, S1 = S::S1, S2 = S::S2;
-  constexpr int Q0 = N2 / 4, QH = N2 / 2;
+  constexpr int LO = P::LO, NR = P::HI - P::LO;
   extern __shared__ __align__(16) float2 smem_k[];
   float2 *s_tile = smem_k;
   const int TC = blockDim.x / G;
@@ -590,33 +608,29 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
   // past L1 (which keeps the twiddle, mask and tilt tables)
   const float2 *cx = rows_in + ((size_t)it * N + col0 + vec) * n_pix;
   float2 r[N2];
+  {
+    const int row0 = lane + N1 * LO - P::OFF;   // pupil row of register LO
+    const float2 *g = gy + (size_t)m * n_pix + row0;
+    const float2 *w = cx + row0;
+    float2 e[NR];
+    bool ok[NR];
 #pragma unroll
-  for (int n2 = 0; n2 < N2; ++n2) r[n2] = make_float2(0.f, 0.f);
-  if (lane < N1) {
-    if constexpr (GEN) {
-      const float2 *g = gy + (size_t)m * n_pix;
+    for (int h = 0; h < NR; ++h) {
+      const int row = row0 + N1 * h;
+      ok[h] = lane < N1 &&
+              (P::ALIGNED || ((h > 0 || row >= 0) && (h < NR - 1 || row < n_pix)));
+      e[h] = ok[h] ? ld_stream2(w + N1 * h) : make_float2(0.f, 0.f);
+    }
 #pragma unroll
-      for (int n2 = 0; n2 < N2; ++n2) {
-        const int row = lane + N1 * n2 - off;                // pupil row
-        if (row >= 0 && row < n_pix) {
-          if constexpr (S::WIDE)
-            r[n2] = cmul(ld_stream2(cx + row), s_gy[row]);
-          else
-            r[n2] = cmul(ld_stream2(cx + row), __ldg(g + row));
-        }
-      }
-    } else {
-      const float2 *g = gy + (size_t)m * n_pix + lane;   // pupil row lane + N1 h
-      const float2 *w = cx + lane;
-      float2 e[QH];
-#pragma unroll
-      for (int h = 0; h < QH; ++h) e[h] = ld_stream2(w + N1 * h);
-#pragma unroll
-      for (int h = 0; h < QH; ++h) r[Q0 + h] = cmul(e[h], __ldg(g + N1 * h));
+    for (int h = 0; h < NR; ++h) {
+      if constexpr (S::WIDE)
+        r[LO + h] = ok[h] ? cmul(e[h], s_gy[row0 + N1 * h]) : make_float2(0.f, 0.f);
+      else
+        r[LO + h] = ok[h] ? cmul(e[h], __ldg(g + N1 * h)) : make_float2(0.f, 0.f);
     }
   }
   float2 *col = s_tile + vec * CS;   // this vector's exchange buffer
-  RegDFT<N2, false>::run(r);
+  RegDFTZ<N2, false, P::NZ>::run(r);
   if (lane < N1) {
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) col[k2 * S1 + lane] = cmulc(r[k2], __ldg(twA + k2 * N1 + lane));
@@ -746,6 +760,19 @@ __global__ void __launch_bounds__(256) k_bin_reduce(const float *__restrict__ pa
 
 constexpr int kColsTile = 8;
 
+// f(integral_constant<int, pad>) for the paddings the two-pass kernels of a
+// split are built for: those that divide N, pad 2 only with N2 % 4 == 0 (the
+// plan refuses the others).
+template <int N1, int N2, class F> static void for_pad(int pad, F &&f) {
+  constexpr int N = N1 * N2;
+  if constexpr (N2 % 4 == 0)
+    if (pad == 2) f(std::integral_constant<int, 2>{});
+  if constexpr (N % 3 == 0)
+    if (pad == 3) f(std::integral_constant<int, 3>{});
+  if constexpr (N % 4 == 0)
+    if (pad == 4) f(std::integral_constant<int, 4>{});
+}
+
 template <int N1, int N2>
 static int configure(PwfsPlan *p) {
   using S = Split<N1, N2>;
@@ -806,22 +833,20 @@ static int configure(PwfsPlan *p) {
     // factors, after a 16-byte boundary)
     p->smemK = ((size_t)tc * p->csK + (S::WIDE ? 1 + p->n_pix : 0)) * sizeof(float2);
     if (p->smemK <= 227 * 1024 && S::N % tc == 0) {
-      if constexpr (S::WIDE) {
-        // general-offset loads only (N2 % 4 != 0 or pad != 2), tiles of up to 128 threads
-        if ((s = ensure_dynamic_smem((const void *)k_rowfilt<N1, N2, true>, p->smemR)) ||
-            (s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, 256, true>, p->smemK)))
-          return s;
-      } else {
-        if ((s = ensure_dynamic_smem((const void *)k_rowfilt<N1, N2>, p->smemR)) ||
-            (s = ensure_dynamic_smem((const void *)k_rowfilt<N1, N2, true>, p->smemR)) ||
-            (s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2>, p->smemK)) ||
-            (s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, 160>, p->smemK)) ||
-            (s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, 256, true>, p->smemK)) ||
-            (s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, 160, true>, p->smemK)) ||
-            (s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, 352>, p->smemK)) ||
-            (s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, 352, true>, p->smemK)))
-          return s;
-      }
+      s = SPECULA_OK;
+      for_pad<N1, N2>(p->pad, [&](auto pc) {
+        constexpr int PAD = decltype(pc)::value;
+        if ((s = ensure_dynamic_smem((const void *)k_rowfilt<N1, N2, PAD>, p->smemR))) return;
+        if constexpr (S::WIDE) {
+          s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 256>, p->smemK);
+        } else if (!(s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 256>,
+                                             p->smemK)) &&
+                   !(s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 160>,
+                                             p->smemK))) {
+          s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 352>, p->smemK);
+        }
+      });
+      if (s) return s;
       p->two_ok = true;
     }
   }
@@ -856,45 +881,37 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
       field_done = b1;
     }
     dim3 gR((Np + vpc - 1) / vpc, (nj + p->ka - 1) / p->ka);
-    const int off = (S::N - Np) / 2;                // the pupil's padded offset
-    const bool gen = p->pad != 2 || N2 % 4 != 0;   // general-offset loads
-#define SPECULA_ROWFILT(GEN_)                                                                  \
-  SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_ROWFILT, st,                                              \
-                 k_rowfilt<N1, N2, GEN_><<<gR, p->blockR, p->smemR, st>>>(                     \
-                     p->field.as<float2>(), p->gx.as<float2>(), p->twA.as<float2>(),           \
-                     p->twB.as<float2>(), p->mask.as<float2>(), p->rows.as<float2>(), Np, nc,  \
-                     p->nbw, j0, nj, p->ka, off, s0))
-#define SPECULA_COLFILT(MAXT_, GEN_)                                                           \
+    dim3 gK(S::N / tc, 2 * nj);
+    int s = SPECULA_EUNSUPPORTED;
+    for_pad<N1, N2>(p->pad, [&](auto pc) {
+      constexpr int PAD = decltype(pc)::value;
+      s = [&]() -> int {
+        SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_ROWFILT, st,
+                       k_rowfilt<N1, N2, PAD><<<gR, p->blockR, p->smemR, st>>>(
+                           p->field.as<float2>(), p->gx.as<float2>(), p->twA.as<float2>(),
+                           p->twB.as<float2>(), p->mask.as<float2>(), p->rows.as<float2>(), Np,
+                           nc, p->nbw, j0, nj, p->ka, s0));
+#define SPECULA_COLFILT(MAXT_)                                                                 \
   SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_COLFILT, st,                                              \
-                 k_colfilt_bin<N1, N2, MAXT_, GEN_><<<gK, p->blockK, p->smemK, st>>>(          \
+                 k_colfilt_bin<N1, N2, PAD, MAXT_><<<gK, p->blockK, p->smemK, st>>>(           \
                      p->rows.as<float2>(), p->gy.as<float2>(), p->twA.as<float2>(),            \
                      p->twB.as<float2>(), p->mask.as<float2>(), p->part.as<float>(), Np, p->fp, \
-                     p->fq, scale, p->n_mod, nc, p->nbw, j0, p->csK, off, s0))
-    dim3 gK(S::N / tc, 2 * nj);
-    const bool k160 = S::G == 32 && p->blockK <= 160;
-    if constexpr (S::WIDE) {
-      SPECULA_ROWFILT(true);   // the plan refuses pad 2 for N2 % 4 != 0; wide tiles <= 128
-      SPECULA_COLFILT(256, true);
-    } else {
-      if (gen)
-        SPECULA_ROWFILT(true);
-      else
-        SPECULA_ROWFILT(false);
-      if (p->blockK > 256 && gen)     // tiles of fractional detector pixels
-        SPECULA_COLFILT(352, true);
-      else if (p->blockK > 256)
-        SPECULA_COLFILT(352, false);
-      else if (k160 && gen)
-        SPECULA_COLFILT(160, true);
-      else if (k160)
-        SPECULA_COLFILT(160, false);
-      else if (gen)
-        SPECULA_COLFILT(256, true);
-      else
-        SPECULA_COLFILT(256, false);
-    }
-#undef SPECULA_ROWFILT
+                     p->fq, scale, p->n_mod, nc, p->nbw, j0, p->csK, s0))
+        if constexpr (S::WIDE) {
+          SPECULA_COLFILT(256);   // wide tiles <= 128 threads
+        } else {
+          if (p->blockK > 256)    // tiles of fractional detector pixels
+            SPECULA_COLFILT(352);
+          else if (S::G == 32 && p->blockK <= 160)
+            SPECULA_COLFILT(160);
+          else
+            SPECULA_COLFILT(256);
+        }
 #undef SPECULA_COLFILT
+        return SPECULA_OK;
+      }();
+    });
+    if (s) return s;
     const int complete = (j0 + nj) / nc - 1;
     if (complete > det_done) {
       dim3 gD((nd * nd + 255) / 256, complete - det_done);
