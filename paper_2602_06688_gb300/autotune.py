@@ -16,9 +16,9 @@ def cache_path():
         os.path.expanduser("~"), ".cache", "specula_gb300", "tiles.json")
 
 
-# bumped whenever the kernels' best tiling can change (v5: the two-pass form's
-# column-major slot blocks and 128-thread row filter)
-_VERSION = "v5"
+# bumped whenever the kernels' best tiling can change (v6: the two-pass form's
+# transforms packed several to a warp, zero inputs left out)
+_VERSION = "v6"
 
 
 def _key(device_name, pupil, pwfs, n_batch):

@@ -98,15 +98,18 @@ struct PwfsPlan {
   int slot_lo = 0;      // cosine slots [slot_lo, slot_hi) imaged (slot_hi < 0: all)
   int slot_hi = -1;
   bool two_ok;          // the two-pass form fits this geometry
-  int blockR, blockK;   // two-pass blocks (K: TC columns x G lanes)
+  int G = 32;           // lanes per transform of the split N1 x N2
+  int M1 = 0, M2 = 0;   // the two-pass form's split of N
+  int blockR, blockK;   // two-pass blocks
   size_t smemR, smemK;
-  int csK = 0;                      // column stride of the column-pass tile (complex)
+  int tcK = 0;          // columns of a column-pass tile
   // a detector pixel is fp / fq grid pixels (N / (pad n_sub) in lowest
   // terms; fq = 1: fp x fp binning, else area-weighted rebinning)
   int fp = 1, fq = 1;
   DevBuf gx, gy;        // [n_mod][n_pix] float2: tilt x pre-phase (x and y parts)
   DevBuf mask;          // [N] float2: pyramid mask factor per axis, x (1/N)
   DevBuf twA, twB;      // [N] float2: inter-step twiddles (cos, sin)
+  DevBuf tpA, tpB;      // the same for the two-pass form's split
   DevBuf field;         // [nbw][n_pix][n_pix] float2: E = amp exp(i phase)
   DevBuf rows;          // [chunk][n_pix][N] float2: after the row transform
   DevBuf cols;          // [chunk][N][N] float2: after the column pass (three-pass form)

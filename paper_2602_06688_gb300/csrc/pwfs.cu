@@ -354,30 +354,72 @@ __global__ void __launch_bounds__(256, 2) k_rows_inv_part(
 // into registers.  The inverse row transform's output phase depends
 // on x only and vanishes in |.|^2.
 
-template <int N1, int N2> struct RowFiltCfg {
+// A warp runs P = 32 / N1 transforms side by side: in the outer stages lane
+// (p, n1) = (lane / N1, lane % N1) holds N2 values of transform p, in the
+// middle stage lane (c, k2) = (lane / N2, lane % N2) holds N1 values of
+// transform PB i + c, i = 0 .. IT-1.  So 320 = 10 x 32 keeps 30 of 32 lanes
+// busy in the outer stages and all in the middle one (as 20 x 16 with a warp
+// per transform: 20 and 16), 128 = 8 x 16 all.  XS: stride (complex) of the
+// exchange buffers; with several transforms per warp XS = N1 (mod 16) puts
+// the lanes of an outer stage on consecutive banks, else it is odd.
+template <int N1, int N2> struct Pack {
   using S = Split<N1, N2>;
-  static constexpr int XBF =
-      S::WIDE ? S::XW : (N2 * S::S1 > N1 * S::S2 ? N2 * S::S1 : N1 * S::S2);
-  static_assert(S::N <= XBF, "a row fits its vector's exchange buffer");
+  static constexpr int P = 32 / N1;
+  static constexpr int PB = N2 <= 32 ? 32 / N2 : 1;
+  static constexpr int IT = (P + PB - 1) / PB;
+  static constexpr bool FULL = PB * N2 == 32 && IT * PB == P;   // no idle lane in the middle
+  static constexpr int base = S::WIDE ? S::XW : imax3(S::N, N2 * S::S1, N1 * S::S2);
+  static constexpr int XS = P > 1 ? base + ((N1 - base) % 16 + 16) % 16 : (base | 1);
+  // the row pass: a one-transform warp's buffer stays even (16-byte loads)
+  static constexpr int XSR = P > 1 ? XS : base;
+  static_assert(S::N <= base, "a transform fits its exchange buffer");
 };
+
+// Middle stage of a warp's P transforms (buffers at wb, wb + stride, ...):
+// N1-point DFT, mask, inverse, twiddle of the swapped split, in place.
+template <int N1, int N2, int STRIDE>
+__device__ __forceinline__ void packed_mid(float2 *wb, const float2 *__restrict__ mask,
+                                           const float2 *__restrict__ twB, int lane) {
+  using S = Split<N1, N2>;
+  using K = Pack<N1, N2>;
+  const int k2 = lane % N2;
+#pragma unroll
+  for (int i = 0; i < K::IT; ++i) {
+    const int c = i * K::PB + lane / N2;
+    const bool act = K::FULL || (lane < K::PB * N2 && c < K::P);
+    float2 *xb = wb + min(c, K::P - 1) * STRIDE;   // idle lanes repeat another's work
+    float2 r2[N1];
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) r2[n1] = xb[k2 * S::S1 + n1];
+    RegDFT<N1, false>::run(r2);
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) r2[k1] = cmul(r2[k1], __ldg(mask + N2 * k1 + k2));
+    RegDFT<N1, true>::run(r2);
+    __syncwarp();
+    if (act) {
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1)
+        xb[k1 * S::S2 + k2] = cmul(r2[k1], __ldg(twB + k1 * N2 + k2));
+    }
+  }
+}
 
 // Points m and n_mod - m share cos(theta), hence the x factor of the tilt;
 // their y factors are constant along a row and commute with the row filter.
 // So the row filter runs once per distinct cosine ("slot" c = 0 .. nc-1,
 // representative m = c) without the y factor, and the column pass applies
 // each item's own y factor gy[m][row] to its input.
-// R: grid (ceil(n_pix / VPC), ceil(n_slots / ka)); block VPC * G threads;
-// writes rows_out[slot][x][row].
+// R: grid (ceil(n_pix / (warps P)), ceil(n_slots / ka)); writes rows_out[slot][x][row].
 // PAD: the padding N / n_pix.  The pupil sits at padded offset PadRegs::OFF,
 // so only registers LO .. HI of a lane can be non-zero: the others are neither
 // loaded nor added (RegDFTZ).  With pad 2 and N2 % 4 == 0 the pupil is exactly
 // registers N2/4 .. 3 N2/4 of every lane; otherwise each lane checks its first
 // and last ones.
-// One-warp transforms (G = 32) run four warps per CTA, five CTAs per SM at
-// 96 registers (four rows per CTA: the transposed output goes out as whole
-// 32-byte sectors), and reload the field row for every slot (caching it
+// Splits with up to 32 values per lane run four warps per CTA, five CTAs per
+// SM at 96 registers (4 P rows per CTA: the transposed output goes out as
+// whole 32-byte sectors), and reload the field row for every slot (caching it
 // across slots needs 32 more registers: spills at that bound); smaller
-// transforms run 256 threads, two CTAs per SM, with the cached row; wide
+// ones (N2 <= 16) run 256 threads, two CTAs per SM, with the cached row; wide
 // splits run 128-thread CTAs (bounded for up to 256 threads, one CTA per SM,
 // so that their 50-point transforms keep their registers).
 template <int N1, int N2, int PAD> struct PadRegs {
@@ -390,9 +432,9 @@ template <int N1, int N2, int PAD> struct PadRegs {
 
 template <int N1, int N2> struct RowFiltLaunch {
   using S = Split<N1, N2>;
-  static constexpr int threads = S::WIDE ? 256 : (S::G == 32 ? 128 : 256);
-  static constexpr int min_blocks = S::WIDE ? 1 : (S::G == 32 ? 5 : 2);
-  static constexpr bool reload = S::G == 32;
+  static constexpr int threads = S::WIDE ? 256 : (N2 > 16 ? 128 : 256);
+  static constexpr int min_blocks = S::WIDE ? 1 : (N2 > 16 ? 5 : 2);
+  static constexpr bool reload = N2 > 16;
 };
 template <int N1, int N2, int PAD>
 __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
@@ -403,20 +445,24 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
     int slot0, int n_slots, int ka, int s0) {
   using S = Split<N1, N2>;
   using P = PadRegs<N1, N2, PAD>;
-  constexpr int N = S::N, G = S::G, S1 = S::S1, S2 = S::S2;
+  using K = Pack<N1, N2>;
+  constexpr int N = S::N, S1 = S::S1, S2 = S::S2;
   constexpr int LO = P::LO, NR = P::HI - P::LO;
-  extern __shared__ float2 smem[];
-  const int vpc = blockDim.x / G;
-  const int vec = threadIdx.x / G, lane = threadIdx.x % G;
-  constexpr int XBF = RowFiltCfg<N1, N2>::XBF;
-  float2 *xb = smem + vec * XBF;
+  extern __shared__ __align__(16) float2 smem[];
+  const int vpc = blockDim.x / 32 * K::P;   // rows per CTA
+  const int wlane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int pa = wlane / N1, lane = wlane % N1;
+  const bool outer = pa < K::P;   // this lane takes part in the outer stages
+  const int vec = warp * K::P + (outer ? pa : 0);
+  constexpr int XBF = K::XSR;
+  float2 *xb = smem + vec * XBF, *wb = smem + warp * K::P * XBF;
   // where vector v's output row sits in its buffer: 4 v complex in, as far
   // as the buffer's slack allows, and even, so that with an even XBF two
   // adjacent columns of a row are one aligned 16-byte load
   auto row_tile_off = [](int v) { return min(4 * v, (XBF - N) & ~1); };
-  const int j = blockIdx.x * vpc + vec;
-  const bool row_ok = j < n_pix;
-  const bool in_lane = row_ok && lane < N1;
+  // lanes that take no part and rows past the pupil repeat valid ones; their
+  // values are not stored
+  const int j = min(blockIdx.x * vpc + vec, n_pix - 1);
   // the pupil column of register LO + h is lane + N1 (LO + h) - OFF
   const auto in_pupil = [&](int h) {
     const int i = lane + N1 * (LO + h) - P::OFF;
@@ -431,13 +477,13 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
     if (it >= n_slots) break;
     const int gi = slot0 + it;
     const int b = gi / nc, c = s0 + (gi - b * nc);   // nc slots per element from s0
-    const float2 *src = field + ((size_t)(b % nbw) * n_pix + (row_ok ? j : 0)) * n_pix +
+    const float2 *src = field + ((size_t)(b % nbw) * n_pix + j) * n_pix +
                         (lane + N1 * LO - P::OFF);
     if constexpr (!kReload) {
       if (b != cur_b) {
         cur_b = b;
 #pragma unroll
-        for (int h = 0; h < NR; ++h) e[h] = in_lane ? src[N1 * h] : make_float2(0.f, 0.f);
+        for (int h = 0; h < NR; ++h) e[h] = src[N1 * h];
       }
     }
     // forward row transform, pruned input (standard split)
@@ -448,57 +494,33 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
 #pragma unroll
       for (int h = 0; h < NR; ++h) {
         if constexpr (kReload)
-          f[h] = in_lane && in_pupil(h) ? src[N1 * h] : make_float2(0.f, 0.f);
+          f[h] = in_pupil(h) ? src[N1 * h] : make_float2(0.f, 0.f);
         else
           f[h] = e[h];
       }
 #pragma unroll
       for (int h = 0; h < NR; ++h)
-        r[LO + h] = in_lane && in_pupil(h) ? cmul(f[h], __ldg(g + N1 * h)) : make_float2(0.f, 0.f);
+        r[LO + h] = in_pupil(h) ? cmul(f[h], __ldg(g + N1 * h)) : make_float2(0.f, 0.f);
     }
     RegDFTZ<N2, false, P::NZ>::run(r);
     __syncwarp();
-    if (lane < N1) {
+    if (outer) {
 #pragma unroll
       for (int k2 = 0; k2 < N2; ++k2) xb[k2 * S1 + lane] = cmulc(r[k2], __ldg(twA + k2 * N1 + lane));
     }
     __syncwarp();
     float2 *x3 = xb;   // input of the last stage
+    // the x mask between the forward and the inverse transform (swapped split)
     if constexpr (S::WIDE) {
       x3 = xb + N2 * S1;
-      wide_mid<N1, N2>(xb, x3, mask, twB, lane);
+      wide_mid<N1, N2>(xb, x3, mask, twB, wlane);
     } else {
-      float2 r2[N1];
-      if (lane < N2) {
-#pragma unroll
-        for (int n1 = 0; n1 < N1; ++n1) r2[n1] = xb[lane * S1 + n1];
-      } else {
-#pragma unroll
-        for (int n1 = 0; n1 < N1; ++n1) r2[n1] = make_float2(0.f, 0.f);
-      }
-      RegDFT<N1, false>::run(r2);
-      // x mask, then the inverse row transform (swapped split)
-      if (lane < N2) {
-#pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) r2[k1] = cmul(r2[k1], __ldg(mask + N2 * k1 + lane));
-      }
-      RegDFT<N1, true>::run(r2);
-      __syncwarp();
-      if (lane < N2) {
-#pragma unroll
-        for (int k2 = 0; k2 < N1; ++k2)
-          xb[k2 * S2 + lane] = cmul(r2[k2], __ldg(twB + k2 * N2 + lane));
-      }
+      packed_mid<N1, N2, XBF>(wb, mask, twB, wlane);
     }
     __syncwarp();
     float2 r3[N2];
-    if (lane < N1) {
 #pragma unroll
-      for (int n1 = 0; n1 < N2; ++n1) r3[n1] = x3[lane * S2 + n1];
-    } else {
-#pragma unroll
-      for (int n1 = 0; n1 < N2; ++n1) r3[n1] = make_float2(0.f, 0.f);
-    }
+    for (int n1 = 0; n1 < N2; ++n1) r3[n1] = x3[lane * S2 + n1];
     RegDFT<N2, true>::run(r3);
     // The slot's block is column-major (rows_out[it][x][row]), so that the
     // column pass loads a column coalesced.  Each vector puts its row in
@@ -506,7 +528,7 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
     // bank conflicts), and the CTA writes one run of vpc rows per column x,
     // as 16-byte row pairs where the rows allow.
     __syncwarp();   // this vector's last-stage loads are done
-    if (lane < N1) {
+    if (outer) {
 #pragma unroll
       for (int k1 = 0; k1 < N2; ++k1) xb[N1 * k1 + lane + row_tile_off(vec)] = r3[k1];   // x = N1 k1 + lane
     }
@@ -516,12 +538,13 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
       float2 *dst = rows_out + ((size_t)it * N) * n_pix + j0;
       if ((vpc & 1) == 0 && (n_pix & 1) == 0) {
         const int hp = vpc / 2, h = threadIdx.x % hp;   // rows 2h and 2h + 1
-        if (j0 + 2 * h < n_pix) {                       // n_pix even: both rows exist
+        const int xt = threadIdx.x / hp, nxt = blockDim.x / hp;
+        if (j0 + 2 * h < n_pix && xt < nxt) {           // n_pix even: both rows exist
           const float2 *ta = smem + (2 * h) * XBF + row_tile_off(2 * h);
           const float2 *tb = smem + (2 * h + 1) * XBF + row_tile_off(2 * h + 1);
           if constexpr (XBF % 2 == 0) {
             // columns x and x + 1 of both rows: two 16-byte loads, two stores
-            for (int x = 2 * (threadIdx.x / hp); x < N; x += 4 * G) {
+            for (int x = 2 * xt; x < N; x += 2 * nxt) {
               const float4 a = *reinterpret_cast<const float4 *>(ta + x);
               const float4 c = *reinterpret_cast<const float4 *>(tb + x);
               *reinterpret_cast<float4 *>(dst + (size_t)x * n_pix + 2 * h) =
@@ -530,7 +553,7 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
                   make_float4(a.z, a.w, c.z, c.w);
             }
           } else {
-            for (int x = threadIdx.x / hp; x < N; x += 2 * G) {
+            for (int x = xt; x < N; x += nxt) {
               const float2 a = ta[x], c = tb[x];
               *reinterpret_cast<float4 *>(dst + (size_t)x * n_pix + 2 * h) =
                   make_float4(a.x, a.y, c.x, c.y);
@@ -538,10 +561,10 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
           }
         }
       } else {
-        const int v = threadIdx.x % vpc;
-        if (j0 + v < n_pix) {
+        const int v = threadIdx.x % vpc, xt = threadIdx.x / vpc, nxt = blockDim.x / vpc;
+        if (j0 + v < n_pix && xt < nxt) {
           const float2 *tv = smem + v * XBF + row_tile_off(v);
-          for (int x = threadIdx.x / vpc; x < N; x += G) dst[(size_t)x * n_pix + v] = tv[x];
+          for (int x = xt; x < N; x += nxt) dst[(size_t)x * n_pix + v] = tv[x];
         }
       }
     }
@@ -549,23 +572,16 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
   }
 }
 
-// K: per tile of TC = blockDim.x / G columns (a multiple of the bin side),
-// read from rows_in[slot][x][row]: the item's y tilt, column filter,
+// K: per tile of up to tc columns (whole detector pixels, at most P per
+// warp), read from rows_in[slot][x][row]: the item's y tilt, column filter,
 // |.|^2 / n_mod, b x b bins ->
-// part[b % nbw][m][ybin][xbin].  grid (N / TC, 2 n_slots): y = 2 p + w is
+// part[b % nbw][m][ybin][xbin].  grid (ceil(N / tc), 2 n_slots): y = 2 p + w is
 // item m = c (w = 0) or m = n_mod - c (w = 1, when distinct) of slot p.
-// Column stride CS (complex) of the exchange buffers: at least the exchange
-// buffer of a column, odd.
-template <int N1, int N2> struct ColFiltCfg {
-  using S = Split<N1, N2>;
-  static constexpr int base = S::WIDE ? S::XW : imax3(S::N, N2 * S::S1, N1 * S::S2);
-  static int stride(int) { return base | 1; }
-};
-
-// One-warp columns in tiles of at most 160 threads (five columns for the
-// 39 m pupil's bin side 5) take the variant bounded at 160 threads x 4 CTAs
-// per SM, the occupancy that 80 registers per thread gave them already:
-// 96 registers per thread, so the twiddle loads can be issued earlier.
+//
+// Tiles of at most 160 threads (five columns for the 39 m pupil's bin side 5,
+// twelve for the 8 m pupil's 4) take the variant bounded at 160 threads x 4
+// CTAs per SM: 96 registers per thread, so the twiddle loads can be issued
+// earlier.
 template <int N1, int N2, int PAD, int MAXT>
 __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
                                               ? 1
@@ -574,26 +590,29 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
     const float2 *__restrict__ rows_in, const float2 *__restrict__ gy,
     const float2 *__restrict__ twA, const float2 *__restrict__ twB,
     const float2 *__restrict__ mask, float *__restrict__ part, int n_pix, int fp, int fq,
-    float scale, int n_mod, int nc, int nbw, int slot0, int CS, int s0) {
+    float scale, int n_mod, int nc, int nbw, int slot0, int tc, int s0) {
   using S = Split<N1, N2>;
   using P = PadRegs<N1, N2, PAD>;
-  constexpr int N = S::N, G = S::G, S1 = S::S1, S2 = S::S2;
+  using K = Pack<N1, N2>;
+  constexpr int N = S::N, S1 = S::S1, S2 = S::S2, CS = K::XS;
   constexpr int LO = P::LO, NR = P::HI - P::LO;
   extern __shared__ __align__(16) float2 smem_k[];
   float2 *s_tile = smem_k;
-  const int TC = blockDim.x / G;
   const int it = blockIdx.y >> 1;              // slot within the chunk
   const int gs = slot0 + it;
   const int b = gs / nc, cslot = s0 + (gs - b * nc);   // nc slots per element from s0
   const int m = (blockIdx.y & 1) ? n_mod - cslot : cslot;
   if ((blockIdx.y & 1) && (cslot == 0 || 2 * cslot == n_mod)) return;   // no second item
-  const int col0 = blockIdx.x * TC;
-  const int vec = threadIdx.x / G, lane = threadIdx.x % G;
+  const int col0 = blockIdx.x * tc, ncol = min(tc, N - col0);
+  const int wlane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int pa = wlane / N1, lane = wlane % N1;
+  const bool outer = pa < K::P;   // this lane takes part in the outer stages
+  const int vec = warp * K::P + (outer ? pa : 0);
   // wide splits stage the item's y factors in shared memory (5% off their
   // column pass; at 960 the factors come through L1 as fast)
   float2 *s_gy = nullptr;
   if constexpr (S::WIDE) {
-    s_gy = s_tile + ((TC * CS + 1) & ~1);   // 16-byte aligned
+    s_gy = s_tile + ((blockDim.x / 32 * CS + 1) & ~1);   // 16-byte aligned
     const float2 *g = gy + (size_t)m * n_pix;
     if ((n_pix & 1) == 0) {
       for (int i = threadIdx.x; 2 * i < n_pix; i += blockDim.x) cp_async16(s_gy + 2 * i, g + 2 * i);
@@ -606,7 +625,9 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
   // this vector's column x = col0 + vec: n_pix contiguous rows of the
   // slot's column-major block, loaded coalesced straight into registers and
   // past L1 (which keeps the twiddle, mask and tilt tables)
-  const float2 *cx = rows_in + ((size_t)it * N + col0 + vec) * n_pix;
+  // (lanes that take no part and columns past the tile repeat valid ones;
+  // their values are not stored, or not binned)
+  const float2 *cx = rows_in + ((size_t)it * N + min(col0 + vec, N - 1)) * n_pix;
   float2 r[N2];
   {
     const int row0 = lane + N1 * LO - P::OFF;   // pupil row of register LO
@@ -617,8 +638,7 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
 #pragma unroll
     for (int h = 0; h < NR; ++h) {
       const int row = row0 + N1 * h;
-      ok[h] = lane < N1 &&
-              (P::ALIGNED || ((h > 0 || row >= 0) && (h < NR - 1 || row < n_pix)));
+      ok[h] = P::ALIGNED || ((h > 0 || row >= 0) && (h < NR - 1 || row < n_pix));
       e[h] = ok[h] ? ld_stream2(w + N1 * h) : make_float2(0.f, 0.f);
     }
 #pragma unroll
@@ -631,7 +651,7 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
   }
   float2 *col = s_tile + vec * CS;   // this vector's exchange buffer
   RegDFTZ<N2, false, P::NZ>::run(r);
-  if (lane < N1) {
+  if (outer) {
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) col[k2 * S1 + lane] = cmulc(r[k2], __ldg(twA + k2 * N1 + lane));
   }
@@ -639,42 +659,18 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
   float2 *x3 = col;   // input of the last stage
   if constexpr (S::WIDE) {
     x3 = col + N2 * S1;
-    wide_mid<N1, N2>(col, x3, mask, twB, lane);
+    wide_mid<N1, N2>(col, x3, mask, twB, wlane);
   } else {
-    float2 r2[N1];
-    if (lane < N2) {
-#pragma unroll
-      for (int n1 = 0; n1 < N1; ++n1) r2[n1] = col[lane * S1 + n1];
-    } else {
-#pragma unroll
-      for (int n1 = 0; n1 < N1; ++n1) r2[n1] = make_float2(0.f, 0.f);
-    }
-    RegDFT<N1, false>::run(r2);
-    if (lane < N2) {
-#pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1) r2[k1] = cmul(r2[k1], __ldg(mask + N2 * k1 + lane));
-    }
-    RegDFT<N1, true>::run(r2);
-    __syncwarp();
-    if (lane < N2) {
-#pragma unroll
-      for (int k2 = 0; k2 < N1; ++k2)
-        col[k2 * S2 + lane] = cmul(r2[k2], __ldg(twB + k2 * N2 + lane));
-    }
+    packed_mid<N1, N2, CS>(s_tile + warp * K::P * CS, mask, twB, wlane);
   }
   __syncwarp();
   float2 r3[N2];
-  if (lane < N1) {
 #pragma unroll
-    for (int n1 = 0; n1 < N2; ++n1) r3[n1] = x3[lane * S2 + n1];
-  } else {
-#pragma unroll
-    for (int n1 = 0; n1 < N2; ++n1) r3[n1] = make_float2(0.f, 0.f);
-  }
+  for (int n1 = 0; n1 < N2; ++n1) r3[n1] = x3[lane * S2 + n1];
   RegDFT<N2, true>::run(r3);
   __syncwarp();
   float *colI = reinterpret_cast<float *>(col);   // this column's intensity, y = N1 k1 + lane
-  if (lane < N1) {
+  if (outer) {
 #pragma unroll
     for (int k1 = 0; k1 < N2; ++k1)
       colI[N1 * k1 + lane] = (r3[k1].x * r3[k1].x + r3[k1].y * r3[k1].y) * scale;
@@ -687,8 +683,8 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
     // rebinning): output pixel o covers [o fp, (o + 1) fp) and grid pixel i
     // covers [i fq, (i + 1) fq) in units of 1 / fq; the weight is their
     // overlap, an integer, and the sum is divided by fq^2 once.  The tile's
-    // TC = k fp columns hold exactly its k fq output columns.
-    const int nd = N * fq / fp, nxo = TC / fp * fq, xo0 = col0 / fp * fq;
+    // ncol = k fp columns hold exactly its k fq output columns.
+    const int nd = N * fq / fp, nxo = ncol / fp * fq, xo0 = col0 / fp * fq;
     const float inv = 1.0f / (float)(fq * fq);
     for (int q = threadIdx.x; q < nd * nxo; q += blockDim.x) {
       const int yo = q / nxo, X = xo0 + (q - yo * nxo);
@@ -706,7 +702,7 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
     }
     return;
   }
-  const int bsz = fp, nd = N / bsz, nbx = TC / bsz;
+  const int bsz = fp, nd = N / bsz, nbx = ncol / bsz;
   if (bsz == 5 && nbx == 1) {
     // the 39 m pupil's 5 x 5 bins, one bin column per tile: unrolled sums
     for (int yb = threadIdx.x; yb < nd; yb += blockDim.x) {
@@ -786,6 +782,7 @@ static int configure(PwfsPlan *p) {
     }
     p->fp = S::N / a;
     p->fq = nd / a;
+    p->G = S::G;
   }
   int s;
   if constexpr (S::WIDE) {
@@ -811,45 +808,55 @@ static int configure(PwfsPlan *p) {
         (s = ensure_dynamic_smem((const void *)k_rows_inv_part<N1, N2>, p->smemC)))
       return s;
   }
-  // two-pass form: column tiles of TC = k fp grid columns (k fq detector
-  // columns, so every detector pixel lies in one CTA), k the largest divisor
-  // of pad n_sub / fq with TC G <= 256 threads (352 where a detector pixel
-  // is a fraction of grid pixels: the SOUL example's 11-column tiles)
-  // (wide splits: 128-thread CTAs, two per SM within the register budget of
-  // their 50-point transforms, so one CTA's barriers do not idle the SM)
+  return SPECULA_OK;
+}
+
+// Two-pass form (its own split of N: N1, N2): column tiles of whole detector
+// pixels, so every detector pixel lies in one CTA.  The number of warps is the
+// one that leaves the fewest lanes idle (a tile narrower than its warps, a
+// last tile that is not full), up to five of 32-value lanes and eight of
+// shorter ones (eleven where a detector pixel is a fraction of grid pixels:
+// the SOUL example's 11-column tiles; wide splits four, so that two CTAs of
+// their 50-point transforms share an SM's registers).
+template <int N1, int N2>
+static int configure_two(PwfsPlan *p) {
+  using S = Split<N1, N2>;
+  using K = Pack<N1, N2>;
+  int s = SPECULA_OK;
   p->two_ok = false;
   p->blockR = S::WIDE ? 128 : RowFiltLaunch<N1, N2>::threads;
-  p->smemR = (size_t)(p->blockR / S::G) * RowFiltCfg<N1, N2>::XBF * sizeof(float2);
-  const int ndq = p->pad * p->n_sub / p->fq;
-  const int maxt = S::WIDE ? 128 : (p->fq == 1 ? 256 : 352);
-  int k = 0;
-  for (int d = 1; d <= ndq; ++d)
-    if (ndq % d == 0 && d * p->fp * S::G <= maxt) k = d;
-  if (k > 0 && p->smemR <= 227 * 1024) {
-    const int tc = k * p->fp;
-    p->blockK = tc * S::G;
-    p->csK = ColFiltCfg<N1, N2>::stride(tc);
-    // the tile's exchange buffers (wide splits: and the item's n_pix y
-    // factors, after a 16-byte boundary)
-    p->smemK = ((size_t)tc * p->csK + (S::WIDE ? 1 + p->n_pix : 0)) * sizeof(float2);
-    if (p->smemK <= 227 * 1024 && S::N % tc == 0) {
-      s = SPECULA_OK;
-      for_pad<N1, N2>(p->pad, [&](auto pc) {
-        constexpr int PAD = decltype(pc)::value;
-        if ((s = ensure_dynamic_smem((const void *)k_rowfilt<N1, N2, PAD>, p->smemR))) return;
-        if constexpr (S::WIDE) {
-          s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 256>, p->smemK);
-        } else if (!(s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 256>,
-                                             p->smemK)) &&
-                   !(s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 160>,
-                                             p->smemK))) {
-          s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 352>, p->smemK);
-        }
-      });
-      if (s) return s;
-      p->two_ok = true;
-    }
+  p->smemR = (size_t)(p->blockR / 32 * K::P) * K::XSR * sizeof(float2);
+  const int fit = (p->fp + K::P - 1) / K::P;   // warps that hold one detector pixel
+  const int most = S::WIDE ? 4 : (p->fq != 1 ? 11 : std::max(fit, N2 >= 32 ? 5 : 8));
+  int best = 0, cost = 0;   // lane columns issued for the N columns of an item
+  for (int w = fit; w <= most; ++w) {
+    const int tc = w * K::P / p->fp * p->fp;
+    const int c = (S::N + tc - 1) / tc * w;
+    if (!best || c <= cost) best = w, cost = c;
   }
+  // a detector pixel's columns at the three-pass split's lanes per transform
+  // fit one CTA: the geometries that the plan takes
+  if (!best || p->fp * p->G > (S::WIDE ? 128 : (p->fq != 1 ? 352 : 256))) return SPECULA_OK;
+  p->tcK = best * K::P / p->fp * p->fp;
+  p->blockK = best * 32;
+  // the tile's exchange buffers (wide splits: and the item's n_pix y factors,
+  // after a 16-byte boundary)
+  p->smemK = ((size_t)best * K::P * K::XS + (S::WIDE ? 1 + p->n_pix : 0)) * sizeof(float2);
+  if (p->smemR > 227 * 1024 || p->smemK > 227 * 1024) return SPECULA_OK;
+  for_pad<N1, N2>(p->pad, [&](auto pc) {
+    constexpr int PAD = decltype(pc)::value;
+    if ((s = ensure_dynamic_smem((const void *)k_rowfilt<N1, N2, PAD>, p->smemR))) return;
+    if constexpr (S::WIDE) {
+      s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 256>, p->smemK);
+    } else if (!(s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 256>,
+                                         p->smemK)) &&
+               !(s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 160>,
+                                         p->smemK))) {
+      s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 352>, p->smemK);
+    }
+  });
+  if (s) return s;
+  p->two_ok = true;
   return SPECULA_OK;
 }
 
@@ -865,8 +872,7 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
   const int s0 = p->slot_lo;
   const int nc = (p->slot_hi < 0 ? p->nc : p->slot_hi) - s0;
   const int total = n_batch * nc;
-  const int vpc = p->blockR / S::G;
-  const int tc = p->blockK / S::G;
+  const int vpc = p->blockR / 32 * Pack<N1, N2>::P;
   const float scale = 1.0f / (float)p->n_mod;
   int field_done = -1, det_done = -1;
   for (int j0 = 0; j0 < total; j0 += p->chunk) {
@@ -881,28 +887,28 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
       field_done = b1;
     }
     dim3 gR((Np + vpc - 1) / vpc, (nj + p->ka - 1) / p->ka);
-    dim3 gK(S::N / tc, 2 * nj);
+    dim3 gK((S::N + p->tcK - 1) / p->tcK, 2 * nj);
     int s = SPECULA_EUNSUPPORTED;
     for_pad<N1, N2>(p->pad, [&](auto pc) {
       constexpr int PAD = decltype(pc)::value;
       s = [&]() -> int {
         SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_ROWFILT, st,
                        k_rowfilt<N1, N2, PAD><<<gR, p->blockR, p->smemR, st>>>(
-                           p->field.as<float2>(), p->gx.as<float2>(), p->twA.as<float2>(),
-                           p->twB.as<float2>(), p->mask.as<float2>(), p->rows.as<float2>(), Np,
+                           p->field.as<float2>(), p->gx.as<float2>(), p->tpA.as<float2>(),
+                           p->tpB.as<float2>(), p->mask.as<float2>(), p->rows.as<float2>(), Np,
                            nc, p->nbw, j0, nj, p->ka, s0));
 #define SPECULA_COLFILT(MAXT_)                                                                 \
   SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_COLFILT, st,                                              \
                  k_colfilt_bin<N1, N2, PAD, MAXT_><<<gK, p->blockK, p->smemK, st>>>(           \
-                     p->rows.as<float2>(), p->gy.as<float2>(), p->twA.as<float2>(),            \
-                     p->twB.as<float2>(), p->mask.as<float2>(), p->part.as<float>(), Np, p->fp, \
-                     p->fq, scale, p->n_mod, nc, p->nbw, j0, p->csK, s0))
+                     p->rows.as<float2>(), p->gy.as<float2>(), p->tpA.as<float2>(),            \
+                     p->tpB.as<float2>(), p->mask.as<float2>(), p->part.as<float>(), Np, p->fp, \
+                     p->fq, scale, p->n_mod, nc, p->nbw, j0, p->tcK, s0))
         if constexpr (S::WIDE) {
           SPECULA_COLFILT(256);   // wide tiles <= 128 threads
         } else {
           if (p->blockK > 256)    // tiles of fractional detector pixels
             SPECULA_COLFILT(352);
-          else if (S::G == 32 && p->blockK <= 160)
+          else if (p->blockK <= 160)
             SPECULA_COLFILT(160);
           else
             SPECULA_COLFILT(256);
@@ -928,7 +934,6 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
 template <int N1, int N2>
 static int run_split(specula_ctx *ctx, PwfsPlan *p, const float *amp, const float *phase,
                      int n_batch, float *det, cudaStream_t st) {
-  if (p->passes == 2) return run_split2<N1, N2>(ctx, p, amp, phase, n_batch, det, st);
   using S = Split<N1, N2>;
   if constexpr (S::WIDE) {
     return SPECULA_EUNSUPPORTED;   // the three-pass kernels hold N2 <= 32
@@ -1070,6 +1075,18 @@ int pwfs_run(specula_ctx *ctx, PwfsPlan *p, const float *amp, const float *phase
   if (p->form == SPECULA_PWFS_FORM_DFTGEMM_BF16 || p->form == SPECULA_PWFS_FORM_DFTGEMM_TF32)
     return pwfs_dftgemm_run(ctx, p, amp, phase, n_batch, det, st);
   if (p->passes == 4) return pwfs_pair_run(ctx, p, amp, phase, n_batch, det, st);
+  if (p->passes == 2) {
+    switch (p->N) {
+      case 64: return run_split2<8, 8>(ctx, p, amp, phase, n_batch, det, st);
+      case 128: return run_split2<8, 16>(ctx, p, amp, phase, n_batch, det, st);
+      case 240: return run_split2<15, 16>(ctx, p, amp, phase, n_batch, det, st);
+      case 320: return run_split2<10, 32>(ctx, p, amp, phase, n_batch, det, st);
+      case 660: return run_split2<30, 22>(ctx, p, amp, phase, n_batch, det, st);
+      case 960: return run_split2<30, 32>(ctx, p, amp, phase, n_batch, det, st);
+      case 1600: return run_split2<32, 50>(ctx, p, amp, phase, n_batch, det, st);
+      default: return SPECULA_EUNSUPPORTED;
+    }
+  }
   switch (p->N) {
     case 64: return run_split<8, 8>(ctx, p, amp, phase, n_batch, det, st);
     case 128: return run_split<8, 16>(ctx, p, amp, phase, n_batch, det, st);
@@ -1139,15 +1156,25 @@ done:
   return status;
 }
 
+// The three-pass form's split, and the two-pass form's: the same but for
+// 320 = 10 x 32, three transforms per warp.
+template <int N1, int N2, int M1 = N1, int M2 = N2>
+static int configure_both(PwfsPlan *p) {
+  p->M1 = M1;
+  p->M2 = M2;
+  const int s = configure<N1, N2>(p);
+  return s ? s : configure_two<M1, M2>(p);
+}
+
 static int configure_for(PwfsPlan *p) {
   switch (p->N) {
-    case 64: return configure<8, 8>(p);
-    case 128: return configure<8, 16>(p);
-    case 240: return configure<15, 16>(p);
-    case 320: return configure<20, 16>(p);
-    case 660: return configure<30, 22>(p);
-    case 960: return configure<30, 32>(p);
-    case 1600: return configure<32, 50>(p);
+    case 64: return configure_both<8, 8>(p);
+    case 128: return configure_both<8, 16>(p);
+    case 240: return configure_both<15, 16>(p);
+    case 320: return configure_both<20, 16, 10, 32>(p);
+    case 660: return configure_both<30, 22>(p);
+    case 960: return configure_both<30, 32>(p);
+    case 1600: return configure_both<32, 50>(p);
     default: return SPECULA_EUNSUPPORTED;
   }
 }
@@ -1168,6 +1195,19 @@ static inline void exp_ipi(long long num, long long den, double *c, double *s) {
   const double a = M_PI * (double)r / (double)den;
   *c = cos(a);
   *s = sin(a);
+}
+
+// inter-step twiddles (cos, sin)(2 pi (a b mod N) / N)
+void pwfs_host_twiddles(int N, int N1, int N2, std::vector<float2> *twA,
+                        std::vector<float2> *twB) {
+  twA->resize(N);
+  twB->resize(N);
+  for (int a = 0; a < N2; ++a)
+    for (int b = 0; b < N1; ++b) {
+      double c, sn;
+      exp_ipi(2LL * ((long long)a * b % N), N, &c, &sn);
+      (*twA)[a * N1 + b] = (*twB)[b * N2 + a] = make_float2((float)c, (float)sn);
+    }
 }
 
 void pwfs_host_tables(int Np, int N, int N1, int N2, int n_mod, double mod_amp, int pup_dist,
@@ -1199,25 +1239,10 @@ void pwfs_host_tables(int Np, int N, int N1, int N2, int n_mod, double mod_amp, 
     exp_ipi(-(long long)pup_dist * a, 2LL * N, &c, &sn);
     mk[k] = make_float2((float)(c / N), (float)(sn / N));
   }
-  // inter-step twiddles (cos, sin)(2 pi (a b mod N) / N)
-  std::vector<float2> ta(N), tb(N);
-  for (int a = 0; a < N2; ++a)
-    for (int b = 0; b < N1; ++b) {
-      double c, sn;
-      exp_ipi(2LL * ((long long)a * b % N), N, &c, &sn);
-      ta[a * N1 + b] = make_float2((float)c, (float)sn);
-    }
-  for (int a = 0; a < N1; ++a)
-    for (int b = 0; b < N2; ++b) {
-      double c, sn;
-      exp_ipi(2LL * ((long long)a * b % N), N, &c, &sn);
-      tb[a * N2 + b] = make_float2((float)c, (float)sn);
-    }
   t->gx = std::move(gx);
   t->gy = std::move(gy);
   t->mask = std::move(mk);
-  t->twA = std::move(ta);
-  t->twB = std::move(tb);
+  pwfs_host_twiddles(N, N1, N2, &t->twA, &t->twB);
 }
 
 int pwfs_plan_build(specula_ctx *ctx, const specula_pupil_desc *pupil,
@@ -1244,6 +1269,10 @@ int pwfs_plan_build(specula_ctx *ctx, const specula_pupil_desc *pupil,
   if ((s = p->mask.upload(mk.data(), mk.size() * sizeof(float2)))) return s;
   if ((s = p->twA.upload(ta.data(), ta.size() * sizeof(float2)))) return s;
   if ((s = p->twB.upload(tb.data(), tb.size() * sizeof(float2)))) return s;
+  std::vector<float2> pa, pb;
+  pwfs_host_twiddles(N, p->M1, p->M2, &pa, &pb);
+  if ((s = p->tpA.upload(pa.data(), pa.size() * sizeof(float2)))) return s;
+  if ((s = p->tpB.upload(pb.data(), pb.size() * sizeof(float2)))) return s;
 
   // Default chunk.  Two-pass form: as many row-filter slots as keep the rows
   // workspace within kRowsBytes, a size that L2 (129 MB) still holds between

@@ -42,6 +42,8 @@ struct PwfsTablesHost {
 };
 void pwfs_host_tables(int Np, int N, int N1, int N2, int n_mod, double mod_amp, int pup_dist,
                       PwfsTablesHost *t);
+void pwfs_host_twiddles(int N, int N1, int N2, std::vector<float2> *twA,
+                        std::vector<float2> *twB);
 bool pwfs_split_for(int N, int *N1, int *N2);
 
 }  // namespace specula
