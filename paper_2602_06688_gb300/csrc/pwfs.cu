@@ -51,10 +51,6 @@ __device__ __forceinline__ void cp_async8(void *smem_dst, const void *gsrc) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"(gsrc) : "memory");
 }
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gsrc) : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
@@ -63,40 +59,6 @@ __device__ __forceinline__ float2 ld_stream2(const float2 *p) {
   float2 v;
   asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
   return v;
-}
-
-// The N1-point middle stage of a wide split (N2 > 32): lane k2 = lane + 32 t
-// (t < NT2) takes column k2 of the exchange xa (xa[k2 S1 + n1]), applies the
-// forward N1-point DFT, the mask factor of frequency N2 k1 + k2, the inverse
-// N1-point DFT and the twiddle of the swapped split, and writes
-// xo[k1 S2 + k2]; xo and xa do not overlap.
-template <int N1, int N2>
-__device__ __forceinline__ void wide_mid(const float2 *xa, float2 *xo,
-                                         const float2 *__restrict__ mask,
-                                         const float2 *__restrict__ twB, int lane) {
-  using S = Split<N1, N2>;
-#pragma unroll 1
-  for (int t = 0; t < S::NT2; ++t) {
-    const int k2 = lane + 32 * t;
-    float2 r2[N1];
-    if (k2 < N2) {
-#pragma unroll
-      for (int n1 = 0; n1 < N1; ++n1) r2[n1] = xa[k2 * S::S1 + n1];
-    } else {
-#pragma unroll
-      for (int n1 = 0; n1 < N1; ++n1) r2[n1] = make_float2(0.f, 0.f);
-    }
-    RegDFT<N1, false>::run(r2);
-    if (k2 < N2) {
-#pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1) r2[k1] = cmul(r2[k1], __ldg(mask + N2 * k1 + k2));
-    }
-    RegDFT<N1, true>::run(r2);
-    if (k2 < N2) {
-#pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1) xo[k1 * S::S2 + k2] = cmul(r2[k1], __ldg(twB + k1 * N2 + k2));
-    }
-  }
 }
 
 // --------------------------------------------------------------------------
@@ -354,52 +316,72 @@ __global__ void __launch_bounds__(256, 2) k_rows_inv_part(
 // into registers.  The inverse row transform's output phase depends
 // on x only and vanishes in |.|^2.
 
-// A warp runs P = 32 / N1 transforms side by side: in the outer stages lane
-// (p, n1) = (lane / N1, lane % N1) holds N2 values of transform p, in the
-// middle stage lane (c, k2) = (lane / N2, lane % N2) holds N1 values of
-// transform PB i + c, i = 0 .. IT-1.  So 320 = 10 x 32 keeps 30 of 32 lanes
-// busy in the outer stages and all in the middle one (as 20 x 16 with a warp
-// per transform: 20 and 16), 128 = 8 x 16 all.  XS: stride (complex) of the
-// exchange buffers; with several transforms per warp XS = N1 (mod 16) puts
-// the lanes of an outer stage on consecutive banks, else it is odd.
+// How a CTA's threads share its transforms.
+// Splits with N1 <= 32: a warp runs P = 32 / N1 transforms side by side: in
+// the outer stages lane (p, n1) = (lane / N1, lane % N1) holds N2 values of
+// transform p, in the middle stage lane (c, k2) = (lane / N2, lane % N2) holds
+// N1 values of transform PB i + c, i = 0 .. IT-1.  So 320 = 10 x 32 keeps 30 of
+// 32 lanes busy in the outer stages and all in the middle one (as 20 x 16 with
+// a warp per transform: 20 and 16), 128 = 8 x 16 all.
+// Square splits with N1 = N2 > 32 (1600 = 40 x 40): thread t holds values t % N1
+// of transform t / N1 in every stage, four transforms on five warps, and the
+// stages are separated by CTA barriers instead of warp ones.  40 values per
+// thread leave 15 warps per SM; as 32 x 50, a warp per transform, the 50-point
+// transforms took 220 registers (8 warps) and the middle stage two lane strides
+// of 50 / 64.
+// XS: stride (complex) of the exchange buffers; where a warp holds lanes of
+// several transforms XS = N1 (mod 16) puts the lanes of an outer stage on
+// consecutive banks, else it is odd.
 template <int N1, int N2> struct Pack {
-  using S = Split<N1, N2>;
-  static constexpr int P = 32 / N1;
-  static constexpr int PB = N2 <= 32 ? 32 / N2 : 1;
+  static constexpr int N = N1 * N2;
+  static constexpr bool CTA = N1 > 32;
+  static constexpr int S1 = N1 | 1, S2 = N2 | 1;   // exchange strides (odd: no conflicts)
+  static constexpr int P = CTA ? 1 : 32 / N1;
+  static constexpr int PB = CTA ? 1 : 32 / N2;
   static constexpr int IT = (P + PB - 1) / PB;
   static constexpr bool FULL = PB * N2 == 32 && IT * PB == P;   // no idle lane in the middle
-  static constexpr int base = S::WIDE ? S::XW : imax3(S::N, N2 * S::S1, N1 * S::S2);
-  static constexpr int XS = P > 1 ? base + ((N1 - base) % 16 + 16) % 16 : (base | 1);
+  static constexpr int base = imax3(N, N2 * S1, N1 * S2);
+  static constexpr bool MANY = CTA || P > 1;
+  static constexpr int XS = MANY ? base + ((N1 - base) % 16 + 16) % 16 : (base | 1);
   // the row pass: a one-transform warp's buffer stays even (16-byte loads)
-  static constexpr int XSR = P > 1 ? XS : base;
-  static_assert(S::N <= base, "a transform fits its exchange buffer");
+  static constexpr int XSR = MANY ? XS : base;
+  static_assert(N2 <= 32 || (CTA && N1 == N2), "wide splits are square");
+  // transforms of a CTA of `threads`
+  static __host__ __device__ constexpr int vecs(int threads) {
+    return CTA ? threads / N1 : threads / 32 * P;
+  }
+  static __device__ __forceinline__ void sync() {
+    if constexpr (CTA) __syncthreads();
+    else __syncwarp();
+  }
 };
 
-// Middle stage of a warp's P transforms (buffers at wb, wb + stride, ...):
+// Middle stage of the CTA's transforms (buffers at sm, sm + STRIDE, ...):
 // N1-point DFT, mask, inverse, twiddle of the swapped split, in place.
 template <int N1, int N2, int STRIDE>
-__device__ __forceinline__ void packed_mid(float2 *wb, const float2 *__restrict__ mask,
-                                           const float2 *__restrict__ twB, int lane) {
-  using S = Split<N1, N2>;
+__device__ __forceinline__ void packed_mid(float2 *sm, const float2 *__restrict__ mask,
+                                           const float2 *__restrict__ twB) {
   using K = Pack<N1, N2>;
-  const int k2 = lane % N2;
+  const int lane = threadIdx.x % 32, k2 = K::CTA ? threadIdx.x % N2 : lane % N2;
 #pragma unroll
   for (int i = 0; i < K::IT; ++i) {
-    const int c = i * K::PB + lane / N2;
-    const bool act = K::FULL || (lane < K::PB * N2 && c < K::P);
-    float2 *xb = wb + min(c, K::P - 1) * STRIDE;   // idle lanes repeat another's work
+    const int c = i * K::PB + lane / N2;   // transform of the warp
+    const bool act = K::CTA || K::FULL || (lane < K::PB * N2 && c < K::P);
+    // idle lanes repeat another's work
+    float2 *xb = sm + (K::CTA ? threadIdx.x / N2
+                              : threadIdx.x / 32 * K::P + min(c, K::P - 1)) * STRIDE;
     float2 r2[N1];
 #pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) r2[n1] = xb[k2 * S::S1 + n1];
+    for (int n1 = 0; n1 < N1; ++n1) r2[n1] = xb[k2 * K::S1 + n1];
     RegDFT<N1, false>::run(r2);
 #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1) r2[k1] = cmul(r2[k1], __ldg(mask + N2 * k1 + k2));
     RegDFT<N1, true>::run(r2);
-    __syncwarp();
+    K::sync();
     if (act) {
 #pragma unroll
       for (int k1 = 0; k1 < N1; ++k1)
-        xb[k1 * S::S2 + k2] = cmul(r2[k1], __ldg(twB + k1 * N2 + k2));
+        xb[k1 * K::S2 + k2] = cmul(r2[k1], __ldg(twB + k1 * N2 + k2));
     }
   }
 }
@@ -419,9 +401,8 @@ __device__ __forceinline__ void packed_mid(float2 *wb, const float2 *__restrict_
 // SM at 96 registers (4 P rows per CTA: the transposed output goes out as
 // whole 32-byte sectors), and reload the field row for every slot (caching it
 // across slots needs 32 more registers: spills at that bound); smaller
-// ones (N2 <= 16) run 256 threads, two CTAs per SM, with the cached row; wide
-// splits run 128-thread CTAs (bounded for up to 256 threads, one CTA per SM,
-// so that their 50-point transforms keep their registers).
+// ones (N2 <= 16) run 256 threads, two CTAs per SM, with the cached row; 40-value
+// threads 160 (four transforms), three CTAs per SM.
 template <int N1, int N2, int PAD> struct PadRegs {
   static constexpr int N = N1 * N2, NP = N / PAD, OFF = (N - NP) / 2;
   static constexpr int LO = OFF / N1, HI = (OFF + NP - 1) / N1 + 1;
@@ -431,9 +412,8 @@ template <int N1, int N2, int PAD> struct PadRegs {
 };
 
 template <int N1, int N2> struct RowFiltLaunch {
-  using S = Split<N1, N2>;
-  static constexpr int threads = S::WIDE ? 256 : (N2 > 16 ? 128 : 256);
-  static constexpr int min_blocks = S::WIDE ? 1 : (N2 > 16 ? 5 : 2);
+  static constexpr int threads = N2 > 32 ? 4 * N1 : (N2 > 16 ? 128 : 256);
+  static constexpr int min_blocks = N2 > 32 ? 3 : (N2 > 16 ? 5 : 2);
   static constexpr bool reload = N2 > 16;
 };
 template <int N1, int N2, int PAD>
@@ -443,19 +423,18 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
     const float2 *__restrict__ twA, const float2 *__restrict__ twB,
     const float2 *__restrict__ mask, float2 *__restrict__ rows_out, int n_pix, int nc, int nbw,
     int slot0, int n_slots, int ka, int s0) {
-  using S = Split<N1, N2>;
   using P = PadRegs<N1, N2, PAD>;
   using K = Pack<N1, N2>;
-  constexpr int N = S::N, S1 = S::S1, S2 = S::S2;
+  constexpr int N = K::N, S1 = K::S1, S2 = K::S2;
   constexpr int LO = P::LO, NR = P::HI - P::LO;
   extern __shared__ __align__(16) float2 smem[];
-  const int vpc = blockDim.x / 32 * K::P;   // rows per CTA
+  const int vpc = K::vecs(blockDim.x);   // rows per CTA
   const int wlane = threadIdx.x % 32, warp = threadIdx.x / 32;
-  const int pa = wlane / N1, lane = wlane % N1;
-  const bool outer = pa < K::P;   // this lane takes part in the outer stages
-  const int vec = warp * K::P + (outer ? pa : 0);
+  const int lane = K::CTA ? threadIdx.x % N1 : wlane % N1;
+  const bool outer = K::CTA || wlane / N1 < K::P;   // this lane takes part in the outer stages
+  const int vec = K::CTA ? threadIdx.x / N1 : warp * K::P + (outer ? wlane / N1 : 0);
   constexpr int XBF = K::XSR;
-  float2 *xb = smem + vec * XBF, *wb = smem + warp * K::P * XBF;
+  float2 *xb = smem + vec * XBF;
   // where vector v's output row sits in its buffer: 4 v complex in, as far
   // as the buffer's slack allows, and even, so that with an even XBF two
   // adjacent columns of a row are one aligned 16-byte load
@@ -503,31 +482,25 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
         r[LO + h] = in_pupil(h) ? cmul(f[h], __ldg(g + N1 * h)) : make_float2(0.f, 0.f);
     }
     RegDFTZ<N2, false, P::NZ>::run(r);
-    __syncwarp();
+    K::sync();
     if (outer) {
 #pragma unroll
       for (int k2 = 0; k2 < N2; ++k2) xb[k2 * S1 + lane] = cmulc(r[k2], __ldg(twA + k2 * N1 + lane));
     }
-    __syncwarp();
-    float2 *x3 = xb;   // input of the last stage
+    K::sync();
     // the x mask between the forward and the inverse transform (swapped split)
-    if constexpr (S::WIDE) {
-      x3 = xb + N2 * S1;
-      wide_mid<N1, N2>(xb, x3, mask, twB, wlane);
-    } else {
-      packed_mid<N1, N2, XBF>(wb, mask, twB, wlane);
-    }
-    __syncwarp();
+    packed_mid<N1, N2, XBF>(smem, mask, twB);
+    K::sync();
     float2 r3[N2];
 #pragma unroll
-    for (int n1 = 0; n1 < N2; ++n1) r3[n1] = x3[lane * S2 + n1];
+    for (int n1 = 0; n1 < N2; ++n1) r3[n1] = xb[lane * S2 + n1];
     RegDFT<N2, true>::run(r3);
     // The slot's block is column-major (rows_out[it][x][row]), so that the
     // column pass loads a column coalesced.  Each vector puts its row in
     // its own exchange buffer (T_v, offset a few complex per vector against
     // bank conflicts), and the CTA writes one run of vpc rows per column x,
     // as 16-byte row pairs where the rows allow.
-    __syncwarp();   // this vector's last-stage loads are done
+    K::sync();   // this vector's last-stage loads are done
     if (outer) {
 #pragma unroll
       for (int k1 = 0; k1 < N2; ++k1) xb[N1 * k1 + lane + row_tile_off(vec)] = r3[k1];   // x = N1 k1 + lane
@@ -583,18 +556,15 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
 // CTAs per SM: 96 registers per thread, so the twiddle loads can be issued
 // earlier.
 template <int N1, int N2, int PAD, int MAXT>
-__global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
-                                              ? 1
-                                              : (MAXT <= 160 ? 4 : (MAXT <= 256 ? 3 : 2)))
+__global__ void __launch_bounds__(MAXT, N2 > 32 ? 3 : (MAXT <= 160 ? 4 : (MAXT <= 256 ? 3 : 2)))
     k_colfilt_bin(
     const float2 *__restrict__ rows_in, const float2 *__restrict__ gy,
     const float2 *__restrict__ twA, const float2 *__restrict__ twB,
     const float2 *__restrict__ mask, float *__restrict__ part, int n_pix, int fp, int fq,
     float scale, int n_mod, int nc, int nbw, int slot0, int tc, int s0) {
-  using S = Split<N1, N2>;
   using P = PadRegs<N1, N2, PAD>;
   using K = Pack<N1, N2>;
-  constexpr int N = S::N, S1 = S::S1, S2 = S::S2, CS = K::XS;
+  constexpr int N = K::N, S1 = K::S1, S2 = K::S2, CS = K::XS;
   constexpr int LO = P::LO, NR = P::HI - P::LO;
   extern __shared__ __align__(16) float2 smem_k[];
   float2 *s_tile = smem_k;
@@ -605,23 +575,9 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
   if ((blockIdx.y & 1) && (cslot == 0 || 2 * cslot == n_mod)) return;   // no second item
   const int col0 = blockIdx.x * tc, ncol = min(tc, N - col0);
   const int wlane = threadIdx.x % 32, warp = threadIdx.x / 32;
-  const int pa = wlane / N1, lane = wlane % N1;
-  const bool outer = pa < K::P;   // this lane takes part in the outer stages
-  const int vec = warp * K::P + (outer ? pa : 0);
-  // wide splits stage the item's y factors in shared memory (5% off their
-  // column pass; at 960 the factors come through L1 as fast)
-  float2 *s_gy = nullptr;
-  if constexpr (S::WIDE) {
-    s_gy = s_tile + ((blockDim.x / 32 * CS + 1) & ~1);   // 16-byte aligned
-    const float2 *g = gy + (size_t)m * n_pix;
-    if ((n_pix & 1) == 0) {
-      for (int i = threadIdx.x; 2 * i < n_pix; i += blockDim.x) cp_async16(s_gy + 2 * i, g + 2 * i);
-    } else {
-      for (int i = threadIdx.x; i < n_pix; i += blockDim.x) cp_async8(s_gy + i, g + i);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-  }
+  const int lane = K::CTA ? threadIdx.x % N1 : wlane % N1;
+  const bool outer = K::CTA || wlane / N1 < K::P;   // this lane takes part in the outer stages
+  const int vec = K::CTA ? threadIdx.x / N1 : warp * K::P + (outer ? wlane / N1 : 0);
   // this vector's column x = col0 + vec: n_pix contiguous rows of the
   // slot's column-major block, loaded coalesced straight into registers and
   // past L1 (which keeps the twiddle, mask and tilt tables)
@@ -643,10 +599,7 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
     }
 #pragma unroll
     for (int h = 0; h < NR; ++h) {
-      if constexpr (S::WIDE)
-        r[LO + h] = ok[h] ? cmul(e[h], s_gy[row0 + N1 * h]) : make_float2(0.f, 0.f);
-      else
-        r[LO + h] = ok[h] ? cmul(e[h], __ldg(g + N1 * h)) : make_float2(0.f, 0.f);
+      r[LO + h] = ok[h] ? cmul(e[h], __ldg(g + N1 * h)) : make_float2(0.f, 0.f);
     }
   }
   float2 *col = s_tile + vec * CS;   // this vector's exchange buffer
@@ -655,20 +608,14 @@ __global__ void __launch_bounds__(MAXT, Split<N1, N2>::WIDE
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) col[k2 * S1 + lane] = cmulc(r[k2], __ldg(twA + k2 * N1 + lane));
   }
-  __syncwarp();
-  float2 *x3 = col;   // input of the last stage
-  if constexpr (S::WIDE) {
-    x3 = col + N2 * S1;
-    wide_mid<N1, N2>(col, x3, mask, twB, wlane);
-  } else {
-    packed_mid<N1, N2, CS>(s_tile + warp * K::P * CS, mask, twB, wlane);
-  }
-  __syncwarp();
+  K::sync();
+  packed_mid<N1, N2, CS>(s_tile, mask, twB);
+  K::sync();
   float2 r3[N2];
 #pragma unroll
-  for (int n1 = 0; n1 < N2; ++n1) r3[n1] = x3[lane * S2 + n1];
+  for (int n1 = 0; n1 < N2; ++n1) r3[n1] = col[lane * S2 + n1];
   RegDFT<N2, true>::run(r3);
-  __syncwarp();
+  K::sync();
   float *colI = reinterpret_cast<float *>(col);   // this column's intensity, y = N1 k1 + lane
   if (outer) {
 #pragma unroll
@@ -757,11 +704,11 @@ __global__ void __launch_bounds__(256) k_bin_reduce(const float *__restrict__ pa
 constexpr int kColsTile = 8;
 
 // f(integral_constant<int, pad>) for the paddings the two-pass kernels of a
-// split are built for: those that divide N, pad 2 only with N2 % 4 == 0 (the
-// plan refuses the others).
+// split are built for: those that divide N, but not pad 2 at 660 and 1600 (the
+// plan refuses it).
 template <int N1, int N2, class F> static void for_pad(int pad, F &&f) {
   constexpr int N = N1 * N2;
-  if constexpr (N2 % 4 == 0)
+  if constexpr (N2 % 4 == 0 && N1 <= 32)
     if (pad == 2) f(std::integral_constant<int, 2>{});
   if constexpr (N % 3 == 0)
     if (pad == 3) f(std::integral_constant<int, 3>{});
@@ -816,38 +763,40 @@ static int configure(PwfsPlan *p) {
 // one that leaves the fewest lanes idle (a tile narrower than its warps, a
 // last tile that is not full), up to five of 32-value lanes and eight of
 // shorter ones (eleven where a detector pixel is a fraction of grid pixels:
-// the SOUL example's 11-column tiles; wide splits four, so that two CTAs of
-// their 50-point transforms share an SM's registers).
+// the SOUL example's 11-column tiles); five for 1600's four columns.
 template <int N1, int N2>
 static int configure_two(PwfsPlan *p) {
-  using S = Split<N1, N2>;
   using K = Pack<N1, N2>;
   int s = SPECULA_OK;
   p->two_ok = false;
-  p->blockR = S::WIDE ? 128 : RowFiltLaunch<N1, N2>::threads;
-  p->smemR = (size_t)(p->blockR / 32 * K::P) * K::XSR * sizeof(float2);
-  const int fit = (p->fp + K::P - 1) / K::P;   // warps that hold one detector pixel
-  const int most = S::WIDE ? 4 : (p->fq != 1 ? 11 : std::max(fit, N2 >= 32 ? 5 : 8));
-  int best = 0, cost = 0;   // lane columns issued for the N columns of an item
-  for (int w = fit; w <= most; ++w) {
-    const int tc = w * K::P / p->fp * p->fp;
-    const int c = (S::N + tc - 1) / tc * w;
-    if (!best || c <= cost) best = w, cost = c;
-  }
+  p->blockR = RowFiltLaunch<N1, N2>::threads;
+  p->smemR = (size_t)K::vecs(p->blockR) * K::XSR * sizeof(float2);
   // a detector pixel's columns at the three-pass split's lanes per transform
   // fit one CTA: the geometries that the plan takes
-  if (!best || p->fp * p->G > (S::WIDE ? 128 : (p->fq != 1 ? 352 : 256))) return SPECULA_OK;
-  p->tcK = best * K::P / p->fp * p->fp;
-  p->blockK = best * 32;
-  // the tile's exchange buffers (wide splits: and the item's n_pix y factors,
-  // after a 16-byte boundary)
-  p->smemK = ((size_t)best * K::P * K::XS + (S::WIDE ? 1 + p->n_pix : 0)) * sizeof(float2);
+  if (p->fp * p->G > (K::CTA ? 128 : (p->fq != 1 ? 352 : 256))) return SPECULA_OK;
+  if constexpr (K::CTA) {
+    p->blockK = 4 * N1;
+    p->tcK = 4 / p->fp * p->fp;   // fp <= 4 from the line above
+  } else {
+    const int fit = (p->fp + K::P - 1) / K::P;   // warps that hold one detector pixel
+    const int most = p->fq != 1 ? 11 : std::max(fit, N2 >= 32 ? 5 : 8);
+    int best = 0, cost = 0;   // lane columns issued for the N columns of an item
+    for (int w = fit; w <= most; ++w) {
+      const int tc = w * K::P / p->fp * p->fp;
+      const int c = (K::N + tc - 1) / tc * w;
+      if (!best || c <= cost) best = w, cost = c;
+    }
+    if (!best || best * 32 > (p->fq != 1 ? 352 : 256)) return SPECULA_OK;
+    p->blockK = best * 32;
+    p->tcK = best * K::P / p->fp * p->fp;
+  }
+  p->smemK = (size_t)K::vecs(p->blockK) * K::XS * sizeof(float2);
   if (p->smemR > 227 * 1024 || p->smemK > 227 * 1024) return SPECULA_OK;
   for_pad<N1, N2>(p->pad, [&](auto pc) {
     constexpr int PAD = decltype(pc)::value;
     if ((s = ensure_dynamic_smem((const void *)k_rowfilt<N1, N2, PAD>, p->smemR))) return;
-    if constexpr (S::WIDE) {
-      s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 256>, p->smemK);
+    if constexpr (K::CTA) {
+      s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 160>, p->smemK);
     } else if (!(s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 256>,
                                          p->smemK)) &&
                !(s = ensure_dynamic_smem((const void *)k_colfilt_bin<N1, N2, PAD, 160>,
@@ -865,14 +814,14 @@ static int configure_two(PwfsPlan *p) {
 template <int N1, int N2>
 static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const float *phase,
                       int n_batch, float *det, cudaStream_t st) {
-  using S = Split<N1, N2>;
+  using K = Pack<N1, N2>;
   const int Np = p->n_pix;
   const int nd = p->pad * p->n_sub;   // detector side
   // the imaged cosine slots [s0, s0 + nc) of every batch element
   const int s0 = p->slot_lo;
   const int nc = (p->slot_hi < 0 ? p->nc : p->slot_hi) - s0;
   const int total = n_batch * nc;
-  const int vpc = p->blockR / 32 * Pack<N1, N2>::P;
+  const int vpc = K::vecs(p->blockR);
   const float scale = 1.0f / (float)p->n_mod;
   int field_done = -1, det_done = -1;
   for (int j0 = 0; j0 < total; j0 += p->chunk) {
@@ -887,7 +836,7 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
       field_done = b1;
     }
     dim3 gR((Np + vpc - 1) / vpc, (nj + p->ka - 1) / p->ka);
-    dim3 gK((S::N + p->tcK - 1) / p->tcK, 2 * nj);
+    dim3 gK((K::N + p->tcK - 1) / p->tcK, 2 * nj);
     int s = SPECULA_EUNSUPPORTED;
     for_pad<N1, N2>(p->pad, [&](auto pc) {
       constexpr int PAD = decltype(pc)::value;
@@ -903,8 +852,8 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
                      p->rows.as<float2>(), p->gy.as<float2>(), p->tpA.as<float2>(),            \
                      p->tpB.as<float2>(), p->mask.as<float2>(), p->part.as<float>(), Np, p->fp, \
                      p->fq, scale, p->n_mod, nc, p->nbw, j0, p->tcK, s0))
-        if constexpr (S::WIDE) {
-          SPECULA_COLFILT(256);   // wide tiles <= 128 threads
+        if constexpr (K::CTA) {
+          SPECULA_COLFILT(160);
         } else {
           if (p->blockK > 256)    // tiles of fractional detector pixels
             SPECULA_COLFILT(352);
@@ -1083,7 +1032,7 @@ int pwfs_run(specula_ctx *ctx, PwfsPlan *p, const float *amp, const float *phase
       case 320: return run_split2<10, 32>(ctx, p, amp, phase, n_batch, det, st);
       case 660: return run_split2<30, 22>(ctx, p, amp, phase, n_batch, det, st);
       case 960: return run_split2<30, 32>(ctx, p, amp, phase, n_batch, det, st);
-      case 1600: return run_split2<32, 50>(ctx, p, amp, phase, n_batch, det, st);
+      case 1600: return run_split2<40, 40>(ctx, p, amp, phase, n_batch, det, st);
       default: return SPECULA_EUNSUPPORTED;
     }
   }
@@ -1156,8 +1105,8 @@ done:
   return status;
 }
 
-// The three-pass form's split, and the two-pass form's: the same but for
-// 320 = 10 x 32, three transforms per warp.
+// The three-pass form's split (none for 1600), and the two-pass form's: the
+// same but for 320 = 10 x 32 and 1600 = 40 x 40.
 template <int N1, int N2, int M1 = N1, int M2 = N2>
 static int configure_both(PwfsPlan *p) {
   p->M1 = M1;
@@ -1174,7 +1123,7 @@ static int configure_for(PwfsPlan *p) {
     case 320: return configure_both<20, 16, 10, 32>(p);
     case 660: return configure_both<30, 22>(p);
     case 960: return configure_both<30, 32>(p);
-    case 1600: return configure_both<32, 50>(p);
+    case 1600: return configure_both<32, 50, 40, 40>(p);
     default: return SPECULA_EUNSUPPORTED;
   }
 }
