@@ -25,7 +25,8 @@
 //                        per thread) to global memory while the next tile
 //                        accumulates in the other one
 // Split-K partials go to a caller workspace and are summed in split order by
-// k_split_reduce (no atomics: bit-reproducible).  Every wait is bounded:
+// k_split_reduce (no atomics: bit-reproducible) or by the caller's next kernel
+// (gemm_bf16_partials).  Every wait is bounded:
 // on timeout the CTA records SPECULA_ETIMEOUT in the context status word,
 // waits for its own copies and MMAs, frees its tensor memory and returns.
 #include <cuda.h>
@@ -338,10 +339,18 @@ static int sm_count() {
   return sms[dev];
 }
 
+int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n, float *C,
+                      cudaStream_t st) {
+  SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
+                 k_split_reduce<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0,
+                                  st>>>(part, splits, n, C));
+  return SPECULA_OK;
+}
+
 template <bool TF32, int BN>
 static int gemm_launch(specula_ctx *ctx, int n_terms, const void *const *A, const void *const *B,
                        int M, int N, int K, float *C, int splits, float *work,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool partials) {
   using Cfg = GCfg<BN>;
   static bool attr_done[64] = {};
   int dev = 0;
@@ -371,38 +380,43 @@ static int gemm_launch(specula_ctx *ctx, int n_terms, const void *const *A, cons
   g.tiles_m = (M + GBM - 1) / GBM;
   g.tiles_n = (N + BN - 1) / BN;
   g.n_items = g.tiles_m * g.tiles_n * g.splits;
-  if (g.splits > 1 && !work) return SPECULA_EINVAL;
-  float *dst = g.splits > 1 ? work : C;
+  const bool to_work = partials || g.splits > 1;
+  if (to_work && !work) return SPECULA_EINVAL;
+  if (partials && g.splits != splits) return SPECULA_EINVAL;
+  float *dst = to_work ? work : C;
   g.vec4 = (N % 4 == 0) && ((uintptr_t)dst % 16 == 0);
   const int grid = std::min(g.n_items, sms);
   SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
                  k_gemm_tn<TF32, BN><<<grid, 256, Cfg::SMEM, st>>>(maps, g, dst,
                                                                    ctx->status_dev));
-  if (g.splits > 1) {
-    const size_t n = (size_t)M * N;
-    SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
-                   k_split_reduce<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0,
-                                    st>>>(work, g.splits, n, C));
-  }
+  if (g.splits > 1 && !partials)
+    return gemm_split_reduce(ctx, work, g.splits, (size_t)M * N, C, st);
   return SPECULA_OK;
 }
 
 template <bool TF32>
 static int gemm_terms(specula_ctx *ctx, int n_terms, const void *const *A, const void *const *B,
-                      int M, int N, int K, float *C, int splits, float *work, cudaStream_t st) {
-  if (!ctx || !C || n_terms < 1 || n_terms > kMaxTerms || splits < 1) return SPECULA_EINVAL;
+                      int M, int N, int K, float *C, int splits, float *work, cudaStream_t st,
+                      bool partials = false) {
+  if (!ctx || (!C && !partials) || n_terms < 1 || n_terms > kMaxTerms || splits < 1)
+    return SPECULA_EINVAL;
   for (int t = 0; t < n_terms; ++t) {
     const int s = gemm_check(A[t], B[t], M, N, K, TF32);
     if (s) return s;
   }
   if (gemm_bn(N) == 128)
-    return gemm_launch<TF32, 128>(ctx, n_terms, A, B, M, N, K, C, splits, work, st);
-  return gemm_launch<TF32, 256>(ctx, n_terms, A, B, M, N, K, C, splits, work, st);
+    return gemm_launch<TF32, 128>(ctx, n_terms, A, B, M, N, K, C, splits, work, st, partials);
+  return gemm_launch<TF32, 256>(ctx, n_terms, A, B, M, N, K, C, splits, work, st, partials);
 }
 
 int gemm_bf16_tn(specula_ctx *ctx, const void *A, const void *B, int M, int N, int K, float *C,
                  int splits, float *work, cudaStream_t st) {
   return gemm_terms<false>(ctx, 1, &A, &B, M, N, K, C, splits, work, st);
+}
+
+int gemm_bf16_partials(specula_ctx *ctx, const void *A, const void *B, int M, int N, int K,
+                       int splits, float *work, cudaStream_t st) {
+  return gemm_terms<false>(ctx, 1, &A, &B, M, N, K, nullptr, splits, work, st, true);
 }
 
 int gemm_bf16_terms(specula_ctx *ctx, int n_terms, const void *const *A, const void *const *B,

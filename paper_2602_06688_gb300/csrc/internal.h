@@ -285,6 +285,13 @@ int gemm_tf32_tn(specula_ctx *ctx, const float *A, const float *B, int M, int N,
                  int splits, float *work, cudaStream_t st);
 int gemm_bf16_tn(specula_ctx *ctx, const void *A, const void *B, int M, int N, int K, float *C,
                  int splits, float *work, cudaStream_t st);
+// the split-K partials work[s][M][N], s < splits (a count from gemm_splits),
+// left for the caller's kernel to add
+int gemm_bf16_partials(specula_ctx *ctx, const void *A, const void *B, int M, int N, int K,
+                       int splits, float *work, cudaStream_t st);
+// C[n] = the sum over s < splits of part[s][n], in order
+int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n, float *C,
+                      cudaStream_t st);
 // C = sum over t < n_terms (<= 3) of A_t B_t^T, one accumulation on the
 // tensor cores (split-precision products); every A_t is M x K, every B_t is
 // N x K, bf16, row-major

@@ -27,6 +27,11 @@
 namespace specula {
 
 constexpr int TT = 32;   // transpose tile
+// Thread rows of a tile kernel: one element per thread.  The training step's
+// kernels cover 256 rows by about 1000 columns, so the time is that of a few
+// rounds of loads; four elements per thread were four times the rounds
+// (gelu' of 256 x 1024 from 16 partials: 13.8 us).
+constexpr int TY = 32;
 
 __device__ __forceinline__ float gelu_f(float z) {
   return 0.5f * z * (1.0f + erff(z * (float)M_SQRT1_2));
@@ -36,15 +41,16 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
   return 0.5f * (1.0f + erff(z * (float)M_SQRT1_2)) + z * expf(-0.5f * z * z) * inv_sqrt_2pi;
 }
 
-// Tiled writer of a bf16 matrix and its transpose.  Block (32, 8), grid
+// Tiled writer of a bf16 matrix and its transpose.  Block (32, TY), grid
 // (C/32, R/32); the value function is evaluated once per element.
 template <class F>
 __device__ __forceinline__ void tile_bf16_pair(int R, int C, __nv_bfloat16 *out,
                                                __nv_bfloat16 *outT, F value) {
   __shared__ __nv_bfloat16 tile[TT][TT + 2];
   const int c0 = blockIdx.x * TT, r0 = blockIdx.y * TT;
-  for (int dr = threadIdx.y; dr < TT; dr += blockDim.y) {
-    const int r = r0 + dr, c = c0 + threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < TT / TY; ++k) {
+    const int dr = threadIdx.y + TY * k, r = r0 + dr, c = c0 + threadIdx.x;
     __nv_bfloat16 v = __float2bfloat16_rn(0.f);
     if (r < R && c < C) {
       v = __float2bfloat16_rn(value(r, c));
@@ -53,47 +59,139 @@ __device__ __forceinline__ void tile_bf16_pair(int R, int C, __nv_bfloat16 *out,
     tile[dr][threadIdx.x] = v;
   }
   __syncthreads();
-  for (int dc = threadIdx.y; dc < TT; dc += blockDim.y) {
-    const int c = c0 + dc, r = r0 + threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < TT / TY; ++k) {
+    const int dc = threadIdx.y + TY * k, c = c0 + dc, r = r0 + threadIdx.x;
     if (r < R && c < C) outT[(size_t)c * R + r] = tile[threadIdx.x][dc];
   }
 }
 
 // X [B][n_in] float -> Xb [Bp][in_pad] and XbT [in_pad][Bp] (zero pads)
-__global__ void k_pack_input(const float *__restrict__ X, int B, int n_in, int Bp, int in_pad,
+__global__ void __launch_bounds__(TT * TY) k_pack_input(const float *__restrict__ X, int B, int n_in, int Bp, int in_pad,
                              __nv_bfloat16 *Xb, __nv_bfloat16 *XbT) {
   tile_bf16_pair(Bp, in_pad, Xb, XbT, [&](int r, int c) {
     return (r < B && c < n_in) ? X[(size_t)r * n_in + c] : 0.f;
   });
 }
 
-// Z += bias (in place); H = gelu(Z) and its transpose in bf16
-__global__ void k_bias_gelu(float *__restrict__ Z, const float *__restrict__ bias, int R, int C,
-                            __nv_bfloat16 *H, __nv_bfloat16 *HT) {
+// A GEMM's result as its split-K partials part[s][R][C], added in split order.
+// The kernel that consumes a product adds them itself: a separate reduction
+// wrote and re-read every product once more (nine launches of a training step).
+struct Partials {
+  const float *p;
+  int splits;
+  size_t n;   // R C
+};
+__device__ __forceinline__ float partial_sum(const Partials &P, size_t e) {
+  // eight loads in flight, added in order
+  float v = 0.f;
+  int s = 0;
+  for (; s + 8 <= P.splits; s += 8) {
+    float x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = __ldg(P.p + (size_t)(s + u) * P.n + e);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v += x[u];
+  }
+  if (s < P.splits) {
+    float x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = s + u < P.splits ? __ldg(P.p + (size_t)(s + u) * P.n + e) : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (s + u < P.splits) v += x[u];
+  }
+  return v;
+}
+
+// Z = sum of partials + bias; H = gelu(Z) and its transpose in bf16
+__global__ void __launch_bounds__(TT * TY) k_bias_gelu(const Partials P,
+                                                      const float *__restrict__ bias,
+                                                      float *__restrict__ Z, int R, int C,
+                                                      __nv_bfloat16 *H, __nv_bfloat16 *HT) {
   tile_bf16_pair(R, C, H, HT, [&](int r, int c) {
-    const float z = Z[(size_t)r * C + c] + bias[c];
-    Z[(size_t)r * C + c] = z;
+    const size_t e = (size_t)r * C + c;
+    const float z = partial_sum(P, e) + bias[c];
+    Z[e] = z;
     return gelu_f(z);
   });
 }
 
-// dA (in place) <- dA * gelu'(Z); bf16 dZ and its transpose
-__global__ void k_gelu_back(float *__restrict__ dA, const float *__restrict__ Z, int R, int C,
-                            __nv_bfloat16 *dZb, __nv_bfloat16 *dZbT) {
+// Y = sum of partials + bias (padded, for the backward pass) and, when given,
+// the caller's [B][n_out]
+__global__ void __launch_bounds__(256) k_output(const Partials P, const float *__restrict__ bias,
+                                                int C, float *__restrict__ Y, int B, int n_out,
+                                                float *__restrict__ out) {
+  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (e >= P.n) return;
+  const int r = (int)(e / C), c = (int)(e - (size_t)r * C);
+  const float y = partial_sum(P, e) + bias[c];
+  Y[e] = y;
+  if (out && r < B && c < n_out) out[(size_t)r * n_out + c] = y;
+}
+
+// Bias gradients: db[c] = sum of D[r][c] over the batch's rows, in order, for
+// a 32 x 32 tile kernel that leaves D in global memory: the block that
+// finishes a tile column last (done[] counts, wrapping to zero) stages its
+// rows in shared memory, 128 at a time, and one thread per column adds them.
+// (A kernel of one thread per column took 18 us for 256 rows, each load
+// waiting for the last.)  Returns, to every thread, whether this block was the
+// last of its tile column.
+__device__ __forceinline__ bool tile_colsum(const float *D, int rows, int C, unsigned *done,
+                                            float *__restrict__ db) {
+  constexpr int CH = 128;
+  __shared__ float s_d[CH][TT];
+  __shared__ bool s_last;
+  __threadfence();   // this thread's part of D
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0)
+    s_last = atomicInc(done + blockIdx.x, gridDim.y - 1) == gridDim.y - 1;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  const int c = blockIdx.x * TT + threadIdx.x;
+  float s = 0.f;
+  for (int r0 = 0; r0 < rows; r0 += CH) {
+#pragma unroll
+    for (int k = 0; k < CH / TY; ++k) {
+      const int r = r0 + threadIdx.y + TY * k;
+      s_d[threadIdx.y + TY * k][threadIdx.x] = r < rows ? __ldcg(D + (size_t)r * C + c) : 0.f;
+    }
+    __syncthreads();
+    if (threadIdx.y == 0) {
+#pragma unroll 16
+      for (int r = 0; r < CH; ++r) s += s_d[r][threadIdx.x];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.y == 0) db[c] = s;
+  return true;
+}
+
+// dA = (sum of partials) gelu'(Z); bf16 dZ and its transpose; db = the column
+// sums over the B rows of the batch
+__global__ void __launch_bounds__(TT * TY) k_gelu_back(const Partials P,
+                                                      const float *__restrict__ Z, float *dA,
+                                                      int B, int R, int C, __nv_bfloat16 *dZb,
+                                                      __nv_bfloat16 *dZbT, unsigned *done,
+                                                      float *__restrict__ db) {
   tile_bf16_pair(R, C, dZb, dZbT, [&](int r, int c) {
     const size_t e = (size_t)r * C + c;
-    const float d = dA[e] * gelu_grad_f(Z[e]);
+    const float d = partial_sum(P, e) * gelu_grad_f(Z[e]);
     dA[e] = d;
     return d;
   });
+  tile_colsum(dA, B, C, done, db);
 }
 
-// dY = scale (Y - T) on the B x n_out block, zero on pads; squared residual
-// sums per tile row into part (one float per (tile, row) pair)
-__global__ void k_loss_grad(const float *__restrict__ Y, const float *__restrict__ T, int B,
-                            int n_out, int Bp, int out_pad, float scale, float *__restrict__ dYf,
-                            __nv_bfloat16 *dYb, __nv_bfloat16 *dYbT, float *__restrict__ part) {
-  __shared__ float s_sq[8][TT];
+// dY = scale (Y - T) on the B x n_out block, zero on pads, in bf16 with its
+// transpose; db = its column sums; loss = inv_count x the squared residuals'
+// sum, each block's in part, added by the block that finishes last
+__global__ void __launch_bounds__(TT * TY) k_loss_grad(
+    const float *__restrict__ Y, const float *__restrict__ T, int B, int n_out, int Bp,
+    int out_pad, float scale, float *dYf, __nv_bfloat16 *dYb, __nv_bfloat16 *dYbT, unsigned *done,
+    float *__restrict__ db, float *__restrict__ part, float inv_count, float *__restrict__ loss) {
+  __shared__ float s_sq[2][TY];
   float sq = 0.f;
   tile_bf16_pair(Bp, out_pad, dYb, dYbT, [&](int r, int c) {
     float d = 0.f;
@@ -103,60 +201,136 @@ __global__ void k_loss_grad(const float *__restrict__ Y, const float *__restrict
     dYf[(size_t)r * out_pad + c] = g;
     return g;
   });
-  s_sq[threadIdx.y][threadIdx.x] = sq;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if (threadIdx.x == 0) s_sq[0][threadIdx.y] = sq;
   __syncthreads();
   if (threadIdx.x == 0 && threadIdx.y == 0) {
     float s = 0.f;
-    for (int y = 0; y < 8; ++y)
-      for (int x = 0; x < TT; ++x) s += s_sq[y][x];
-    part[blockIdx.y * gridDim.x + blockIdx.x] = s;
+    for (int y = 0; y < TY; ++y) s += s_sq[0][y];
+    __stcg(part + blockIdx.y * gridDim.x + blockIdx.x, s);
   }
-}
-
-__global__ void k_loss_final(const float *__restrict__ part, int n, float inv_count,
-                             float *__restrict__ loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    float s = 0.f;
-    for (int i = 0; i < n; ++i) s += part[i];
+  // the tile columns' last blocks count themselves; the last of them sees
+  // every block's residual sum
+  if (!tile_colsum(dYf, B, out_pad, done, db)) return;
+  __shared__ bool s_end;
+  if (threadIdx.x == 0 && threadIdx.y == 0)
+    s_end = atomicInc(done + gridDim.x, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_end) return;
+  __threadfence();
+  const int n = gridDim.x * gridDim.y, t = threadIdx.y * TT + threadIdx.x;
+  float s = 0.f;
+  for (int i = t; i < n; i += TT * TY) s += __ldcg(part + i);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (threadIdx.x == 0) s_sq[1][threadIdx.y] = s;
+  __syncthreads();
+  if (t == 0) {
+    s = 0.f;
+    for (int y = 0; y < TY; ++y) s += s_sq[1][y];
     *loss = s * inv_count;
   }
 }
 
-__global__ void k_add_bias(float *__restrict__ Y, const float *__restrict__ bias, int R, int C) {
-  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (e < (size_t)R * C) Y[e] += bias[e % C];
+__device__ __forceinline__ void adam_step(float &p, float &m, float &v, float g, float lr_t,
+                                          float b1, float b2, float eps) {
+  m = b1 * m + (1.f - b1) * g;
+  v = b2 * v + (1.f - b2) * g * g;
+  p -= lr_t * m / (sqrtf(v) + eps);
 }
 
-__global__ void k_unpack_out(const float *__restrict__ Y, int B, int n_out, int out_pad,
-                             float *__restrict__ out) {
-  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (e < (size_t)B * n_out) out[e] = Y[(e / n_out) * out_pad + e % n_out];
-}
-
-// db[c] = sum over r < R of D[r][c], rows in order
-__global__ void k_colsum(const float *__restrict__ D, int R, int C, float *__restrict__ db) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= C) return;
-  float s = 0.f;
-  for (int r = 0; r < R; ++r) s += D[(size_t)r * C + c];
-  db[c] = s;
-}
-
-__global__ void k_adam(float *__restrict__ p, float *__restrict__ m, float *__restrict__ v,
-                       const float *__restrict__ g, size_t n, float lr_t, float b1, float b2,
-                       float eps) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr_t * mi / (sqrtf(vi) + eps);
+// Adam on every layer's weights and biases in one launch; the updated
+// weights' bf16 copy and its transpose come from the same registers (three
+// launches per layer and one more pass over the weights before).  Blocks
+// [first[l], first[l + 1]) are layer l's 32 x 128 weight tiles, a row of
+// four-float loads per warp; the rest 256 bias entries each.  The weight
+// gradients are read as their GEMMs' partials.  Bound by L2: at least 32 bytes
+// per weight.
+constexpr int kAdamC = 128;
+struct AdamLayer {
+  float *W, *mW, *vW, *b, *mb, *vb;
+  Partials gW;   // the gradient as its GEMM left it
+  const float *gb;
+  __nv_bfloat16 *Wb, *WbT;
+  int R, C;
+};
+struct AdamArgs {
+  AdamLayer L[3];
+  int first[4], bias_first[4];
+};
+__global__ void __launch_bounds__(TT * 8) k_adam(const AdamArgs A, float lr_t, float b1, float b2,
+                                                 float eps) {
+  __shared__ __nv_bfloat16 tile[kAdamC][TT + 2];   // transposed
+  const int blk = blockIdx.x, lane = threadIdx.x, warp = threadIdx.y;
+  if (blk >= A.first[3]) {
+    const int q = blk - A.first[3];
+    const int l = q >= A.bias_first[2] ? 2 : (q >= A.bias_first[1] ? 1 : 0);
+    const AdamLayer &L = A.L[l];
+    const int i = (q - A.bias_first[l]) * (TT * 8) + warp * TT + lane;
+    if (i < L.R) adam_step(L.b[i], L.mb[i], L.vb[i], L.gb[i], lr_t, b1, b2, eps);
+    return;
+  }
+  const int l = blk >= A.first[2] ? 2 : (blk >= A.first[1] ? 1 : 0);
+  const AdamLayer &L = A.L[l];
+  const int tiles_c = L.C / kAdamC, q = blk - A.first[l];   // widths are multiples of 128
+  const int r0 = q / tiles_c * TT, c0 = q % tiles_c * kAdamC;
+  constexpr int NR = TT / 8;
+  float4 p[NR], m[NR], v[NR], g[NR];
+#pragma unroll
+  for (int k = 0; k < NR; ++k) {
+    const size_t e = (size_t)(r0 + warp + 8 * k) * L.C + c0 + 4 * lane;
+    p[k] = *reinterpret_cast<const float4 *>(L.W + e);
+    m[k] = *reinterpret_cast<const float4 *>(L.mW + e);
+    v[k] = *reinterpret_cast<const float4 *>(L.vW + e);
+    g[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+#pragma unroll 2
+  for (int s = 0; s < L.gW.splits; ++s) {
+    float4 x[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k)
+      x[k] = __ldg(reinterpret_cast<const float4 *>(
+          L.gW.p + (size_t)s * L.gW.n + (size_t)(r0 + warp + 8 * k) * L.C + c0 + 4 * lane));
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+      g[k].x += x[k].x;
+      g[k].y += x[k].y;
+      g[k].z += x[k].z;
+      g[k].w += x[k].w;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < NR; ++k) {
+    const int dr = warp + 8 * k;
+    const size_t e = (size_t)(r0 + dr) * L.C + c0 + 4 * lane;
+    adam_step(p[k].x, m[k].x, v[k].x, g[k].x, lr_t, b1, b2, eps);
+    adam_step(p[k].y, m[k].y, v[k].y, g[k].y, lr_t, b1, b2, eps);
+    adam_step(p[k].z, m[k].z, v[k].z, g[k].z, lr_t, b1, b2, eps);
+    adam_step(p[k].w, m[k].w, v[k].w, g[k].w, lr_t, b1, b2, eps);
+    *reinterpret_cast<float4 *>(L.W + e) = p[k];
+    *reinterpret_cast<float4 *>(L.mW + e) = m[k];
+    *reinterpret_cast<float4 *>(L.vW + e) = v[k];
+    __nv_bfloat162 w[2] = {__floats2bfloat162_rn(p[k].x, p[k].y),
+                           __floats2bfloat162_rn(p[k].z, p[k].w)};
+    *reinterpret_cast<uint2 *>(L.Wb + e) = *reinterpret_cast<const uint2 *>(w);
+    tile[4 * lane][dr] = w[0].x;
+    tile[4 * lane + 1][dr] = w[0].y;
+    tile[4 * lane + 2][dr] = w[1].x;
+    tile[4 * lane + 3][dr] = w[1].y;
+  }
+  __syncthreads();
+  // a column's 32 rows are 64 bytes: two columns per warp
+  const int half = lane / 16, pr = 2 * (lane % 16);
+#pragma unroll
+  for (int k = 0; k < kAdamC / 16; ++k) {
+    const int c = 16 * k + 2 * warp + half;
+    *reinterpret_cast<uint32_t *>(L.WbT + (size_t)(c0 + c) * L.R + r0 + pr) =
+        *reinterpret_cast<const uint32_t *>(&tile[c][pr]);
   }
 }
 
-__global__ void k_cast_w(const float *__restrict__ W, int R, int C, __nv_bfloat16 *Wb,
+__global__ void __launch_bounds__(TT * TY) k_cast_w(const float *__restrict__ W, int R, int C, __nv_bfloat16 *Wb,
                          __nv_bfloat16 *WbT) {
   tile_bf16_pair(R, C, Wb, WbT, [&](int r, int c) { return W[(size_t)r * C + c]; });
 }
@@ -224,9 +398,11 @@ struct specula_mlp {
   int bmax;        // padded batch capacity
   int t = 0;       // Adam steps taken
   int last_b = 0;  // batch of the last forward
+  int gsplits[3] = {1, 1, 1};   // partials of the weight gradients in gW
   DevBuf W[3], b[3], mW[3], vW[3], mb[3], vb[3], Wb[3], WbT[3], gW[3], gb[3];
   DevBuf Xb, XbT, Z[2], H[2], HT[2], Y, dYf, dYb, dYbT, dA[2], dZb[2], dZbT[2];
   DevBuf work, part, loss;
+  DevBuf done;     // finished-block counts of the loss and GELU-backward kernels
   DevBuf Hi[2];    // inference activations, [kInferMax][np] float32
   size_t work_floats = 0;
 };
@@ -353,18 +529,31 @@ static int mlp_splits(int M, int N, int K) {
   return gemm_splits(K, want);
 }
 
-static int mlp_gemm(specula_mlp *p, const void *A, const void *B, int M, int N, int K, float *C,
-                    cudaStream_t st) {
+// C = A B^T left as split-K partials in the workspace, for the kernel that
+// follows on the stream to add
+static int mlp_gemm(specula_mlp *p, const void *A, const void *B, int M, int N, int K,
+                    Partials *out, cudaStream_t st) {
   const int s = mlp_splits(M, N, K);
-  if ((size_t)s * M * N > p->work_floats && s > 1) return SPECULA_EINVAL;
-  return gemm_bf16_tn(p->ctx, A, B, M, N, K, C, s, p->work.as<float>(), st);
+  if ((size_t)s * M * N > p->work_floats) return SPECULA_EINVAL;
+  *out = Partials{p->work.as<float>(), s, (size_t)M * N};
+  return gemm_bf16_partials(p->ctx, A, B, M, N, K, s, p->work.as<float>(), st);
+}
+
+// dW_l = A B^T over the batch (M = np[l + 1], N = np[l]) as partials in the
+// layer's own buffer: Adam adds them as it reads them, get_grad when asked
+static int mlp_gemm_dw(specula_mlp *p, int l, const void *A, const void *B, int K,
+                       cudaStream_t st) {
+  const int M = p->np[l + 1], N = p->np[l];
+  p->gsplits[l] = mlp_splits(M, N, K);
+  if ((size_t)p->gsplits[l] * M * N * 4 > p->gW[l].bytes) return SPECULA_EINVAL;
+  return gemm_bf16_partials(p->ctx, A, B, M, N, K, p->gsplits[l], p->gW[l].as<float>(), st);
 }
 
 static int cast_layer(specula_mlp *p, int l, cudaStream_t st) {
   const int R = p->np[l + 1], C = p->np[l];
   dim3 g((C + TT - 1) / TT, (R + TT - 1) / TT);
   SPECULA_LAUNCH(p->ctx, SPECULA_K_MLP, st,
-                 k_cast_w<<<g, dim3(TT, 8), 0, st>>>(p->W[l].as<float>(), R, C,
+                 k_cast_w<<<g, dim3(TT, TY), 0, st>>>(p->W[l].as<float>(), R, C,
                                                     p->Wb[l].as<__nv_bfloat16>(),
                                                     p->WbT[l].as<__nv_bfloat16>()));
   return SPECULA_OK;
@@ -387,15 +576,18 @@ extern "C" int specula_mlp_create(specula_ctx *ctx, int32_t n_in, int32_t n_h1, 
   int s;
   for (int l = 0; l < 3; ++l) {
     const size_t nw = (size_t)p->np[l + 1] * p->np[l], nb = p->np[l + 1];
+    size_t gw = nw;   // the gradient's partials, for every padded batch up to the capacity
+    for (int b = 128; b <= Bp; b += 128)
+      gw = std::max(gw, nw * mlp_splits(p->np[l + 1], p->np[l], b));
     if ((s = p->W[l].alloc(nw * 4)) || (s = p->mW[l].alloc(nw * 4)) || (s = p->vW[l].alloc(nw * 4)) ||
-        (s = p->gW[l].alloc(nw * 4)) || (s = p->Wb[l].alloc(nw * 2)) || (s = p->WbT[l].alloc(nw * 2)) ||
+        (s = p->gW[l].alloc(gw * 4)) || (s = p->Wb[l].alloc(nw * 2)) || (s = p->WbT[l].alloc(nw * 2)) ||
         (s = p->b[l].alloc(nb * 4)) || (s = p->mb[l].alloc(nb * 4)) || (s = p->vb[l].alloc(nb * 4)) ||
         (s = p->gb[l].alloc(nb * 4)))
       return s;
     SPECULA_CK(cudaMemset(p->W[l].p, 0, nw * 4));
     SPECULA_CK(cudaMemset(p->mW[l].p, 0, nw * 4));
     SPECULA_CK(cudaMemset(p->vW[l].p, 0, nw * 4));
-    SPECULA_CK(cudaMemset(p->gW[l].p, 0, nw * 4));
+    SPECULA_CK(cudaMemset(p->gW[l].p, 0, gw * 4));
     SPECULA_CK(cudaMemset(p->b[l].p, 0, nb * 4));
     SPECULA_CK(cudaMemset(p->mb[l].p, 0, nb * 4));
     SPECULA_CK(cudaMemset(p->vb[l].p, 0, nb * 4));
@@ -407,17 +599,16 @@ extern "C" int specula_mlp_create(specula_ctx *ctx, int32_t n_in, int32_t n_h1, 
       (s = p->H[0].alloc((size_t)Bp * h1 * 2)) || (s = p->H[1].alloc((size_t)Bp * h2 * 2)) ||
       (s = p->HT[0].alloc((size_t)Bp * h1 * 2)) || (s = p->HT[1].alloc((size_t)Bp * h2 * 2)) ||
       (s = p->Y.alloc((size_t)Bp * o * 4)) || (s = p->dYf.alloc((size_t)Bp * o * 4)) ||
-      (s = p->dYb.alloc((size_t)Bp * o * 2)) || (s = p->dYbT.alloc((size_t)Bp * o * 2)) ||
       (s = p->dA[0].alloc((size_t)Bp * h1 * 4)) || (s = p->dA[1].alloc((size_t)Bp * h2 * 4)) ||
+      (s = p->dYb.alloc((size_t)Bp * o * 2)) || (s = p->dYbT.alloc((size_t)Bp * o * 2)) ||
       (s = p->dZb[0].alloc((size_t)Bp * h1 * 2)) || (s = p->dZb[1].alloc((size_t)Bp * h2 * 2)) ||
       (s = p->dZbT[0].alloc((size_t)Bp * h1 * 2)) || (s = p->dZbT[1].alloc((size_t)Bp * h2 * 2)))
     return s;
-  // split-K workspace: the largest of the eight GEMMs of a step, for every
+  // split-K workspace: the largest of the forward and input-gradient GEMMs, for every
   // padded batch up to the capacity
   size_t wf = 1;
   for (int b = 128; b <= Bp; b += 128) {
-    const int shapes[8][3] = {{b, h1, in}, {b, h2, h1}, {b, o, h2}, {o, h2, b},
-                              {b, h2, o},  {h2, h1, b}, {b, h1, h2}, {h1, in, b}};
+    const int shapes[5][3] = {{b, h1, in}, {b, h2, h1}, {b, o, h2}, {b, h2, o}, {b, h1, h2}};
     for (auto &sh : shapes)
       wf = std::max(wf, (size_t)mlp_splits(sh[0], sh[1], sh[2]) * sh[0] * sh[1]);
   }
@@ -427,7 +618,11 @@ extern "C" int specula_mlp_create(specula_ctx *ctx, int32_t n_in, int32_t n_h1, 
       (s = p->Hi[1].alloc((size_t)kInferMax * h2 * 4)))
     return s;
   const int tiles = ((o + TT - 1) / TT) * ((Bp + TT - 1) / TT);
-  if ((s = p->part.alloc((size_t)tiles * 4)) || (s = p->loss.alloc(4))) return s;
+  const int wide = std::max(o, std::max(h1, h2));
+  if ((s = p->part.alloc((size_t)tiles * 4)) || (s = p->loss.alloc(4)) ||
+      (s = p->done.alloc((size_t)(wide / TT + 1) * 4)))
+    return s;
+  SPECULA_CK(cudaMemset(p->done.p, 0, p->done.bytes));
   for (int l = 0; l < 3; ++l)
     if ((s = cast_layer(p.get(), l, 0))) return s;
   SPECULA_CK(cudaDeviceSynchronize());
@@ -468,8 +663,8 @@ static int copy_out(specula_mlp *p, int layer, const DevBuf &W, const DevBuf &b,
   SPECULA_CK(cudaSetDevice(p->ctx->device));
   SPECULA_CK(cudaDeviceSynchronize());
   const int R = p->n[layer + 1], C = p->n[layer], CP = p->np[layer];
-  std::vector<float> w(W.bytes / 4), bb(b.bytes / 4);
-  SPECULA_CK(cudaMemcpy(w.data(), W.p, W.bytes, cudaMemcpyDeviceToHost));
+  std::vector<float> w((size_t)p->np[layer + 1] * CP), bb(b.bytes / 4);
+  SPECULA_CK(cudaMemcpy(w.data(), W.p, w.size() * 4, cudaMemcpyDeviceToHost));
   SPECULA_CK(cudaMemcpy(bb.data(), b.p, b.bytes, cudaMemcpyDeviceToHost));
   for (int r = 0; r < R; ++r)
     for (int c = 0; c < C; ++c) W_host[(size_t)r * C + c] = w[(size_t)r * CP + c];
@@ -486,7 +681,15 @@ extern "C" int specula_mlp_get_layer(specula_mlp *p, int32_t layer, float *W_hos
 extern "C" int specula_mlp_get_grad(specula_mlp *p, int32_t layer, float *dW_host,
                                     float *db_host) {
   if (!p || layer < 0 || layer > 2 || !dW_host || !db_host) return SPECULA_EINVAL;
-  return copy_out(p, layer, p->gW[layer], p->gb[layer], dW_host, db_host);
+  if (p->gsplits[layer] == 1) return copy_out(p, layer, p->gW[layer], p->gb[layer], dW_host, db_host);
+  SPECULA_CK(cudaSetDevice(p->ctx->device));
+  SPECULA_CK(cudaDeviceSynchronize());
+  const size_t n = (size_t)p->np[layer + 1] * p->np[layer];
+  DevBuf g;
+  int s = g.alloc(n * 4);
+  if (!s)
+    s = gemm_split_reduce(p->ctx, p->gW[layer].as<float>(), p->gsplits[layer], n, g.as<float>(), 0);
+  return s ? s : copy_out(p, layer, g, p->gb[layer], dW_host, db_host);
 }
 
 extern "C" int specula_mlp_forward(specula_mlp *p, const float *X_dev, int32_t batch,
@@ -497,33 +700,27 @@ extern "C" int specula_mlp_forward(specula_mlp *p, const float *X_dev, int32_t b
   cudaStream_t st = (cudaStream_t)stream;
   specula_ctx *ctx = p->ctx;
   const int in = p->np[0], h1 = p->np[1], h2 = p->np[2], o = p->np[3];
-  const dim3 tb(TT, 8);
+  const dim3 tb(TT, TY);
   int s;
   SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
                  k_pack_input<<<dim3(in / TT, Bp / TT), tb, 0, st>>>(
                      X_dev, batch, p->n[0], Bp, in, p->Xb.as<__nv_bfloat16>(),
                      p->XbT.as<__nv_bfloat16>()));
   const void *Hin = p->Xb.p;
+  Partials P;
   for (int l = 0; l < 2; ++l) {
     const int K = p->np[l], N = p->np[l + 1];
-    if ((s = mlp_gemm(p, Hin, p->Wb[l].p, Bp, N, K, p->Z[l].as<float>(), st))) return s;
+    if ((s = mlp_gemm(p, Hin, p->Wb[l].p, Bp, N, K, &P, st))) return s;
     SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
                    k_bias_gelu<<<dim3(N / TT, Bp / TT), tb, 0, st>>>(
-                       p->Z[l].as<float>(), p->b[l].as<float>(), Bp, N,
+                       P, p->b[l].as<float>(), p->Z[l].as<float>(), Bp, N,
                        p->H[l].as<__nv_bfloat16>(), p->HT[l].as<__nv_bfloat16>()));
     Hin = p->H[l].p;
   }
-  if ((s = mlp_gemm(p, Hin, p->Wb[2].p, Bp, o, h2, p->Y.as<float>(), st))) return s;
-  const size_t ny = (size_t)Bp * o;
+  if ((s = mlp_gemm(p, Hin, p->Wb[2].p, Bp, o, h2, &P, st))) return s;
   SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                 k_add_bias<<<(unsigned)((ny + 255) / 256), 256, 0, st>>>(
-                     p->Y.as<float>(), p->b[2].as<float>(), Bp, o));
-  if (Y_dev) {
-    const size_t n = (size_t)batch * p->n[3];
-    SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                   k_unpack_out<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-                       p->Y.as<float>(), batch, p->n[3], o, Y_dev));
-  }
+                 k_output<<<(unsigned)((P.n + 255) / 256), 256, 0, st>>>(
+                     P, p->b[2].as<float>(), o, p->Y.as<float>(), batch, p->n[3], Y_dev));
   p->last_b = batch;
   (void)h1;
   return SPECULA_OK;
@@ -576,39 +773,32 @@ extern "C" int specula_mlp_backward(specula_mlp *p, const float *T_dev, int32_t 
   cudaStream_t st = (cudaStream_t)stream;
   specula_ctx *ctx = p->ctx;
   const int in = p->np[0], h1 = p->np[1], h2 = p->np[2], o = p->np[3];
-  const dim3 tb(TT, 8);
+  const dim3 tb(TT, TY);
   const float scale = 2.0f / ((float)batch * (float)p->n[3]);
   const dim3 gl(o / TT, Bp / TT);
   int s;
   SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                 k_loss_grad<<<gl, tb, 0, st>>>(p->Y.as<float>(), T_dev, batch, p->n[3], Bp, o,
-                                                scale, p->dYf.as<float>(),
-                                                p->dYb.as<__nv_bfloat16>(),
-                                                p->dYbT.as<__nv_bfloat16>(), p->part.as<float>()));
-  SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                 k_loss_final<<<1, 32, 0, st>>>(p->part.as<float>(), (int)(gl.x * gl.y),
-                                                1.0f / ((float)batch * (float)p->n[3]),
-                                                loss_dev ? loss_dev : p->loss.as<float>()));
-  SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                 k_colsum<<<(o + 255) / 256, 256, 0, st>>>(p->dYf.as<float>(), batch, o,
-                                                           p->gb[2].as<float>()));
+                 k_loss_grad<<<gl, tb, 0, st>>>(
+                     p->Y.as<float>(), T_dev, batch, p->n[3], Bp, o, scale,
+                     p->dYf.as<float>(), p->dYb.as<__nv_bfloat16>(), p->dYbT.as<__nv_bfloat16>(),
+                     p->done.as<unsigned>(), p->gb[2].as<float>(),
+                     p->part.as<float>(), 1.0f / ((float)batch * (float)p->n[3]),
+                     loss_dev ? loss_dev : p->loss.as<float>()));
   // layer 3: dW3 = dY^T H2, dH2 = dY W3
-  if ((s = mlp_gemm(p, p->dYbT.p, p->HT[1].p, o, h2, Bp, p->gW[2].as<float>(), st))) return s;
-  if ((s = mlp_gemm(p, p->dYb.p, p->WbT[2].p, Bp, h2, o, p->dA[1].as<float>(), st))) return s;
+  Partials P;
+  if ((s = mlp_gemm_dw(p, 2, p->dYbT.p, p->HT[1].p, Bp, st))) return s;
+  if ((s = mlp_gemm(p, p->dYb.p, p->WbT[2].p, Bp, h2, o, &P, st))) return s;
   for (int l = 1; l >= 0; --l) {
-    const int N = p->np[l + 1], K = p->np[l];
+    const int N = p->np[l + 1];
     SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
                    k_gelu_back<<<dim3(N / TT, Bp / TT), tb, 0, st>>>(
-                       p->dA[l].as<float>(), p->Z[l].as<float>(), Bp, N,
-                       p->dZb[l].as<__nv_bfloat16>(), p->dZbT[l].as<__nv_bfloat16>()));
-    SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                   k_colsum<<<(N + 255) / 256, 256, 0, st>>>(p->dA[l].as<float>(), batch, N,
-                                                             p->gb[l].as<float>()));
+                       P, p->Z[l].as<float>(), p->dA[l].as<float>(), batch, Bp, N,
+                       p->dZb[l].as<__nv_bfloat16>(), p->dZbT[l].as<__nv_bfloat16>(),
+                       p->done.as<unsigned>(), p->gb[l].as<float>()));
     const void *HinT = l == 1 ? p->HT[0].p : p->XbT.p;
-    if ((s = mlp_gemm(p, p->dZbT[l].p, HinT, N, K, Bp, p->gW[l].as<float>(), st))) return s;
+    if ((s = mlp_gemm_dw(p, l, p->dZbT[l].p, HinT, Bp, st))) return s;
     if (l == 1)
-      if ((s = mlp_gemm(p, p->dZb[1].p, p->WbT[1].p, Bp, h1, h2, p->dA[0].as<float>(), st)))
-        return s;
+      if ((s = mlp_gemm(p, p->dZb[1].p, p->WbT[1].p, Bp, h1, h2, &P, st))) return s;
   }
   (void)in;
   return SPECULA_OK;
@@ -621,18 +811,20 @@ extern "C" int specula_mlp_adam(specula_mlp *p, float lr, float b1, float b2, fl
   cudaStream_t st = (cudaStream_t)stream;
   p->t += 1;
   const double lr_t = lr * sqrt(1.0 - pow((double)b2, p->t)) / (1.0 - pow((double)b1, p->t));
+  AdamArgs A;
+  A.first[0] = A.bias_first[0] = 0;
   for (int l = 0; l < 3; ++l) {
-    const size_t nw = (size_t)p->np[l + 1] * p->np[l], nb = p->np[l + 1];
-    SPECULA_LAUNCH(p->ctx, SPECULA_K_MLP, st,
-                   k_adam<<<(unsigned)std::min<size_t>((nw + 255) / 256, 4096), 256, 0, st>>>(
-                       p->W[l].as<float>(), p->mW[l].as<float>(), p->vW[l].as<float>(),
-                       p->gW[l].as<float>(), nw, (float)lr_t, b1, b2, eps));
-    SPECULA_LAUNCH(p->ctx, SPECULA_K_MLP, st,
-                   k_adam<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(
-                       p->b[l].as<float>(), p->mb[l].as<float>(), p->vb[l].as<float>(),
-                       p->gb[l].as<float>(), nb, (float)lr_t, b1, b2, eps));
-    int s = cast_layer(p, l, st);
-    if (s) return s;
+    const int R = p->np[l + 1], C = p->np[l];
+    A.L[l] = AdamLayer{p->W[l].as<float>(),  p->mW[l].as<float>(), p->vW[l].as<float>(),
+                       p->b[l].as<float>(),  p->mb[l].as<float>(), p->vb[l].as<float>(),
+                       Partials{p->gW[l].as<float>(), p->gsplits[l], (size_t)R * C},
+                       p->gb[l].as<float>(),
+                       p->Wb[l].as<__nv_bfloat16>(), p->WbT[l].as<__nv_bfloat16>(), R, C};
+    A.first[l + 1] = A.first[l] + (R / TT) * (C / kAdamC);
+    A.bias_first[l + 1] = A.bias_first[l] + (R + TT * 8 - 1) / (TT * 8);
   }
+  SPECULA_LAUNCH(p->ctx, SPECULA_K_MLP, st,
+                 k_adam<<<A.first[3] + A.bias_first[3], dim3(TT, 8), 0, st>>>(A, (float)lr_t, b1,
+                                                                           b2, eps));
   return SPECULA_OK;
 }
