@@ -22,7 +22,8 @@
 //                        stage back to the producer and each finished tile
 //                        to the epilogue
 //   warps 4-7          : drain a finished accumulator (tcgen05.ld, one row
-//                        per thread) to global memory while the next tile
+//                        per thread, transposed in shared memory to whole
+//                        lines) to global memory while the next tile
 //                        accumulates in the other one
 // Split-K partials go to a caller workspace and are summed in split order by
 // k_split_reduce (no atomics: bit-reproducible) or by the caller's next kernel
@@ -46,11 +47,13 @@ constexpr int kMaxTerms = 3;
 constexpr uint32_t G_A_BYTES = GBM * 128;   // 128 rows x 128 bytes of K
 // K elements per 128-byte row of a stage: 64 bf16 (TF32 = false) or 32 tf32
 template <bool TF32> constexpr int gbk() { return TF32 ? 32 : 64; }
+constexpr int kOutLd = 36;   // row stride (floats) of an epilogue warp's 32 x 32 block
 template <int BN> struct GCfg {
   static constexpr int STAGES = BN == 256 ? 4 : 6;
   static constexpr uint32_t B_BYTES = BN * 128;
   static constexpr uint32_t TMEM_COLS = 2 * BN;
-  static constexpr size_t SMEM = 1024 + STAGES * (G_A_BYTES + B_BYTES) + 256;
+  static constexpr size_t SMEM =
+      1024 + STAGES * (G_A_BYTES + B_BYTES) + 4 * 32 * kOutLd * sizeof(float) + 256;
 };
 
 // the operand maps of every term (kernel parameter space)
@@ -107,7 +110,8 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
   uint8_t *base = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
   uint8_t *sA = base;
   uint8_t *sB = base + C::STAGES * G_A_BYTES;
-  uint64_t *full = reinterpret_cast<uint64_t *>(sB + C::STAGES * C::B_BYTES);
+  float *s_out = reinterpret_cast<float *>(sB + C::STAGES * C::B_BYTES);
+  uint64_t *full = reinterpret_cast<uint64_t *>(s_out + 4 * 32 * kOutLd);
   uint64_t *empty = full + C::STAGES;
   uint64_t *acc_full = empty + C::STAGES;   // [2]
   uint64_t *acc_empty = acc_full + 2;       // [2]
@@ -222,25 +226,37 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
         break;
       }
       tc::fence_after();
-      const int row = m0 + wl * 32 + lane;
+      // 32 x 32 blocks through shared memory, so that rows go out as whole
+      // 128-byte lines (one row per lane wrote 32 half sectors per store)
+      const int row0 = m0 + wl * 32;
+      float *blk = s_out + wl * 32 * kOutLd;
+      float *dst0 = out + (size_t)split * g.M * g.N;
 #pragma unroll 1
       for (int c0 = 0; c0 < BN; c0 += 32) {
         float v[32];
         tc::tmem_ld32(tmem + ((uint32_t)(wl * 32) << 16) + (uint32_t)(buf * BN + c0), v);
         const int col = n0 + c0;
-        if (row < g.M && col < g.N) {
-          float *dst = out + ((size_t)split * g.M + row) * g.N + col;
-          if (g.vec4 && col + 32 <= g.N) {
-            float4 *d4 = reinterpret_cast<float4 *>(dst);
+        if (col >= g.N) break;   // warp-uniform
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-              d4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-          } else {
+        for (int q = 0; q < 8; ++q)
+          *reinterpret_cast<float4 *>(blk + lane * kOutLd + 4 * q) =
+              make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        __syncwarp();
+        if (g.vec4) {   // N % 4 == 0: four columns are inside together
+          const int r = lane >> 3, c = (lane & 7) * 4;
 #pragma unroll
-            for (int q = 0; q < 32; ++q)
-              if (col + q < g.N) dst[q] = v[q];
+          for (int q = 0; q < 8; ++q) {
+            const int row = row0 + r + 4 * q;
+            if (row < g.M && col + c < g.N)
+              *reinterpret_cast<float4 *>(dst0 + (size_t)row * g.N + col + c) =
+                  *reinterpret_cast<const float4 *>(blk + (r + 4 * q) * kOutLd + c);
           }
+        } else {
+          for (int r = 0; r < 32; ++r)
+            if (row0 + r < g.M && col + lane < g.N)
+              dst0[(size_t)(row0 + r) * g.N + col + lane] = blk[r * kOutLd + lane];
         }
+        __syncwarp();
       }
       tc::fence_before();
       __syncwarp();
@@ -256,13 +272,33 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
   if (threadIdx.x == 0 && *abort_flag) atomicExch(status, SPECULA_ETIMEOUT);
 }
 
-__global__ void k_split_reduce(const float *__restrict__ part, int splits, size_t n,
-                               float *__restrict__ out) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n;
+// out[e] = sum of part[s][e] over the splits, in order; V = 4 floats per load
+// where n and the pointers allow, four splits' loads in flight.
+template <int V>
+__global__ void __launch_bounds__(256) k_split_reduce(const float *__restrict__ part, int splits,
+                                                      size_t n, float *__restrict__ out) {
+  const size_t nv = n / V;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < nv;
        e += (size_t)gridDim.x * blockDim.x) {
-    float v = 0.f;
-    for (int s = 0; s < splits; ++s) v += part[(size_t)s * n + e];
-    out[e] = v;
+    float v[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) v[q] = 0.f;
+#pragma unroll 4
+    for (int s = 0; s < splits; ++s) {
+      if constexpr (V == 4) {
+        const float4 x = __ldcs(reinterpret_cast<const float4 *>(part + (size_t)s * n) + e);
+        v[0] += x.x;
+        v[1] += x.y;
+        v[2] += x.z;
+        v[3] += x.w;
+      } else {
+        v[0] += part[(size_t)s * n + e];
+      }
+    }
+    if constexpr (V == 4)
+      reinterpret_cast<float4 *>(out)[e] = make_float4(v[0], v[1], v[2], v[3]);
+    else
+      out[e] = v[0];
   }
 }
 
@@ -341,9 +377,15 @@ static int sm_count() {
 
 int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n, float *C,
                       cudaStream_t st) {
-  SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
-                 k_split_reduce<<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0,
-                                  st>>>(part, splits, n, C));
+  const bool v4 = n % 4 == 0 && (((uintptr_t)part | (uintptr_t)C) % 16) == 0;
+  const size_t threads = v4 ? n / 4 : n;
+  const unsigned grid = (unsigned)std::min<size_t>((threads + 255) / 256, 8192);
+  if (v4)
+    SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
+                   k_split_reduce<4><<<grid, 256, 0, st>>>(part, splits, n, C));
+  else
+    SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
+                   k_split_reduce<1><<<grid, 256, 0, st>>>(part, splits, n, C));
   return SPECULA_OK;
 }
 

@@ -87,15 +87,42 @@ __global__ void __launch_bounds__(kReconWarps * 32) k_mvm_bf16(
   }
 }
 
-__global__ void k_convert_bf16(const float *__restrict__ R, uint16_t *__restrict__ hi,
-                               uint16_t *__restrict__ lo, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const float v = R[i];
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    hi[i] = __bfloat16_as_ushort(h);
-    if (lo) lo[i] = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(h)));
+// hi = bf16(R), lo = bf16(R - hi) (lo may be NULL), eight values per thread by
+// 16-byte accesses where n and the pointers allow, the rest one by one.
+__device__ __forceinline__ void split_bf16(float v, uint32_t &h, uint32_t &l) {
+  const __nv_bfloat16 b = __float2bfloat16_rn(v);
+  h = __bfloat16_as_ushort(b);
+  l = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(b)));
+}
+__global__ void __launch_bounds__(256) k_convert_bf16(const float *__restrict__ R,
+                                                      uint16_t *__restrict__ hi,
+                                                      uint16_t *__restrict__ lo, size_t n,
+                                                      int vec) {
+  const size_t nt = (size_t)gridDim.x * blockDim.x;
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  const size_t n8 = vec ? n / 8 : 0;
+  for (size_t i = t; i < n8; i += nt) {
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(R) + 2 * i);
+    const float4 b = __ldg(reinterpret_cast<const float4 *>(R) + 2 * i + 1);
+    const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    uint32_t h[8], l[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) split_bf16(x[q], h[q], l[q]);
+    reinterpret_cast<uint4 *>(hi)[i] = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16,
+                                                  h[4] | h[5] << 16, h[6] | h[7] << 16);
+    if (lo)
+      reinterpret_cast<uint4 *>(lo)[i] = make_uint4(l[0] | l[1] << 16, l[2] | l[3] << 16,
+                                                    l[4] | l[5] << 16, l[6] | l[7] << 16);
   }
+  for (size_t i = 8 * n8 + t; i < n; i += nt) {
+    uint32_t h, l;
+    split_bf16(R[i], h, l);
+    hi[i] = (uint16_t)h;
+    if (lo) lo[i] = (uint16_t)l;
+  }
+}
+static int convert_vec(const void *R, const void *hi, const void *lo) {
+  return (((uintptr_t)R | (uintptr_t)hi | (uintptr_t)lo) % 16) == 0;
 }
 
 // Batched bf16 products on the tensor cores: the slopes are split into
@@ -156,8 +183,8 @@ static int recon_gemm(specula_ctx *ctx, const specula_recon_desc *rec, const flo
   uint16_t *xh = reinterpret_cast<uint16_t *>(w), *xl = reinterpret_cast<uint16_t *>(w + xb);
   float *part = reinterpret_cast<float *>(w + 2 * xb);
   SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st,
-                 k_convert_bf16<<<(unsigned)std::min<size_t>((nx + 255) / 256, 4096), 256, 0,
-                                  st>>>(X, xh, xl, nx));
+                 k_convert_bf16<<<(unsigned)std::min<size_t>((nx / 8 + 255) / 256 + 1, 8192), 256,
+                                  0, st>>>(X, xh, xl, nx, convert_vec(X, xh, xl)));
   const void *A3[3] = {xh, xh, xl}, *B3[3] = {rec->R_dev, rec->R_lo_dev, rec->R_dev};
   const void *A2[2] = {xh, xl}, *B2[2] = {rec->R_dev, rec->R_dev};
   return split ? gemm_bf16_terms(ctx, 3, A3, B3, nb, N, K, modes, splits, part, st)
@@ -236,8 +263,9 @@ extern "C" int specula_recon_convert(specula_ctx *ctx, int32_t n_modes, int32_t 
   if (precision != SPECULA_PREC_BF16 && precision != SPECULA_PREC_BF16X2) return SPECULA_EINVAL;
   if (precision == SPECULA_PREC_BF16X2 && !lo_dev) return SPECULA_EINVAL;
   const size_t n = (size_t)n_modes * n_slopes;
-  k_convert_bf16<<<1216, 256, 0, (cudaStream_t)stream>>>(
-      R_dev, (uint16_t *)hi_dev, precision == SPECULA_PREC_BF16X2 ? (uint16_t *)lo_dev : nullptr, n);
+  uint16_t *lo = precision == SPECULA_PREC_BF16X2 ? (uint16_t *)lo_dev : nullptr;
+  k_convert_bf16<<<1216, 256, 0, (cudaStream_t)stream>>>(R_dev, (uint16_t *)hi_dev, lo, n,
+                                                         convert_vec(R_dev, hi_dev, lo));
   SPECULA_CK_LAUNCH();
   return SPECULA_OK;
 }
