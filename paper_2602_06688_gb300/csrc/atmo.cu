@@ -45,6 +45,7 @@ __global__ void __launch_bounds__(256) k_atmo_coords(const AtmoParams P, double 
                                                      const double *__restrict__ t_dev,
                                                      int *__restrict__ tab_i,
                                                      float *__restrict__ tab_f) {
+  pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = P.n_pix;
   if (e >= P.n_layers * 2 * n) return;
@@ -72,6 +73,7 @@ __global__ void __launch_bounds__(256) k_atmo_extract(const AtmoParams P,
                                                       const int *__restrict__ tab_i,
                                                       const float *__restrict__ tab_f,
                                                       float *__restrict__ phase) {
+  pdl_wait();
   __shared__ int s_ix[kMaxLayers][kTileX], s_iy[kMaxLayers][kTileY];
   __shared__ float s_fx[kMaxLayers][kTileX], s_fy[kMaxLayers][kTileY];
   const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * kTileY;
@@ -162,14 +164,12 @@ extern "C" int specula_atmo_extract(specula_ctx *ctx, int32_t n_layers,
   }
   cudaStream_t st = (cudaStream_t)stream;
   const int nc = n_layers * 2 * pupil->n_pix;
-  SPECULA_LAUNCH(ctx, SPECULA_K_ATMO, st,
-                 k_atmo_coords<<<(nc + 255) / 256, 256, 0, st>>>(P, t_s, t_dev, ctx->atmo_tab_i,
-                                                                 ctx->atmo_tab_f));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_ATMO, st, k_atmo_coords, (nc + 255) / 256, 256, 0, P, t_s,
+                     t_dev, ctx->atmo_tab_i, ctx->atmo_tab_f);
   dim3 grid((pupil->n_pix + kTileX - 1) / kTileX, (pupil->n_pix + kTileY - 1) / kTileY);
   dim3 block(32, 8);
-  SPECULA_LAUNCH(ctx, SPECULA_K_ATMO, st,
-                 k_atmo_extract<<<grid, block, 0, st>>>(P, ctx->atmo_tab_i, ctx->atmo_tab_f,
-                                                        phase_dev));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_ATMO, st, k_atmo_extract, grid, block, 0, P, ctx->atmo_tab_i,
+                     ctx->atmo_tab_f, phase_dev);
   return SPECULA_OK;
 }
 

@@ -139,6 +139,7 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();   // barriers and tensor memory are set up under the kernel before
   if (warp == 0) {
     if (lane == 0) {
       uint32_t it = 0;   // stage fills issued (ring position)
@@ -277,6 +278,7 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
 template <int V>
 __global__ void __launch_bounds__(256) k_split_reduce(const float *__restrict__ part, int splits,
                                                       size_t n, float *__restrict__ out) {
+  pdl_wait();
   const size_t nv = n / V;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < nv;
        e += (size_t)gridDim.x * blockDim.x) {
@@ -381,11 +383,11 @@ int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n,
   const size_t threads = v4 ? n / 4 : n;
   const unsigned grid = (unsigned)std::min<size_t>((threads + 255) / 256, 8192);
   if (v4)
-    SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
-                   k_split_reduce<4><<<grid, 256, 0, st>>>(part, splits, n, C));
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_GEMM, st, k_split_reduce<4>, grid, 256, 0, part, splits, n,
+                       C);
   else
-    SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
-                   k_split_reduce<1><<<grid, 256, 0, st>>>(part, splits, n, C));
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_GEMM, st, k_split_reduce<1>, grid, 256, 0, part, splits, n,
+                       C);
   return SPECULA_OK;
 }
 
@@ -428,9 +430,8 @@ static int gemm_launch(specula_ctx *ctx, int n_terms, const void *const *A, cons
   float *dst = to_work ? work : C;
   g.vec4 = (N % 4 == 0) && ((uintptr_t)dst % 16 == 0);
   const int grid = std::min(g.n_items, sms);
-  SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
-                 k_gemm_tn<TF32, BN><<<grid, 256, Cfg::SMEM, st>>>(maps, g, dst,
-                                                                   ctx->status_dev));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_GEMM, st, (k_gemm_tn<TF32, BN>), grid, 256, Cfg::SMEM, maps, g,
+                     dst, ctx->status_dev);
   if (g.splits > 1 && !partials)
     return gemm_split_reduce(ctx, work, g.splits, (size_t)M * N, C, st);
   return SPECULA_OK;

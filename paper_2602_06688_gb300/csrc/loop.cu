@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(kDmWarps * 32, 4) k_dm_shape(const float *__re
                                                             int n_modes, int n_pix2) {
   using T = typename DmVec<V>::T;
   __shared__ T s_p[kDmWarps][32];
+  pdl_wait();
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(kLoopThreads) k_loop_residual(
     const float *__restrict__ amp, const float *__restrict__ atm, const float *__restrict__ dm,
     float *__restrict__ resid, double *__restrict__ part, unsigned *__restrict__ done,
     double *__restrict__ stats, int n_pix2, float k) {
+  pdl_wait();
   __shared__ double s_p[5][kLoopThreads / 32];
   __shared__ bool s_last;
   double a[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
@@ -157,6 +159,7 @@ __global__ void __launch_bounds__(kLoopThreads) k_loop_residual(
 __global__ void __launch_bounds__(256) k_loop_integrate(const float *__restrict__ m,
                                                         float *__restrict__ cmd, int n,
                                                         float keep, float gain) {
+  pdl_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < n) cmd[j] = keep * cmd[j] + gain * m[j];
 }
@@ -190,24 +193,16 @@ extern "C" int specula_dm_shape(specula_ctx *ctx, int32_t n_modes, int32_t n_pix
   while (cs < kDmMaxCluster && tiles * cs < 2 * sms &&
          n_modes / (kDmWarps * cs * 2) >= kDmUnroll)
     cs *= 2;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)tiles * cs);
-  cfg.blockDim = dim3(kDmWarps * 32);
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cs;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
+  const unsigned grid = (unsigned)tiles * cs;
+  const int cluster = cs > 1 ? cs : 0;
   if (v4)
     SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
-                   SPECULA_CK(cudaLaunchKernelEx(&cfg, k_dm_shape<4>, basis_dev, cmd_dev,
-                                                 phase_dev, n_modes, n_pix2)));
+                   SPECULA_CK(launch_pdl(k_dm_shape<4>, grid, kDmWarps * 32, 0, st, cluster,
+                                         basis_dev, cmd_dev, phase_dev, n_modes, n_pix2)));
   else
     SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
-                   SPECULA_CK(cudaLaunchKernelEx(&cfg, k_dm_shape<1>, basis_dev, cmd_dev,
-                                                 phase_dev, n_modes, n_pix2)));
+                   SPECULA_CK(launch_pdl(k_dm_shape<1>, grid, kDmWarps * 32, 0, st, cluster,
+                                         basis_dev, cmd_dev, phase_dev, n_modes, n_pix2)));
   return SPECULA_OK;
 }
 
@@ -221,10 +216,9 @@ extern "C" int specula_loop_residual(specula_ctx *ctx, int32_t n_pix2, const flo
   int blocks = (n_pix2 + kLoopThreads - 1) / kLoopThreads;
   blocks = blocks > kLoopMaxBlocks ? kLoopMaxBlocks : blocks;
   unsigned *done = reinterpret_cast<unsigned *>(ctx->loop_part + (size_t)kLoopMaxBlocks * 5);
-  SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
-                 k_loop_residual<<<blocks, kLoopThreads, 0, st>>>(
-                     amp_dev, atm_dev, dm_dev, resid_dev, ctx->loop_part, done, stats_dev, n_pix2,
-                     (float)wfs_over_sci));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_LOOP, st, k_loop_residual, blocks, kLoopThreads, 0, amp_dev,
+                     atm_dev, dm_dev, resid_dev, ctx->loop_part, done, stats_dev, n_pix2,
+                     (float)wfs_over_sci);
   return SPECULA_OK;
 }
 
@@ -233,9 +227,7 @@ extern "C" int specula_loop_integrate(specula_ctx *ctx, int32_t n_modes, float g
   if (!ctx || !modes_dev || !cmd_dev || n_modes < 1) return SPECULA_EINVAL;
   if (!isfinite(gain) || !isfinite(leak) || leak < 0.f || leak > 1.f) return SPECULA_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
-                 k_loop_integrate<<<(n_modes + 255) / 256, 256, 0, st>>>(modes_dev, cmd_dev,
-                                                                         n_modes, 1.f - leak,
-                                                                         gain));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_LOOP, st, k_loop_integrate, (n_modes + 255) / 256, 256, 0,
+                     modes_dev, cmd_dev, n_modes, 1.f - leak, gain);
   return SPECULA_OK;
 }

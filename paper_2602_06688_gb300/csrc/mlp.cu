@@ -69,6 +69,7 @@ __device__ __forceinline__ void tile_bf16_pair(int R, int C, __nv_bfloat16 *out,
 // X [B][n_in] float -> Xb [Bp][in_pad] and XbT [in_pad][Bp] (zero pads)
 __global__ void __launch_bounds__(TT * TY) k_pack_input(const float *__restrict__ X, int B, int n_in, int Bp, int in_pad,
                              __nv_bfloat16 *Xb, __nv_bfloat16 *XbT) {
+  pdl_wait();
   tile_bf16_pair(Bp, in_pad, Xb, XbT, [&](int r, int c) {
     return (r < B && c < n_in) ? X[(size_t)r * n_in + c] : 0.f;
   });
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(TT * TY) k_bias_gelu(const Partials P,
                                                       const float *__restrict__ bias,
                                                       float *__restrict__ Z, int R, int C,
                                                       __nv_bfloat16 *H, __nv_bfloat16 *HT) {
+  pdl_wait();
   tile_bf16_pair(R, C, H, HT, [&](int r, int c) {
     const size_t e = (size_t)r * C + c;
     const float z = partial_sum(P, e) + bias[c];
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(TT * TY) k_bias_gelu(const Partials P,
 __global__ void __launch_bounds__(256) k_output(const Partials P, const float *__restrict__ bias,
                                                 int C, float *__restrict__ Y, int B, int n_out,
                                                 float *__restrict__ out) {
+  pdl_wait();
   const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (e >= P.n) return;
   const int r = (int)(e / C), c = (int)(e - (size_t)r * C);
@@ -175,6 +178,7 @@ __global__ void __launch_bounds__(TT * TY) k_gelu_back(const Partials P,
                                                       int B, int R, int C, __nv_bfloat16 *dZb,
                                                       __nv_bfloat16 *dZbT, unsigned *done,
                                                       float *__restrict__ db) {
+  pdl_wait();
   tile_bf16_pair(R, C, dZb, dZbT, [&](int r, int c) {
     const size_t e = (size_t)r * C + c;
     const float d = partial_sum(P, e) * gelu_grad_f(Z[e]);
@@ -191,6 +195,7 @@ __global__ void __launch_bounds__(TT * TY) k_loss_grad(
     const float *__restrict__ Y, const float *__restrict__ T, int B, int n_out, int Bp,
     int out_pad, float scale, float *dYf, __nv_bfloat16 *dYb, __nv_bfloat16 *dYbT, unsigned *done,
     float *__restrict__ db, float *__restrict__ part, float inv_count, float *__restrict__ loss) {
+  pdl_wait();
   __shared__ float s_sq[2][TY];
   float sq = 0.f;
   tile_bf16_pair(Bp, out_pad, dYb, dYbT, [&](int r, int c) {
@@ -261,6 +266,7 @@ struct AdamArgs {
 };
 __global__ void __launch_bounds__(TT * 8) k_adam(const AdamArgs A, float lr_t, float b1, float b2,
                                                  float eps) {
+  pdl_wait();
   __shared__ __nv_bfloat16 tile[kAdamC][TT + 2];   // transposed
   const int blk = blockIdx.x, lane = threadIdx.x, warp = threadIdx.y;
   if (blk >= A.first[3]) {
@@ -439,6 +445,7 @@ template <int NB, bool GELU, bool VX>
 __global__ void __launch_bounds__(kGemvWarps * 32) k_mlp_gemv(
     const __nv_bfloat16 *__restrict__ W, int ldw, const float *__restrict__ x, int ldx, int K,
     int n_out, int nb, const float *__restrict__ bias, float *__restrict__ out, int ldo) {
+  pdl_wait();
   __shared__ float s_w[kGemvWarps][kGemvRows * NB];
   const int o0 = blockIdx.x * kGemvRows;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -702,25 +709,22 @@ extern "C" int specula_mlp_forward(specula_mlp *p, const float *X_dev, int32_t b
   const int in = p->np[0], h1 = p->np[1], h2 = p->np[2], o = p->np[3];
   const dim3 tb(TT, TY);
   int s;
-  SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                 k_pack_input<<<dim3(in / TT, Bp / TT), tb, 0, st>>>(
-                     X_dev, batch, p->n[0], Bp, in, p->Xb.as<__nv_bfloat16>(),
-                     p->XbT.as<__nv_bfloat16>()));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_pack_input, dim3(in / TT, Bp / TT), tb, 0, X_dev,
+                     batch, p->n[0], Bp, in, p->Xb.as<__nv_bfloat16>(),
+                     p->XbT.as<__nv_bfloat16>());
   const void *Hin = p->Xb.p;
   Partials P;
   for (int l = 0; l < 2; ++l) {
     const int K = p->np[l], N = p->np[l + 1];
     if ((s = mlp_gemm(p, Hin, p->Wb[l].p, Bp, N, K, &P, st))) return s;
-    SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                   k_bias_gelu<<<dim3(N / TT, Bp / TT), tb, 0, st>>>(
-                       P, p->b[l].as<float>(), p->Z[l].as<float>(), Bp, N,
-                       p->H[l].as<__nv_bfloat16>(), p->HT[l].as<__nv_bfloat16>()));
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_bias_gelu, dim3(N / TT, Bp / TT), tb, 0, P,
+                       p->b[l].as<float>(), p->Z[l].as<float>(), Bp, N,
+                       p->H[l].as<__nv_bfloat16>(), p->HT[l].as<__nv_bfloat16>());
     Hin = p->H[l].p;
   }
   if ((s = mlp_gemm(p, Hin, p->Wb[2].p, Bp, o, h2, &P, st))) return s;
-  SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                 k_output<<<(unsigned)((P.n + 255) / 256), 256, 0, st>>>(
-                     P, p->b[2].as<float>(), o, p->Y.as<float>(), batch, p->n[3], Y_dev));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_output, (unsigned)((P.n + 255) / 256), 256, 0, P,
+                     p->b[2].as<float>(), o, p->Y.as<float>(), batch, p->n[3], Y_dev);
   p->last_b = batch;
   (void)h1;
   return SPECULA_OK;
@@ -739,23 +743,21 @@ extern "C" int specula_mlp_infer(specula_mlp *p, const float *X_dev, int32_t bat
   const bool vx = p->n[0] % 4 == 0 && (uintptr_t)X_dev % 16 == 0;
   auto grid = [](int n) { return (unsigned)((n + kGemvRows - 1) / kGemvRows); };
 #define SPECULA_GEMV1(NB, VX)                                                                \
-  SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,                                                     \
-                 (k_mlp_gemv<NB, true, VX><<<grid(h1), kGemvWarps * 32, 0, st>>>(            \
-                     W0, p->np[0], X_dev, p->n[0], p->n[0], h1, batch, p->b[0].as<float>(),  \
-                     H0, h1)))
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, (k_mlp_gemv<NB, true, VX>), grid(h1),                \
+                     kGemvWarps * 32, 0, W0, p->np[0], X_dev, p->n[0], p->n[0], h1, batch,        \
+                     p->b[0].as<float>(), H0, h1)
 #define SPECULA_GEMV(NB)                                                                     \
   do {                                                                                       \
     if (vx)                                                                                  \
       SPECULA_GEMV1(NB, true);                                                               \
     else                                                                                     \
       SPECULA_GEMV1(NB, false);                                                              \
-    SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,                                                   \
-                   (k_mlp_gemv<NB, true, true><<<grid(h2), kGemvWarps * 32, 0, st>>>(        \
-                       W1, p->np[1], H0, h1, h1, h2, batch, p->b[1].as<float>(), H1, h2)));  \
-    SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,                                                   \
-                   (k_mlp_gemv<NB, false, true><<<grid(p->n[3]), kGemvWarps * 32, 0, st>>>(  \
-                       W2, p->np[2], H1, h2, h2, p->n[3], batch, p->b[2].as<float>(), Y_dev, \
-                       p->n[3])));                                                           \
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, (k_mlp_gemv<NB, true, true>), grid(h2),            \
+                       kGemvWarps * 32, 0, W1, p->np[1], H0, h1, h1, h2, batch,                   \
+                       p->b[1].as<float>(), H1, h2); \
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, (k_mlp_gemv<NB, false, true>), grid(p->n[3]),      \
+                       kGemvWarps * 32, 0, W2, p->np[2], H1, h2, h2, p->n[3], batch,              \
+                       p->b[2].as<float>(), Y_dev, p->n[3]); \
   } while (0)
   if (batch == 1)
     SPECULA_GEMV(1);
@@ -777,24 +779,21 @@ extern "C" int specula_mlp_backward(specula_mlp *p, const float *T_dev, int32_t 
   const float scale = 2.0f / ((float)batch * (float)p->n[3]);
   const dim3 gl(o / TT, Bp / TT);
   int s;
-  SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                 k_loss_grad<<<gl, tb, 0, st>>>(
-                     p->Y.as<float>(), T_dev, batch, p->n[3], Bp, o, scale,
-                     p->dYf.as<float>(), p->dYb.as<__nv_bfloat16>(), p->dYbT.as<__nv_bfloat16>(),
-                     p->done.as<unsigned>(), p->gb[2].as<float>(),
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_loss_grad, gl, tb, 0, p->Y.as<float>(), T_dev,
+                     batch, p->n[3], Bp, o, scale, p->dYf.as<float>(), p->dYb.as<__nv_bfloat16>(),
+                     p->dYbT.as<__nv_bfloat16>(), p->done.as<unsigned>(), p->gb[2].as<float>(),
                      p->part.as<float>(), 1.0f / ((float)batch * (float)p->n[3]),
-                     loss_dev ? loss_dev : p->loss.as<float>()));
+                     loss_dev ? loss_dev : p->loss.as<float>());
   // layer 3: dW3 = dY^T H2, dH2 = dY W3
   Partials P;
   if ((s = mlp_gemm_dw(p, 2, p->dYbT.p, p->HT[1].p, Bp, st))) return s;
   if ((s = mlp_gemm(p, p->dYb.p, p->WbT[2].p, Bp, h2, o, &P, st))) return s;
   for (int l = 1; l >= 0; --l) {
     const int N = p->np[l + 1];
-    SPECULA_LAUNCH(ctx, SPECULA_K_MLP, st,
-                   k_gelu_back<<<dim3(N / TT, Bp / TT), tb, 0, st>>>(
-                       P, p->Z[l].as<float>(), p->dA[l].as<float>(), batch, Bp, N,
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_gelu_back, dim3(N / TT, Bp / TT), tb, 0, P,
+                       p->Z[l].as<float>(), p->dA[l].as<float>(), batch, Bp, N,
                        p->dZb[l].as<__nv_bfloat16>(), p->dZbT[l].as<__nv_bfloat16>(),
-                       p->done.as<unsigned>(), p->gb[l].as<float>()));
+                       p->done.as<unsigned>(), p->gb[l].as<float>());
     const void *HinT = l == 1 ? p->HT[0].p : p->XbT.p;
     if ((s = mlp_gemm_dw(p, l, p->dZbT[l].p, HinT, Bp, st))) return s;
     if (l == 1)
@@ -823,8 +822,7 @@ extern "C" int specula_mlp_adam(specula_mlp *p, float lr, float b1, float b2, fl
     A.first[l + 1] = A.first[l] + (R / TT) * (C / kAdamC);
     A.bias_first[l + 1] = A.bias_first[l] + (R + TT * 8 - 1) / (TT * 8);
   }
-  SPECULA_LAUNCH(p->ctx, SPECULA_K_MLP, st,
-                 k_adam<<<A.first[3] + A.bias_first[3], dim3(TT, 8), 0, st>>>(A, (float)lr_t, b1,
-                                                                           b2, eps));
+  SPECULA_LAUNCH_PDL(p->ctx, SPECULA_K_MLP, st, k_adam, A.first[3] + A.bias_first[3], dim3(TT, 8),
+                     0, A, (float)lr_t, b1, b2, eps);
   return SPECULA_OK;
 }

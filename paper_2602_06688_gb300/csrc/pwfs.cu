@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(256) k_field(const float *__restrict__ amp,
                                                const float *__restrict__ phase,
                                                float2 *__restrict__ field, int npix2, int b0,
                                                int nbw, float phase_scale) {
+  pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= npix2) return;
   const int b = b0 + blockIdx.y;
@@ -423,6 +424,7 @@ __global__ void __launch_bounds__(RowFiltLaunch<N1, N2>::threads,
     const float2 *__restrict__ twA, const float2 *__restrict__ twB,
     const float2 *__restrict__ mask, float2 *__restrict__ rows_out, int n_pix, int nc, int nbw,
     int slot0, int n_slots, int ka, int s0) {
+  pdl_wait();
   using P = PadRegs<N1, N2, PAD>;
   using K = Pack<N1, N2>;
   constexpr int N = K::N, S1 = K::S1, S2 = K::S2;
@@ -562,6 +564,7 @@ __global__ void __launch_bounds__(MAXT, N2 > 32 ? 3 : (MAXT <= 160 ? 4 : (MAXT <
     const float2 *__restrict__ twA, const float2 *__restrict__ twB,
     const float2 *__restrict__ mask, float *__restrict__ part, int n_pix, int fp, int fq,
     float scale, int n_mod, int nc, int nbw, int slot0, int tc, int s0) {
+  pdl_wait();
   using P = PadRegs<N1, N2, PAD>;
   using K = Pack<N1, N2>;
   constexpr int N = K::N, S1 = K::S1, S2 = K::S2, CS = K::XS;
@@ -678,6 +681,7 @@ __global__ void __launch_bounds__(MAXT, N2 > 32 ? 3 : (MAXT <= 160 ? 4 : (MAXT <
 __global__ void __launch_bounds__(256) k_bin_reduce(const float *__restrict__ part,
                                                     float *__restrict__ det, int nd2, int n_mod,
                                                     int nbw, int b0, float alpha, float beta) {
+  pdl_wait();
   const int pix = blockIdx.x * blockDim.x + threadIdx.x;
   if (pix >= nd2) return;
   const int b = b0 + blockIdx.y;
@@ -830,9 +834,8 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
     const int fb = std::max(b0, field_done + 1);
     if (fb <= b1) {
       dim3 gF((Np * Np + 255) / 256, b1 - fb + 1);
-      SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_FIELD, st,
-                     k_field<<<gF, 256, 0, st>>>(amp, phase, p->field.as<float2>(), Np * Np, fb,
-                                                 p->nbw, p->run_phase_scale));
+      SPECULA_LAUNCH_PDL(ctx, SPECULA_K_PWFS_FIELD, st, k_field, gF, 256, 0, amp, phase,
+                         p->field.as<float2>(), Np * Np, fb, p->nbw, p->run_phase_scale);
       field_done = b1;
     }
     dim3 gR((Np + vpc - 1) / vpc, (nj + p->ka - 1) / p->ka);
@@ -841,17 +844,16 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
     for_pad<N1, N2>(p->pad, [&](auto pc) {
       constexpr int PAD = decltype(pc)::value;
       s = [&]() -> int {
-        SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_ROWFILT, st,
-                       k_rowfilt<N1, N2, PAD><<<gR, p->blockR, p->smemR, st>>>(
-                           p->field.as<float2>(), p->gx.as<float2>(), p->tpA.as<float2>(),
-                           p->tpB.as<float2>(), p->mask.as<float2>(), p->rows.as<float2>(), Np,
-                           nc, p->nbw, j0, nj, p->ka, s0));
+        SPECULA_LAUNCH_PDL(ctx, SPECULA_K_PWFS_ROWFILT, st, (k_rowfilt<N1, N2, PAD>), gR,
+                           p->blockR, p->smemR, p->field.as<float2>(), p->gx.as<float2>(),
+                           p->tpA.as<float2>(), p->tpB.as<float2>(), p->mask.as<float2>(),
+                           p->rows.as<float2>(), Np, nc, p->nbw, j0, nj, p->ka, s0);
 #define SPECULA_COLFILT(MAXT_)                                                                 \
-  SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_COLFILT, st,                                              \
-                 k_colfilt_bin<N1, N2, PAD, MAXT_><<<gK, p->blockK, p->smemK, st>>>(           \
-                     p->rows.as<float2>(), p->gy.as<float2>(), p->tpA.as<float2>(),            \
-                     p->tpB.as<float2>(), p->mask.as<float2>(), p->part.as<float>(), Np, p->fp, \
-                     p->fq, scale, p->n_mod, nc, p->nbw, j0, p->tcK, s0))
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_PWFS_COLFILT, st, (k_colfilt_bin<N1, N2, PAD, MAXT_>), gK,    \
+                     p->blockK, p->smemK, p->rows.as<float2>(), p->gy.as<float2>(),               \
+                     p->tpA.as<float2>(), p->tpB.as<float2>(), p->mask.as<float2>(),              \
+                     p->part.as<float>(), Np, p->fp, p->fq, scale, p->n_mod, nc, p->nbw, j0,      \
+                     p->tcK, s0)
         if constexpr (K::CTA) {
           SPECULA_COLFILT(160);
         } else {
@@ -870,10 +872,9 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
     const int complete = (j0 + nj) / nc - 1;
     if (complete > det_done) {
       dim3 gD((nd * nd + 255) / 256, complete - det_done);
-      SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_BIN, st,
-                     k_bin_reduce<<<gD, 256, 0, st>>>(p->part.as<float>(), det, nd * nd,
-                                                      p->n_mod, p->nbw, det_done + 1,
-                                                      p->run_alpha, p->run_beta));
+      SPECULA_LAUNCH_PDL(ctx, SPECULA_K_PWFS_BIN, st, k_bin_reduce, gD, 256, 0,
+                         p->part.as<float>(), det, nd * nd, p->n_mod, p->nbw, det_done + 1,
+                         p->run_alpha, p->run_beta);
       det_done = complete;
     }
   }
@@ -901,9 +902,8 @@ static int run_split(specula_ctx *ctx, PwfsPlan *p, const float *amp, const floa
       const int fb = std::max(b0, field_done + 1);
       if (fb <= b1) {
         dim3 gF((Np * Np + 255) / 256, b1 - fb + 1);
-        SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_FIELD, st,
-                       k_field<<<gF, 256, 0, st>>>(amp, phase, p->field.as<float2>(), Np * Np, fb,
-                                                   p->nbw, p->run_phase_scale));
+        SPECULA_LAUNCH_PDL(ctx, SPECULA_K_PWFS_FIELD, st, k_field, gF, 256, 0, amp, phase,
+                           p->field.as<float2>(), Np * Np, fb, p->nbw, p->run_phase_scale);
         field_done = b1;
       }
       dim3 gA((Np + vpcA - 1) / vpcA, (ni + p->ka - 1) / p->ka);
@@ -928,10 +928,9 @@ static int run_split(specula_ctx *ctx, PwfsPlan *p, const float *amp, const floa
       const int complete = (i0 + ni) / p->n_mod - 1;
       if (complete > det_done) {
         dim3 gD((nd * nd + 255) / 256, complete - det_done);
-        SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_BIN, st,
-                       k_bin_reduce<<<gD, 256, 0, st>>>(p->part.as<float>(), det, nd * nd,
-                                                        p->n_mod, p->nbw, det_done + 1,
-                                                        p->run_alpha, p->run_beta));
+        SPECULA_LAUNCH_PDL(ctx, SPECULA_K_PWFS_BIN, st, k_bin_reduce, gD, 256, 0,
+                           p->part.as<float>(), det, nd * nd, p->n_mod, p->nbw, det_done + 1,
+                           p->run_alpha, p->run_beta);
         det_done = complete;
       }
     }
@@ -990,9 +989,8 @@ int pwfs_set_tiles(PwfsPlan *p, int chunk, int ka, int passes) {
 
 int pwfs_bin_reduce(specula_ctx *ctx, const float *part, float *det, int nd2, int n_mod,
                     float alpha, float beta, cudaStream_t st) {
-  SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_BIN, st,
-                 k_bin_reduce<<<dim3((nd2 + 255) / 256, 1), 256, 0, st>>>(part, det, nd2, n_mod,
-                                                                          1, 0, alpha, beta));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_PWFS_BIN, st, k_bin_reduce, dim3((nd2 + 255) / 256, 1), 256, 0,
+                     part, det, nd2, n_mod, 1, 0, alpha, beta);
   return SPECULA_OK;
 }
 
@@ -1000,18 +998,16 @@ int pwfs_field_launch(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
                       int fb, int nb, cudaStream_t st) {
   const int Np = p->n_pix;
   dim3 gF((Np * Np + 255) / 256, nb);
-  SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_FIELD, st,
-                 k_field<<<gF, 256, 0, st>>>(amp, phase, p->field.as<float2>(), Np * Np, fb, p->nbw,
-                                             p->run_phase_scale));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_PWFS_FIELD, st, k_field, gF, 256, 0, amp, phase,
+                     p->field.as<float2>(), Np * Np, fb, p->nbw, p->run_phase_scale);
   return SPECULA_OK;
 }
 
 int pwfs_bin_reduce_range(specula_ctx *ctx, PwfsPlan *p, float *det, int nd2, int b0, int nb,
                           cudaStream_t st) {
   dim3 gD((nd2 + 255) / 256, nb);
-  SPECULA_LAUNCH(ctx, SPECULA_K_PWFS_BIN, st,
-                 k_bin_reduce<<<gD, 256, 0, st>>>(p->part.as<float>(), det, nd2, p->n_mod, p->nbw,
-                                                  b0, p->run_alpha, p->run_beta));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_PWFS_BIN, st, k_bin_reduce, gD, 256, 0, p->part.as<float>(),
+                     det, nd2, p->n_mod, p->nbw, b0, p->run_alpha, p->run_beta);
   return SPECULA_OK;
 }
 

@@ -39,6 +39,7 @@ template <int NB, bool SPLIT>
 __global__ void __launch_bounds__(kReconWarps * 32) k_mvm_bf16(
     const uint16_t *__restrict__ Rh, const uint16_t *__restrict__ Rl, const float *__restrict__ s,
     float *__restrict__ m, int n_modes, int n_slopes, int n_batch, int b0) {
+  pdl_wait();
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= n_modes) return;
@@ -98,6 +99,7 @@ __global__ void __launch_bounds__(256) k_convert_bf16(const float *__restrict__ 
                                                       uint16_t *__restrict__ hi,
                                                       uint16_t *__restrict__ lo, size_t n,
                                                       int vec) {
+  pdl_wait();
   const size_t nt = (size_t)gridDim.x * blockDim.x;
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   const size_t n8 = vec ? n / 8 : 0;
@@ -182,9 +184,9 @@ static int recon_gemm(specula_ctx *ctx, const specula_recon_desc *rec, const flo
   uint8_t *w = static_cast<uint8_t *>(ctx->recon_ws.p);
   uint16_t *xh = reinterpret_cast<uint16_t *>(w), *xl = reinterpret_cast<uint16_t *>(w + xb);
   float *part = reinterpret_cast<float *>(w + 2 * xb);
-  SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st,
-                 k_convert_bf16<<<(unsigned)std::min<size_t>((nx / 8 + 255) / 256 + 1, 8192), 256,
-                                  0, st>>>(X, xh, xl, nx, convert_vec(X, xh, xl)));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_RECON, st, k_convert_bf16,
+                     (unsigned)std::min<size_t>((nx / 8 + 255) / 256 + 1, 8192), 256, 0, X, xh, xl,
+                     nx, convert_vec(X, xh, xl));
   const void *A3[3] = {xh, xh, xl}, *B3[3] = {rec->R_dev, rec->R_lo_dev, rec->R_dev};
   const void *A2[2] = {xh, xl}, *B2[2] = {rec->R_dev, rec->R_dev};
   return split ? gemm_bf16_terms(ctx, 3, A3, B3, nb, N, K, modes, splits, part, st)
@@ -225,11 +227,19 @@ extern "C" int specula_recon(specula_ctx *ctx, const specula_recon_desc *rec,
         const bool one = n_batch - b0 == 1;
         const uint16_t *h = (const uint16_t *)rec->R_dev, *l = (const uint16_t *)rec->R_lo_dev;
         if (split) {
-          if (one) SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st, k_mvm_bf16<1, true><<<grid1, blk1, 0, st>>>(h, l, slopes_dev, modes_dev, rec->n_modes, rec->n_slopes, n_batch, b0));
-          else SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st, k_mvm_bf16<NB, true><<<grid, blk, 0, st>>>(h, l, slopes_dev, modes_dev, rec->n_modes, rec->n_slopes, n_batch, b0));
+          if (one) SPECULA_LAUNCH_PDL(ctx, SPECULA_K_RECON, st, (k_mvm_bf16<1, true>), grid1, blk1,
+                                      0, h, l, slopes_dev, modes_dev, rec->n_modes, rec->n_slopes,
+                                      n_batch, b0);
+          else SPECULA_LAUNCH_PDL(ctx, SPECULA_K_RECON, st, (k_mvm_bf16<NB, true>), grid, blk, 0,
+                                  h, l, slopes_dev, modes_dev, rec->n_modes, rec->n_slopes,
+                                  n_batch, b0);
         } else {
-          if (one) SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st, k_mvm_bf16<1, false><<<grid1, blk1, 0, st>>>(h, l, slopes_dev, modes_dev, rec->n_modes, rec->n_slopes, n_batch, b0));
-          else SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st, k_mvm_bf16<NB, false><<<grid, blk, 0, st>>>(h, l, slopes_dev, modes_dev, rec->n_modes, rec->n_slopes, n_batch, b0));
+          if (one) SPECULA_LAUNCH_PDL(ctx, SPECULA_K_RECON, st, (k_mvm_bf16<1, false>), grid1,
+                                      blk1, 0, h, l, slopes_dev, modes_dev, rec->n_modes,
+                                      rec->n_slopes, n_batch, b0);
+          else SPECULA_LAUNCH_PDL(ctx, SPECULA_K_RECON, st, (k_mvm_bf16<NB, false>), grid, blk, 0,
+                                  h, l, slopes_dev, modes_dev, rec->n_modes, rec->n_slopes,
+                                  n_batch, b0);
         }
       }
       return SPECULA_OK;

@@ -69,6 +69,7 @@ template <int V>
 __global__ void __launch_bounds__(kSplitWarps * 32) k_mvm_f32_split(
     const float *__restrict__ R, const float *__restrict__ s, float *__restrict__ m, int n_modes,
     int n_slopes) {
+  pdl_wait();
   using T = typename VecOf<V>::T;
   __shared__ float s_w[kSplitWarps];
   const int row = blockIdx.x;
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(256, TileCfg<RM, RN>::CTAS) k_mvm_f32_tile(
   constexpr int BN = C::BN, STAGES = C::STAGES, LM = C::LM, LN = C::LN;
   constexpr int kStage = (kTm + BN) * kTld;
   extern __shared__ __align__(16) float sm_f[];
+  pdl_wait();
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int tile = blockIdx.x / cs;
@@ -275,20 +277,10 @@ static int launch_tile(specula_ctx *ctx, const float *R, const float *s, float *
   if (tiles * cs > 0x7fffffffLL) return SPECULA_EUNSUPPORTED;
   int e = ensure_dynamic_smem((const void *)k_mvm_f32_tile<RM, RN, V>, C::smem);
   if (e) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles * cs));
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = C::smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cs;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
   SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st,
-                 SPECULA_CK(cudaLaunchKernelEx(&cfg, k_mvm_f32_tile<RM, RN, V>, R, s, m, n_modes,
-                                               n_slopes, nb, tiles_n)));
+                 SPECULA_CK(launch_pdl((k_mvm_f32_tile<RM, RN, V>), (unsigned)(tiles * cs), 256,
+                                       C::smem, st, cs > 1 ? cs : 0, R, s, m, n_modes, n_slopes,
+                                       nb, tiles_n)));
   return SPECULA_OK;
 }
 
@@ -296,9 +288,8 @@ template <int V>
 static int run_v(specula_ctx *ctx, const float *R, const float *s, float *m, int n_modes,
                  int n_slopes, int nb, cudaStream_t st) {
   if (nb == 1)
-    SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st,
-                   k_mvm_f32_split<V><<<n_modes, kSplitWarps * 32, 0, st>>>(R, s, m, n_modes,
-                                                                            n_slopes));
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_RECON, st, (k_mvm_f32_split<V>), n_modes, kSplitWarps * 32,
+                       0, R, s, m, n_modes, n_slopes);
   else if (nb <= 8)
     return launch_tile<4, 2, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
   else if (nb <= 16)

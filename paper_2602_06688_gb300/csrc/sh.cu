@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(kShWarps * 32) k_sh_spots(
     const float *__restrict__ amp, const float *__restrict__ phase,
     const int32_t *__restrict__ valid, const float2 *__restrict__ pre, int n_pix, int n_sub,
     int n_valid, int n_batch, float phase_scale, float *__restrict__ spots) {
+  pdl_wait();
   constexpr int OFF = (NF - SP) / 2;
   constexpr int XS = SP | 1;
   __shared__ float2 s_x[kShWarps][NF * XS];
@@ -127,25 +128,21 @@ int sh_run(specula_ctx *ctx, ShPlan *p, const float *amp, const float *phase, in
   if (tasks == 0) return SPECULA_OK;
   const unsigned grid = (unsigned)((tasks + kShWarps - 1) / kShWarps);
   if (p->fft_n == 24 && p->sub_pix == 12)
-    SPECULA_LAUNCH(ctx, SPECULA_K_SH, st,
-                   k_sh_spots<24, 12><<<grid, kShWarps * 32, 0, st>>>(
-                       amp, phase, valid, p->pre.as<float2>(), p->n_pix, p->n_sub, nv, n_batch,
-                       phase_scale, spots));
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_SH, st, (k_sh_spots<24, 12>), grid, kShWarps * 32, 0, amp,
+                       phase, valid, p->pre.as<float2>(), p->n_pix, p->n_sub, nv, n_batch,
+                       phase_scale, spots);
   else if (p->fft_n == 16 && p->sub_pix == 8)
-    SPECULA_LAUNCH(ctx, SPECULA_K_SH, st,
-                   k_sh_spots<16, 8><<<grid, kShWarps * 32, 0, st>>>(
-                       amp, phase, valid, p->pre.as<float2>(), p->n_pix, p->n_sub, nv, n_batch,
-                       phase_scale, spots));
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_SH, st, (k_sh_spots<16, 8>), grid, kShWarps * 32, 0, amp,
+                       phase, valid, p->pre.as<float2>(), p->n_pix, p->n_sub, nv, n_batch,
+                       phase_scale, spots);
   else if (p->fft_n == 56 && p->sub_pix == 8)   // Tab. 2's SCAO SH spots (56 = 8 x 7)
-    SPECULA_LAUNCH(ctx, SPECULA_K_SH, st,
-                   k_sh_spots<56, 8><<<grid, kShWarps * 32, 0, st>>>(
-                       amp, phase, valid, p->pre.as<float2>(), p->n_pix, p->n_sub, nv, n_batch,
-                       phase_scale, spots));
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_SH, st, (k_sh_spots<56, 8>), grid, kShWarps * 32, 0, amp,
+                       phase, valid, p->pre.as<float2>(), p->n_pix, p->n_sub, nv, n_batch,
+                       phase_scale, spots);
   else if (p->fft_n == 68 && p->sub_pix == 4)   // Tab. 2's ERIS spots (68 = 4 x 17)
-    SPECULA_LAUNCH(ctx, SPECULA_K_SH, st,
-                   k_sh_spots<68, 4><<<grid, kShWarps * 32, 0, st>>>(
-                       amp, phase, valid, p->pre.as<float2>(), p->n_pix, p->n_sub, nv, n_batch,
-                       phase_scale, spots));
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_SH, st, (k_sh_spots<68, 4>), grid, kShWarps * 32, 0, amp,
+                       phase, valid, p->pre.as<float2>(), p->n_pix, p->n_sub, nv, n_batch,
+                       phase_scale, spots);
   else
     return SPECULA_EUNSUPPORTED;
   return SPECULA_OK;

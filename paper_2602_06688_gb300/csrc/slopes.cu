@@ -32,6 +32,7 @@ __device__ __forceinline__ void guard_finite(float a, float b, int32_t *nf_statu
 __global__ void __launch_bounds__(kPyrThreads) k_pyr_slopes(
     const float *__restrict__ det, const int32_t *__restrict__ idx, const float *__restrict__ ref,
     int n_sub, int n_valid, float *__restrict__ out, int32_t *status, int32_t *nf_status) {
+  pdl_wait();
   __shared__ float s_w[kPyrThreads / 32];
   __shared__ float s_T;
   const int b = blockIdx.y;
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(kPyrThreads) k_pyr_slopes(
 __global__ void __launch_bounds__(kPyrThreads) k_pyr_slopes_maps(
     const float *__restrict__ det, const int32_t *__restrict__ map, const float *__restrict__ ref,
     int n_det2, int n_valid, float *__restrict__ out, int32_t *status, int32_t *nf_status) {
+  pdl_wait();
   __shared__ float s_w[kPyrThreads / 32];
   __shared__ float s_T;
   const int b = blockIdx.y;
@@ -175,6 +177,7 @@ __global__ void __launch_bounds__(256) k_sh_cog(const float *__restrict__ spots,
                                                 const float *__restrict__ ref, int nf,
                                                 int n_valid, int n_batch,
                                                 float *__restrict__ out, int32_t *nf_status) {
+  pdl_wait();
   const long long task = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (task >= (long long)n_valid * n_batch) return;   // warp-uniform
@@ -206,11 +209,10 @@ __global__ void __launch_bounds__(256) k_sh_cog(const float *__restrict__ spots,
 
 int slopes_pyr_run(specula_ctx *ctx, const int32_t *idx, int n_sub, int n_valid,
                    const float *det, const float *ref, int n_batch, float *out, cudaStream_t st) {
-  SPECULA_LAUNCH(ctx, SPECULA_K_SLOPES, st,
-                 k_pyr_slopes<<<dim3((n_valid + kPyrThreads - 1) / kPyrThreads, n_batch),
-                                kPyrThreads, 0, st>>>(det, idx, ref, n_sub, n_valid, out,
-                                                      ctx->status_dev,
-                                                      ctx->guard ? ctx->status_dev : nullptr));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_SLOPES, st, k_pyr_slopes,
+                     dim3((n_valid + kPyrThreads - 1) / kPyrThreads, n_batch), kPyrThreads, 0, det,
+                     idx, ref, n_sub, n_valid, out, ctx->status_dev,
+                     ctx->guard ? ctx->status_dev : nullptr);
   return SPECULA_OK;
 }
 
@@ -231,18 +233,16 @@ extern "C" int specula_slopes(specula_ctx *ctx, const specula_slopec_desc *d, co
                           slopes_dev, st);
   } else if (d->kind == SPECULA_SLOPES_PYR_MAPS) {
     if (!d->subap_idx_dev || d->n_sub < 1) return SPECULA_EINVAL;
-    SPECULA_LAUNCH(ctx, SPECULA_K_SLOPES, st,
-                   k_pyr_slopes_maps<<<dim3((d->n_valid + kPyrThreads - 1) / kPyrThreads, n_batch),
-                                       kPyrThreads, 0, st>>>(
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_SLOPES, st, k_pyr_slopes_maps,
+                       dim3((d->n_valid + kPyrThreads - 1) / kPyrThreads, n_batch), kPyrThreads, 0,
                        img_dev, d->subap_idx_dev, ref_dev, d->n_sub * d->n_sub, d->n_valid,
-                       slopes_dev, ctx->status_dev, ctx->guard ? ctx->status_dev : nullptr));
+                       slopes_dev, ctx->status_dev, ctx->guard ? ctx->status_dev : nullptr);
   } else if (d->kind == SPECULA_SLOPES_SH) {
     if (d->fft_n < 2) return SPECULA_EINVAL;
     const long long tasks = (long long)d->n_valid * n_batch;
-    SPECULA_LAUNCH(ctx, SPECULA_K_SLOPES, st,
-                   k_sh_cog<<<(unsigned)((tasks + 7) / 8), 256, 0, st>>>(
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_SLOPES, st, k_sh_cog, (unsigned)((tasks + 7) / 8), 256, 0,
                        img_dev, ref_dev, d->fft_n, d->n_valid, n_batch, slopes_dev,
-                       ctx->guard ? ctx->status_dev : nullptr));
+                       ctx->guard ? ctx->status_dev : nullptr);
   } else {
     return SPECULA_EINVAL;
   }
