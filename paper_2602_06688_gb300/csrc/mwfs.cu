@@ -406,16 +406,15 @@ __device__ void mw_field(const MwParams &P, const MwSensor &S, int y0, int y1, f
 // The CTA extracts the phase of their pixels as one strip of SP rows x
 // W = kMwShSubPerTask SP column slots (slot c: subaperture c / SP, column
 // c % SP), then one warp per subaperture images it: the spot arithmetic of
-// k_sh_spots, with the centre of gravity taken in registers.
+// centre of gravity taken in registers.
 template <int NF, int SP>
 struct MwShSmem {
   static constexpr int W = kMwShSubPerTask * SP;                        // column slots
   static constexpr int kPh = kMwShSubPerTask * SP * SP;                 // floats
   static constexpr int kTab = 2 * kMwLayerChunk * (W + SP);             // int + float
   static constexpr int kWin = 4096;                                     // one screen window
-  static constexpr int kFft = kMwWarps * NF * (SP | 1) * 2;            // floats
+  static constexpr int kFft = kMwShSubPerTask * NF * (SP | 1) * 2;     // floats
   static_assert(kFft <= kTab + 2 * kWin, "the FFT exchange reuses the extraction space");
-  static_assert((W * SP) % kMwThreads == 0, "whole pixels per thread");
   static constexpr size_t bytes = (size_t)(kPh + kTab + 2 * kWin + 2 * kMwShSubPerTask) * 4;
 };
 
@@ -427,14 +426,24 @@ struct MwShSmem {
 // star, so slots 0 and ns SP - 1, rows 0 and SP - 1 bound it) and the
 // interpolation reads it there; otherwise it gathers from the screen.  Both
 // read the same samples: the result is that of k_atmo_extract.
-template <int SP, int PPT>
+//
+// One thread per column slot, all SP rows: the column's index and fraction are
+// read once per layer, and a screen row's horizontal interpolation serves the
+// pupil rows above and below it (the rows' indices are the same for every
+// thread, so the reuse is a uniform branch).  About 9 instructions per pixel
+// and layer; one thread per pixel, each with its own index arithmetic and four
+// samples, took about 35 (39 m system frame, with the packed rows below:
+// 320.1 -> 275.4 us).
+template <int SP>
 __device__ __forceinline__ void mw_sh_extract(const MwParams &P, const MwSensor &S, int ns,
                                               const int *s_ab, int *s_i, float *s_f,
-                                              float *s_win, int win_cap, float (&acc)[PPT]) {
+                                              float *s_win, int win_cap, float (&acc)[SP]) {
   constexpr int W = kMwShSubPerTask * SP, PER = W + SP;
+  static_assert(W <= kMwThreads, "a thread per column slot");
 #pragma unroll
-  for (int i = 0; i < PPT; ++i) acc[i] = 0.f;
+  for (int i = 0; i < SP; ++i) acc[i] = 0.f;
   if (P.flat) return;
+  const int c = threadIdx.x;   // this thread's column slot
   const int n = S.n_pix, wc = ns * SP, arow = s_ab[0];
   for (int l0 = 0; l0 < P.n_layers; l0 += kMwLayerChunk) {
     const int lc = min(kMwLayerChunk, P.n_layers - l0);
@@ -509,46 +518,51 @@ __device__ __forceinline__ void mw_sh_extract(const MwParams &P, const MwSensor 
       const int *ti = s_i + l * PER;
       const float *tf = s_f + l * PER;
       int x0, y0, wx, wy;
-      if (win_geom(l, x0, y0, wx, wy)) {   // uniform over the CTA
+      const bool win = win_geom(l, x0, y0, wx, wy);   // uniform over the CTA
+      if (c < wc) {
+        const float fx = tf[c];
+        const int ix = ti[c];
+        // one column of the strip: rowY gives the screen row below a pupil
+        // row, next the one above it, row(y) the screen row y at this column
+        const auto column = [&](auto rowY, auto next, auto row) {
+          int at = -2;   // the row that `lo` holds
+          float lo = 0.f, hi = 0.f;
 #pragma unroll
-        for (int i = 0; i < PPT; ++i) {
-          const int q = threadIdx.x + i * kMwThreads;
-          const int r = q / W, c = q - r * W;
-          if (c < wc) {
-            int cx = ti[c] - x0, cy = ti[W + r] - y0;
-            if (cx < 0) cx += M;
-            if (cy < 0) cy += M;
-            if (cx > wx - 2 || cy > wy - 2) {   // never with the host's task split
-              atomicExch(P.status, SPECULA_EINVAL);
-              cx = min(cx, wx - 2);
-              cy = min(cy, wy - 2);
+          for (int r = 0; r < SP; ++r) {
+            const int cy = rowY(ti[W + r]);
+            const float fy = tf[W + r];
+            if (cy != at) {   // uniform over the CTA
+              lo = cy == at + 1 ? hi : row(cy);
+              hi = row(next(cy));
+              at = cy;
             }
-            const float fx = tf[c], fy = tf[W + r];
-            const float *w0 = cur + cy * wx + cx;
-            const float s00 = w0[0], s01 = w0[1], s10 = w0[wx], s11 = w0[wx + 1];
-            const float a = s00 + fx * (s01 - s00);
-            const float b = s10 + fx * (s11 - s10);
-            acc[i] += a + fy * (b - a);
+            acc[r] += lo + fy * (hi - lo);
           }
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < PPT; ++i) {
-          const int q = threadIdx.x + i * kMwThreads;
-          const int r = q / W, c = q - r * W;
-          if (c < wc) {
-            const int ix0 = ti[c], iy0 = ti[W + r];
-            const float fx = tf[c], fy = tf[W + r];
-            const int ix1 = ix0 + 1 == M ? 0 : ix0 + 1;
-            const int iy1 = iy0 + 1 == M ? 0 : iy0 + 1;
-            const float s00 = __ldg(Sc + (size_t)iy0 * M + ix0);
-            const float s01 = __ldg(Sc + (size_t)iy0 * M + ix1);
-            const float s10 = __ldg(Sc + (size_t)iy1 * M + ix0);
-            const float s11 = __ldg(Sc + (size_t)iy1 * M + ix1);
-            const float a = s00 + fx * (s01 - s00);
-            const float b = s10 + fx * (s11 - s10);
-            acc[i] += a + fy * (b - a);
-          }
+        };
+        if (win) {
+          const auto inside = [&](int v, int v0, int w) {   // offset in the window
+            int q = v - v0;
+            if (q < 0) q += M;
+            if (q > w - 2) {   // never with the host's task split
+              atomicExch(P.status, SPECULA_EINVAL);
+              q = w - 2;
+            }
+            return q;
+          };
+          const float *base = cur + inside(ix, x0, wx);
+          column([&](int y) { return inside(y, y0, wy); }, [&](int y) { return y + 1; },
+                 [&](int y) {
+                   const float s0 = base[y * wx], s1 = base[y * wx + 1];
+                   return s0 + fx * (s1 - s0);
+                 });
+        } else {
+          const int ix1 = ix + 1 == M ? 0 : ix + 1;
+          column([&](int y) { return y; }, [&](int y) { return y + 1 == M ? 0 : y + 1; },
+                 [&](int y) {
+                   const float s0 = __ldg(Sc + (size_t)y * M + ix);
+                   const float s1 = __ldg(Sc + (size_t)y * M + ix1);
+                   return s0 + fx * (s1 - s0);
+                 });
         }
       }
       __syncthreads();   // readers of `cur` are done before it is refilled
@@ -562,7 +576,6 @@ __device__ void mw_sh(const MwParams &P, const MwSensor &S, int v0, int v1, floa
   constexpr int XS = SP | 1;
   using L = MwShSmem<NF, SP>;
   constexpr int W = L::W;
-  constexpr int PPT = W * SP / kMwThreads;
   float *ph = reinterpret_cast<float *>(smem);
   float *region = ph + L::kPh;                     // tables + window, then FFT exchange
   float *s_win = region + L::kTab;                 // two windows
@@ -576,55 +589,52 @@ __device__ void mw_sh(const MwParams &P, const MwSensor &S, int v0, int v1, floa
   __syncthreads();
   int *s_i = reinterpret_cast<int *>(region);
   float *s_f = region + kMwLayerChunk * (W + SP);
-  float acc[PPT];
-  mw_sh_extract<SP, PPT>(P, S, ns, s_ab, s_i, s_f, s_win, L::kWin, acc);
-  const int n = S.n_pix;
+  float acc[SP];
+  mw_sh_extract<SP>(P, S, ns, s_ab, s_i, s_f, s_win, L::kWin, acc);
+  const int n = S.n_pix, cs = threadIdx.x;
+  if (cs < ns * SP) {
+    const int sub = cs / SP, c = cs % SP;
+    float *dst = S.phase + (size_t)s_ab[sub] * SP * n + (size_t)s_ab[kMwShSubPerTask + sub] * SP + c;
 #pragma unroll
-  for (int i = 0; i < PPT; ++i) {
-    const int q = threadIdx.x + i * kMwThreads;
-    const int r = q / W, cs = q - r * W;
-    if (cs < ns * SP) {
-      const int sub = cs / SP, c = cs % SP;
-      const float f = acc[i] * S.scale;
+    for (int r = 0; r < SP; ++r) {
+      const float f = acc[r] * S.scale;
       ph[sub * SP * SP + r * SP + c] = f;
-      S.phase[(size_t)(s_ab[sub] * SP + r) * n + (size_t)s_ab[kMwShSubPerTask + sub] * SP + c] = f;
+      dst[(size_t)r * n] = f;
     }
   }
   __syncthreads();
-  const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
-  float2 *xs = reinterpret_cast<float2 *>(region) + w * (NF * XS);
-  for (int sub = w; sub < ns; sub += kMwWarps) {
-    const int v = v0 + sub;
-    const int a = s_ab[sub], bc = s_ab[kMwShSubPerTask + sub];
-    const float *phs = ph + sub * SP * SP;
+  // Rows: one thread per (subaperture, row), packed over the CTA (a warp per
+  // subaperture kept 12 of 32 lanes); the padded half of the inputs is zero
+  // and left out.
+  constexpr nzmask NZ = nz_range(OFF, OFF + SP);
+  float2 *xs = reinterpret_cast<float2 *>(region);
+  if (threadIdx.x < ns * SP) {
+    const int sub = threadIdx.x / SP, r = threadIdx.x % SP;
+    const float *phs = ph + sub * SP * SP + r * SP;
+    const float *am = S.amp + (size_t)(s_ab[sub] * SP + r) * n +
+                      (size_t)s_ab[kMwShSubPerTask + sub] * SP;
+    const float2 py = __ldg(S.pre + OFF + r);
     float2 vv[NF];
 #pragma unroll
-    for (int q = 0; q < NF; ++q) vv[q] = make_float2(0.f, 0.f);
-    if (lane < SP) {
-      const float *am = S.amp + (size_t)(a * SP + lane) * n + (size_t)bc * SP;
-      const float2 py = __ldg(S.pre + OFF + lane);
-#pragma unroll
-      for (int c = 0; c < SP; ++c) {
-        float sv, cv;
-        sincosf(phs[lane * SP + c], &sv, &cv);
-        const float A = __ldg(am + c);
-        vv[OFF + c] = cmul(cmul(make_float2(A * cv, A * sv), __ldg(S.pre + OFF + c)), py);
-      }
+    for (int c = 0; c < SP; ++c) {
+      float sv, cv;
+      sincosf(phs[c], &sv, &cv);
+      const float A = __ldg(am + c);
+      vv[OFF + c] = cmul(cmul(make_float2(A * cv, A * sv), __ldg(S.pre + OFF + c)), py);
     }
-    RegDFT<NF, false>::run(vv);
-    __syncwarp();
-    if (lane < SP) {
+    RegDFTZ<NF, false, NZ>::run(vv);
 #pragma unroll
-      for (int k = 0; k < NF; ++k) xs[k * XS + lane] = vv[k];
-    }
-    __syncwarp();
+    for (int k = 0; k < NF; ++k) xs[(sub * NF + k) * XS + r] = vv[k];
+  }
+  __syncthreads();
+  const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
+  for (int sub = w; sub < ns; sub += kMwWarps) {
+    const int v = v0 + sub;
+    float2 vv[NF];
+    const float2 *xk = xs + (sub * NF + min(lane, NF - 1)) * XS;
 #pragma unroll
-    for (int q = 0; q < NF; ++q) vv[q] = make_float2(0.f, 0.f);
-    if (lane < NF) {
-#pragma unroll
-      for (int r = 0; r < SP; ++r) vv[OFF + r] = xs[lane * XS + r];
-    }
-    RegDFT<NF, false>::run(vv);
+    for (int r = 0; r < SP; ++r) vv[OFF + r] = xk[r];
+    RegDFTZ<NF, false, NZ>::run(vv);
     // lane k holds column k of the spot: vv[q] at row q
     float si = 0.f, sx = 0.f, sy = 0.f;
     if (lane < NF) {
@@ -652,7 +662,6 @@ __device__ void mw_sh(const MwParams &P, const MwSensor &S, int v0, int v1, floa
       P.slopes[S.slope_off + S.n_valid + v] = gy;
       mw_guard(gx, gy, P.nf_status);
     }
-    __syncwarp();
   }
 }
 
