@@ -55,6 +55,7 @@ extern "C" int specula_ctx_create(specula_ctx **out, int device) {
   }
   int s = pwfs_init_device();
   if (!s) s = sh_init_device();
+  if (!s) s = screens_init_device();
   if (!s) s = mwfs_init_device();
   if (!s) s = pwfs_shifted_init_device();
   if (!s) s = pwfs_pair_init_device();

@@ -257,6 +257,7 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
 
 // per-translation-unit device initialisation (constant tables)
 int pwfs_init_device();
+int screens_init_device();
 int sh_init_device();
 int mwfs_init_device();
 // float64 helpers of the calibration file, shared with the infinite screens:

@@ -103,11 +103,112 @@ __global__ void k_screen_final(const double2 *__restrict__ T, const double2 *__r
   }
 }
 
-// four standard normals for counter (pair index, sample, stream)
+// ---- Box-Muller in float64 ------------------------------------------------------
+// (r cos 2 pi v, r sin 2 pi v), r = sqrt(-2 ln u), with the uniforms u, v =
+// (x + 1/2) 2^-32 of two Philox words.  float64 runs at 2 operations per clock
+// and SM here and the normals are most of a batch of screens, so the functions
+// are written for these arguments, 33-bit integers over 2^33: table lookups
+// after exact integer range reduction and short polynomials (the table-driven
+// method of Tang, ACM TOMS 16, 378, 1990, for the logarithm; addition theorems
+// for sine and cosine; Goldschmidt's iteration for the square root), about 39
+// float64 operations per pair where log, sqrt and sincospi took about twice
+// that (256 screens of 256^2, pass 1: 2.79 -> 1.63 ms).  Largest errors
+// on the CPU over 6 million arguments: radius 1.7e-16 relative, angle 2.1e-16.
+constexpr int kLogFirst = 90, kLogCount = 91;   // j = 90 .. 180
+// c = 128 / j rounded, and 2 ln c and 2 n ln 2 as multiples of 2^-40, whose sums
+// are exact, with their remainders
+static __device__ double2 d_bm_log[kLogCount];  // (c, 2 ln c high)
+static __device__ double d_bm_log_lo[kLogCount];
+static __device__ double2 d_bm_exp[34];
+static __device__ double2 d_bm_trig[257];       // (cos, sin) 2 pi k / 256
+
+int screens_init_device() {
+  double2 lg[kLogCount], ex[34], tr[257];
+  double lo[kLogCount];
+  const auto high = [](long double v) { return rint((double)(v * 0x1p40L)) * 0x1p-40; };
+  for (int j = 0; j < kLogCount; ++j) {
+    const double c = 128.0 / (double)(kLogFirst + j);
+    const long double l = 2.0L * logl((long double)c);
+    lg[j] = make_double2(c, high(l));
+    lo[j] = (double)(l - (long double)lg[j].y);
+  }
+  for (int n = 0; n < 34; ++n) {
+    const long double l = 2.0L * n * logl(2.0L);
+    ex[n].x = high(l);
+    ex[n].y = (double)(l - (long double)ex[n].x);
+  }
+  for (int k = 0; k <= 256; ++k) {
+    // reduced to an eighth of a turn: the argument's rounding stays below 2^-54
+    const int a = k % 64, q = (k / 64) % 4;
+    const double x = M_PI * (a <= 32 ? a : 64 - a) / 128.0;
+    const double c = a <= 32 ? cos(x) : sin(x), s = a <= 32 ? sin(x) : cos(x);
+    const double cq[4] = {c, -s, -c, s}, sq[4] = {s, c, -s, -c};
+    tr[k] = make_double2(cq[q], sq[q]);
+  }
+  SPECULA_CK(cudaMemcpyToSymbol(d_bm_log, lg, sizeof(lg)));
+  SPECULA_CK(cudaMemcpyToSymbol(d_bm_log_lo, lo, sizeof(lo)));
+  SPECULA_CK(cudaMemcpyToSymbol(d_bm_exp, ex, sizeof(ex)));
+  SPECULA_CK(cudaMemcpyToSymbol(d_bm_trig, tr, sizeof(tr)));
+  return SPECULA_OK;
+}
+
+// sqrt(-2 ln((x + 1/2) 2^-32)).  With m = 2 x + 1 = f 2^k, f in [1, 2) or, from
+// 181/128 on, halved: -2 ln u = 2 (33 - k) ln 2 + 2 ln c - 2 ln(1 + r), r = f c - 1,
+// c = 128 / j for the nearest j / 128 to f, |r| <= 0.5 / 90; near u = 1 both
+// table terms are zero, so small results keep their relative accuracy.
+__device__ __forceinline__ double bm_radius(uint32_t x) {
+  const int k = 32 - __clz(x);   // bit length of x: m has its top bit there
+  const uint64_t m = 2ull * x + 1ull;
+  const uint64_t mant = (m << (52 - k)) & 0xFFFFFFFFFFFFFull;
+  const int j1 = 128 + (((int)(mant >> 44) + 1) >> 1);
+  const bool half = j1 > 180;
+  const int j = half ? 64 + (((int)(mant >> 45) + 1) >> 1) : j1;
+  const double f = __longlong_as_double((long long)(mant | ((half ? 1022ull : 1023ull) << 52)));
+  const double2 cl = __ldg(d_bm_log + (j - kLogFirst));
+  const double2 en = __ldg(d_bm_exp + (33 - k - (half ? 1 : 0)));
+  const double lo = en.y + __ldg(d_bm_log_lo + (j - kLogFirst));
+  const double r = fma(f, cl.x, -1.0), r2 = r * r;
+  double p = fma(r, -2.0 / 7.0, 1.0 / 3.0);
+  p = fma(r, p, -2.0 / 5.0);
+  p = fma(r, p, 0.5);
+  p = fma(r, p, -2.0 / 3.0);
+  p = fma(r, p, 1.0);
+  const double t = (en.x + cl.y) + fma(-2.0, r, fma(r2, p, lo));
+  const double y = (double)rsqrtf((float)t);
+  double g = t * y, h = 0.5 * y;
+  const double e = fma(-g, h, 0.5);
+  g = fma(g, e, g);
+  h = fma(h, e, h);
+  return fma(fma(-g, g, t), h, g);
+}
+
+// (cos, sin) of 2 pi (x + 1/2) 2^-32: the nearest k / 256 of a turn from the
+// table, the rest |theta| <= pi / 256 by Taylor polynomials to theta^7
+__device__ __forceinline__ double2 bm_angle(uint32_t x) {
+  const uint32_t k = (uint32_t)(((uint64_t)x + (1u << 23)) >> 24);
+  const int q = (int)(2ll * x + 1ll - ((long long)k << 25));   // 2^33 of a turn
+  const double th = (__longlong_as_double(0x4338000000000000ll + q) - 6755399441055744.0) *
+                    (2.0 * M_PI / 8589934592.0);
+  const double2 cs = __ldg(d_bm_trig + k);
+  const double t2 = th * th;
+  const double s = fma(th * t2, fma(t2, fma(t2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0), th);
+  const double c1 = t2 * fma(t2, fma(t2, -1.0 / 720.0, 1.0 / 24.0), -0.5);   // cos - 1
+  return make_double2(fma(cs.x, c1, fma(-cs.y, s, cs.x)), fma(cs.y, c1, fma(cs.x, s, cs.y)));
+}
+
+// four standard normals for counter (pair index, sample, stream): words 0 / 1
+// and 2 / 3, each (r cos, r sin)
 __device__ __forceinline__ void normals4(uint64_t pair, uint32_t sample, uint32_t stream,
                                          uint64_t seed, double g[4]) {
   uint32_t c[4] = {(uint32_t)pair, (uint32_t)(pair >> 32), sample, stream};
-  philox_normals4(c, seed, g);
+  philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double r = bm_radius(c[2 * i]);
+    const double2 a = bm_angle(c[2 * i + 1]);
+    g[2 * i] = r * a.x;
+    g[2 * i + 1] = r * a.y;
+  }
 }
 
 // n complex normals per sample: element 2i, 2i+1 from counter i
@@ -134,8 +235,8 @@ __global__ void k_rng_complex(uint64_t seed, int sample0, int stream_id, long lo
 //    transforms take two real columns at a time: half the transforms.
 //  * The subharmonics are separable: per column nine products, per pixel six
 //    fused multiply-adds.
-// 256 screens of 256^2 now: 2.79 ms (pass 1, of which the Box-Muller normals
-// are about 2.3) and 0.81 ms (pass 2).
+// 256 screens of 256^2 now: 1.63 ms (pass 1, most of it the Box-Muller
+// normals) and 0.81 ms (pass 2).
 // Pass 1 (k_screen_rows) draws rows ky and -ky, combines and transforms them;
 // pass 2 (k_screen_cols) transforms the columns, adds the subharmonics and
 // rounds to float32 once.
