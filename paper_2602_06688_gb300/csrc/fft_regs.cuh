@@ -377,7 +377,8 @@ template <bool A, bool X> __device__ __forceinline__ float2 cfma_z(float2 c, flo
 
 typedef unsigned long long nzmask;
 constexpr nzmask nz_full(int n) { return n >= 64 ? ~0ull : ((1ull << n) - 1ull); }
-constexpr bool nz_bit(nzmask m, int j) { return (m >> j) & 1ull; }
+// (inputs from 64 on are zero)
+constexpr bool nz_bit(nzmask m, int j) { return j < 64 && ((m >> j) & 1ull); }
 constexpr nzmask nz_range(int lo, int hi) { return nz_full(hi) & ~nz_full(lo); }
 // masks of the sub-transforms: inputs n1 + P n2 (Cooley-Tukey), (a B + b A) mod N
 // (prime factor)
