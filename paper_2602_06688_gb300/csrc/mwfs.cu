@@ -41,6 +41,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <queue>
 
 #include "fft_regs.cuh"
 #include "internal.h"
@@ -59,7 +60,8 @@ constexpr int kMwMaxLayers = 64;
 constexpr int kMwShSubPerTask = 16;
 constexpr int kMwCoordsPerTask = kMwThreads;
 constexpr int kMwBinPerTask = 1024;
-constexpr int kMwMvmRows = 32;
+constexpr int kMwMvmRows = 16;
+constexpr int kMwShLayers = 16;              // layers whose tables an SH task stages at once
 constexpr int kMwFinalRows = 1024;
 constexpr unsigned long long kMwWaitNs = 2000000000ull;      // default wait limit
 constexpr long long kMwWaitMaxNs = 10000000000ll;            // largest settable limit
@@ -105,6 +107,7 @@ struct MwParams {
   int *ctr;                    // [0] ticket, [1] CTAs done, [2] abort, [3..] dependencies
   double t_host;
   const double *t_dev;
+  unsigned long long scr_vec;  // bit l set if layer l's rows start on 16-byte boundaries
   int flat;                    // 1: flat wavefront (reference slopes)
   const float *R;
   int n_modes, n_slopes, r_vec4;
@@ -176,8 +179,12 @@ __device__ __forceinline__ void cp_async4(void *smem_dst, const void *gsrc) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gsrc) : "memory");
 }
+__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gsrc) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // ---- extraction ------------------------------------------------------------------
 // Table entries [e0, e1) of [layer][axis][pixel] (same arithmetic as
@@ -409,155 +416,191 @@ __device__ void mw_field(const MwParams &P, const MwSensor &S, int y0, int y1, f
 // centre of gravity taken in registers.
 template <int NF, int SP>
 struct MwShSmem {
-  static constexpr int W = kMwShSubPerTask * SP;                        // column slots
   static constexpr int kPh = kMwShSubPerTask * SP * SP;                 // floats
-  static constexpr int kTab = 2 * kMwLayerChunk * (W + SP);             // int + float
   static constexpr int kWin = 4096;                                     // one screen window
-  static constexpr int kFft = kMwShSubPerTask * NF * (SP | 1) * 2;     // floats
-  static_assert(kFft <= kTab + 2 * kWin, "the FFT exchange reuses the extraction space");
-  static constexpr size_t bytes = (size_t)(kPh + kTab + 2 * kWin + 2 * kMwShSubPerTask) * 4;
+  static constexpr int kGeo = kMwShLayers * (SP * 2 + 8);               // rows, windows
+  static constexpr int kFft = kMwShSubPerTask * NF * (SP | 1) * 2;
+  static constexpr int kRegion = kFft > 2 * kWin ? kFft : 2 * kWin;     // windows, then FFTs
+  static constexpr size_t bytes = (size_t)(kPh + kRegion + kGeo + 2 * kMwShSubPerTask) * 4;
+  static_assert(kPh % 4 == 0 && kRegion % 4 == 0 && kWin % 4 == 0, "16-byte windows");
 };
 
-// Strip extraction: per chunk of layers the table entries of the W column
-// slots and SP rows go to shared memory; per layer, when the host marked
-// the layer's span as shorter than the screen (S.win_ok), the screen window
-// the strip samples is staged in shared memory with coalesced row loads
+// Strip extraction: when the host marked a layer's span as shorter than the
+// screen (S.win_ok), the screen window the strip samples is staged in shared
+// memory with coalesced row loads
 // (the sampling coordinate grows with the pupil coordinate below the guide
 // star, so slots 0 and ns SP - 1, rows 0 and SP - 1 bound it) and the
 // interpolation reads it there; otherwise it gathers from the screen.  Both
 // read the same samples: the result is that of k_atmo_extract.
 //
 // One thread per column slot, all SP rows: the column's index and fraction are
-// read once per layer, and a screen row's horizontal interpolation serves the
+// read once per layer (a layer ahead, straight from the tables), and a screen row's horizontal interpolation serves the
 // pupil rows above and below it (the rows' indices are the same for every
-// thread, so the reuse is a uniform branch).  About 9 instructions per pixel
-// and layer; one thread per pixel, each with its own index arithmetic and four
-// samples, took about 35 (39 m system frame, with the packed rows below:
-// 320.1 -> 275.4 us).
+// thread, so the reuse is a uniform branch).  What bounds it is instructions:
+// the rows' offsets in the window and each layer's window are worked out once
+// per chunk of layers (mw_sh_window), and windows are copied 16 bytes at a
+// time where the screen's rows allow it.  At 13.8 subapertures and ten layers
+// a task's extraction went from 45800 cycles to 26300, three CTAs to an SM
+// (4-byte copies, index arithmetic per row and thread, the columns' tables
+// through shared memory); more shared memory than this costs it again: the
+// table of 12 layers took 36300, of 8 layers 32900 (less L1 for the rest).
+struct MwWin {
+  int xa, y0, nu, wy;        // first screen column copied, first row, units per row, rows
+  int stride, x0, wx, unit;  // floats per window row, first column used, its width; floats
+                             // per unit (4 or 1; 0: no window, gather from the screen)
+};
+
+// The window of a strip on one layer: x0..x1, y0..y1 the screen samples of its
+// first and last column and row.
+__device__ __forceinline__ MwWin mw_sh_window(int x0, int x1, int y0, int y1, int M, bool ok,
+                                              bool vec, int cap) {
+  MwWin g;
+  g.x0 = x0;
+  g.y0 = y0;
+  g.wx = (x1 - x0 + M) % M + 2;
+  g.wy = (y1 - y0 + M) % M + 2;
+  g.xa = x0 & ~3;
+  g.nu = (x0 - g.xa + g.wx + 3) / 4;
+  g.stride = 4 * g.nu;
+  g.unit = 4;
+  if (!vec || g.stride * g.wy > cap) {
+    g.xa = x0;
+    g.nu = g.stride = g.wx;
+    g.unit = 1;
+  }
+  if (!ok || g.stride * g.wy > cap) g.unit = 0;
+  return g;
+}
+
 template <int SP>
 __device__ __forceinline__ void mw_sh_extract(const MwParams &P, const MwSensor &S, int ns,
-                                              const int *s_ab, int *s_i, float *s_f,
-                                              float *s_win, int win_cap, float (&acc)[SP]) {
-  constexpr int W = kMwShSubPerTask * SP, PER = W + SP;
-  static_assert(W <= kMwThreads, "a thread per column slot");
+                                              const int *s_ab, float *s_win, int win_cap,
+                                              MwWin *s_geo, int2 *s_row, float (&acc)[SP]) {
+  static_assert(kMwShSubPerTask * SP <= kMwThreads && kMwShLayers * SP <= kMwThreads,
+                "a thread per column slot, per row of a layer");
+  constexpr int CL = 64;      // threads along a window row in the copy
 #pragma unroll
   for (int i = 0; i < SP; ++i) acc[i] = 0.f;
   if (P.flat) return;
-  const int c = threadIdx.x;   // this thread's column slot
-  const int n = S.n_pix, wc = ns * SP, arow = s_ab[0];
-  for (int l0 = 0; l0 < P.n_layers; l0 += kMwLayerChunk) {
-    const int lc = min(kMwLayerChunk, P.n_layers - l0);
+  const int c = threadIdx.x, n = S.n_pix, wc = ns * SP;   // this thread's column slot
+  const int row0 = s_ab[0] * SP, colA = s_ab[kMwShSubPerTask] * SP;
+  const int colZ = s_ab[kMwShSubPerTask + ns - 1] * SP + SP - 1;
+  // this column's table entries, read a layer ahead
+  const int col = c < wc ? s_ab[kMwShSubPerTask + c / SP] * SP + c % SP : colA;
+  int nix = __ldcg(S.tab_i + col);
+  float nfx = __ldcg(S.tab_f + col);
+  for (int l0 = 0; l0 < P.n_layers; l0 += kMwShLayers) {
+    const int lc = min(kMwShLayers, P.n_layers - l0);
     __syncthreads();
-    // all of this thread's table loads in flight before any store
-    constexpr int TPT = (kMwLayerChunk * PER + kMwThreads - 1) / kMwThreads;
-    int vi[TPT];
-    float vf[TPT];
-#pragma unroll
-    for (int k = 0; k < TPT; ++k) {
-      const int e = threadIdx.x + k * kMwThreads;
-      if (e < lc * PER) {
-        const int l = e / PER, r = e - l * PER;
-        int pix, axis = 0;
-        if (r < W) {
-          const int c = r < wc ? r : wc - 1;   // unused slots repeat the last column
-          pix = s_ab[kMwShSubPerTask + c / SP] * SP + c % SP;
-        } else {
-          pix = arow * SP + (r - W);
-          axis = 1;
+    // per layer its window, per row of a layer its offset there and fraction
+    if (threadIdx.x < lc * SP) {
+      const int l = threadIdx.x / SP, r = threadIdx.x % SP;
+      const int *tx = S.tab_i + (size_t)(2 * (l0 + l)) * n, *ty = tx + n + row0;
+      const int x0 = __ldcg(tx + colA), x1 = __ldcg(tx + colZ);
+      const int y0 = __ldcg(ty), y1 = __ldcg(ty + SP - 1);
+      int y = __ldcg(ty + r);
+      const float fy = __ldcg(S.tab_f + (size_t)(2 * (l0 + l) + 1) * n + row0 + r);
+      const int M = P.L[l0 + l].side;
+      const MwWin g = mw_sh_window(x0, x1, y0, y1, M, (S.win_ok >> (l0 + l)) & 1ull,
+                                   (P.scr_vec >> (l0 + l)) & 1ull, win_cap);
+      if (g.unit) {
+        y -= g.y0;
+        if (y < 0) y += M;
+        if (y > g.wy - 2) {    // never with the host's task split
+          atomicExch(P.status, SPECULA_EINVAL);
+          y = g.wy - 2;
         }
-        const size_t o = (size_t)(2 * (l0 + l) + axis) * n + pix;
-        vi[k] = __ldcg(S.tab_i + o);
-        vf[k] = __ldcg(S.tab_f + o);
+        y *= g.stride;
       }
-    }
-#pragma unroll
-    for (int k = 0; k < TPT; ++k) {
-      const int e = threadIdx.x + k * kMwThreads;
-      if (e < lc * PER) {
-        s_i[e] = vi[k];
-        s_f[e] = vf[k];
-      }
+      s_row[l * SP + r] = make_int2(y, __float_as_int(fy));
+      if (r == 0) s_geo[l] = g;
     }
     __syncthreads();
     // windows double-buffered: layer l + 1's window is copied (cp.async)
     // while layer l interpolates from the other buffer
-    auto win_geom = [&](int l, int &x0, int &y0, int &wx, int &wy) {
-      const int *ti = s_i + l * PER;
-      const int M = P.L[l0 + l].side;
-      x0 = ti[0];
-      y0 = ti[W];
-      wx = (ti[wc - 1] - x0 + M) % M + 2;
-      wy = (ti[W + SP - 1] - y0 + M) % M + 2;
-      return ((S.win_ok >> (l0 + l)) & 1ull) && wx * wy <= win_cap;
-    };
-    auto issue = [&](int l, float *buf) {
-      int x0, y0, wx, wy;
-      if (!win_geom(l, x0, y0, wx, wy)) return;
+    auto issue = [&](int l) {
+      const MwWin g = s_geo[l];
       const float *Sc = P.L[l0 + l].scr;
       const int M = P.L[l0 + l].side;
-      for (int c = threadIdx.x; c < wx; c += kMwThreads) {
-        int xx = x0 + c;
-        if (xx >= M) xx -= M;
-        for (int r = 0; r < wy; ++r) {
-          int yy = y0 + r;
-          if (yy >= M) yy -= M;
-          cp_async4(buf + r * wx + c, Sc + (size_t)yy * M + xx);
+      float *buf = s_win + (l & 1) * win_cap;
+      if (g.unit) {
+        for (int u = threadIdx.x % CL; u < g.nu; u += CL) {
+          int xx = g.xa + u * g.unit;
+          if (xx >= M) xx -= M;
+          for (int r = threadIdx.x / CL; r < g.wy; r += kMwThreads / CL) {
+            int yy = g.y0 + r;
+            if (yy >= M) yy -= M;
+            float *d = buf + r * g.stride + u * g.unit;
+            const float *src = Sc + (size_t)yy * M + xx;
+            if (g.unit == 4) cp_async16(d, src);
+            else cp_async4(d, src);
+          }
         }
       }
-    };
-    issue(0, s_win);
-    cp_async_commit();
-    for (int l = 0; l < lc; ++l) {
-      float *cur = s_win + (l & 1) * win_cap;
-      if (l + 1 < lc) issue(l + 1, s_win + ((l + 1) & 1) * win_cap);
       cp_async_commit();
-      cp_async_wait_1();     // all but the newest group: layer l's window is in
-      __syncthreads();
-      const float *Sc = P.L[l0 + l].scr;
-      const int M = P.L[l0 + l].side;
-      const int *ti = s_i + l * PER;
-      const float *tf = s_f + l * PER;
-      int x0, y0, wx, wy;
-      const bool win = win_geom(l, x0, y0, wx, wy);   // uniform over the CTA
+    };
+    issue(0);
+    for (int l = 0; l < lc; ++l) {
+      cp_async_wait_all();     // layer l's window
+      __syncthreads();         // everyone's part of it; readers of the other buffer are done
+      if (l + 1 < lc) issue(l + 1);
+      const int ix = nix;
+      const float fx = nfx;
+      if (l0 + l + 1 < P.n_layers) {
+        const size_t o = (size_t)(2 * (l0 + l + 1)) * n + col;
+        nix = __ldcg(S.tab_i + o);
+        nfx = __ldcg(S.tab_f + o);
+      }
       if (c < wc) {
-        const float fx = tf[c];
-        const int ix = ti[c];
-        // one column of the strip: rowY gives the screen row below a pupil
-        // row, next the one above it, row(y) the screen row y at this column
-        const auto column = [&](auto rowY, auto next, auto row) {
-          int at = -2;   // the row that `lo` holds
-          float lo = 0.f, hi = 0.f;
+        const float *Sc = P.L[l0 + l].scr;
+        const int M = P.L[l0 + l].side;
+        const int2 *rows = s_row + l * SP;
+        const MwWin g = s_geo[l];
+        // one column of the strip: next(o) is the row below row o, row(o) the
+        // row's horizontal interpolation at this column.  The rows below are
+        // loaded for every pupil row, so the loads wait for no comparison; the
+        // row itself is the last one's, the row below that, or (screen samples
+        // closer than the pixels) one more load.
+        const auto column = [&](auto next, auto row) {
+          constexpr int B = 4;             // rows whose loads are in flight together
+          int at = rows[0].x;
+          float lo = row(at), below = 0.f;
 #pragma unroll
-          for (int r = 0; r < SP; ++r) {
-            const int cy = rowY(ti[W + r]);
-            const float fy = tf[W + r];
-            if (cy != at) {   // uniform over the CTA
-              lo = cy == at + 1 ? hi : row(cy);
-              hi = row(next(cy));
-              at = cy;
+          for (int r0 = 0; r0 < SP; r0 += B) {
+            int o[B];
+            float hi[B];
+#pragma unroll
+            for (int r = 0; r < B && r0 + r < SP; ++r) {
+              o[r] = rows[r0 + r].x;
+              hi[r] = row(next(o[r]));
             }
-            acc[r] += lo + fy * (hi - lo);
+#pragma unroll
+            for (int r = 0; r < B && r0 + r < SP; ++r) {
+              if (o[r] != at) {            // uniform over the CTA
+                lo = o[r] == next(at) ? below : row(o[r]);
+                at = o[r];
+              }
+              below = hi[r];
+              acc[r0 + r] += lo + __int_as_float(rows[r0 + r].y) * (below - lo);
+            }
           }
         };
-        if (win) {
-          const auto inside = [&](int v, int v0, int w) {   // offset in the window
-            int q = v - v0;
-            if (q < 0) q += M;
-            if (q > w - 2) {   // never with the host's task split
-              atomicExch(P.status, SPECULA_EINVAL);
-              q = w - 2;
-            }
-            return q;
-          };
-          const float *base = cur + inside(ix, x0, wx);
-          column([&](int y) { return inside(y, y0, wy); }, [&](int y) { return y + 1; },
-                 [&](int y) {
-                   const float s0 = base[y * wx], s1 = base[y * wx + 1];
+        if (g.unit) {
+          int q = ix - g.x0;
+          if (q < 0) q += M;
+          if (q > g.wx - 2) {      // never with the host's task split
+            atomicExch(P.status, SPECULA_EINVAL);
+            q = g.wx - 2;
+          }
+          const float *base = s_win + (l & 1) * win_cap + (g.x0 - g.xa) + q;
+          column([&](int o) { return o + g.stride; },
+                 [&](int o) {
+                   const float s0 = base[o], s1 = base[o + 1];
                    return s0 + fx * (s1 - s0);
                  });
         } else {
           const int ix1 = ix + 1 == M ? 0 : ix + 1;
-          column([&](int y) { return y; }, [&](int y) { return y + 1 == M ? 0 : y + 1; },
+          column([&](int y) { return y + 1 == M ? 0 : y + 1; },
                  [&](int y) {
                    const float s0 = __ldg(Sc + (size_t)y * M + ix);
                    const float s1 = __ldg(Sc + (size_t)y * M + ix1);
@@ -565,7 +608,6 @@ __device__ __forceinline__ void mw_sh_extract(const MwParams &P, const MwSensor 
                  });
         }
       }
-      __syncthreads();   // readers of `cur` are done before it is refilled
     }
   }
 }
@@ -575,11 +617,11 @@ __device__ void mw_sh(const MwParams &P, const MwSensor &S, int v0, int v1, floa
   constexpr int OFF = (NF - SP) / 2;
   constexpr int XS = SP | 1;
   using L = MwShSmem<NF, SP>;
-  constexpr int W = L::W;
   float *ph = reinterpret_cast<float *>(smem);
-  float *region = ph + L::kPh;                     // tables + window, then FFT exchange
-  float *s_win = region + L::kTab;                 // two windows
-  int *s_ab = reinterpret_cast<int *>(s_win + 2 * L::kWin);
+  float *region = ph + L::kPh;                     // two windows, then FFT exchange
+  MwWin *s_geo = reinterpret_cast<MwWin *>(region + L::kRegion);
+  int2 *s_row = reinterpret_cast<int2 *>(s_geo + kMwShLayers);
+  int *s_ab = reinterpret_cast<int *>(s_row + kMwShLayers * SP);
   const int ns = v1 - v0;
   for (int k = threadIdx.x; k < ns; k += kMwThreads) {
     const int idx = __ldg(S.valid + v0 + k);
@@ -587,10 +629,8 @@ __device__ void mw_sh(const MwParams &P, const MwSensor &S, int v0, int v1, floa
     s_ab[kMwShSubPerTask + k] = idx % S.n_sub;
   }
   __syncthreads();
-  int *s_i = reinterpret_cast<int *>(region);
-  float *s_f = region + kMwLayerChunk * (W + SP);
   float acc[SP];
-  mw_sh_extract<SP>(P, S, ns, s_ab, s_i, s_f, s_win, L::kWin, acc);
+  mw_sh_extract<SP>(P, S, ns, s_ab, region, L::kWin, s_geo, s_row, acc);
   const int n = S.n_pix, cs = threadIdx.x;
   if (cs < ns * SP) {
     const int sub = cs / SP, c = cs % SP;
@@ -1064,50 +1104,80 @@ struct specula_mwfs {
 
 namespace {
 
-// Emit A in order and release the (independent of each other) tasks of B
-// once the last producer of their dependency went out at least `lag`
-// positions earlier (about two waves of CTAs: by the time a CTA takes such
-// a task, its dependency has most likely completed, so it does not idle).
-// From the first position where some B task is eligible, B tasks leave at a
-// steady rate over the rest of A, in the order they became eligible; what is
-// left follows A.
-void release_when_ready(const std::vector<MwTask> &A, const std::vector<MwTask> &B,
-                        const std::vector<int> &produced_total, std::vector<int> &emitted,
-                        std::vector<MwTask> &out, int lag) {
-  std::vector<long> last_pos(produced_total.size(), -1);
-  std::vector<char> pooled(B.size(), 0);
-  std::vector<size_t> pool;
-  size_t head = 0, n_out = 0;
-  long first = -1;
-  auto eligible = [&](const MwTask &t, long pos) {
-    if (t.wait_ctr < 0) return true;
-    return emitted[t.wait_ctr] >= produced_total[t.wait_ctr] && pos - last_pos[t.wait_ctr] >= lag;
+// Order of the tasks: list scheduling on the host.  The frame is played
+// through with `workers` CTAs: whenever one is free it takes the first task
+// whose dependency has completed, groups searched in priority order, and the
+// order of taking is the ticket order.  A task so placed waits for nothing if
+// the costs are right, and only briefly if they are not (a CTA that draws a
+// ticket early waits for its dependency, so a completion is seen a quarter of
+// the task's cost late here).
+//
+// Groups are tasks of one kind and sensor; tasks of a group go in list order.
+// At most `mvm_cap` CTAs take reconstructor tasks while others are left: a
+// third of the slots draws half the HBM rate while the rest keep computing (a
+// 39 m frame with a half instead: 247 us against 242).  The order before this,
+// sensor after sensor with the pyramids last, left their chains of passes and
+// the last MVM tasks alone on the chip: 274 us against 261.
+struct MwGroup {
+  std::vector<MwTask> t;
+  double cost = 0.;    // per task, microseconds
+  size_t head = 0;
+};
+
+bool schedule_tasks(std::vector<MwGroup> &groups, int n_ctr, int workers, int mvm_cap,
+                    std::vector<MwTask> &out) {
+  struct Ev {
+    double t;
+    int ctr;         // -1: a worker comes free; else a completion is seen
+    bool mvm;
+    bool operator<(const Ev &o) const { return t > o.t; }
   };
-  auto refill = [&](long pos) {
-    for (size_t i = 0; i < B.size(); ++i)
-      if (!pooled[i] && eligible(B[i], pos)) {
-        pooled[i] = 1;
-        pool.push_back(i);
+  std::priority_queue<Ev> q;
+  std::vector<int> done(n_ctr, 0);
+  size_t left = 0, left_other = 0;
+  for (auto &g : groups) {
+    left += g.t.size();
+    if (!g.t.empty() && g.t[0].type != MT_MVM) left_other += g.t.size();
+  }
+  int idle = workers, mvm = 0;
+  double now = 0.;
+  while (left) {
+    bool took = true;
+    while (idle > 0 && took) {
+      took = false;
+      for (auto &g : groups) {
+        if (g.head == g.t.size()) continue;
+        const MwTask &t = g.t[g.head];
+        const bool is_mvm = t.type == MT_MVM;
+        if (is_mvm && left_other && mvm >= mvm_cap) continue;
+        if (t.wait_ctr >= 0 && done[t.wait_ctr] < t.wait_val) continue;
+        out.push_back(t);
+        g.head++;
+        left--;
+        if (!is_mvm) left_other--;
+        idle--;
+        mvm += is_mvm;
+        q.push({now + g.cost, -1, is_mvm});
+        q.push({now + 1.25 * g.cost, t.done_ctr, false});
+        took = true;
+        break;
       }
-  };
-  auto emit = [&](const MwTask &t) {
-    last_pos[t.done_ctr] = (long)out.size();
-    out.push_back(t);
-    emitted[t.done_ctr]++;
-  };
-  for (size_t ia = 0; ia < A.size(); ++ia) {
-    emit(A[ia]);
-    refill((long)out.size());
-    if (first < 0 && head < pool.size()) first = (long)ia;
-    if (first < 0) continue;
-    const double frac = (double)(ia + 1 - first) / (double)(A.size() - first);
-    while (head < pool.size() && (double)n_out < frac * B.size()) {
-      emit(B[pool[head++]]);
-      n_out++;
+    }
+    if (!left) break;
+    if (q.empty()) return false;      // a dependency nothing fulfils
+    now = q.top().t;
+    while (!q.empty() && q.top().t <= now) {
+      const Ev e = q.top();
+      q.pop();
+      if (e.ctr >= 0) {
+        done[e.ctr]++;
+      } else {
+        idle++;
+        mvm -= e.mvm;
+      }
     }
   }
-  refill(1L << 40);
-  while (head < pool.size()) emit(B[pool[head++]]);
+  return true;
 }
 
 MwTask mk(int type, int sensor, int a, int b, int wait_ctr, int wait_val, int done_ctr) {
@@ -1183,6 +1253,7 @@ extern "C" int specula_mwfs_create(specula_ctx *ctx, int32_t n_sensors,
   for (int l = 0; l < n_layers; ++l) {
     P.L[l].scr = screens_dev[l];
     P.L[l].side = layers[l].side;
+    if (layers[l].side % 4 == 0 && (uintptr_t)screens_dev[l] % 16 == 0) P.scr_vec |= 1ull << l;
     P.L[l].pitch = layers[l].pitch_m;
     P.L[l].h = layers[l].height_m;
     P.L[l].vx = layers[l].vx_mps;
@@ -1306,8 +1377,15 @@ extern "C" int specula_mwfs_create(specula_ctx *ctx, int32_t n_sensors,
       n_field(n_sensors, 0), c_sh(n_sensors, -1), n_sh(n_sensors, 0), c_slopes(n_sensors, -1),
       c_rinv(n_sensors, -1), c_bin(n_sensors, -1), n_binv(n_sensors, 0);
   std::vector<std::vector<int>> c_rows(n_sensors), c_cols(n_sensors);
-  std::vector<MwTask> L_coords, L_field, L_pyr, L_sh, L_mvm, L_final;
-  std::vector<std::vector<MwTask>> L_sh_by(n_sensors);
+  // groups by kind and sensor; kinds in the order of MT_*
+  std::vector<std::vector<MwGroup>> by(MT_FINAL + 1, std::vector<MwGroup>(n_sensors));
+  auto add = [&](const MwTask &t, double cost) {
+    MwGroup &g = by[t.type][t.sensor];
+    g.t.push_back(t);
+    g.cost = std::max(g.cost, cost);
+  };
+  // costs in microseconds: each kind's mean with three CTAs to an SM (FIELD and
+  // SH at ten layers, the passes at a 240-point transform, MVM at 27 KB rows)
   const int TC = kMwThreads / G, VPC = kMwThreads / G;
   for (int pass = 0; pass < 2; ++pass)   // pyramids first, then SH
     for (int k = 0; k < n_sensors; ++k) {
@@ -1316,8 +1394,7 @@ extern "C" int specula_mwfs_create(specula_ctx *ctx, int32_t n_sensors,
       c_coords[k] = new_ctr();
       const int ne = n_layers * 2 * n;
       for (int e0 = 0; e0 < ne; e0 += kMwCoordsPerTask) {
-        L_coords.push_back(mk(MT_COORDS, k, e0, std::min(ne, e0 + kMwCoordsPerTask), -1, 0,
-                              c_coords[k]));
+        add(mk(MT_COORDS, k, e0, std::min(ne, e0 + kMwCoordsPerTask), -1, 0, c_coords[k]), 9.);
         n_coords[k]++;
       }
     }
@@ -1325,6 +1402,7 @@ extern "C" int specula_mwfs_create(specula_ctx *ctx, int32_t n_sensors,
     const MwSensor &S = P.S[k];
     const int n = S.n_pix;
     if (m->kind[k] == SPECULA_WFS_SH) {
+      const double sh_px = (double)(n / S.n_sub) * (n / S.n_sub);
       c_sh[k] = new_ctr();
       // runs of valid subapertures in one row spanning < 16 columns, so a
       // task's screen window stays small
@@ -1336,7 +1414,8 @@ extern "C" int specula_mwfs_create(specula_ctx *ctx, int32_t n_sensors,
         while (v1 < S.n_valid && v1 - v0 < kMwShSubPerTask && vl[v1] / S.n_sub == a0 &&
                vl[v1] % S.n_sub - b0 < kMwShSubPerTask)
           ++v1;
-        L_sh_by[k].push_back(mk(MT_SH, k, v0, v1, c_coords[k], n_coords[k], c_sh[k]));
+        add(mk(MT_SH, k, v0, v1, c_coords[k], n_coords[k], c_sh[k]),
+            (v1 - v0) * sh_px * (4e-3 + 0.85e-3 * n_layers));
         n_sh[k]++;
         v0 = v1;
       }
@@ -1348,8 +1427,8 @@ extern "C" int specula_mwfs_create(specula_ctx *ctx, int32_t n_sensors,
     max_field_slots = std::max(max_field_slots, n + rpt);
     if (kMwLayerChunk * (n + rpt) > 4 * kMwThreads) return SPECULA_EUNSUPPORTED;
     for (int y0 = 0; y0 < n; y0 += rpt) {
-      L_field.push_back(mk(MT_FIELD, k, y0, std::min(n, y0 + rpt), c_coords[k], n_coords[k],
-                           c_field[k]));
+      add(mk(MT_FIELD, k, y0, std::min(n, y0 + rpt), c_coords[k], n_coords[k], c_field[k]),
+          2.5 + n_layers);
       n_field[k]++;
     }
     const int nrg = (n + VPC - 1) / VPC, nct = N / TC, nsg = (S.nd + S.spt - 1) / S.spt;
@@ -1360,59 +1439,69 @@ extern "C" int specula_mwfs_create(specula_ctx *ctx, int32_t n_sensors,
     }
     for (int mm = 0; mm < S.n_mod; ++mm)
       for (int rg = 0; rg < nrg; ++rg)
-        L_pyr.push_back(mk(MT_ROWS, k, mm, rg, c_field[k], n_field[k], c_rows[k][mm]));
+        add(mk(MT_ROWS, k, mm, rg, c_field[k], n_field[k], c_rows[k][mm]), 4.);
     for (int mm = 0; mm < S.n_mod; ++mm)
       for (int ct = 0; ct < nct; ++ct)
-        L_pyr.push_back(mk(MT_COLS, k, mm, ct, c_rows[k][mm], nrg, c_cols[k][mm]));
+        add(mk(MT_COLS, k, mm, ct, c_rows[k][mm], nrg, c_cols[k][mm]), 7.);
     for (int mm = 0; mm < S.n_mod; ++mm)
       for (int sg = 0; sg < nsg; ++sg)
-        L_pyr.push_back(mk(MT_RINV, k, mm, sg, c_cols[k][mm], nct, c_rinv[k]));
+        add(mk(MT_RINV, k, mm, sg, c_cols[k][mm], nct, c_rinv[k]), 5.);
     c_bin[k] = new_ctr();
     const int nd2 = S.nd * S.nd;
     for (int p0 = 0; p0 < nd2; p0 += kMwBinPerTask) {
-      L_pyr.push_back(mk(MT_BIN, k, p0, std::min(nd2, p0 + kMwBinPerTask), c_rinv[k],
-                         S.n_mod * nsg, c_bin[k]));
+      add(mk(MT_BIN, k, p0, std::min(nd2, p0 + kMwBinPerTask), c_rinv[k], S.n_mod * nsg, c_bin[k]),
+          5.);
       n_binv[k]++;
     }
     c_slopes[k] = new_ctr();
-    L_pyr.push_back(mk(MT_SLOPES, k, 0, 0, c_bin[k], n_binv[k], c_slopes[k]));
+    add(mk(MT_SLOPES, k, 0, 0, c_bin[k], n_binv[k], c_slopes[k]), 11.);
   }
   const int c_mvm = new_ctr(), c_final = new_ctr();
   int n_mvm = 0;
   if (n_modes > 0) {
-    // pyramids' MVM first: their slopes come first in the ALU list
-    for (int pass = 0; pass < 2; ++pass)
-      for (int k = 0; k < n_sensors; ++k) {
-        const bool pyr = m->kind[k] == SPECULA_WFS_PYR;
-        if ((pass == 0) != pyr) continue;
-        for (int r0 = 0; r0 < n_modes; r0 += kMwMvmRows) {
-          L_mvm.push_back(mk(MT_MVM, k, r0, std::min(n_modes, r0 + kMwMvmRows),
-                             pyr ? c_slopes[k] : c_sh[k], pyr ? 1 : n_sh[k], c_mvm));
-          n_mvm++;
-        }
+    for (int k = 0; k < n_sensors; ++k) {
+      const bool pyr = m->kind[k] == SPECULA_WFS_PYR;
+      for (int r0 = 0; r0 < n_modes; r0 += kMwMvmRows) {
+        add(mk(MT_MVM, k, r0, std::min(n_modes, r0 + kMwMvmRows), pyr ? c_slopes[k] : c_sh[k],
+               pyr ? 1 : n_sh[k], c_mvm),
+            kMwMvmRows * 2. * P.S[k].n_valid * 4. / 30e3);
+        n_mvm++;
       }
+    }
     for (int r0 = 0; r0 < n_modes; r0 += kMwFinalRows)
-      L_final.push_back(mk(MT_FINAL, 0, r0, std::min(n_modes, r0 + kMwFinalRows), c_mvm, n_mvm,
-                           c_final));
+      add(mk(MT_FINAL, 0, r0, std::min(n_modes, r0 + kMwFinalRows), c_mvm, n_mvm, c_final), 5.);
   }
-  // producers per counter, for the merge
-  std::vector<int> produced(nctr, 0), emitted(nctr, 0);
-  auto count = [&](const std::vector<MwTask> &v) { for (auto &t : v) produced[t.done_ctr]++; };
-  count(L_coords); count(L_field); count(L_pyr); count(L_mvm); count(L_final);
-  for (auto &v : L_sh_by) count(v);
-  std::vector<MwTask> A, order;
-  for (auto &t : L_coords) { order.push_back(t); emitted[t.done_ctr]++; }
-  for (auto &t : L_field) { order.push_back(t); emitted[t.done_ctr]++; }
-  // SH sensors one after another (each finishes early and its MVM tasks can
-  // stream R from HBM while the rest compute), then the pyramid passes, whose
-  // dependency chains the MVM tasks fill; the pyramids' own MVM tasks end
-  // the frame.
-  for (int k = 0; k < n_sensors; ++k) A.insert(A.end(), L_sh_by[k].begin(), L_sh_by[k].end());
-  A.insert(A.end(), L_pyr.begin(), L_pyr.end());
-  int sms = 0;
+  m->smem = var->smem(max_slopes, max_field_slots);
+  if (m->smem > 227 * 1024) return SPECULA_EUNSUPPORTED;
+  if ((st = ensure_dynamic_smem((const void *)var->fn, m->smem))) return st;
+  int occ = 0, sms = 0;
+  SPECULA_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, var->fn, kMwThreads, m->smem));
+  if (occ < 1) return SPECULA_EUNSUPPORTED;
   SPECULA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
-  release_when_ready(A, L_mvm, produced, emitted, order, 4 * sms);
-  for (auto &t : L_final) { order.push_back(t); emitted[t.done_ctr]++; }
+  // Priorities: the reconstructor's tasks first (HBM is what the frame cannot
+  // do without, so it streams from the first sensor that is done), then the
+  // first SH sensor, whose slopes release the first of them, then the
+  // pyramids' chains, latest stage first, then the other SH sensors, which
+  // fill every gap the chains leave.
+  std::vector<MwGroup> groups;
+  auto put = [&](int type, int k) { groups.push_back(std::move(by[type][k])); };
+  int first_sh = -1;
+  for (int k = n_sensors - 1; k >= 0; --k)
+    if (m->kind[k] == SPECULA_WFS_SH) first_sh = k;
+  for (int k = 0; k < n_sensors; ++k) put(MT_MVM, k);
+  for (int pass = 0; pass < 2; ++pass)
+    for (int k = 0; k < n_sensors; ++k)
+      if ((pass == 0) == (m->kind[k] == SPECULA_WFS_PYR)) put(MT_COORDS, k);
+  if (first_sh >= 0) put(MT_SH, first_sh);
+  for (int type : {(int)MT_SLOPES, (int)MT_BIN, (int)MT_RINV, (int)MT_COLS, (int)MT_ROWS,
+                   (int)MT_FIELD})
+    for (int k = 0; k < n_sensors; ++k) put(type, k);
+  for (int k = 0; k < n_sensors; ++k)
+    if (k != first_sh) put(MT_SH, k);
+  put(MT_FINAL, 0);
+  std::vector<MwTask> order;
+  if (!schedule_tasks(groups, nctr, sms * occ, std::max(1, sms * occ / 3), order))
+    return SPECULA_EINVAL;
   // every dependency precedes its consumer
   {
     std::vector<int> seen(nctr, 0);
@@ -1433,12 +1522,6 @@ extern "C" int specula_mwfs_create(specula_ctx *ctx, int32_t n_sensors,
   P.wait_ns = kMwWaitNs;
   P.stall_task = -1;
 
-  m->smem = var->smem(max_slopes, max_field_slots);
-  if (m->smem > 227 * 1024) return SPECULA_EUNSUPPORTED;
-  if ((st = ensure_dynamic_smem((const void *)var->fn, m->smem))) return st;
-  int occ = 0;
-  SPECULA_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, var->fn, kMwThreads, m->smem));
-  if (occ < 1) return SPECULA_EUNSUPPORTED;
   m->sm_count = sms;
   m->occupancy = occ;
   m->max_grid = sms * occ;
