@@ -332,7 +332,8 @@ int specula_rng_complex(specula_ctx *ctx, uint64_t seed, int32_t sample0, int32_
  * the Philox complex normals of sample sample0 + b, stream 0 for the FFT
  * grid (element ky * side + kx) and stream 1 for the 27 subharmonic values
  * (element (p * 3 + b) * 3 + a).  screens_dev: n_screens * side^2 floats.
- * Set-up call: the context keeps the float64 work arrays (at most 80 MB of
+ * Values are pairs of float32 (about 48 bits) until the one rounding to float32.
+ * Set-up call: the context keeps the work arrays (at most 80 MB of
  * spectra, or one screen's) for the next one. */
 int specula_screen_generate_batch(specula_ctx *ctx, int32_t n_screens, int32_t side,
                                   double pitch_m, double r0_m, double L0_m, uint64_t seed,

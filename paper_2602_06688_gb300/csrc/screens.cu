@@ -5,7 +5,7 @@
 //   screen[y][x] = Re sum_k c_k sqrt(Phi(f_k)) df exp(2 pi i f_k . (x, y) pitch)
 //                + subharmonics - their spatial mean
 //
-// Everything runs in float64 on the device (a set-up cost, not per frame).
+// A set-up cost, not per frame: float64, and pairs of float32 in the batched form.
 // The single screen from given noise: spectral weighting, a radix-2 Stockham FFT along rows in shared memory, a
 // tiled transpose, the second row pass, and a final kernel that adds the
 // separable subharmonic sum and rounds to float32 once.
@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "float_pair.cuh"
 #include "internal.h"
 #include "philox.cuh"
 
@@ -105,14 +106,15 @@ __global__ void k_screen_final(const double2 *__restrict__ T, const double2 *__r
 
 // ---- Box-Muller in float64 ------------------------------------------------------
 // (r cos 2 pi v, r sin 2 pi v), r = sqrt(-2 ln u), with the uniforms u, v =
-// (x + 1/2) 2^-32 of two Philox words.  float64 runs at 2 operations per clock
-// and SM here and the normals are most of a batch of screens, so the functions
+// (x + 1/2) 2^-32 of two Philox words: the values of specula_rng_complex and the
+// batched screens' subharmonic coefficients (their grids take float32 pairs).
+// float64 runs at 2 operations per clock and SM here, so the functions
 // are written for these arguments, 33-bit integers over 2^33: table lookups
 // after exact integer range reduction and short polynomials (the table-driven
 // method of Tang, ACM TOMS 16, 378, 1990, for the logarithm; addition theorems
 // for sine and cosine; Goldschmidt's iteration for the square root), about 39
 // float64 operations per pair where log, sqrt and sincospi took about twice
-// that (256 screens of 256^2, pass 1: 2.79 -> 1.63 ms).  Largest errors
+// that (16.8 million pairs and their transforms: 2.79 -> 1.63 ms).  Largest errors
 // on the CPU over 6 million arguments: radius 1.7e-16 relative, angle 2.1e-16.
 constexpr int kLogFirst = 90, kLogCount = 91;   // j = 90 .. 180
 // c = 128 / j rounded, and 2 ln c and 2 n ln 2 as multiples of 2^-40, whose sums
@@ -121,6 +123,10 @@ static __device__ double2 d_bm_log[kLogCount];  // (c, 2 ln c high)
 static __device__ double d_bm_log_lo[kLogCount];
 static __device__ double2 d_bm_exp[34];
 static __device__ double2 d_bm_trig[257];       // (cos, sin) 2 pi k / 256
+// the same as pairs of float32 for the batched screens (float_pair.cuh)
+static __device__ BmLog d_bmp_log[kBmCount];
+static __device__ fpair d_bmp_exp[34];
+static __device__ cpair d_bmp_trig[257];
 
 int screens_init_device() {
   double2 lg[kLogCount], ex[34], tr[257];
@@ -145,6 +151,23 @@ int screens_init_device() {
     const double cq[4] = {c, -s, -c, s}, sq[4] = {s, c, -s, -c};
     tr[k] = make_double2(cq[q], sq[q]);
   }
+  BmLog plg[kBmCount];
+  fpair pex[34];
+  cpair ptr[257];
+  const auto pair = [](long double v) {
+    const float h = (float)v;
+    return fpair{h, (float)(v - (long double)h)};
+  };
+  for (int j = 0; j < kBmCount; ++j) {
+    const double c = rint(128.0 / (double)(kBmFirst + j) * 2048.0) / 2048.0;
+    const fpair l = pair(2.0L * logl((long double)c));
+    plg[j] = BmLog{(float)c, l.h, l.l, 0.f};
+  }
+  for (int n = 0; n < 34; ++n) pex[n] = pair(2.0L * n * logl(2.0L));
+  for (int k = 0; k <= 256; ++k) ptr[k] = cpair{pair(tr[k].x), pair(tr[k].y)};
+  SPECULA_CK(cudaMemcpyToSymbol(d_bmp_log, plg, sizeof(plg)));
+  SPECULA_CK(cudaMemcpyToSymbol(d_bmp_exp, pex, sizeof(pex)));
+  SPECULA_CK(cudaMemcpyToSymbol(d_bmp_trig, ptr, sizeof(ptr)));
   SPECULA_CK(cudaMemcpyToSymbol(d_bm_log, lg, sizeof(lg)));
   SPECULA_CK(cudaMemcpyToSymbol(d_bm_log_lo, lo, sizeof(lo)));
   SPECULA_CK(cudaMemcpyToSymbol(d_bm_exp, ex, sizeof(ex)));
@@ -211,6 +234,19 @@ __device__ __forceinline__ void normals4(uint64_t pair, uint32_t sample, uint32_
   }
 }
 
+// the same four normals as pairs of float32
+__device__ __forceinline__ void normals4_pair(uint64_t pair, uint32_t sample, uint32_t stream,
+                                              uint64_t seed, cpair g[2]) {
+  uint32_t c[4] = {(uint32_t)pair, (uint32_t)(pair >> 32), sample, stream};
+  philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const fpair r = bm_radius(c[2 * i], d_bmp_log, d_bmp_exp);
+    const cpair a = bm_angle(c[2 * i + 1], d_bmp_trig);
+    g[i] = cpair{fp_mul(r, a.re), fp_mul(r, a.im)};
+  }
+}
+
 // n complex normals per sample: element 2i, 2i+1 from counter i
 __global__ void k_rng_complex(uint64_t seed, int sample0, int stream_id, long long n,
                               double2 *__restrict__ out) {
@@ -224,19 +260,20 @@ __global__ void k_rng_complex(uint64_t seed, int sample0, int stream_id, long lo
 }
 
 // ---- batched screens ---------------------------------------------------------------
-// Everything is float64, whose rate bounds it (about 2 fused multiply-adds per
-// clock and SM): 256 screens of 256^2 took 6.5 ms for the noise (two pow per
-// pair of pixels), 2.0 ms for radix-2 transforms, 5.1 ms for the subharmonics
-// (24 complex products per pixel) before this form.
+// The result is rounded to float32 once; until then values are pairs of float32
+// (float_pair.cuh, about 48 bits; the tables are made in float64).  The float64
+// rate, 2 fused multiply-adds per clock and SM, bounded the same passes in float64:
+// 256 screens of 256^2 took 2.5 ms there (pass 1 1.63, pass 2 0.81); now 0.55 ms.
+// Error against float64 unchanged to nine digits (2.5e-8 of the screen's norm, the
+// final rounding; 0 to 15 values in a million round the other way).
 //  * The spectral amplitude depends on (|kx|, |ky|) and not on the screen: one
-//    quadrant table per call.
+//    quadrant table per call.  It is divided by a power of two that takes the
+//    largest near 1, so that the pairs' exponents never leave their range; the
+//    rounded result is multiplied by it again.
 //  * Only the real part is wanted: Re IDFT(a) = IDFT(h), h the Hermitian part
 //    of a, so the row transforms run for ky = 0 .. M/2 only and the column
 //    transforms take two real columns at a time: half the transforms.
-//  * The subharmonics are separable: per column nine products, per pixel six
-//    fused multiply-adds.
-// 256 screens of 256^2 now: 1.63 ms (pass 1, most of it the Box-Muller
-// normals) and 0.81 ms (pass 2).
+//  * The subharmonics are separable: per column nine products, per pixel six.
 // Pass 1 (k_screen_rows) draws rows ky and -ky, combines and transforms them;
 // pass 2 (k_screen_cols) transforms the columns, adds the subharmonics and
 // rounds to float32 once.
@@ -250,16 +287,17 @@ __device__ __forceinline__ double2 dmul(double2 a, double2 w) {
 __device__ __forceinline__ double2 dadd(double2 a, double2 b) {
   return make_double2(a.x + b.x, a.y + b.y);
 }
-__device__ __forceinline__ double2 dsub(double2 a, double2 b) {
-  return make_double2(a.x - b.x, a.y - b.y);
+__device__ __forceinline__ cpair ldg_cpair(const cpair *p) {
+  const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+  return cpair{{v.x, v.y}, {v.z, v.w}};
 }
-__device__ __forceinline__ void dfft4(double2 (&x)[4]) {   // natural order, sign +
-  const double2 a = dadd(x[0], x[2]), b = dsub(x[0], x[2]);
-  const double2 c = dadd(x[1], x[3]), e = dsub(x[1], x[3]);
-  x[0] = dadd(a, c);
-  x[2] = dsub(a, c);
-  x[1] = make_double2(b.x - e.y, b.y + e.x);
-  x[3] = make_double2(b.x + e.y, b.y - e.x);
+__device__ __forceinline__ void dft4(cpair (&x)[4]) {   // natural order, sign +
+  const cpair a = cp_add(x[0], x[2]), b = cp_sub(x[0], x[2]);
+  const cpair c = cp_add(x[1], x[3]), e = cp_sub(x[1], x[3]);
+  x[0] = cp_add(a, c);
+  x[2] = cp_sub(a, c);
+  x[1] = cpair{fp_sub(b.re, e.im), fp_add(b.im, e.re)};
+  x[3] = cpair{fp_add(b.re, e.im), fp_sub(b.im, e.re)};
 }
 
 // M-point inverse DFT of one vector by M/4 threads.  load(i): input i of the
@@ -267,10 +305,10 @@ __device__ __forceinline__ void dfft4(double2 (&x)[4]) {   // natural order, sig
 // after the last barrier (every load and exchange of the CTA is done).  tw[m]
 // = exp(2 pi i m / M).  Odd LOGM ends with a radix-2 pass.
 template <int LOGM, class Load, class Store>
-__device__ __forceinline__ void dfft(double2 *buf, int t, const double2 *__restrict__ tw,
+__device__ __forceinline__ void dft(cpair *buf, int t, const cpair *__restrict__ tw,
                                      Load load, Store store) {
   constexpr int M = 1 << LOGM, P4 = LOGM / 2;
-  double2 x[4];
+  cpair x[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) x[q] = load(t + q * (M / 4));
 #pragma unroll
@@ -281,9 +319,9 @@ __device__ __forceinline__ void dfft(double2 *buf, int t, const double2 *__restr
 #pragma unroll
       for (int q = 0; q < 4; ++q) x[q] = buf[t + q * (M / 4)];
 #pragma unroll
-      for (int q = 1; q < 4; ++q) x[q] = dmul(x[q], __ldg(tw + q * k * (M / (4 * L))));
+      for (int q = 1; q < 4; ++q) x[q] = cp_mul(x[q], ldg_cpair(tw + q * k * (M / (4 * L))));
     }
-    dfft4(x);
+    dft4(x);
     __syncthreads();   // every input of this pass is in registers
     if (s == P4 - 1 && LOGM % 2 == 0) {
 #pragma unroll
@@ -299,14 +337,14 @@ __device__ __forceinline__ void dfft(double2 *buf, int t, const double2 *__restr
     for (int h = 0; h < 2; ++h) {   // L = M/2: output i and i + M/2 from inputs i, i + M/2
       const int i = t + h * (M / 4);
       x[2 * h] = buf[i];
-      x[2 * h + 1] = dmul(buf[i + M / 2], __ldg(tw + i));
+      x[2 * h + 1] = cp_mul(buf[i + M / 2], ldg_cpair(tw + i));
     }
     __syncthreads();
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int i = t + h * (M / 4);
-      store(i, dadd(x[2 * h], x[2 * h + 1]));
-      store(i + M / 2, dsub(x[2 * h], x[2 * h + 1]));
+      store(i, cp_add(x[2 * h], x[2 * h + 1]));
+      store(i + M / 2, cp_sub(x[2 * h], x[2 * h + 1]));
     }
   }
 }
@@ -315,29 +353,32 @@ constexpr int kScrThreads = 256;
 constexpr int kSubLevels = 3;
 
 // tw[m] = exp(2 pi i m / M), m < M; per level p: sub[p][x] = exp(2 pi i x /
-// (M 3^(p+1))); amp[j][i] = sqrt(Phi) df / 2 at |ky| = j, |kx| = i <= M/2 (the
-// half of the Hermitian part).
-__global__ void __launch_bounds__(256) k_screen_tables(double2 *__restrict__ tw,
+// (M 3^(p+1))), subp the same in pairs; amp[j][i] = inv_s sqrt(Phi) df / 2 at
+// |ky| = j, |kx| = i <= M/2 (the half of the Hermitian part).
+__global__ void __launch_bounds__(256) k_screen_tables(cpair *__restrict__ tw,
                                                        double2 *__restrict__ sub,
-                                                       double *__restrict__ amp, int M, double Md,
-                                                       double coef, double k0) {
+                                                       cpair *__restrict__ subp,
+                                                       fpair *__restrict__ amp, int M, double Md,
+                                                       double coef, double k0, double inv_s) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const int H = M / 2 + 1;
   if (e < M) {
     double sn, cs;
     sincospi(2.0 * (double)e / (double)M, &sn, &cs);
-    tw[e] = make_double2(cs, sn);
+    tw[e] = cpair{fp_from(cs), fp_from(sn)};
     double w = 1.0;
     for (int p = 0; p < kSubLevels; ++p) {
       w *= 3.0;
       sincospi(2.0 * (double)e / ((double)M * w), &sn, &cs);
       sub[(size_t)p * M + e] = make_double2(cs, sn);
+      subp[(size_t)p * M + e] = cpair{fp_from(cs), fp_from(sn)};
     }
   }
   if (e < H * H) {
     const double fx = (double)(e % H) / Md, fy = (double)(e / H) / Md;
     const double f2 = fx * fx + fy * fy;
-    amp[e] = f2 > 0.0 ? 0.5 * (sqrt(coef * pow(f2 + k0, -11.0 / 6.0)) / Md) : 0.0;
+    amp[e] = fp_from(
+        f2 > 0.0 ? inv_s * (0.5 * (sqrt(coef * pow(f2 + k0, -11.0 / 6.0)) / Md)) : 0.0);
   }
 }
 
@@ -361,7 +402,7 @@ __global__ void __launch_bounds__(256) k_screen_sub_mean(const double2 *__restri
 // and the spatial mean of their sum.
 __global__ void __launch_bounds__(256) k_screen_sub_coef(const double2 *__restrict__ mean,
                                                          double Md, double psd, double k0,
-                                                         uint64_t seed, int sample0,
+                                                         double inv_s, uint64_t seed, int sample0,
                                                          int n_screens, double2 *__restrict__ coef,
                                                          double *__restrict__ sub_mean) {
   __shared__ double2 s_c[8][28];
@@ -379,7 +420,7 @@ __global__ void __launch_bounds__(256) k_screen_sub_coef(const double2 *__restri
     const int p = lane / 9, bb = (lane / 3) % 3, a = lane % 3;
     const double df = 1.0 / (Md * (p == 0 ? 3.0 : (p == 1 ? 9.0 : 27.0)));
     const double fx = (a - 1) * df, fy = (bb - 1) * df, f2 = fx * fx + fy * fy;
-    const double amp = f2 > 0.0 ? sqrt(psd * pow(f2 + k0, -11.0 / 6.0)) * df : 0.0;
+    const double amp = f2 > 0.0 ? inv_s * (sqrt(psd * pow(f2 + k0, -11.0 / 6.0)) * df) : 0.0;
     const double2 c = make_double2(s_c[w][lane].x * amp, s_c[w][lane].y * amp);
     coef[(size_t)b * 27 + lane] = c;
     const double2 e = mean[p];
@@ -398,53 +439,55 @@ template <int LOGM> struct ScrCfg {
   static constexpr int TPR = M / 4;                       // threads per transform
   // rows per CTA of pass 1
   static constexpr int RPB = TPR >= kScrThreads ? 1 : kScrThreads / TPR;
-  static constexpr size_t smem1 = (size_t)RPB * 2 * M * sizeof(double2);
+  static constexpr size_t smem1 = (size_t)RPB * 2 * M * sizeof(cpair);
   // pass 2: TB transforms per CTA, two columns each (eight columns give the
   // row tiles whole 128-byte lines; fewer where M/4 threads fill a CTA)
   static constexpr int TB0 = TPR >= 1024 ? 1 : (TPR >= 512 ? 2 : (TPR >= 64 ? 4 : 256 / TPR));
   static constexpr int TB = TB0 * 2 > M ? M / 2 : TB0;
   static constexpr int W = 2 * TB, LD = H | 1;
   static constexpr size_t smem2 =
-      ((size_t)W * LD > (size_t)TB * M ? (size_t)W * LD : (size_t)TB * M) * sizeof(double2) +
-      (size_t)W * 7 * sizeof(double);
+      ((size_t)W * LD > (size_t)TB * M ? (size_t)W * LD : (size_t)TB * M) * sizeof(cpair) +
+      (size_t)W * 7 * sizeof(fpair);
 };
 
 // Pass 1: rows ky = 0 .. M/2 of the Hermitian part, transformed along kx.
 // grid (ceil(H / RPB), n_screens).
 template <int LOGM>
 __global__ void __launch_bounds__(ScrCfg<LOGM>::RPB *ScrCfg<LOGM>::TPR) k_screen_rows(
-    const double2 *__restrict__ tw, const double *__restrict__ amp, uint64_t seed, int sample0,
-    double2 *__restrict__ rows) {
+    const cpair *__restrict__ tw, const fpair *__restrict__ amp, uint64_t seed, int sample0,
+    cpair *__restrict__ rows) {
   using C = ScrCfg<LOGM>;
   constexpr int M = C::M, TPR = C::TPR;
-  extern __shared__ __align__(16) double2 sm_d[];
+  extern __shared__ __align__(16) cpair sm_c[];
   const int v = threadIdx.x / TPR, t = threadIdx.x % TPR, b = blockIdx.y;
   const int ky = blockIdx.x * C::RPB + v;
   const bool ok = ky < C::H;
-  double2 *c1 = sm_d + (size_t)v * 2 * M, *c2 = c1 + M;   // noise rows ky and -ky
+  cpair *c1 = sm_c + (size_t)v * 2 * M, *c2 = c1 + M;   // noise rows ky and -ky
   const int kyn = ky == 0 ? 0 : M - ky;
   if (ok) {
     for (int i = t; i < M; i += TPR) {   // M/2 counters per row, two rows
       const bool second = i >= M / 2;
       const int pr = second ? i - M / 2 : i;
-      double g[4];
-      normals4((uint64_t)(second ? kyn : ky) * (M / 2) + pr, (uint32_t)(sample0 + b), 0u, seed, g);
-      double2 *d = (second ? c2 : c1) + 2 * pr;
-      d[0] = make_double2(g[0], g[1]);
-      d[1] = make_double2(g[2], g[3]);
+      cpair g[2];
+      normals4_pair((uint64_t)(second ? kyn : ky) * (M / 2) + pr, (uint32_t)(sample0 + b), 0u,
+                    seed, g);
+      cpair *d = (second ? c2 : c1) + 2 * pr;
+      d[0] = g[0];
+      d[1] = g[1];
     }
   }
   __syncthreads();
-  const double *am = amp + (size_t)(ok ? ky : 0) * C::H;
-  double2 *dst = rows + ((size_t)b * C::H + (ok ? ky : 0)) * M;
-  dfft<LOGM>(
+  const fpair *am = amp + (size_t)(ok ? ky : 0) * C::H;
+  cpair *dst = rows + ((size_t)b * C::H + (ok ? ky : 0)) * M;
+  dft<LOGM>(
       c1, t, tw,
       [&](int i) {
-        const double a = __ldg(am + (i > M / 2 ? M - i : i));
-        const double2 p = c1[i], q = c2[i == 0 ? 0 : M - i];
-        return make_double2(a * (p.x + q.x), a * (p.y - q.y));
+        const float2 a = __ldg(reinterpret_cast<const float2 *>(am + (i > M / 2 ? M - i : i)));
+        const cpair p = c1[i], q = c2[i == 0 ? 0 : M - i];
+        return cpair{fp_mul(fpair{a.x, a.y}, fp_add(p.re, q.re)),
+                     fp_mul(fpair{a.x, a.y}, fp_sub(p.im, q.im))};
       },
-      [&](int i, double2 z) {
+      [&](int i, cpair z) {
         if (ok) dst[i] = z;
       });
 }
@@ -452,21 +495,22 @@ __global__ void __launch_bounds__(ScrCfg<LOGM>::RPB *ScrCfg<LOGM>::TPR) k_screen
 // Pass 2: W columns of one screen, two at a time.  grid (M / W, n_screens).
 template <int LOGM>
 __global__ void __launch_bounds__(ScrCfg<LOGM>::TB *ScrCfg<LOGM>::TPR) k_screen_cols(
-    const double2 *__restrict__ rows, const double2 *__restrict__ tw,
-    const double2 *__restrict__ sub, const double2 *__restrict__ coef,
-    const double *__restrict__ sub_mean, float *__restrict__ out) {
+    const cpair *__restrict__ rows, const cpair *__restrict__ tw,
+    const double2 *__restrict__ sub, const cpair *__restrict__ subp,
+    const double2 *__restrict__ coef, const double *__restrict__ sub_mean, float s1, float s2,
+    float *__restrict__ out) {
   using C = ScrCfg<LOGM>;
   constexpr int M = C::M, TPR = C::TPR, W = C::W, LD = C::LD, NT = C::TB * TPR;
-  extern __shared__ __align__(16) double2 sm_d[];
+  extern __shared__ __align__(16) cpair sm_c[];
   const int v = threadIdx.x / TPR, t = threadIdx.x % TPR, b = blockIdx.y;
   const int x0 = blockIdx.x * W;
-  double *s_sub = reinterpret_cast<double *>(
-      sm_d + ((size_t)W * LD > (size_t)C::TB * M ? (size_t)W * LD : (size_t)C::TB * M));
+  fpair *s_sub = reinterpret_cast<fpair *>(
+      sm_c + ((size_t)W * LD > (size_t)C::TB * M ? (size_t)W * LD : (size_t)C::TB * M));
   // the columns' half spectra, column-major
-  const double2 *src = rows + (size_t)b * C::H * M + x0;
+  const cpair *src = rows + (size_t)b * C::H * M + x0;
   for (int e = threadIdx.x; e < C::H * W; e += NT) {
     const int c = e % W, ky = e / W;
-    sm_d[(size_t)c * LD + ky] = src[(size_t)ky * M + c];
+    sm_c[(size_t)c * LD + ky] = src[(size_t)ky * M + c];
   }
   // column x's subharmonics: s_sub[c][2p] cos + s_sub[c][2p + 1] sin of level
   // p's row phase, plus s_sub[c][6]
@@ -483,36 +527,37 @@ __global__ void __launch_bounds__(ScrCfg<LOGM>::TB *ScrCfg<LOGM>::TPR) k_screen_
         G[bb] = dadd(dmul(q[0], en), dmul(q[2], e));
         if (bb != 1) G[bb] = dadd(G[bb], q[1]);
       }
-      s_sub[c * 7 + 2 * p] = G[2].x + G[0].x;
-      s_sub[c * 7 + 2 * p + 1] = G[0].y - G[2].y;
+      s_sub[c * 7 + 2 * p] = fp_from(G[2].x + G[0].x);
+      s_sub[c * 7 + 2 * p + 1] = fp_from(G[0].y - G[2].y);
       k += G[1].x;
     }
-    s_sub[c * 7 + 6] = k;
+    s_sub[c * 7 + 6] = fp_from(k);
   }
   __syncthreads();
-  const double2 *r1 = sm_d + (size_t)(2 * v) * LD, *r2 = r1 + LD;
-  const double *u1 = s_sub + (2 * v) * 7, *u2 = u1 + 7;
-  float *tile = reinterpret_cast<float *>(sm_d);
+  const cpair *r1 = sm_c + (size_t)(2 * v) * LD, *r2 = r1 + LD;
+  const fpair *u1 = s_sub + (2 * v) * 7, *u2 = u1 + 7;
+  float *tile = reinterpret_cast<float *>(sm_c);
   constexpr int TLD = M + 1;
-  dfft<LOGM>(
-      sm_d + (size_t)v * M, t, tw,
+  dft<LOGM>(
+      sm_c + (size_t)v * M, t, tw,
       [&](int i) {
-        if (i == 0 || i == M / 2) return make_double2(r1[i].x, r2[i].x);
+        if (i == 0 || i == M / 2) return cpair{r1[i].re, r2[i].re};
         const int k = i < M / 2 ? i : M - i;
-        const double s = i < M / 2 ? 1.0 : -1.0;   // conjugates above M/2
-        const double2 a = r1[k], c = r2[k];
-        return make_double2(a.x - s * c.y, s * a.y + c.x);
+        const cpair a = r1[k], c = r2[k];
+        // conjugates above M/2
+        return i < M / 2 ? cpair{fp_sub(a.re, c.im), fp_add(a.im, c.re)}
+                         : cpair{fp_add(a.re, c.im), fp_sub(c.re, a.im)};
       },
-      [&](int y, double2 z) {
-        double v1 = u1[6], v2 = u2[6];
+      [&](int y, cpair z) {
+        fpair v1 = fp_add(z.re, u1[6]), v2 = fp_add(z.im, u2[6]);
 #pragma unroll
         for (int p = 0; p < kSubLevels; ++p) {
-          const double2 e = __ldg(sub + (size_t)p * M + y);
-          v1 += u1[2 * p] * e.x + u1[2 * p + 1] * e.y;
-          v2 += u2[2 * p] * e.x + u2[2 * p + 1] * e.y;
+          const cpair e = ldg_cpair(subp + (size_t)p * M + y);
+          v1 = fp_add(v1, fp_dot(u1[2 * p], e.re, u1[2 * p + 1], e.im));
+          v2 = fp_add(v2, fp_dot(u2[2 * p], e.re, u2[2 * p + 1], e.im));
         }
-        tile[(2 * v) * TLD + y] = (float)(z.x + v1);
-        tile[(2 * v + 1) * TLD + y] = (float)(z.y + v2);
+        tile[(2 * v) * TLD + y] = __fadd_rn(v1.h, v1.l) * s1 * s2;
+        tile[(2 * v + 1) * TLD + y] = __fadd_rn(v2.h, v2.l) * s1 * s2;
       });
   __syncthreads();
   float *dst = out + (size_t)b * M * M + x0;
@@ -524,7 +569,7 @@ __global__ void __launch_bounds__(ScrCfg<LOGM>::TB *ScrCfg<LOGM>::TPR) k_screen_
 
 // Bytes of the half spectra of one screen, and the most a group of screens
 // takes: a group stays in L2 between the two passes.
-static size_t screen_bytes(int M) { return (size_t)(M / 2 + 1) * M * sizeof(double2); }
+static size_t screen_bytes(int M) { return (size_t)(M / 2 + 1) * M * sizeof(cpair); }
 constexpr size_t kScreenGroupBytes = (size_t)80 << 20;
 
 template <int LOGM>
@@ -538,34 +583,44 @@ static int screen_batch(specula_ctx *ctx, int n_screens, double pitch_m, double 
   const int groups = (int)(((size_t)n_screens * screen_bytes(M) + kScreenGroupBytes - 1) /
                            kScreenGroupBytes);
   const int G = std::min(n_screens, std::max(1, (n_screens + groups - 1) / groups));
+  // the power of two that takes the largest amplitude to [1, 2), in two factors
+  // of at most 2^126
+  int ex = 0;
+  frexp(0.5 * sqrt(coef * pow(1.0 / (Md * Md) + k0, -11.0 / 6.0)) / Md, &ex);
+  ex = std::max(-252, std::min(252, ex - 1));
+  const double inv_s = ldexp(1.0, -ex);
+  const float s1 = (float)ldexp(1.0, ex / 2), s2 = (float)ldexp(1.0, ex - ex / 2);
   // workspace, kept by the context: half spectra, twiddles, subharmonic row
-  // phases and their means, coefficients, amplitude quadrant
-  const size_t nd2 = (size_t)G * H * M + M + (size_t)kSubLevels * M + 4 + (size_t)G * 27;
+  // phases (in pairs and in float64) and their means, coefficients, amplitude
+  // quadrant; entries of 16 bytes but the last two
+  static_assert(sizeof(cpair) == sizeof(double2) && sizeof(fpair) == sizeof(double), "");
+  const size_t nd2 = (size_t)G * H * M + M + (size_t)2 * kSubLevels * M + 4 + (size_t)G * 27;
   const size_t need = nd2 * sizeof(double2) + ((size_t)G + (size_t)H * H) * sizeof(double);
   int s;
   if (ctx->screen_ws.bytes < need && (s = ctx->screen_ws.alloc(need))) return s;
-  double2 *rows = ctx->screen_ws.as<double2>(), *tw = rows + (size_t)G * H * M;
-  double2 *sub = tw + M, *mean = sub + (size_t)kSubLevels * M, *cf = mean + 4;
-  double *sm = reinterpret_cast<double *>(cf + (size_t)G * 27), *amp = sm + G;
+  cpair *rows = ctx->screen_ws.as<cpair>(), *tw = rows + (size_t)G * H * M, *subp = tw + M;
+  double2 *sub = reinterpret_cast<double2 *>(subp + (size_t)kSubLevels * M), *mean = sub + (size_t)kSubLevels * M, *cf = mean + 4;
+  double *sm = reinterpret_cast<double *>(cf + (size_t)G * 27);
+  fpair *amp = reinterpret_cast<fpair *>(sm + G);
   if ((s = ensure_dynamic_smem((const void *)k_screen_rows<LOGM>, C::smem1)) ||
       (s = ensure_dynamic_smem((const void *)k_screen_cols<LOGM>, C::smem2)))
     return s;
   SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
                  k_screen_tables<<<(std::max(H * H, M) + 255) / 256, 256, 0, st>>>(
-                     tw, sub, amp, M, Md, coef, k0));
+                     tw, sub, subp, amp, M, Md, coef, k0, inv_s));
   SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
                  k_screen_sub_mean<<<kSubLevels, 256, 0, st>>>(sub, M, mean));
   for (int g0 = 0; g0 < n_screens; g0 += G) {
     const int ng = std::min(G, n_screens - g0);
     SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
-                   k_screen_sub_coef<<<(ng + 7) / 8, 256, 0, st>>>(mean, Md, coef, k0, seed,
-                                                                   sample0 + g0, ng, cf, sm));
+                   k_screen_sub_coef<<<(ng + 7) / 8, 256, 0, st>>>(mean, Md, coef, k0, inv_s,
+                                                                   seed, sample0 + g0, ng, cf, sm));
     SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
                    k_screen_rows<LOGM><<<dim3((H + C::RPB - 1) / C::RPB, ng), C::RPB * C::TPR,
                                          C::smem1, st>>>(tw, amp, seed, sample0 + g0, rows));
     SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
                    k_screen_cols<LOGM><<<dim3(M / C::W, ng), C::TB * C::TPR, C::smem2, st>>>(
-                       rows, tw, sub, cf, sm, out + (size_t)g0 * M * M));
+                       rows, tw, sub, subp, cf, sm, s1, s2, out + (size_t)g0 * M * M));
   }
   // the workspace is the context's, whatever stream its next call runs on
   SPECULA_CK(cudaStreamSynchronize(st));

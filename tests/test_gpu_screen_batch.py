@@ -37,6 +37,19 @@ def test_sides(env, M, ns, L0):
         assert np.max(np.abs(got[b] - ref)) <= 2.0 ** -23 * np.max(np.abs(ref)) * 1.01
 
 
+@pytest.mark.parametrize("delta,r0,L0", [(1e-6, 1e-4, 1e-3), (1e4, 1e8, 1e3), (0.05, 1e-12, 40.0)])
+def test_scales(env, delta, r0, L0):
+    """Amplitudes far from 1: the pairs' common power of two."""
+    torch, sp, ctx = env
+    M = 128
+    out = torch.empty(M, M, device="cuda")
+    sp.specula_screen_generate_batch(ctx, 1, M, delta, r0, L0, 99, 5, out)
+    ref = screens.fft_screen(M, delta, r0, L0, philox.complex_noise(99, 5, 0, M * M).reshape(M, M),
+                             philox.complex_noise(99, 5, 1, 27).reshape(3, 3, 3))
+    err = np.max(np.abs(out.cpu().numpy().astype(np.float64) - ref))
+    assert err <= 2.0 ** -23 * np.max(np.abs(ref)) * 1.01
+
+
 def test_groups_do_not_change_a_screen(env):
     """More screens than one group of the workspace holds; each equals the
     screen generated alone."""
