@@ -72,6 +72,13 @@ struct GemmShape {
   int kb_per_split;
   int vec4;                 // N % 4 == 0 and a 16-byte aligned output
 };
+// Products of one K in one launch: term q of the maps is a product of its own,
+// work items [first[q], first[q + 1]) its tiles.
+struct GemmGroup {
+  int first[kMaxTerms + 1];
+  int M[kMaxTerms], N[kMaxTerms], tiles_n[kMaxTerms];
+  float *out[kMaxTerms];
+};
 
 __device__ __forceinline__ bool wait_noabort(uint64_t *bar, uint32_t parity) {
   return tc::mbar_wait(bar, parity, nullptr);
@@ -100,10 +107,26 @@ __device__ __forceinline__ void gemm_item(const GemmShape &g, int w, int BN, int
   n0 = (nb0 + (r - tm * gw)) * BN;
 }
 
-template <bool TF32, int BN>
+// the same for a group: split is the product, whose K blocks are its term's
+__device__ __forceinline__ void gemm_item(const GemmGroup &g, int w, int BN, int &m0, int &n0,
+                                          int &q) {
+  q = 0;
+  while (q + 1 < kMaxTerms && w >= g.first[q + 1]) ++q;
+  const int t = w - g.first[q], tm = t / g.tiles_n[q];
+  m0 = tm * GBM;
+  n0 = (t - tm * g.tiles_n[q]) * BN;
+}
+
+template <bool TF32, int BN, bool GROUP>
 __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ GemmMaps maps,
-                                                    const GemmShape g, float *__restrict__ out,
-                                                    int32_t *status) {
+                                                    const GemmShape g, const GemmGroup gg,
+                                                    float *__restrict__ out, int32_t *status) {
+  const auto item = [&](int w, int &m0, int &n0, int &split) {
+    if constexpr (GROUP)
+      gemm_item(gg, w, BN, m0, n0, split);
+    else
+      gemm_item(g, w, BN, m0, n0, split);
+  };
   using C = GCfg<BN>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = tc::smem_u32(smem_raw);
@@ -146,7 +169,7 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
       bool ok = true;
       for (int w = blockIdx.x; w < g.n_items && ok; w += gridDim.x) {
         int m0, n0, split;
-        gemm_item(g, w, BN, m0, n0, split);
+        item(w, m0, n0, split);
         const int kb0 = split * g.kb_per_split;
         const int nk = min(g.kb_per_split, g.kb_total - kb0);
         for (int i = 0; i < nk; ++i, ++it) {
@@ -179,7 +202,7 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
       bool ok = true;
       for (int w = blockIdx.x; w < g.n_items && ok; w += gridDim.x, ++j) {
         int m0, n0, split;
-        gemm_item(g, w, BN, m0, n0, split);
+        item(w, m0, n0, split);
         const int nk = min(g.kb_per_split, g.kb_total - split * g.kb_per_split);
         const int buf = j & 1;
         // the epilogue has drained this accumulator's previous tile
@@ -218,7 +241,8 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
     int j = 0;
     for (int w = blockIdx.x; w < g.n_items; w += gridDim.x, ++j) {
       int m0, n0, split;
-      gemm_item(g, w, BN, m0, n0, split);
+      item(w, m0, n0, split);
+      const int gM = GROUP ? gg.M[split] : g.M, gN = GROUP ? gg.N[split] : g.N;
       const int buf = j & 1;
       bool go = tc::mbar_wait(acc_full + buf, (j >> 1) & 1, abort_flag);
       go = __all_sync(0xffffffffu, go);
@@ -231,13 +255,13 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
       // 128-byte lines (one row per lane wrote 32 half sectors per store)
       const int row0 = m0 + wl * 32;
       float *blk = s_out + wl * 32 * kOutLd;
-      float *dst0 = out + (size_t)split * g.M * g.N;
+      float *dst0 = GROUP ? gg.out[split] : out + (size_t)split * g.M * g.N;
 #pragma unroll 1
       for (int c0 = 0; c0 < BN; c0 += 32) {
         float v[32];
         tc::tmem_ld32(tmem + ((uint32_t)(wl * 32) << 16) + (uint32_t)(buf * BN + c0), v);
         const int col = n0 + c0;
-        if (col >= g.N) break;   // warp-uniform
+        if (col >= gN) break;   // warp-uniform
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           *reinterpret_cast<float4 *>(blk + lane * kOutLd + 4 * q) =
@@ -248,14 +272,14 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             const int row = row0 + r + 4 * q;
-            if (row < g.M && col + c < g.N)
-              *reinterpret_cast<float4 *>(dst0 + (size_t)row * g.N + col + c) =
+            if (row < gM && col + c < gN)
+              *reinterpret_cast<float4 *>(dst0 + (size_t)row * gN + col + c) =
                   *reinterpret_cast<const float4 *>(blk + (r + 4 * q) * kOutLd + c);
           }
         } else {
           for (int r = 0; r < 32; ++r)
-            if (row0 + r < g.M && col + lane < g.N)
-              dst0[(size_t)(row0 + r) * g.N + col + lane] = blk[r * kOutLd + lane];
+            if (row0 + r < gM && col + lane < gN)
+              dst0[(size_t)(row0 + r) * gN + col + lane] = blk[r * kOutLd + lane];
         }
         __syncwarp();
       }
@@ -391,25 +415,32 @@ int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n,
   return SPECULA_OK;
 }
 
+// the kernel's shared-memory limit, once per device
+template <bool TF32, int BN, bool GROUP>
+static int gemm_attr() {
+  static bool attr_done[64] = {};
+  int dev = 0;
+  SPECULA_CK(cudaGetDevice(&dev));
+  if (dev < 64 && !attr_done[dev]) {
+    SPECULA_CK(cudaFuncSetAttribute(k_gemm_tn<TF32, BN, GROUP>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)GCfg<BN>::SMEM));
+    attr_done[dev] = true;
+  }
+  return SPECULA_OK;
+}
+
 template <bool TF32, int BN>
 static int gemm_launch(specula_ctx *ctx, int n_terms, const void *const *A, const void *const *B,
                        int M, int N, int K, float *C, int splits, float *work,
                        cudaStream_t st, bool partials) {
   using Cfg = GCfg<BN>;
-  static bool attr_done[64] = {};
-  int dev = 0;
-  SPECULA_CK(cudaGetDevice(&dev));
-  if (dev < 64 && !attr_done[dev]) {
-    SPECULA_CK(cudaFuncSetAttribute(k_gemm_tn<TF32, BN>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)Cfg::SMEM));
-    attr_done[dev] = true;
-  }
+  int s;
+  if ((s = gemm_attr<TF32, BN, false>())) return s;
   const int sms = sm_count();
   if (sms < 1) return SPECULA_ECUDA;
   GemmMaps maps;
   memset(&maps, 0, sizeof(maps));
-  int s;
   for (int t = 0; t < n_terms; ++t) {
     if ((s = make_map(&maps.a[t], A[t], M, K, GBM, TF32))) return s;
     if ((s = make_map(&maps.b[t], B[t], N, K, BN, TF32))) return s;
@@ -430,8 +461,8 @@ static int gemm_launch(specula_ctx *ctx, int n_terms, const void *const *A, cons
   float *dst = to_work ? work : C;
   g.vec4 = (N % 4 == 0) && ((uintptr_t)dst % 16 == 0);
   const int grid = std::min(g.n_items, sms);
-  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_GEMM, st, (k_gemm_tn<TF32, BN>), grid, 256, Cfg::SMEM, maps, g,
-                     dst, ctx->status_dev);
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_GEMM, st, (k_gemm_tn<TF32, BN, false>), grid, 256, Cfg::SMEM,
+                     maps, g, GemmGroup{}, dst, ctx->status_dev);
   if (g.splits > 1 && !partials)
     return gemm_split_reduce(ctx, work, g.splits, (size_t)M * N, C, st);
   return SPECULA_OK;
@@ -460,6 +491,41 @@ int gemm_bf16_tn(specula_ctx *ctx, const void *A, const void *B, int M, int N, i
 int gemm_bf16_partials(specula_ctx *ctx, const void *A, const void *B, int M, int N, int K,
                        int splits, float *work, cudaStream_t st) {
   return gemm_terms<false>(ctx, 1, &A, &B, M, N, K, nullptr, splits, work, st, true);
+}
+
+int gemm_bf16_group(specula_ctx *ctx, int n, const void *const *A, const void *const *B,
+                    const int *M, const int *N, int K, float *const *C, cudaStream_t st) {
+  constexpr int BN = 128;
+  if (!ctx || n < 1 || n > kMaxTerms) return SPECULA_EINVAL;
+  GemmMaps maps;
+  memset(&maps, 0, sizeof(maps));
+  GemmShape g{};
+  GemmGroup gg{};
+  int s;
+  if ((s = gemm_attr<false, BN, true>())) return s;
+  const int sms = sm_count();
+  if (sms < 1) return SPECULA_ECUDA;
+  g.kb_term = g.kb_per_split = (K + gbk<false>() - 1) / gbk<false>();
+  g.kb_total = g.kb_term * n;
+  g.vec4 = 1;
+  for (int q = 0; q < kMaxTerms; ++q) {
+    gg.first[q + 1] = gg.first[q];
+    if (q >= n) continue;
+    if ((s = gemm_check(A[q], B[q], M[q], N[q], K, false))) return s;
+    if ((s = make_map(&maps.a[q], A[q], M[q], K, GBM))) return s;
+    if ((s = make_map(&maps.b[q], B[q], N[q], K, BN))) return s;
+    gg.M[q] = M[q];
+    gg.N[q] = N[q];
+    gg.out[q] = C[q];
+    gg.tiles_n[q] = (N[q] + BN - 1) / BN;
+    gg.first[q + 1] += (M[q] + GBM - 1) / GBM * gg.tiles_n[q];
+    if (N[q] % 4 || (uintptr_t)C[q] % 16) g.vec4 = 0;
+  }
+  g.n_items = gg.first[kMaxTerms];
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_GEMM, st, (k_gemm_tn<false, BN, true>),
+                     std::min(g.n_items, sms), 256, GCfg<BN>::SMEM, maps, g, gg, (float *)nullptr,
+                     ctx->status_dev);
+  return SPECULA_OK;
 }
 
 int gemm_bf16_terms(specula_ctx *ctx, int n_terms, const void *const *A, const void *const *B,

@@ -330,6 +330,9 @@ int gemm_bf16_tn(specula_ctx *ctx, const void *A, const void *B, int M, int N, i
 // left for the caller's kernel to add
 int gemm_bf16_partials(specula_ctx *ctx, const void *A, const void *B, int M, int N, int K,
                        int splits, float *work, cudaStream_t st);
+// C_q = A_q B_q^T for up to three products of one K in one launch (no split-K)
+int gemm_bf16_group(specula_ctx *ctx, int n, const void *const *A, const void *const *B,
+                    const int *M, const int *N, int K, float *const *C, cudaStream_t st);
 // C[n] = the sum over s < splits of part[s][n], in order
 int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n, float *C,
                       cudaStream_t st);

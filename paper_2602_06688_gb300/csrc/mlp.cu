@@ -41,7 +41,7 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
   return 0.5f * (1.0f + erff(z * (float)M_SQRT1_2)) + z * expf(-0.5f * z * z) * inv_sqrt_2pi;
 }
 
-// Tiled writer of a bf16 matrix and its transpose.  Block (32, TY), grid
+// Tiled writer of a bf16 matrix and, where outT is given, its transpose.  Block (32, TY), grid
 // (C/32, R/32); the value function is evaluated once per element.
 template <class F>
 __device__ __forceinline__ void tile_bf16_pair(int R, int C, __nv_bfloat16 *out,
@@ -58,6 +58,7 @@ __device__ __forceinline__ void tile_bf16_pair(int R, int C, __nv_bfloat16 *out,
     }
     tile[dr][threadIdx.x] = v;
   }
+  if (!outT) return;   // the whole launch
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < TT / TY; ++k) {
@@ -325,6 +326,7 @@ __global__ void __launch_bounds__(TT * 8) k_adam(const AdamArgs A, float lr_t, f
     tile[4 * lane + 2][dr] = w[1].x;
     tile[4 * lane + 3][dr] = w[1].y;
   }
+  if (!L.WbT) return;   // the first layer's: nothing multiplies by it
   __syncthreads();
   // a column's 32 rows are 64 bytes: two columns per warp
   const int half = lane / 16, pr = 2 * (lane % 16);
@@ -546,14 +548,33 @@ static int mlp_gemm(specula_mlp *p, const void *A, const void *B, int M, int N, 
   return gemm_bf16_partials(p->ctx, A, B, M, N, K, s, p->work.as<float>(), st);
 }
 
-// dW_l = A B^T over the batch (M = np[l + 1], N = np[l]) as partials in the
-// layer's own buffer: Adam adds them as it reads them, get_grad when asked
-static int mlp_gemm_dw(specula_mlp *p, int l, const void *A, const void *B, int K,
+// Splits of the weight gradients' K = the padded batch: none up to kDwGroupK,
+// where one launch does all three layers
+constexpr int kDwGroupK = 1024;
+static int dw_splits(int M, int N, int Bp) { return Bp <= kDwGroupK ? 1 : mlp_splits(M, N, Bp); }
+
+// Weight gradients dW_l = dZ_l^T H_{l-1}, l = 0 .. 2 (M = np[l + 1], N = np[l]), over
+// the padded batch.  Up to kDwGroupK rows the products are short (four K blocks at a
+// batch of 256) and bound by what they write: one launch over all the layers'
+// 128 x 128 tiles, no partials.  Beyond, each layer's own launch, its K split over
+// the SMs; the partials stay in the layer's buffer: Adam adds them as it reads
+// them, get_grad when asked.
+static int mlp_gemm_dw(specula_mlp *p, const void *const *A, const void *const *B, int Bp,
                        cudaStream_t st) {
-  const int M = p->np[l + 1], N = p->np[l];
-  p->gsplits[l] = mlp_splits(M, N, K);
-  if ((size_t)p->gsplits[l] * M * N * 4 > p->gW[l].bytes) return SPECULA_EINVAL;
-  return gemm_bf16_partials(p->ctx, A, B, M, N, K, p->gsplits[l], p->gW[l].as<float>(), st);
+  int M[3], N[3], s;
+  float *out[3];
+  for (int l = 0; l < 3; ++l) {
+    M[l] = p->np[l + 1];
+    N[l] = p->np[l];
+    out[l] = p->gW[l].as<float>();
+    p->gsplits[l] = dw_splits(M[l], N[l], Bp);
+    if ((size_t)p->gsplits[l] * M[l] * N[l] * 4 > p->gW[l].bytes) return SPECULA_EINVAL;
+  }
+  if (Bp <= kDwGroupK) return gemm_bf16_group(p->ctx, 3, A, B, M, N, Bp, out, st);
+  for (int l = 2; l >= 0; --l)
+    if ((s = gemm_bf16_partials(p->ctx, A[l], B[l], M[l], N[l], Bp, p->gsplits[l], out[l], st)))
+      return s;
+  return SPECULA_OK;
 }
 
 static int cast_layer(specula_mlp *p, int l, cudaStream_t st) {
@@ -585,9 +606,9 @@ extern "C" int specula_mlp_create(specula_ctx *ctx, int32_t n_in, int32_t n_h1, 
     const size_t nw = (size_t)p->np[l + 1] * p->np[l], nb = p->np[l + 1];
     size_t gw = nw;   // the gradient's partials, for every padded batch up to the capacity
     for (int b = 128; b <= Bp; b += 128)
-      gw = std::max(gw, nw * mlp_splits(p->np[l + 1], p->np[l], b));
+      gw = std::max(gw, nw * dw_splits(p->np[l + 1], p->np[l], b));
     if ((s = p->W[l].alloc(nw * 4)) || (s = p->mW[l].alloc(nw * 4)) || (s = p->vW[l].alloc(nw * 4)) ||
-        (s = p->gW[l].alloc(gw * 4)) || (s = p->Wb[l].alloc(nw * 2)) || (s = p->WbT[l].alloc(nw * 2)) ||
+        (s = p->gW[l].alloc(gw * 4)) || (s = p->Wb[l].alloc(nw * 2)) || (l > 0 && (s = p->WbT[l].alloc(nw * 2))) ||
         (s = p->b[l].alloc(nb * 4)) || (s = p->mb[l].alloc(nb * 4)) || (s = p->vb[l].alloc(nb * 4)) ||
         (s = p->gb[l].alloc(nb * 4)))
       return s;
@@ -774,7 +795,7 @@ extern "C" int specula_mlp_backward(specula_mlp *p, const float *T_dev, int32_t 
   const int Bp = round_up(batch, 128);
   cudaStream_t st = (cudaStream_t)stream;
   specula_ctx *ctx = p->ctx;
-  const int in = p->np[0], h1 = p->np[1], h2 = p->np[2], o = p->np[3];
+  const int h1 = p->np[1], h2 = p->np[2], o = p->np[3];
   const dim3 tb(TT, TY);
   const float scale = 2.0f / ((float)batch * (float)p->n[3]);
   const dim3 gl(o / TT, Bp / TT);
@@ -784,9 +805,7 @@ extern "C" int specula_mlp_backward(specula_mlp *p, const float *T_dev, int32_t 
                      p->dYbT.as<__nv_bfloat16>(), p->done.as<unsigned>(), p->gb[2].as<float>(),
                      p->part.as<float>(), 1.0f / ((float)batch * (float)p->n[3]),
                      loss_dev ? loss_dev : p->loss.as<float>());
-  // layer 3: dW3 = dY^T H2, dH2 = dY W3
   Partials P;
-  if ((s = mlp_gemm_dw(p, 2, p->dYbT.p, p->HT[1].p, Bp, st))) return s;
   if ((s = mlp_gemm(p, p->dYb.p, p->WbT[2].p, Bp, h2, o, &P, st))) return s;
   for (int l = 1; l >= 0; --l) {
     const int N = p->np[l + 1];
@@ -794,13 +813,12 @@ extern "C" int specula_mlp_backward(specula_mlp *p, const float *T_dev, int32_t 
                        p->Z[l].as<float>(), p->dA[l].as<float>(), batch, Bp, N,
                        p->dZb[l].as<__nv_bfloat16>(), p->dZbT[l].as<__nv_bfloat16>(),
                        p->done.as<unsigned>(), p->gb[l].as<float>());
-    const void *HinT = l == 1 ? p->HT[0].p : p->XbT.p;
-    if ((s = mlp_gemm_dw(p, l, p->dZbT[l].p, HinT, Bp, st))) return s;
     if (l == 1)
       if ((s = mlp_gemm(p, p->dZb[1].p, p->WbT[1].p, Bp, h1, h2, &P, st))) return s;
   }
-  (void)in;
-  return SPECULA_OK;
+  const void *dT[3] = {p->dZbT[0].p, p->dZbT[1].p, p->dYbT.p};
+  const void *HinT[3] = {p->XbT.p, p->HT[0].p, p->HT[1].p};
+  return mlp_gemm_dw(p, dT, HinT, Bp, st);
 }
 
 extern "C" int specula_mlp_adam(specula_mlp *p, float lr, float b1, float b2, float eps,
