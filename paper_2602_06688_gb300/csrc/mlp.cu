@@ -693,12 +693,9 @@ static int copy_out(specula_mlp *p, int layer, const DevBuf &W, const DevBuf &b,
   SPECULA_CK(cudaSetDevice(p->ctx->device));
   SPECULA_CK(cudaDeviceSynchronize());
   const int R = p->n[layer + 1], C = p->n[layer], CP = p->np[layer];
-  std::vector<float> w((size_t)p->np[layer + 1] * CP), bb(b.bytes / 4);
-  SPECULA_CK(cudaMemcpy(w.data(), W.p, w.size() * 4, cudaMemcpyDeviceToHost));
-  SPECULA_CK(cudaMemcpy(bb.data(), b.p, b.bytes, cudaMemcpyDeviceToHost));
-  for (int r = 0; r < R; ++r)
-    for (int c = 0; c < C; ++c) W_host[(size_t)r * C + c] = w[(size_t)r * CP + c];
-  for (int r = 0; r < R; ++r) b_host[r] = bb[r];
+  SPECULA_CK(cudaMemcpy2D(W_host, (size_t)C * 4, W.p, (size_t)CP * 4, (size_t)C * 4, R,
+                          cudaMemcpyDeviceToHost));
+  SPECULA_CK(cudaMemcpy(b_host, b.p, (size_t)R * 4, cudaMemcpyDeviceToHost));
   return SPECULA_OK;
 }
 
