@@ -6,7 +6,8 @@
 // variant run here.  The TF32 kernel reads float32 storage (the tensor cores
 // use its upper 19 bits).
 //
-// Persistent kernel, one CTA per SM, looping over (128 x BN output tile, K
+// Large products run on CTA pairs (k_gemm_pair below), the rest on k_gemm_tn:
+// persistent, one CTA per SM, looping over (128 x BN output tile, K
 // slice) work items, BN = 256 (128 where N is a multiple of 128 but not of
 // 256); M and N need not be tile multiples (TMA fills rows beyond the
 // operands with zeros, the epilogue masks its stores).  K is a sum of up to
@@ -94,7 +95,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 // (70 MB at K = 8192) stay in L2, instead of every row of A per wave.
 constexpr int kBand = 8;
 __device__ __forceinline__ void gemm_item(const GemmShape &g, int w, int BN, int &m0, int &n0,
-                                          int &split) {
+                                          int &split, int bm = GBM) {
   const int tiles = g.tiles_m * g.tiles_n;
   split = w / tiles;
   const int t = w - split * tiles;
@@ -103,7 +104,7 @@ __device__ __forceinline__ void gemm_item(const GemmShape &g, int w, int BN, int
   const int gw = min(kBand, g.tiles_n - nb0);
   const int r = t - band * kBand * g.tiles_m;
   const int tm = r / gw;
-  m0 = tm * GBM;
+  m0 = tm * bm;
   n0 = (nb0 + (r - tm * gw)) * BN;
 }
 
@@ -115,6 +116,42 @@ __device__ __forceinline__ void gemm_item(const GemmGroup &g, int w, int BN, int
   const int t = w - g.first[q], tm = t / g.tiles_n[q];
   m0 = tm * GBM;
   n0 = (t - tm * g.tiles_n[q]) * BN;
+}
+
+// One epilogue warp's 32 rows of an accumulator (tensor-memory address acc) to
+// dst [M][N] from (row0, n0) on: 32 x 32 blocks through shared memory, so that
+// rows go out as whole 128-byte lines (one row per lane wrote 32 half sectors per
+// store).
+template <int BN>
+__device__ __forceinline__ void store_tile(uint32_t acc, float *blk, int lane, int row0, int n0,
+                                           int M, int N, int vec4, float *__restrict__ dst) {
+#pragma unroll 1
+  for (int c0 = 0; c0 < BN; c0 += 32) {
+    float v[32];
+    tc::tmem_ld32(acc + (uint32_t)c0, v);
+    const int col = n0 + c0;
+    if (col >= N) break;   // warp-uniform
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      *reinterpret_cast<float4 *>(blk + lane * kOutLd + 4 * q) =
+          make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    __syncwarp();
+    if (vec4) {   // N % 4 == 0: four columns are inside together
+      const int r = lane >> 3, c = (lane & 7) * 4;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int row = row0 + r + 4 * q;
+        if (row < M && col + c < N)
+          *reinterpret_cast<float4 *>(dst + (size_t)row * N + col + c) =
+              *reinterpret_cast<const float4 *>(blk + (r + 4 * q) * kOutLd + c);
+      }
+    } else {
+      for (int r = 0; r < 32; ++r)
+        if (row0 + r < M && col + lane < N)
+          dst[(size_t)(row0 + r) * N + col + lane] = blk[r * kOutLd + lane];
+    }
+    __syncwarp();
+  }
 }
 
 template <bool TF32, int BN, bool GROUP>
@@ -251,38 +288,9 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
         break;
       }
       tc::fence_after();
-      // 32 x 32 blocks through shared memory, so that rows go out as whole
-      // 128-byte lines (one row per lane wrote 32 half sectors per store)
-      const int row0 = m0 + wl * 32;
-      float *blk = s_out + wl * 32 * kOutLd;
-      float *dst0 = GROUP ? gg.out[split] : out + (size_t)split * g.M * g.N;
-#pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        float v[32];
-        tc::tmem_ld32(tmem + ((uint32_t)(wl * 32) << 16) + (uint32_t)(buf * BN + c0), v);
-        const int col = n0 + c0;
-        if (col >= gN) break;   // warp-uniform
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          *reinterpret_cast<float4 *>(blk + lane * kOutLd + 4 * q) =
-              make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        __syncwarp();
-        if (g.vec4) {   // N % 4 == 0: four columns are inside together
-          const int r = lane >> 3, c = (lane & 7) * 4;
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int row = row0 + r + 4 * q;
-            if (row < gM && col + c < gN)
-              *reinterpret_cast<float4 *>(dst0 + (size_t)row * gN + col + c) =
-                  *reinterpret_cast<const float4 *>(blk + (r + 4 * q) * kOutLd + c);
-          }
-        } else {
-          for (int r = 0; r < 32; ++r)
-            if (row0 + r < gM && col + lane < gN)
-              dst0[(size_t)(row0 + r) * gN + col + lane] = blk[r * kOutLd + lane];
-        }
-        __syncwarp();
-      }
+      store_tile<BN>(tmem + ((uint32_t)(wl * 32) << 16) + (uint32_t)(buf * BN),
+                     s_out + wl * 32 * kOutLd, lane, m0 + wl * 32, n0, gM, gN, g.vec4,
+                     GROUP ? gg.out[split] : out + (size_t)split * g.M * g.N);
       tc::fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty + buf);
@@ -295,6 +303,162 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
     tc::tmem_dealloc(tmem, C::TMEM_COLS);
   }
   if (threadIdx.x == 0 && *abort_flag) atomicExch(status, SPECULA_ETIMEOUT);
+}
+
+// The same over CTA pairs (cta_group::2): a pair owns 256 x 256 tiles, each CTA
+// 128 rows of A, 128 rows of B and 128 rows of the accumulator; one thread of the
+// leader issues the MMAs for both.  An SM's port from L2 (64 bytes per clock) was what
+// bounded the single-CTA form: 48 KB per 128 x 256 x 64 step, 768 clocks for 512
+// of the tensor cores, measured 60 bytes per clock; a pair's CTA takes 32 KB
+// for the same step.  4000 x 13344 on 2048 frames in split bf16 (three terms, five
+// slices, their sum included): 481 -> 413 us, 1.59 PFLOP/s; on 512 frames one term
+// 74 -> 66 us.  Bit-identical.
+constexpr int kPairM = 2 * GBM, kPairN = 256, kPairStages = 6;
+constexpr uint32_t kPairStage = 2 * G_A_BYTES;   // 128 rows of A and of B
+constexpr size_t kPairSmem =
+    1024 + kPairStages * kPairStage + 4 * 32 * kOutLd * sizeof(float) + 256;
+template <bool TF32>
+__global__ void __launch_bounds__(256, 1) k_gemm_pair(const __grid_constant__ GemmMaps maps,
+                                                      const GemmShape g, float *__restrict__ out,
+                                                      int32_t *status) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = tc::smem_u32(smem_raw);
+  uint8_t *base = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
+  float *s_out = reinterpret_cast<float *>(base + kPairStages * kPairStage);
+  uint64_t *full = reinterpret_cast<uint64_t *>(s_out + 4 * 32 * kOutLd);   // the leader's count
+  uint64_t *empty = full + kPairStages;
+  uint64_t *acc_full = empty + kPairStages;   // [2]
+  uint64_t *acc_empty = acc_full + 2;         // [2], the leader's count
+  uint64_t *done = acc_empty + 2;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)tc::cluster_rank();
+  const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kPairStages; ++s) {
+      tc::mbar_init(full + s, 1);
+      tc::mbar_init(empty + s, 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(acc_full + b, 1);
+      tc::mbar_init(acc_empty + b, 8);   // the epilogue warps of both CTAs
+    }
+    tc::mbar_init(done, 1);
+    *abort_flag = 0;
+    tc::mbar_fence_init();
+  }
+  if (warp == 1) tc::tmem_alloc_pair(tmem_slot, 2 * kPairN);
+  tc::fence_before();
+  __syncthreads();
+  tc::cluster_sync();   // both CTAs' barriers are initialised
+  tc::fence_after();
+  const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t it = 0;
+      bool ok = true;
+      for (int w = pair; w < g.n_items && ok; w += pairs) {
+        int m0, n0, split;
+        gemm_item(g, w, kPairN, m0, n0, split, kPairM);
+        const int kb0 = split * g.kb_per_split;
+        const int nk = min(g.kb_per_split, g.kb_total - kb0);
+        for (int i = 0; i < nk; ++i, ++it) {
+          const uint32_t s = it % kPairStages;
+          if (it >= (uint32_t)kPairStages &&
+              !tc::mbar_wait(empty + s, ((it / kPairStages) & 1) ^ 1, abort_flag)) {
+            *abort_flag = 1;
+            ok = false;
+            break;
+          }
+          const int gk = kb0 + i, term = gk / g.kb_term;
+          const int kx = (gk - term * g.kb_term) * gbk<TF32>();
+          if (rank == 0) tc::mbar_arrive_expect_tx(full + s, 2 * kPairStage);
+          const uint32_t bar = tc::leader_addr(full + s);
+          uint8_t *st = base + s * kPairStage;
+          tc::tma_load_2d_pair(st, &maps.a[term], bar, kx, m0 + rank * GBM);
+          tc::tma_load_2d_pair(st + G_A_BYTES, &maps.b[term], bar, kx, n0 + rank * GBM);
+        }
+      }
+      // every issued copy has landed and been read before the CTA may leave
+      for (uint32_t s = 0; s < (uint32_t)kPairStages && s < it; ++s) {
+        const uint32_t last = s + ((it - 1 - s) / kPairStages) * kPairStages;
+        wait_noabort(empty + s, (last / kPairStages) & 1);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t idesc =
+          TF32 ? tc::idesc_tf32_f32(kPairM, kPairN) : tc::idesc_bf16_f32(kPairM, kPairN);
+      uint32_t it = 0;
+      int j = 0;
+      bool ok = true;
+      for (int w = pair; w < g.n_items && ok; w += pairs, ++j) {
+        int m0, n0, split;
+        gemm_item(g, w, kPairN, m0, n0, split, kPairM);
+        const int nk = min(g.kb_per_split, g.kb_total - split * g.kb_per_split);
+        const int buf = j & 1;
+        // both CTAs have drained this accumulator's previous tile
+        if (j >= 2 && !tc::mbar_wait(acc_empty + buf, ((j >> 1) - 1) & 1, abort_flag)) {
+          *abort_flag = 1;
+          break;
+        }
+        tc::fence_after();
+        const uint32_t d = tmem + (uint32_t)(buf * kPairN);
+        for (int i = 0; i < nk; ++i, ++it) {
+          const uint32_t s = it % kPairStages;
+          if (!tc::mbar_wait(full + s, (it / kPairStages) & 1, abort_flag)) {
+            *abort_flag = 1;
+            ok = false;
+            break;
+          }
+          tc::fence_after();
+          const uint64_t ad = tc::desc_sw128(tc::smem_u32(base + s * kPairStage));
+          const uint64_t bd = tc::desc_sw128(tc::smem_u32(base + s * kPairStage + G_A_BYTES));
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            tc::mma_pair<TF32>(d, ad + 2 * kk, bd + 2 * kk, idesc, (i | kk) ? 1u : 0u);
+          tc::mma_commit_pair(empty + s);
+        }
+        if (ok) tc::mma_commit_pair(acc_full + buf);
+      }
+      tc::mma_commit_leader(done);   // arrives once every MMA issued has finished
+      wait_noabort(done, 0);         // before the tensor memory is freed
+    }
+  } else if (warp >= 4) {
+    const int wl = warp - 4;
+    int j = 0;
+    for (int w = pair; w < g.n_items; w += pairs, ++j) {
+      int m0, n0, split;
+      gemm_item(g, w, kPairN, m0, n0, split, kPairM);
+      const int buf = j & 1;
+      bool go = tc::mbar_wait(acc_full + buf, (j >> 1) & 1, abort_flag);
+      go = __all_sync(0xffffffffu, go);
+      if (!go) {
+        *abort_flag = 1;
+        break;
+      }
+      tc::fence_after();
+      store_tile<kPairN>(tmem + ((uint32_t)(wl * 32) << 16) + (uint32_t)(buf * kPairN),
+                         s_out + wl * 32 * kOutLd, lane, m0 + rank * GBM + wl * 32, n0, g.M, g.N,
+                         g.vec4, out + (size_t)split * g.M * g.N);
+      tc::fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive_cluster(tc::leader_addr(acc_empty + buf));
+    }
+  }
+  __syncwarp();
+  tc::fence_before();
+  __syncthreads();
+  tc::cluster_sync();   // neither CTA's memory is used by the other from here on
+  if (warp == 1) {
+    tc::fence_after();
+    tc::tmem_dealloc_pair(tmem, 2 * kPairN);
+  }
+  if (threadIdx.x == 0 && *abort_flag) atomicExch(status, SPECULA_ETIMEOUT);
+  tc::cluster_sync();
 }
 
 // out[e] = sum of part[s][e] over the splits, in order; V = 4 floats per load
@@ -415,19 +579,14 @@ int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n,
   return SPECULA_OK;
 }
 
-// the kernel's shared-memory limit, once per device
-template <bool TF32, int BN, bool GROUP>
-static int gemm_attr() {
-  static bool attr_done[64] = {};
-  int dev = 0;
-  SPECULA_CK(cudaGetDevice(&dev));
-  if (dev < 64 && !attr_done[dev]) {
-    SPECULA_CK(cudaFuncSetAttribute(k_gemm_tn<TF32, BN, GROUP>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)GCfg<BN>::SMEM));
-    attr_done[dev] = true;
-  }
-  return SPECULA_OK;
+// Whether a product runs on CTA pairs: enough 256 x 256 x kb items for every pair
+// (below that the single CTAs' finer tiles fill the SMs better), no more than an
+// eighth of the rows padding, and K long enough that loading bounds it: 4096 x
+// 4096 at 16 K blocks takes 37.5 us either way, 2048 x 4000 at 209 139 against 169.
+static bool gemm_pairs(int M, int tiles_n, int splits, int kb_per_split, int sms) {
+  const int tiles_m = (M + GBM - 1) / GBM;
+  return (tiles_m % 2 == 0 || tiles_m >= 8) && kb_per_split >= 16 &&
+         (long long)(tiles_m + 1) / 2 * tiles_n * splits >= sms / 2;
 }
 
 template <bool TF32, int BN>
@@ -436,15 +595,8 @@ static int gemm_launch(specula_ctx *ctx, int n_terms, const void *const *A, cons
                        cudaStream_t st, bool partials) {
   using Cfg = GCfg<BN>;
   int s;
-  if ((s = gemm_attr<TF32, BN, false>())) return s;
   const int sms = sm_count();
   if (sms < 1) return SPECULA_ECUDA;
-  GemmMaps maps;
-  memset(&maps, 0, sizeof(maps));
-  for (int t = 0; t < n_terms; ++t) {
-    if ((s = make_map(&maps.a[t], A[t], M, K, GBM, TF32))) return s;
-    if ((s = make_map(&maps.b[t], B[t], N, K, BN, TF32))) return s;
-  }
   GemmShape g;
   g.M = M;
   g.N = N;
@@ -452,16 +604,32 @@ static int gemm_launch(specula_ctx *ctx, int n_terms, const void *const *A, cons
   g.kb_total = g.kb_term * n_terms;
   g.splits = splits_for(g.kb_total, splits);
   g.kb_per_split = (g.kb_total + g.splits - 1) / g.splits;
-  g.tiles_m = (M + GBM - 1) / GBM;
   g.tiles_n = (N + BN - 1) / BN;
+  const bool pairs =
+      BN == kPairN && gemm_pairs(M, g.tiles_n, g.splits, g.kb_per_split, sms);
+  const int bm = pairs ? kPairM : GBM;
+  g.tiles_m = (M + bm - 1) / bm;
   g.n_items = g.tiles_m * g.tiles_n * g.splits;
   const bool to_work = partials || g.splits > 1;
   if (to_work && !work) return SPECULA_EINVAL;
   if (partials && g.splits != splits) return SPECULA_EINVAL;
   float *dst = to_work ? work : C;
   g.vec4 = (N % 4 == 0) && ((uintptr_t)dst % 16 == 0);
+  GemmMaps maps;
+  memset(&maps, 0, sizeof(maps));
+  for (int t = 0; t < n_terms; ++t) {
+    if ((s = make_map(&maps.a[t], A[t], M, K, GBM, TF32))) return s;
+    if ((s = make_map(&maps.b[t], B[t], N, K, pairs ? GBM : BN, TF32))) return s;
+  }
+  const void *fn = pairs ? (const void *)k_gemm_pair<TF32> : (const void *)k_gemm_tn<TF32, BN, false>;
+  if ((s = ensure_dynamic_smem(fn, pairs ? kPairSmem : Cfg::SMEM))) return s;
   const int grid = std::min(g.n_items, sms);
-  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_GEMM, st, (k_gemm_tn<TF32, BN, false>), grid, 256, Cfg::SMEM,
+  if (pairs)
+    SPECULA_LAUNCH(ctx, SPECULA_K_GEMM, st,
+                   SPECULA_CK(launch_pdl(k_gemm_pair<TF32>, 2 * std::min(g.n_items, sms / 2), 256,
+                                         kPairSmem, st, 2, maps, g, dst, ctx->status_dev)));
+  else
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_GEMM, st, (k_gemm_tn<TF32, BN, false>), grid, 256, Cfg::SMEM,
                      maps, g, GemmGroup{}, dst, ctx->status_dev);
   if (g.splits > 1 && !partials)
     return gemm_split_reduce(ctx, work, g.splits, (size_t)M * N, C, st);
@@ -502,7 +670,7 @@ int gemm_bf16_group(specula_ctx *ctx, int n, const void *const *A, const void *c
   GemmShape g{};
   GemmGroup gg{};
   int s;
-  if ((s = gemm_attr<false, BN, true>())) return s;
+  if ((s = ensure_dynamic_smem((const void *)k_gemm_tn<false, BN, true>, GCfg<BN>::SMEM))) return s;
   const int sms = sm_count();
   if (sms < 1) return SPECULA_ECUDA;
   g.kb_term = g.kb_per_split = (K + gbk<false>() - 1) / gbk<false>();
