@@ -233,6 +233,17 @@ inline void prof_end(specula_ctx *c, int slot, int kid, cudaStream_t st) {
 // (griddepcontrol.launch_dependents first) was slower: its waiting CTAs hold
 // slots and registers (39 m frame 258.4, step 70.9, inference 20.6 us).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel's CTAs start once every CTA of this one has called it or
+// left: for short kernels in front of one that prefetches.
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// `bytes` (a multiple of 16) from p (16-byte aligned) on their way to L2.  A hint
+// without a value, so it may stand before pdl_wait for memory that an earlier
+// kernel may still write.
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 template <class... P, class... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t st, int cluster, A &&...args) {
