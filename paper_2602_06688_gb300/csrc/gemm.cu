@@ -79,6 +79,7 @@ struct GemmGroup {
   int first[kMaxTerms + 1];
   int M[kMaxTerms], N[kMaxTerms], tiles_n[kMaxTerms];
   float *out[kMaxTerms];
+  ColSums sums;   // by the two warps of each CTA that have no other part
 };
 
 __device__ __forceinline__ bool wait_noabort(uint64_t *bar, uint32_t parity) {
@@ -273,7 +274,9 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
       tc::mma_commit(done);      // arrives once every MMA issued has finished
       wait_noabort(done, 0);     // before the tensor memory is freed
     }
-  } else if (warp >= 4) {
+  } else if (warp < 4) {
+    if constexpr (GROUP) column_sums(gg.sums, 2 * blockIdx.x + warp - 2, 2 * gridDim.x);
+  } else {
     const int wl = warp - 4;   // tensor-memory lanes 32 wl .. 32 wl + 31
     int j = 0;
     for (int w = blockIdx.x; w < g.n_items; w += gridDim.x, ++j) {
@@ -662,13 +665,15 @@ int gemm_bf16_partials(specula_ctx *ctx, const void *A, const void *B, int M, in
 }
 
 int gemm_bf16_group(specula_ctx *ctx, int n, const void *const *A, const void *const *B,
-                    const int *M, const int *N, int K, float *const *C, cudaStream_t st) {
+                    const int *M, const int *N, int K, float *const *C, const ColSums &cs,
+                    cudaStream_t st) {
   constexpr int BN = 128;
   if (!ctx || n < 1 || n > kMaxTerms) return SPECULA_EINVAL;
   GemmMaps maps;
   memset(&maps, 0, sizeof(maps));
   GemmShape g{};
   GemmGroup gg{};
+  gg.sums = cs;
   int s;
   if ((s = ensure_dynamic_smem((const void *)k_gemm_tn<false, BN, true>, GCfg<BN>::SMEM))) return s;
   const int sms = sm_count();

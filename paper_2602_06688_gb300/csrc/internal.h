@@ -341,9 +341,44 @@ int gemm_bf16_tn(specula_ctx *ctx, const void *A, const void *B, int M, int N, i
 // left for the caller's kernel to add
 int gemm_bf16_partials(specula_ctx *ctx, const void *A, const void *B, int M, int N, int K,
                        int splits, float *work, cudaStream_t st);
-// C_q = A_q B_q^T for up to three products of one K in one launch (no split-K)
+// Column sums sum[c] = the sum over r < rows of D[r][c], rows in order; n of a
+// multiple of 32 columns.
+struct ColSums {
+  int n = 0, rows = 0;
+  int cols[3] = {};
+  const float *D[3] = {};
+  float *sum[3] = {};
+};
+#ifdef __CUDACC__
+// the column sums by whole warps, 32 columns each: warp w of nw
+__device__ __forceinline__ void column_sums(const ColSums &S, int w, int nw) {
+  for (int l = 0; l < S.n; ++l) {
+    const int C = S.cols[l], groups = C / 32;
+    for (int g = w; g < groups; g += nw) {
+      const int c = g * 32 + (threadIdx.x & 31);
+      const float *d = S.D[l] + c;
+      float s = 0.f;
+      int r = 0;
+      for (; r + 32 <= S.rows; r += 32) {
+        float x[32];
+#pragma unroll
+        for (int u = 0; u < 32; ++u) x[u] = __ldg(d + (size_t)(r + u) * C);
+#pragma unroll
+        for (int u = 0; u < 32; ++u) s += x[u];
+      }
+      for (; r < S.rows; ++r) s += __ldg(d + (size_t)r * C);
+      S.sum[l][c] = s;
+    }
+    w -= groups % nw;   // the next layer's groups go to the warps after these
+    if (w < 0) w += nw;
+  }
+}
+#endif
+// C_q = A_q B_q^T for up to three products of one K in one launch (no split-K),
+// and the column sums beside them
 int gemm_bf16_group(specula_ctx *ctx, int n, const void *const *A, const void *const *B,
-                    const int *M, const int *N, int K, float *const *C, cudaStream_t st);
+                    const int *M, const int *N, int K, float *const *C, const ColSums &cs,
+                    cudaStream_t st);
 // C[n] = the sum over s < splits of part[s][n], in order
 int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n, float *C,
                       cudaStream_t st);

@@ -134,51 +134,11 @@ __global__ void __launch_bounds__(256) k_output(const Partials P, const float *_
   if (out && r < B && c < n_out) out[(size_t)r * n_out + c] = y;
 }
 
-// Bias gradients: db[c] = sum of D[r][c] over the batch's rows, in order, for
-// a 32 x 32 tile kernel that leaves D in global memory: the block that
-// finishes a tile column last (done[] counts, wrapping to zero) stages its
-// rows in shared memory, 128 at a time, and one thread per column adds them.
-// (A kernel of one thread per column took 18 us for 256 rows, each load
-// waiting for the last.)  Returns, to every thread, whether this block was the
-// last of its tile column.
-__device__ __forceinline__ bool tile_colsum(const float *D, int rows, int C, unsigned *done,
-                                            float *__restrict__ db) {
-  constexpr int CH = 128;
-  __shared__ float s_d[CH][TT];
-  __shared__ bool s_last;
-  __threadfence();   // this thread's part of D
-  __syncthreads();
-  if (threadIdx.x == 0 && threadIdx.y == 0)
-    s_last = atomicInc(done + blockIdx.x, gridDim.y - 1) == gridDim.y - 1;
-  __syncthreads();
-  if (!s_last) return false;
-  __threadfence();
-  const int c = blockIdx.x * TT + threadIdx.x;
-  float s = 0.f;
-  for (int r0 = 0; r0 < rows; r0 += CH) {
-#pragma unroll
-    for (int k = 0; k < CH / TY; ++k) {
-      const int r = r0 + threadIdx.y + TY * k;
-      s_d[threadIdx.y + TY * k][threadIdx.x] = r < rows ? __ldcg(D + (size_t)r * C + c) : 0.f;
-    }
-    __syncthreads();
-    if (threadIdx.y == 0) {
-#pragma unroll 16
-      for (int r = 0; r < CH; ++r) s += s_d[r][threadIdx.x];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.y == 0) db[c] = s;
-  return true;
-}
-
-// dA = (sum of partials) gelu'(Z); bf16 dZ and its transpose; db = the column
-// sums over the B rows of the batch
+// dA = (sum of partials) gelu'(Z); bf16 dZ and its transpose
 __global__ void __launch_bounds__(TT * TY) k_gelu_back(const Partials P,
                                                       const float *__restrict__ Z, float *dA,
-                                                      int B, int R, int C, __nv_bfloat16 *dZb,
-                                                      __nv_bfloat16 *dZbT, unsigned *done,
-                                                      float *__restrict__ db) {
+                                                      int R, int C, __nv_bfloat16 *dZb,
+                                                      __nv_bfloat16 *dZbT) {
   pdl_wait();
   tile_bf16_pair(R, C, dZb, dZbT, [&](int r, int c) {
     const size_t e = (size_t)r * C + c;
@@ -186,16 +146,22 @@ __global__ void __launch_bounds__(TT * TY) k_gelu_back(const Partials P,
     dA[e] = d;
     return d;
   });
-  tile_colsum(dA, B, C, done, db);
+}
+
+// The bias gradients, the column sums of dZ, where the weight gradients' launch does
+// not take them along
+__global__ void __launch_bounds__(128) k_bias_grad(const ColSums S) {
+  pdl_wait();
+  column_sums(S, blockIdx.x * 4 + (threadIdx.x >> 5), gridDim.x * 4);
 }
 
 // dY = scale (Y - T) on the B x n_out block, zero on pads, in bf16 with its
-// transpose; db = its column sums; loss = inv_count x the squared residuals'
-// sum, each block's in part, added by the block that finishes last
+// transpose; loss = inv_count x the squared residuals' sum, each block's in part,
+// added by the block that finishes last (done counts, wrapping to zero)
 __global__ void __launch_bounds__(TT * TY) k_loss_grad(
     const float *__restrict__ Y, const float *__restrict__ T, int B, int n_out, int Bp,
     int out_pad, float scale, float *dYf, __nv_bfloat16 *dYb, __nv_bfloat16 *dYbT, unsigned *done,
-    float *__restrict__ db, float *__restrict__ part, float inv_count, float *__restrict__ loss) {
+    float *__restrict__ part, float inv_count, float *__restrict__ loss) {
   pdl_wait();
   __shared__ float s_sq[2][TY];
   float sq = 0.f;
@@ -211,17 +177,15 @@ __global__ void __launch_bounds__(TT * TY) k_loss_grad(
   for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
   if (threadIdx.x == 0) s_sq[0][threadIdx.y] = sq;
   __syncthreads();
+  __shared__ bool s_end;
   if (threadIdx.x == 0 && threadIdx.y == 0) {
     float s = 0.f;
     for (int y = 0; y < TY; ++y) s += s_sq[0][y];
     __stcg(part + blockIdx.y * gridDim.x + blockIdx.x, s);
+    __threadfence();
+    const unsigned last = gridDim.x * gridDim.y - 1;
+    s_end = atomicInc(done, last) == last;
   }
-  // the tile columns' last blocks count themselves; the last of them sees
-  // every block's residual sum
-  if (!tile_colsum(dYf, B, out_pad, done, db)) return;
-  __shared__ bool s_end;
-  if (threadIdx.x == 0 && threadIdx.y == 0)
-    s_end = atomicInc(done + gridDim.x, gridDim.x - 1) == gridDim.x - 1;
   __syncthreads();
   if (!s_end) return;
   __threadfence();
@@ -410,7 +374,7 @@ struct specula_mlp {
   DevBuf W[3], b[3], mW[3], vW[3], mb[3], vb[3], Wb[3], WbT[3], gW[3], gb[3];
   DevBuf Xb, XbT, Z[2], H[2], HT[2], Y, dYf, dYb, dYbT, dA[2], dZb[2], dZbT[2];
   DevBuf work, part, loss;
-  DevBuf done;     // finished-block counts of the loss and GELU-backward kernels
+  DevBuf done;     // finished-block count of the loss kernel
   DevBuf Hi[2];    // inference activations, [kInferMax][np] float32
   size_t work_floats = 0;
 };
@@ -566,8 +530,8 @@ static int dw_splits(int M, int N, int Bp) { return Bp <= kDwGroupK ? 1 : mlp_sp
 // them, get_grad when asked.  A step of 300-128-128-60, four tiles in all, split /
 // grouped: 97.6 / 86.6 us at 1024 rows, 225 / 201 at 4096; of
 // 2512-1024-1024-500: 123 / 95 at 256, 294 / 263 at 2048.
-static int mlp_gemm_dw(specula_mlp *p, const void *const *A, const void *const *B, int Bp,
-                       cudaStream_t st) {
+static int mlp_gemm_dw(specula_mlp *p, const void *const *A, const void *const *B, int batch,
+                       int Bp, cudaStream_t st) {
   int M[3], N[3], s;
   float *out[3];
   for (int l = 0; l < 3; ++l) {
@@ -577,7 +541,21 @@ static int mlp_gemm_dw(specula_mlp *p, const void *const *A, const void *const *
     p->gsplits[l] = dw_splits(M[l], N[l], Bp);
     if ((size_t)p->gsplits[l] * M[l] * N[l] * 4 > p->gW[l].bytes) return SPECULA_EINVAL;
   }
-  if (Bp <= kDwGroupK) return gemm_bf16_group(p->ctx, 3, A, B, M, N, Bp, out, st);
+  // the bias gradients in the same launch, by warps that the products leave idle: a
+  // block that summed its tile column last made each producer of dZ 4 us longer
+  // (a step of 2512-1024-1024-500 at 256 rows 95 -> 82 us)
+  ColSums cs;
+  cs.n = 3;
+  cs.rows = batch;
+  const DevBuf *D[3] = {&p->dA[0], &p->dA[1], &p->dYf};
+  for (int l = 0; l < 3; ++l) {
+    cs.cols[l] = M[l];
+    cs.D[l] = D[l]->as<float>();
+    cs.sum[l] = p->gb[l].as<float>();
+  }
+  if (Bp <= kDwGroupK) return gemm_bf16_group(p->ctx, 3, A, B, M, N, Bp, out, cs, st);
+  SPECULA_LAUNCH_PDL(p->ctx, SPECULA_K_MLP, st, k_bias_grad, (M[0] + M[1] + M[2]) / 128, 128, 0,
+                     cs);
   for (int l = 2; l >= 0; --l)
     if ((s = gemm_bf16_partials(p->ctx, A[l], B[l], M[l], N[l], Bp, p->gsplits[l], out[l], st)))
       return s;
@@ -653,9 +631,8 @@ extern "C" int specula_mlp_create(specula_ctx *ctx, int32_t n_in, int32_t n_h1, 
       (s = p->Hi[1].alloc((size_t)kInferMax * h2 * 4)))
     return s;
   const int tiles = ((o + TT - 1) / TT) * ((Bp + TT - 1) / TT);
-  const int wide = std::max(o, std::max(h1, h2));
   if ((s = p->part.alloc((size_t)tiles * 4)) || (s = p->loss.alloc(4)) ||
-      (s = p->done.alloc((size_t)(wide / TT + 1) * 4)))
+      (s = p->done.alloc(4)))
     return s;
   SPECULA_CK(cudaMemset(p->done.p, 0, p->done.bytes));
   for (int l = 0; l < 3; ++l)
@@ -806,23 +783,22 @@ extern "C" int specula_mlp_backward(specula_mlp *p, const float *T_dev, int32_t 
   int s;
   SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_loss_grad, gl, tb, 0, p->Y.as<float>(), T_dev,
                      batch, p->n[3], Bp, o, scale, p->dYf.as<float>(), p->dYb.as<__nv_bfloat16>(),
-                     p->dYbT.as<__nv_bfloat16>(), p->done.as<unsigned>(), p->gb[2].as<float>(),
-                     p->part.as<float>(), 1.0f / ((float)batch * (float)p->n[3]),
+                     p->dYbT.as<__nv_bfloat16>(), p->done.as<unsigned>(), p->part.as<float>(),
+                     1.0f / ((float)batch * (float)p->n[3]),
                      loss_dev ? loss_dev : p->loss.as<float>());
   Partials P;
   if ((s = mlp_gemm(p, p->dYb.p, p->WbT[2].p, Bp, h2, o, &P, st))) return s;
   for (int l = 1; l >= 0; --l) {
     const int N = p->np[l + 1];
     SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_gelu_back, dim3(N / TT, Bp / TT), tb, 0, P,
-                       p->Z[l].as<float>(), p->dA[l].as<float>(), batch, Bp, N,
-                       p->dZb[l].as<__nv_bfloat16>(), p->dZbT[l].as<__nv_bfloat16>(),
-                       p->done.as<unsigned>(), p->gb[l].as<float>());
+                       p->Z[l].as<float>(), p->dA[l].as<float>(), Bp, N,
+                       p->dZb[l].as<__nv_bfloat16>(), p->dZbT[l].as<__nv_bfloat16>());
     if (l == 1)
       if ((s = mlp_gemm(p, p->dZb[1].p, p->WbT[1].p, Bp, h1, h2, &P, st))) return s;
   }
   const void *dT[3] = {p->dZbT[0].p, p->dZbT[1].p, p->dYbT.p};
   const void *HinT[3] = {p->XbT.p, p->HT[0].p, p->HT[1].p};
-  return mlp_gemm_dw(p, dT, HinT, Bp, st);
+  return mlp_gemm_dw(p, dT, HinT, batch, Bp, st);
 }
 
 extern "C" int specula_mlp_adam(specula_mlp *p, float lr, float b1, float b2, float eps,
