@@ -32,12 +32,12 @@ __device__ __forceinline__ void dm_axpy(float &a, float c, float v) { a += c * v
 
 // phase[p] = sum over j of cmd[j] B[j][p].  Bound by reading B once: one
 // thread per pixel over all modes kept 5 KB in flight per SM (500 modes of
-// 160^2 pixels: 33 us for 51 MB).  A CTA of eight warps takes 32 V pixels (V
+// 160^2 pixels: 33 us for 51 MB).  A CTA of eight warps takes LT V pixels (V
 // = 4 floats per lane where the size and alignment allow, else 1), the modes
-// split over the warps and over a cluster of CTAs; eight rows' loads in
-// flight per lane.  Each warp adds its modes in order, then the warps' and
-// the CTAs' sums are added in order.
-template <int V>
+// split over the warps, over 32 / LT parts of a warp and, on small pupils, over a
+// cluster of CTAs; eight rows' loads in flight per lane.  Each part adds its
+// modes in order, then the parts' and the CTAs' sums are added in order.
+template <int V, int LT>
 __global__ void __launch_bounds__(kDmWarps * 32, 4) k_dm_shape(const float *__restrict__ B,
                                                             const float *__restrict__ cmd,
                                                             float *__restrict__ phase,
@@ -49,8 +49,10 @@ __global__ void __launch_bounds__(kDmWarps * 32, 4) k_dm_shape(const float *__re
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nv = n_pix2 / V;
-  const int p = blockIdx.x / cs * 32 + lane;
-  const int part = rank * kDmWarps + warp, parts = cs * kDmWarps;
+  constexpr int SUB = 32 / LT, NP = kDmWarps * SUB;   // parts of the modes per CTA
+  const int ln = lane % LT;
+  const int p = blockIdx.x / cs * LT + ln;
+  const int part = rank * NP + warp * SUB + lane / LT, parts = cs * NP;
   int j = (int)((long long)n_modes * part / parts);
   const int j1 = (int)((long long)n_modes * (part + 1) / parts);
   const T *b = reinterpret_cast<const T *>(B) + min(p, nv - 1);
@@ -66,19 +68,19 @@ __global__ void __launch_bounds__(kDmWarps * 32, 4) k_dm_shape(const float *__re
   s_p[warp][lane] = acc;
   __syncthreads();
   if (warp == 0) {
-    acc = s_p[0][lane];
+    acc = s_p[0][ln];
 #pragma unroll
-    for (int w = 1; w < kDmWarps; ++w) dm_axpy(acc, 1.f, s_p[w][lane]);
-    s_p[0][lane] = acc;
+    for (int i = 1; i < NP; ++i) dm_axpy(acc, 1.f, s_p[i / SUB][i % SUB * LT + ln]);
+    if (lane < LT) s_p[0][lane] = acc;
   }
   if (cs > 1) {
     cl.sync();
     if (rank == 0 && warp == 0) {
-      for (int c = 1; c < cs; ++c) dm_axpy(acc, 1.f, cl.map_shared_rank(&s_p[0][0], c)[lane]);
+      for (int c = 1; c < cs; ++c) dm_axpy(acc, 1.f, cl.map_shared_rank(&s_p[0][0], c)[ln]);
     }
     cl.sync();   // no CTA leaves before its sums are read
   }
-  if (rank == 0 && warp == 0 && p < nv) reinterpret_cast<T *>(phase)[p] = acc;
+  if (rank == 0 && warp == 0 && lane < LT && p < nv) reinterpret_cast<T *>(phase)[p] = acc;
 }
 
 // residual = atm - dm over the grid, and its statistics: float64 sums over
@@ -91,12 +93,25 @@ __global__ void __launch_bounds__(kDmWarps * 32, 4) k_dm_shape(const float *__re
 // runs at 2 operations per clock and SM, so 13 CTAs of 8 pixels per thread
 // took 13 us, and the statistics in a kernel of one thread 6.5 us.
 __device__ __forceinline__ void loop_block_sum(double (&a)[5], double (*s_p)[kLoopThreads / 32]) {
+  // five butterflies at once: each level halves the values a lane carries, nine
+  // additions instead of 25 with the same pairs (value 4 and zeros in the upper half)
+  const int lane = threadIdx.x & 31;
+  const bool u = lane & 16, h = lane & 8, t = lane & 4;
+  double b[4];
 #pragma unroll
-  for (int q = 0; q < 5; ++q) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a[q] += __shfl_xor_sync(0xffffffffu, a[q], o);
-    if ((threadIdx.x & 31) == 0) s_p[q][threadIdx.x >> 5] = a[q];
+  for (int i = 0; i < 4; ++i) {
+    const double hi = i == 0 ? a[4] : 0.0;
+    b[i] = (u ? hi : a[i]) + __shfl_xor_sync(0xffffffffu, u ? a[i] : hi, 16);
   }
+  double c[2], d;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    c[i] = (h ? b[2 + i] : b[i]) + __shfl_xor_sync(0xffffffffu, h ? b[i] : b[2 + i], 8);
+  d = (t ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, t ? c[0] : c[1], 4);
+  d += __shfl_xor_sync(0xffffffffu, d, 2);
+  d += __shfl_xor_sync(0xffffffffu, d, 1);
+  const int q = (u ? 4 : 0) + (h ? 2 : 0) + (t ? 1 : 0);
+  if (lane % 4 == 0 && q < 5) s_p[q][threadIdx.x >> 5] = d;
   __syncthreads();
 }
 
@@ -186,23 +201,29 @@ extern "C" int specula_dm_shape(specula_ctx *ctx, int32_t n_modes, int32_t n_pix
   const bool v4 = n_pix2 % 4 == 0 && (((uintptr_t)basis_dev | (uintptr_t)phase_dev) % 16) == 0;
   int sms = 0;
   SPECULA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
-  // modes over a cluster until there are two CTAs per SM, while every warp
-  // keeps a full unroll of modes
-  const int tiles = (n_pix2 / (v4 ? 4 : 1) + 31) / 32;
+  // tiles of 32, 16 or 8 lanes, the widest that give two CTAs per SM; then the modes
+  // over a cluster until there are, while every part keeps a full unroll of
+  // modes.  (Narrow tiles before clusters, whose CTAs share SMs while others stand
+  // idle; with the shorter butterflies of the residual, 8 m step 64.9 -> 62.3 us.)
+  const int px = v4 ? 4 : 1;
+  const auto tiles_of = [&](int lt) { return (n_pix2 / px + lt - 1) / lt; };
+  int lt = 32;
+  while (v4 && lt > 8 && tiles_of(lt) < 2 * sms &&
+         n_modes / (kDmWarps * (64 / lt)) >= kDmUnroll)
+    lt /= 2;
+  const int tiles = tiles_of(lt);
   int cs = 1;
   while (cs < kDmMaxCluster && tiles * cs < 2 * sms &&
-         n_modes / (kDmWarps * cs * 2) >= kDmUnroll)
+         n_modes / (kDmWarps * (32 / lt) * cs * 2) >= kDmUnroll)
     cs *= 2;
   const unsigned grid = (unsigned)tiles * cs;
   const int cluster = cs > 1 ? cs : 0;
-  if (v4)
-    SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
-                   SPECULA_CK(launch_pdl(k_dm_shape<4>, grid, kDmWarps * 32, 0, st, cluster,
-                                         basis_dev, cmd_dev, phase_dev, n_modes, n_pix2)));
-  else
-    SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
-                   SPECULA_CK(launch_pdl(k_dm_shape<1>, grid, kDmWarps * 32, 0, st, cluster,
-                                         basis_dev, cmd_dev, phase_dev, n_modes, n_pix2)));
+  void (*fn)(const float *, const float *, float *, int, int) =
+      !v4 ? k_dm_shape<1, 32>
+          : (lt == 32 ? k_dm_shape<4, 32> : (lt == 16 ? k_dm_shape<4, 16> : k_dm_shape<4, 8>));
+  SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
+                 SPECULA_CK(launch_pdl(fn, grid, kDmWarps * 32, 0, st, cluster, basis_dev, cmd_dev,
+                                       phase_dev, n_modes, n_pix2)));
   return SPECULA_OK;
 }
 
