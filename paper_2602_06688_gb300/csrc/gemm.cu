@@ -52,7 +52,6 @@ constexpr int kOutLd = 36;   // row stride (floats) of an epilogue warp's 32 x 3
 template <int BN> struct GCfg {
   static constexpr int STAGES = BN == 256 ? 4 : 6;
   static constexpr uint32_t B_BYTES = BN * 128;
-  static constexpr uint32_t TMEM_COLS = 2 * BN;
   static constexpr size_t SMEM =
       1024 + STAGES * (G_A_BYTES + B_BYTES) + 4 * 32 * kOutLd * sizeof(float) + 256;
 };
@@ -79,6 +78,7 @@ struct GemmGroup {
   int first[kMaxTerms + 1];
   int M[kMaxTerms], N[kMaxTerms], tiles_n[kMaxTerms];
   float *out[kMaxTerms];
+  int kb_slice[kMaxTerms];   // K blocks accumulated together; the slices are added in order
   ColSums sums;   // by the two warps of each CTA that have no other part
 };
 
@@ -119,17 +119,17 @@ __device__ __forceinline__ void gemm_item(const GemmGroup &g, int w, int BN, int
   n0 = (t - tm * g.tiles_n[q]) * BN;
 }
 
-// One epilogue warp's 32 rows of an accumulator (tensor-memory address acc) to
+// One epilogue warp's 32 rows of a tile (load(c0, v): 32 columns of this lane's row) to
 // dst [M][N] from (row0, n0) on: 32 x 32 blocks through shared memory, so that
 // rows go out as whole 128-byte lines (one row per lane wrote 32 half sectors per
 // store).
-template <int BN>
-__device__ __forceinline__ void store_tile(uint32_t acc, float *blk, int lane, int row0, int n0,
+template <int BN, int UNROLL, class Load>
+__device__ __forceinline__ void store_tile(Load load, float *blk, int lane, int row0, int n0,
                                            int M, int N, int vec4, float *__restrict__ dst) {
-#pragma unroll 1
+#pragma unroll UNROLL
   for (int c0 = 0; c0 < BN; c0 += 32) {
     float v[32];
-    tc::tmem_ld32(acc + (uint32_t)c0, v);
+    load(c0, v);
     const int col = n0 + c0;
     if (col >= N) break;   // warp-uniform
 #pragma unroll
@@ -166,6 +166,8 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
       gemm_item(g, w, BN, m0, n0, split);
   };
   using C = GCfg<BN>;
+  constexpr int NACC = GROUP ? 4 : 2;   // accumulators in tensor memory
+  constexpr uint32_t TMEM_COLS = NACC * BN;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = tc::smem_u32(smem_raw);
   uint8_t *base = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
@@ -174,9 +176,9 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
   float *s_out = reinterpret_cast<float *>(sB + C::STAGES * C::B_BYTES);
   uint64_t *full = reinterpret_cast<uint64_t *>(s_out + 4 * 32 * kOutLd);
   uint64_t *empty = full + C::STAGES;
-  uint64_t *acc_full = empty + C::STAGES;   // [2]
-  uint64_t *acc_empty = acc_full + 2;       // [2]
-  uint64_t *done = acc_empty + 2;
+  uint64_t *acc_full = empty + C::STAGES;   // [NACC]
+  uint64_t *acc_empty = acc_full + NACC;    // [NACC]
+  uint64_t *done = acc_empty + NACC;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
@@ -187,7 +189,7 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
       tc::mbar_init(full + s, 1);
       tc::mbar_init(empty + s, 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < NACC; ++b) {
       tc::mbar_init(acc_full + b, 1);
       tc::mbar_init(acc_empty + b, 4);   // one arrival per epilogue warp
     }
@@ -195,7 +197,7 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
     *abort_flag = 0;
     tc::mbar_fence_init();
   }
-  if (warp == 1) tc::tmem_alloc(tmem_slot, C::TMEM_COLS);
+  if (warp == 1) tc::tmem_alloc(tmem_slot, TMEM_COLS);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
@@ -236,40 +238,44 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
       constexpr uint32_t idesc =
           TF32 ? tc::idesc_tf32_f32(GBM, BN) : tc::idesc_bf16_f32(GBM, BN);
       uint32_t it = 0;
-      int j = 0;   // tiles of this CTA so far
+      int j = 0;   // accumulations of this CTA so far
       bool ok = true;
-      for (int w = blockIdx.x; w < g.n_items && ok; w += gridDim.x, ++j) {
+      for (int w = blockIdx.x; w < g.n_items && ok; w += gridDim.x) {
         int m0, n0, split;
         item(w, m0, n0, split);
         const int nk = min(g.kb_per_split, g.kb_total - split * g.kb_per_split);
-        const int buf = j & 1;
-        // the epilogue has drained this accumulator's previous tile
-        if (j >= 2 && !tc::mbar_wait(acc_empty + buf, ((j >> 1) - 1) & 1, abort_flag)) {
-          *abort_flag = 1;
-          break;
-        }
-        tc::fence_after();
-        const uint32_t d = tmem + (uint32_t)(buf * BN);
-        for (int i = 0; i < nk; ++i, ++it) {
-          const uint32_t s = it % C::STAGES;
-          if (!tc::mbar_wait(full + s, (it / C::STAGES) & 1, abort_flag)) {
+        const int per = GROUP ? gg.kb_slice[split] : nk;
+        for (int i0 = 0; i0 < nk && ok; i0 += per, ++j) {
+          const int buf = j % NACC, n = min(per, nk - i0);
+          // the epilogue has drained this accumulator's previous use
+          if (j >= NACC && !tc::mbar_wait(acc_empty + buf, (j / NACC - 1) & 1, abort_flag)) {
             *abort_flag = 1;
             ok = false;
             break;
           }
           tc::fence_after();
-          const uint64_t ad = tc::desc_sw128(tc::smem_u32(sA + s * G_A_BYTES));
-          const uint64_t bd = tc::desc_sw128(tc::smem_u32(sB + s * C::B_BYTES));
+          const uint32_t d = tmem + (uint32_t)(buf * BN);
+          for (int i = 0; i < n; ++i, ++it) {
+            const uint32_t s = it % C::STAGES;
+            if (!tc::mbar_wait(full + s, (it / C::STAGES) & 1, abort_flag)) {
+              *abort_flag = 1;
+              ok = false;
+              break;
+            }
+            tc::fence_after();
+            const uint64_t ad = tc::desc_sw128(tc::smem_u32(sA + s * G_A_BYTES));
+            const uint64_t bd = tc::desc_sw128(tc::smem_u32(sB + s * C::B_BYTES));
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {   // +32 bytes of K per step (16 bf16 or 8 tf32)
-            if constexpr (TF32)
-              tc::mma_tf32(d, ad + 2 * kk, bd + 2 * kk, idesc, (i | kk) ? 1u : 0u);
-            else
-              tc::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (i | kk) ? 1u : 0u);
+            for (int kk = 0; kk < 4; ++kk) {   // +32 bytes of K per step (16 bf16 or 8 tf32)
+              if constexpr (TF32)
+                tc::mma_tf32(d, ad + 2 * kk, bd + 2 * kk, idesc, (i | kk) ? 1u : 0u);
+              else
+                tc::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (i | kk) ? 1u : 0u);
+            }
+            tc::mma_commit(empty + s);
           }
-          tc::mma_commit(empty + s);
+          if (ok) tc::mma_commit(acc_full + buf);
         }
-        if (ok) tc::mma_commit(acc_full + buf);
       }
       tc::mma_commit(done);      // arrives once every MMA issued has finished
       wait_noabort(done, 0);     // before the tensor memory is freed
@@ -278,32 +284,66 @@ __global__ void __launch_bounds__(256, 1) k_gemm_tn(const __grid_constant__ Gemm
     if constexpr (GROUP) column_sums(gg.sums, 2 * blockIdx.x + warp - 2, 2 * gridDim.x);
   } else {
     const int wl = warp - 4;   // tensor-memory lanes 32 wl .. 32 wl + 31
+    const uint32_t lanes = tmem + ((uint32_t)(wl * 32) << 16);
+    float *blk = s_out + wl * 32 * kOutLd;
     int j = 0;
-    for (int w = blockIdx.x; w < g.n_items; w += gridDim.x, ++j) {
-      int m0, n0, split;
-      item(w, m0, n0, split);
-      const int gM = GROUP ? gg.M[split] : g.M, gN = GROUP ? gg.N[split] : g.N;
-      const int buf = j & 1;
-      bool go = tc::mbar_wait(acc_full + buf, (j >> 1) & 1, abort_flag);
+    bool go = true;
+    // the next accumulator, once it is finished; released by the lambda below
+    const auto finished = [&]() {
+      go = tc::mbar_wait(acc_full + j % NACC, (j / NACC) & 1, abort_flag);
       go = __all_sync(0xffffffffu, go);
-      if (!go) {
-        *abort_flag = 1;
-        break;
-      }
+      if (!go) *abort_flag = 1;
       tc::fence_after();
-      store_tile<BN>(tmem + ((uint32_t)(wl * 32) << 16) + (uint32_t)(buf * BN),
-                     s_out + wl * 32 * kOutLd, lane, m0 + wl * 32, n0, gM, gN, g.vec4,
-                     GROUP ? gg.out[split] : out + (size_t)split * g.M * g.N);
+      return lanes + (uint32_t)(j % NACC * BN);
+    };
+    const auto release = [&]() {
       tc::fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty + buf);
+      if (lane == 0) mbar_arrive(acc_empty + j % NACC);
+      ++j;
+    };
+    for (int w = blockIdx.x; w < g.n_items && go; w += gridDim.x) {
+      int m0, n0, split;
+      item(w, m0, n0, split);
+      const int row0 = m0 + wl * 32;
+      if constexpr (GROUP) {
+        // the slices' sums, in order, in registers
+        float sum[BN];
+#pragma unroll
+        for (int c = 0; c < BN; ++c) sum[c] = 0.f;
+        for (int i0 = 0; i0 < g.kb_per_split; i0 += gg.kb_slice[split]) {
+          const uint32_t acc = finished();
+          if (!go) break;
+#pragma unroll
+          for (int c0 = 0; c0 < BN; c0 += 32) {
+            float v[32];
+            tc::tmem_ld32(acc + (uint32_t)c0, v);
+#pragma unroll
+            for (int c = 0; c < 32; ++c) sum[c0 + c] += v[c];
+          }
+          release();
+        }
+        if (!go) break;
+        store_tile<BN, BN / 32>(
+            [&](int c0, float (&v)[32]) {
+#pragma unroll
+              for (int c = 0; c < 32; ++c) v[c] = sum[c0 + c];
+            },
+            blk, lane, row0, n0, gg.M[split], gg.N[split], g.vec4, gg.out[split]);
+      } else {
+        const uint32_t acc = finished();
+        if (!go) break;
+        store_tile<BN, 1>([&](int c0, float (&v)[32]) { tc::tmem_ld32(acc + (uint32_t)c0, v); },
+                          blk, lane, row0, n0, g.M, g.N, g.vec4, out + (size_t)split * g.M * g.N);
+        release();
+      }
     }
   }
   tc::fence_before();
   __syncthreads();
   if (warp == 1) {
     tc::fence_after();
-    tc::tmem_dealloc(tmem, C::TMEM_COLS);
+    tc::tmem_dealloc(tmem, TMEM_COLS);
   }
   if (threadIdx.x == 0 && *abort_flag) atomicExch(status, SPECULA_ETIMEOUT);
 }
@@ -444,9 +484,10 @@ __global__ void __launch_bounds__(256, 1) k_gemm_pair(const __grid_constant__ Ge
         break;
       }
       tc::fence_after();
-      store_tile<kPairN>(tmem + ((uint32_t)(wl * 32) << 16) + (uint32_t)(buf * kPairN),
-                         s_out + wl * 32 * kOutLd, lane, m0 + rank * GBM + wl * 32, n0, g.M, g.N,
-                         g.vec4, out + (size_t)split * g.M * g.N);
+      const uint32_t acc = tmem + ((uint32_t)(wl * 32) << 16) + (uint32_t)(buf * kPairN);
+      store_tile<kPairN, 1>([&](int c0, float (&v)[32]) { tc::tmem_ld32(acc + (uint32_t)c0, v); },
+                            s_out + wl * 32 * kOutLd, lane, m0 + rank * GBM + wl * 32, n0, g.M,
+                            g.N, g.vec4, out + (size_t)split * g.M * g.N);
       tc::fence_before();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive_cluster(tc::leader_addr(acc_empty + buf));
@@ -665,8 +706,8 @@ int gemm_bf16_partials(specula_ctx *ctx, const void *A, const void *B, int M, in
 }
 
 int gemm_bf16_group(specula_ctx *ctx, int n, const void *const *A, const void *const *B,
-                    const int *M, const int *N, int K, float *const *C, const ColSums &cs,
-                    cudaStream_t st) {
+                    const int *M, const int *N, int K, const int *splits, float *const *C,
+                    const ColSums &cs, cudaStream_t st) {
   constexpr int BN = 128;
   if (!ctx || n < 1 || n > kMaxTerms) return SPECULA_EINVAL;
   GemmMaps maps;
@@ -690,6 +731,7 @@ int gemm_bf16_group(specula_ctx *ctx, int n, const void *const *A, const void *c
     gg.M[q] = M[q];
     gg.N[q] = N[q];
     gg.out[q] = C[q];
+    gg.kb_slice[q] = (g.kb_term + splits[q] - 1) / splits[q];
     gg.tiles_n[q] = (N[q] + BN - 1) / BN;
     gg.first[q + 1] += (M[q] + GBM - 1) / GBM * gg.tiles_n[q];
     if (N[q] % 4 || (uintptr_t)C[q] % 16) g.vec4 = 0;

@@ -374,11 +374,12 @@ __device__ __forceinline__ void column_sums(const ColSums &S, int w, int nw) {
   }
 }
 #endif
-// C_q = A_q B_q^T for up to three products of one K in one launch (no split-K),
-// and the column sums beside them
+// C_q = A_q B_q^T for up to three products of one K in one launch, and the column
+// sums beside them.  K is summed in splits[q] slices (a count from gemm_splits),
+// added in order as gemm_split_reduce adds partials.
 int gemm_bf16_group(specula_ctx *ctx, int n, const void *const *A, const void *const *B,
-                    const int *M, const int *N, int K, float *const *C, const ColSums &cs,
-                    cudaStream_t st);
+                    const int *M, const int *N, int K, const int *splits, float *const *C,
+                    const ColSums &cs, cudaStream_t st);
 // C[n] = the sum over s < splits of part[s][n], in order
 int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n, float *C,
                       cudaStream_t st);

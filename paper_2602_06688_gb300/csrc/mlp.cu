@@ -517,28 +517,29 @@ static int mlp_gemm(specula_mlp *p, const void *A, const void *B, int M, int N, 
   return gemm_bf16_partials(p->ctx, A, B, M, N, K, s, p->work.as<float>(), st);
 }
 
-// Splits of the weight gradients' K = the padded batch: none up to kDwGroupK,
-// where one launch does all three layers
+// Padded batch up to which the weight gradients run in one launch
 constexpr int kDwGroupK = 4096;
-static int dw_splits(int M, int N, int Bp) { return Bp <= kDwGroupK ? 1 : mlp_splits(M, N, Bp); }
 
 // Weight gradients dW_l = dZ_l^T H_{l-1}, l = 0 .. 2 (M = np[l + 1], N = np[l]), over
-// the padded batch.  Up to kDwGroupK rows the products are short (four K blocks at a
-// batch of 256) and bound by what they write: one launch over all the layers'
-// 128 x 128 tiles, no partials.  Beyond, each layer's own launch, its K split over
-// the SMs; the partials stay in the layer's buffer: Adam adds them as it reads
-// them, get_grad when asked.  A step of 300-128-128-60, four tiles in all, split /
-// grouped: 97.6 / 86.6 us at 1024 rows, 225 / 201 at 4096; of
-// 2512-1024-1024-500: 123 / 95 at 256, 294 / 263 at 2048.
+// the padded batch.  The products are short (four K blocks at a batch of 256) and
+// bound by what they write: one launch over all the layers' 128 x 128 tiles, a
+// tile's K slices added in registers, so the sums are those of the split-K
+// products to the last bit.  Beyond kDwGroupK each layer's own launch, its K split
+// over the SMs; the partials stay in the layer's buffer: Adam adds them as it reads
+// them, get_grad when asked.  Own launches / one launch, a step of 2512-1024-1024-500:
+// 123 / 95 us at 256 rows, 294 / 263 at 2048; of 300-128-128-60, four tiles in all:
+// 98 / 74 at 1024, 225 / 169 at 4096 (the bias gradients in it, as below).
 static int mlp_gemm_dw(specula_mlp *p, const void *const *A, const void *const *B, int batch,
                        int Bp, cudaStream_t st) {
-  int M[3], N[3], s;
+  const bool group = Bp <= kDwGroupK;
+  int M[3], N[3], splits[3], s;
   float *out[3];
   for (int l = 0; l < 3; ++l) {
     M[l] = p->np[l + 1];
     N[l] = p->np[l];
     out[l] = p->gW[l].as<float>();
-    p->gsplits[l] = dw_splits(M[l], N[l], Bp);
+    splits[l] = mlp_splits(M[l], N[l], Bp);
+    p->gsplits[l] = group ? 1 : splits[l];
     if ((size_t)p->gsplits[l] * M[l] * N[l] * 4 > p->gW[l].bytes) return SPECULA_EINVAL;
   }
   // the bias gradients in the same launch, by warps that the products leave idle: a
@@ -553,7 +554,7 @@ static int mlp_gemm_dw(specula_mlp *p, const void *const *A, const void *const *
     cs.D[l] = D[l]->as<float>();
     cs.sum[l] = p->gb[l].as<float>();
   }
-  if (Bp <= kDwGroupK) return gemm_bf16_group(p->ctx, 3, A, B, M, N, Bp, out, cs, st);
+  if (group) return gemm_bf16_group(p->ctx, 3, A, B, M, N, Bp, splits, out, cs, st);
   SPECULA_LAUNCH_PDL(p->ctx, SPECULA_K_MLP, st, k_bias_grad, (M[0] + M[1] + M[2]) / 128, 128, 0,
                      cs);
   for (int l = 2; l >= 0; --l)
@@ -591,7 +592,7 @@ extern "C" int specula_mlp_create(specula_ctx *ctx, int32_t n_in, int32_t n_h1, 
     const size_t nw = (size_t)p->np[l + 1] * p->np[l], nb = p->np[l + 1];
     size_t gw = nw;   // the gradient's partials, for every padded batch up to the capacity
     for (int b = 128; b <= Bp; b += 128)
-      gw = std::max(gw, nw * dw_splits(p->np[l + 1], p->np[l], b));
+      if (b > kDwGroupK) gw = std::max(gw, nw * mlp_splits(p->np[l + 1], p->np[l], b));
     if ((s = p->W[l].alloc(nw * 4)) || (s = p->mW[l].alloc(nw * 4)) || (s = p->vW[l].alloc(nw * 4)) ||
         (s = p->gW[l].alloc(gw * 4)) || (s = p->Wb[l].alloc(nw * 2)) || (l > 0 && (s = p->WbT[l].alloc(nw * 2))) ||
         (s = p->b[l].alloc(nb * 4)) || (s = p->mb[l].alloc(nb * 4)) || (s = p->vb[l].alloc(nb * 4)) ||
