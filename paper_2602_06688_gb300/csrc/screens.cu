@@ -263,7 +263,9 @@ __global__ void k_rng_complex(uint64_t seed, int sample0, int stream_id, long lo
 // The result is rounded to float32 once; until then values are pairs of float32
 // (float_pair.cuh, about 48 bits; the tables are made in float64).  The float64
 // rate, 2 fused multiply-adds per clock and SM, bounded the same passes in float64:
-// 256 screens of 256^2 took 2.5 ms there (pass 1 1.63, pass 2 0.81); now 0.55 ms.
+// 256 screens of 256^2 took 2.5 ms there (pass 1 1.63, pass 2 0.81); now 0.46 ms
+// (0.55 while pass 2 took its columns in five dependent rounds of loads and their
+// subharmonics in float64 on eight threads).
 // Error against float64 unchanged to nine digits (2.5e-8 of the screen's norm, the
 // final rounding; 0 to 15 values in a million round the other way).
 //  * The spectral amplitude depends on (|kx|, |ky|) and not on the screen: one
@@ -352,10 +354,13 @@ __device__ __forceinline__ void dft(cpair *buf, int t, const cpair *__restrict__
 constexpr int kScrThreads = 256;
 constexpr int kSubLevels = 3;
 
+// small CTAs: the float64 work spreads over every SM (with 256 threads 27 us at M =
+// 256, now 17; one warp per CTA in k_screen_sub_coef: 18.6 -> 12.2 us for 64 screens)
+constexpr int kTabThreads = 64;
 // tw[m] = exp(2 pi i m / M), m < M; per level p: sub[p][x] = exp(2 pi i x /
 // (M 3^(p+1))), subp the same in pairs; amp[j][i] = inv_s sqrt(Phi) df / 2 at
 // |ky| = j, |kx| = i <= M/2 (the half of the Hermitian part).
-__global__ void __launch_bounds__(256) k_screen_tables(cpair *__restrict__ tw,
+__global__ void __launch_bounds__(kTabThreads) k_screen_tables(cpair *__restrict__ tw,
                                                        double2 *__restrict__ sub,
                                                        cpair *__restrict__ subp,
                                                        fpair *__restrict__ amp, int M, double Md,
@@ -400,29 +405,28 @@ __global__ void __launch_bounds__(256) k_screen_sub_mean(const double2 *__restri
 // One warp per screen: its 27 subharmonic coefficients (Philox stream 1,
 // element e = (p * 3 + b) * 3 + a, frequencies (a - 1, b - 1) df / 3^(p+1))
 // and the spatial mean of their sum.
-__global__ void __launch_bounds__(256) k_screen_sub_coef(const double2 *__restrict__ mean,
+__global__ void __launch_bounds__(32) k_screen_sub_coef(const double2 *__restrict__ mean,
                                                          double Md, double psd, double k0,
                                                          double inv_s, uint64_t seed, int sample0,
-                                                         int n_screens, double2 *__restrict__ coef,
-                                                         double *__restrict__ sub_mean) {
-  __shared__ double2 s_c[8][28];
-  const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int b = blockIdx.x * 8 + w;
-  if (b < n_screens && lane < 14) {
+                                                         cpair *__restrict__ coef,
+                                                         fpair *__restrict__ sub_mean) {
+  __shared__ double2 s_c[28];
+  const int lane = threadIdx.x, b = blockIdx.x;
+  if (lane < 14) {
     double g[4];
     normals4((uint64_t)lane, (uint32_t)(sample0 + b), 1u, seed, g);
-    s_c[w][2 * lane] = make_double2(g[0], g[1]);
-    s_c[w][2 * lane + 1] = make_double2(g[2], g[3]);
+    s_c[2 * lane] = make_double2(g[0], g[1]);
+    s_c[2 * lane + 1] = make_double2(g[2], g[3]);
   }
   __syncwarp();
   double m = 0.0;
-  if (b < n_screens && lane < 27) {
+  if (lane < 27) {
     const int p = lane / 9, bb = (lane / 3) % 3, a = lane % 3;
     const double df = 1.0 / (Md * (p == 0 ? 3.0 : (p == 1 ? 9.0 : 27.0)));
     const double fx = (a - 1) * df, fy = (bb - 1) * df, f2 = fx * fx + fy * fy;
     const double amp = f2 > 0.0 ? inv_s * (sqrt(psd * pow(f2 + k0, -11.0 / 6.0)) * df) : 0.0;
-    const double2 c = make_double2(s_c[w][lane].x * amp, s_c[w][lane].y * amp);
-    coef[(size_t)b * 27 + lane] = c;
+    const double2 c = make_double2(s_c[lane].x * amp, s_c[lane].y * amp);
+    coef[(size_t)b * 27 + lane] = cpair{fp_from(c.x), fp_from(c.y)};
     const double2 e = mean[p];
     const double2 mx = a == 1 ? make_double2(1.0, 0.0) : make_double2(e.x, a == 2 ? e.y : -e.y);
     const double2 my = bb == 1 ? make_double2(1.0, 0.0) : make_double2(e.x, bb == 2 ? e.y : -e.y);
@@ -431,7 +435,7 @@ __global__ void __launch_bounds__(256) k_screen_sub_coef(const double2 *__restri
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-  if (b < n_screens && lane == 0) sub_mean[b] = m;
+  if (lane == 0) sub_mean[b] = fp_from(m);
 }
 
 template <int LOGM> struct ScrCfg {
@@ -447,7 +451,7 @@ template <int LOGM> struct ScrCfg {
   static constexpr int W = 2 * TB, LD = H | 1;
   static constexpr size_t smem2 =
       ((size_t)W * LD > (size_t)TB * M ? (size_t)W * LD : (size_t)TB * M) * sizeof(cpair) +
-      (size_t)W * 7 * sizeof(fpair);
+      (size_t)W * 10 * sizeof(fpair);
 };
 
 // Pass 1: rows ky = 0 .. M/2 of the Hermitian part, transformed along kx.
@@ -496,9 +500,8 @@ __global__ void __launch_bounds__(ScrCfg<LOGM>::RPB *ScrCfg<LOGM>::TPR) k_screen
 template <int LOGM>
 __global__ void __launch_bounds__(ScrCfg<LOGM>::TB *ScrCfg<LOGM>::TPR) k_screen_cols(
     const cpair *__restrict__ rows, const cpair *__restrict__ tw,
-    const double2 *__restrict__ sub, const cpair *__restrict__ subp,
-    const double2 *__restrict__ coef, const double *__restrict__ sub_mean, float s1, float s2,
-    float *__restrict__ out) {
+    const cpair *__restrict__ subp, const cpair *__restrict__ coef,
+    const fpair *__restrict__ sub_mean, float s1, float s2, float *__restrict__ out) {
   using C = ScrCfg<LOGM>;
   constexpr int M = C::M, TPR = C::TPR, W = C::W, LD = C::LD, NT = C::TB * TPR;
   extern __shared__ __align__(16) cpair sm_c[];
@@ -506,34 +509,47 @@ __global__ void __launch_bounds__(ScrCfg<LOGM>::TB *ScrCfg<LOGM>::TPR) k_screen_
   const int x0 = blockIdx.x * W;
   fpair *s_sub = reinterpret_cast<fpair *>(
       sm_c + ((size_t)W * LD > (size_t)C::TB * M ? (size_t)W * LD : (size_t)C::TB * M));
-  // the columns' half spectra, column-major
+  // the columns' half spectra, column-major: four loads of a thread in flight, and
+  // the row M/2
   const cpair *src = rows + (size_t)b * C::H * M + x0;
-  for (int e = threadIdx.x; e < C::H * W; e += NT) {
-    const int c = e % W, ky = e / W;
-    sm_c[(size_t)c * LD + ky] = src[(size_t)ky * M + c];
+  cpair in[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int e = threadIdx.x + i * NT;
+    in[i] = src[(size_t)(e / W) * M + e % W];
   }
+  if (threadIdx.x < W) sm_c[(size_t)threadIdx.x * LD + M / 2] = src[(size_t)(M / 2) * M + threadIdx.x];
   // column x's subharmonics: s_sub[c][2p] cos + s_sub[c][2p + 1] sin of level
-  // p's row phase, plus s_sub[c][6]
-  for (int c = threadIdx.x; c < W; c += NT) {
-    double k = -sub_mean[b];
-    const double2 *cf = coef + (size_t)b * 27;
+  // p's row phase, plus s_sub[c][6], the sum of the levels' s_k[c]
+  fpair *s_k = s_sub + W * 7;
+  for (int i = threadIdx.x; i < kSubLevels * W; i += NT) {
+    const int c = i % W, p = i / W;
+    const cpair *cf = coef + (size_t)b * 27 + p * 9;
+    const cpair e = ldg_cpair(subp + (size_t)p * M + x0 + c), en = cpair{e.re, fp_neg(e.im)};
+    cpair G[3];
 #pragma unroll
-    for (int p = 0; p < kSubLevels; ++p) {
-      const double2 e = sub[(size_t)p * M + x0 + c], en = make_double2(e.x, -e.y);
-      double2 G[3];
-#pragma unroll
-      for (int bb = 0; bb < 3; ++bb) {
-        const double2 *q = cf + (p * 3 + bb) * 3;
-        G[bb] = dadd(dmul(q[0], en), dmul(q[2], e));
-        if (bb != 1) G[bb] = dadd(G[bb], q[1]);
-      }
-      s_sub[c * 7 + 2 * p] = fp_from(G[2].x + G[0].x);
-      s_sub[c * 7 + 2 * p + 1] = fp_from(G[0].y - G[2].y);
-      k += G[1].x;
+    for (int bb = 0; bb < 3; ++bb) {
+      const cpair *q = cf + bb * 3;
+      G[bb] = cp_add(cp_mul(ldg_cpair(q), en), cp_mul(ldg_cpair(q + 2), e));
+      if (bb != 1) G[bb] = cp_add(G[bb], ldg_cpair(q + 1));
     }
-    s_sub[c * 7 + 6] = fp_from(k);
+    const fpair sc = fp_add(G[2].re, G[0].re), ss = fp_sub(G[0].im, G[2].im);
+    s_sub[c * 7 + 2 * p] = fp_norm(sc.h, sc.l);
+    s_sub[c * 7 + 2 * p + 1] = fp_norm(ss.h, ss.l);
+    s_k[c * kSubLevels + p] = G[1].re;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int e = threadIdx.x + i * NT;
+    sm_c[(size_t)(e % W) * LD + e / W] = in[i];
   }
   __syncthreads();
+  if (threadIdx.x < W) {   // read after the transforms' barriers
+    fpair k = fp_neg(sub_mean[b]);
+#pragma unroll
+    for (int p = 0; p < kSubLevels; ++p) k = fp_add(k, s_k[threadIdx.x * kSubLevels + p]);
+    s_sub[threadIdx.x * 7 + 6] = fp_norm(k.h, k.l);
+  }
   const cpair *r1 = sm_c + (size_t)(2 * v) * LD, *r2 = r1 + LD;
   const fpair *u1 = s_sub + (2 * v) * 7, *u2 = u1 + 7;
   float *tile = reinterpret_cast<float *>(sm_c);
@@ -599,28 +615,29 @@ static int screen_batch(specula_ctx *ctx, int n_screens, double pitch_m, double 
   int s;
   if (ctx->screen_ws.bytes < need && (s = ctx->screen_ws.alloc(need))) return s;
   cpair *rows = ctx->screen_ws.as<cpair>(), *tw = rows + (size_t)G * H * M, *subp = tw + M;
-  double2 *sub = reinterpret_cast<double2 *>(subp + (size_t)kSubLevels * M), *mean = sub + (size_t)kSubLevels * M, *cf = mean + 4;
-  double *sm = reinterpret_cast<double *>(cf + (size_t)G * 27);
-  fpair *amp = reinterpret_cast<fpair *>(sm + G);
+  double2 *sub = reinterpret_cast<double2 *>(subp + (size_t)kSubLevels * M);
+  double2 *mean = sub + (size_t)kSubLevels * M;
+  cpair *cf = reinterpret_cast<cpair *>(mean + 4);
+  fpair *sm = reinterpret_cast<fpair *>(cf + (size_t)G * 27), *amp = sm + G;
   if ((s = ensure_dynamic_smem((const void *)k_screen_rows<LOGM>, C::smem1)) ||
       (s = ensure_dynamic_smem((const void *)k_screen_cols<LOGM>, C::smem2)))
     return s;
   SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
-                 k_screen_tables<<<(std::max(H * H, M) + 255) / 256, 256, 0, st>>>(
+                 k_screen_tables<<<(std::max(H * H, M) + kTabThreads - 1) / kTabThreads, kTabThreads, 0, st>>>(
                      tw, sub, subp, amp, M, Md, coef, k0, inv_s));
   SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
                  k_screen_sub_mean<<<kSubLevels, 256, 0, st>>>(sub, M, mean));
   for (int g0 = 0; g0 < n_screens; g0 += G) {
     const int ng = std::min(G, n_screens - g0);
     SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
-                   k_screen_sub_coef<<<(ng + 7) / 8, 256, 0, st>>>(mean, Md, coef, k0, inv_s,
-                                                                   seed, sample0 + g0, ng, cf, sm));
+                   k_screen_sub_coef<<<ng, 32, 0, st>>>(mean, Md, coef, k0, inv_s, seed, sample0 + g0,
+                                                       cf, sm));
     SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
                    k_screen_rows<LOGM><<<dim3((H + C::RPB - 1) / C::RPB, ng), C::RPB * C::TPR,
                                          C::smem1, st>>>(tw, amp, seed, sample0 + g0, rows));
     SPECULA_LAUNCH(ctx, SPECULA_K_CALIB, st,
                    k_screen_cols<LOGM><<<dim3(M / C::W, ng), C::TB * C::TPR, C::smem2, st>>>(
-                       rows, tw, sub, subp, cf, sm, s1, s2, out + (size_t)g0 * M * M));
+                       rows, tw, subp, cf, sm, s1, s2, out + (size_t)g0 * M * M));
   }
   // the workspace is the context's, whatever stream its next call runs on
   SPECULA_CK(cudaStreamSynchronize(st));
