@@ -688,7 +688,7 @@ def systems_leg(ctx, steps=50):
     gs = fs.capture(st)
     time_graph(gs, lambda k: fs.t_dev.fill_(ws.dt_s * k), 5)
     mss = time_graph(gs, lambda k: fs.t_dev.fill_(ws.dt_s * k), steps)
-    out["andes400"] = {"config": "39 m, 400 px pupil padded 4x (1600^2 FFT = 32 x 50), 24 mod "
+    out["andes400"] = {"config": "39 m, 400 px pupil padded 4x (1600^2 FFT = 40 x 40), 24 mod "
                                  "points, 100x100 subaps of 4 px, images 120 subaps apart on a "
                                  "400 px detector, 35 layers, 4000 x %d MVM, FP32"
                                  % fs.R.shape[1],
@@ -746,8 +746,8 @@ def gemm_leg(ctx, pk, n=8192, reps=10):
         tot += e0.elapsed_time(e1)
     tf = 2.0 * n ** 3 / (best / 1e3) / 1e12
     peak = pk.get("bf16_tflops")
-    out = {"kernel": "k_gemm_tn<bf16, 256> (persistent, one CTA per SM; TMA ring of 4 x 48 KB; "
-                     "tcgen05 128x256x16 MMAs; two TMEM accumulators, epilogue overlapped)",
+    out = {"kernel": "k_gemm_pair<bf16> (persistent, CTA pairs; TMA ring of 6 x 32 KB per CTA; "
+                     "tcgen05 256x256x16 MMAs; two TMEM accumulators, epilogue overlapped)",
            "shape": [n, n, n], "best_ms": best, "mean_ms": tot / reps, "achieved_tflops": tf,
            "achieved_tflops_mean": 2.0 * n ** 3 / (tot / reps / 1e3) / 1e12,
            "peak_tflops": peak, "frac": (tf / peak) if peak else None,
