@@ -827,9 +827,13 @@ static int run_split2(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
   const int total = n_batch * nc;
   const int vpc = K::vecs(p->blockR);
   const float scale = 1.0f / (float)p->n_mod;
+  // The workspace has a field and a partial detector for each of nbw batch
+  // elements, the most that `chunk` slots of the whole circle touch; of a slot
+  // range's fewer slots per element as many as touch no more.
+  const int chunk = std::min(p->chunk, (p->nbw - 1) * nc);
   int field_done = -1, det_done = -1;
-  for (int j0 = 0; j0 < total; j0 += p->chunk) {
-    const int nj = std::min(p->chunk, total - j0);
+  for (int j0 = 0; j0 < total; j0 += chunk) {
+    const int nj = std::min(chunk, total - j0);
     const int b0 = j0 / nc, b1 = (j0 + nj - 1) / nc;
     const int fb = std::max(b0, field_done + 1);
     if (fb <= b1) {

@@ -639,8 +639,9 @@ static int pair_run_t(specula_ctx *ctx, PwfsPlan *p, const float *amp, const flo
   const int nc = (p->slot_hi < 0 ? p->nc : p->slot_hi) - s0;
   int s = pair_units(p, s0, nc);
   if (s) return s;
-  // whole batch elements per chunk
-  const int per = std::max(1, p->chunk / nc);
+  // whole batch elements per chunk, at most the nbw that the workspace has fields
+  // for (a slot range has fewer slots per element than the chunk was made for)
+  const int per = std::min(std::max(1, p->chunk / nc), p->nbw);
   constexpr bool two = N1 % 2 == 0 && (N1 / 2) % 2 == 1;
   const int tc = p->pair_blockK / (two ? 64 : 32);
   const int vpc = p->pair_blockR / 32;
