@@ -390,8 +390,10 @@ static inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 // in flight per lane and every activation load used for both rows.  (One warp
 // per row with scalar activation loads took 51 us for 13344-2048-2048-4000,
 // 1.5 TB/s: four times the load instructions and half the bytes in flight;
-// now 18.8 us.)  Every layer's CTAs start under the layer before and send their
-// weight rows to L2 first (19.4 us without).
+// now 19.7 us.)  A hidden layer's CTAs start under the layer before and send their
+// weight rows to L2 first.  The first layer's start when the kernel before the
+// network has left.  (Under the last layer of the call before: 18.6 us, but then every
+// kernel that reads the network's output starts while it is being written.)
 constexpr int kInferMax = 4;
 constexpr int kGemvWarps = 4, kGemvRows = 2;
 
@@ -402,6 +404,23 @@ __device__ __forceinline__ uint4 ld_stream_w(const uint4 *p) {
                : "l"(p));
   return v;
 }
+// Activations: plain loads.  A layer's CTAs are resident while the layer before
+// still writes them, and the non-coherent path (ld.global.nc, what __ldg and const
+// __restrict__ give) is only defined for memory that is not written during the
+// kernel's life.
+__device__ __forceinline__ float4 ld_act4(const float *p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_act(const float *p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
 
@@ -410,9 +429,11 @@ __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u 
 // VX (ldx % 4 == 0 and x aligned); grid ceil(n_out / 2), block 128.
 template <int NB, bool GELU, bool VX>
 __global__ void __launch_bounds__(kGemvWarps * 32) k_mlp_gemv(
-    const __nv_bfloat16 *__restrict__ W, int ldw, const float *__restrict__ x, int ldx, int K,
-    int n_out, int nb, const float *__restrict__ bias, float *__restrict__ out, int ldo) {
-  pdl_trigger();
+    const __nv_bfloat16 *__restrict__ W, int ldw, const float *x, int ldx, int K, int n_out, int nb,
+    const float *__restrict__ bias, float *out, int ldo) {
+  // the last layer (no GELU) does not: a kernel behind the network starts once its
+  // CTAs have left, as behind any other kernel
+  if constexpr (GELU) pdl_trigger();
   __shared__ float s_w[kGemvWarps][kGemvRows * NB];
   const int o0 = blockIdx.x * kGemvRows;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -450,13 +471,12 @@ __global__ void __launch_bounds__(kGemvWarps * 32) k_mlp_gemv(
             const float *xp = x + (size_t)q * ldx + 8 * j;
             float xv[8];
             if constexpr (VX) {
-              const float4 a = __ldg(reinterpret_cast<const float4 *>(xp));
-              const float4 c = __ldg(reinterpret_cast<const float4 *>(xp) + 1);
+              const float4 a = ld_act4(xp), c = ld_act4(xp + 4);
               xv[0] = a.x; xv[1] = a.y; xv[2] = a.z; xv[3] = a.w;
               xv[4] = c.x; xv[5] = c.y; xv[6] = c.z; xv[7] = c.w;
             } else {
 #pragma unroll
-              for (int e = 0; e < 8; ++e) xv[e] = __ldg(xp + e);
+              for (int e = 0; e < 8; ++e) xv[e] = ld_act(xp + e);
             }
 #pragma unroll
             for (int i = 0; i < kGemvRows; ++i) {
@@ -478,7 +498,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32) k_mlp_gemv(
       const float wk = __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(w8[i])[kt]);
 #pragma unroll
       for (int q = 0; q < NB; ++q)
-        if (q < nb) acc[i][q] += wk * __ldg(x + (size_t)q * ldx + kt);
+        if (q < nb) acc[i][q] += wk * ld_act(x + (size_t)q * ldx + kt);
     }
   }
 #pragma unroll
