@@ -609,8 +609,8 @@ static int sm_count() {
   return sms[dev];
 }
 
-int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n, float *C,
-                      cudaStream_t st) {
+static int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n, float *C,
+                             cudaStream_t st) {
   const bool v4 = n % 4 == 0 && (((uintptr_t)part | (uintptr_t)C) % 16) == 0;
   const size_t threads = v4 ? n / 4 : n;
   const unsigned grid = (unsigned)std::min<size_t>((threads + 255) / 256, 8192);

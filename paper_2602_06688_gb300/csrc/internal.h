@@ -376,13 +376,10 @@ __device__ __forceinline__ void column_sums(const ColSums &S, int w, int nw) {
 #endif
 // C_q = A_q B_q^T for up to three products of one K in one launch, and the column
 // sums beside them.  K is summed in splits[q] slices (a count from gemm_splits),
-// added in order as gemm_split_reduce adds partials.
+// added in order as k_split_reduce adds partials.
 int gemm_bf16_group(specula_ctx *ctx, int n, const void *const *A, const void *const *B,
                     const int *M, const int *N, int K, const int *splits, float *const *C,
                     const ColSums &cs, cudaStream_t st);
-// C[n] = the sum over s < splits of part[s][n], in order
-int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, size_t n, float *C,
-                      cudaStream_t st);
 // C = sum over t < n_terms (<= 3) of A_t B_t^T, one accumulation on the
 // tensor cores (split-precision products); every A_t is M x K, every B_t is
 // N x K, bf16, row-major

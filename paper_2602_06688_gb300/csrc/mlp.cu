@@ -214,14 +214,12 @@ __device__ __forceinline__ void adam_step(float &p, float &m, float &v, float g,
 // weights' bf16 copy and its transpose come from the same registers (three
 // launches per layer and one more pass over the weights before).  Blocks
 // [first[l], first[l + 1]) are layer l's 32 x 128 weight tiles, a row of
-// four-float loads per warp; the rest 256 bias entries each.  The weight
-// gradients are read as their GEMMs' partials.  Bound by L2: at least 32 bytes
-// per weight.
+// four-float loads per warp; the rest 256 bias entries each.  Bound by L2: 32
+// bytes per weight.
 constexpr int kAdamC = 128;
 struct AdamLayer {
   float *W, *mW, *vW, *b, *mb, *vb;
-  Partials gW;   // the gradient as its GEMM left it
-  const float *gb;
+  const float *gW, *gb;
   __nv_bfloat16 *Wb, *WbT;
   int R, C;
 };
@@ -254,22 +252,7 @@ __global__ void __launch_bounds__(TT * 8) k_adam(const AdamArgs A, float lr_t, f
     p[k] = *reinterpret_cast<const float4 *>(L.W + e);
     m[k] = *reinterpret_cast<const float4 *>(L.mW + e);
     v[k] = *reinterpret_cast<const float4 *>(L.vW + e);
-    g[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-#pragma unroll 2
-  for (int s = 0; s < L.gW.splits; ++s) {
-    float4 x[NR];
-#pragma unroll
-    for (int k = 0; k < NR; ++k)
-      x[k] = __ldg(reinterpret_cast<const float4 *>(
-          L.gW.p + (size_t)s * L.gW.n + (size_t)(r0 + warp + 8 * k) * L.C + c0 + 4 * lane));
-#pragma unroll
-    for (int k = 0; k < NR; ++k) {
-      g[k].x += x[k].x;
-      g[k].y += x[k].y;
-      g[k].z += x[k].z;
-      g[k].w += x[k].w;
-    }
+    g[k] = __ldg(reinterpret_cast<const float4 *>(L.gW + e));
   }
 #pragma unroll
   for (int k = 0; k < NR; ++k) {
@@ -370,7 +353,6 @@ struct specula_mlp {
   int bmax;        // padded batch capacity
   int t = 0;       // Adam steps taken
   int last_b = 0;  // batch of the last forward
-  int gsplits[3] = {1, 1, 1};   // partials of the weight gradients in gW
   DevBuf W[3], b[3], mW[3], vW[3], mb[3], vb[3], Wb[3], WbT[3], gW[3], gb[3];
   DevBuf Xb, XbT, Z[2], H[2], HT[2], Y, dYf, dYb, dYbT, dA[2], dZb[2], dZbT[2];
   DevBuf work, part, loss;
@@ -545,8 +527,9 @@ constexpr int kDwGroupK = 4096;
 // bound by what they write: one launch over all the layers' 128 x 128 tiles, a
 // tile's K slices added in registers, so the sums are those of the split-K
 // products to the last bit.  Beyond kDwGroupK each layer's own launch, its K split
-// over the SMs; the partials stay in the layer's buffer: Adam adds them as it reads
-// them, get_grad when asked.  Own launches / one launch, a step of 2512-1024-1024-500:
+// over the SMs, and their sum: gW holds the gradient whatever the batch, so a replayed
+// graph's Adam or get_grad needs no state of the host's.  Own launches (their sums
+// left to Adam then) / one launch, a step of 2512-1024-1024-500:
 // 123 / 95 us at 256 rows, 294 / 263 at 2048; of 300-128-128-60, four tiles in all:
 // 98 / 74 at 1024, 225 / 169 at 4096 (the bias gradients in it, as below).
 static int mlp_gemm_dw(specula_mlp *p, const void *const *A, const void *const *B, int batch,
@@ -559,8 +542,7 @@ static int mlp_gemm_dw(specula_mlp *p, const void *const *A, const void *const *
     N[l] = p->np[l];
     out[l] = p->gW[l].as<float>();
     splits[l] = mlp_splits(M[l], N[l], Bp);
-    p->gsplits[l] = group ? 1 : splits[l];
-    if ((size_t)p->gsplits[l] * M[l] * N[l] * 4 > p->gW[l].bytes) return SPECULA_EINVAL;
+    if (!group && (size_t)splits[l] * M[l] * N[l] > p->work_floats) return SPECULA_EINVAL;
   }
   // the bias gradients in the same launch, by warps that the products leave idle: a
   // block that summed its tile column last made each producer of dZ 4 us longer
@@ -578,7 +560,8 @@ static int mlp_gemm_dw(specula_mlp *p, const void *const *A, const void *const *
   SPECULA_LAUNCH_PDL(p->ctx, SPECULA_K_MLP, st, k_bias_grad, (M[0] + M[1] + M[2]) / 128, 128, 0,
                      cs);
   for (int l = 2; l >= 0; --l)
-    if ((s = gemm_bf16_partials(p->ctx, A[l], B[l], M[l], N[l], Bp, p->gsplits[l], out[l], st)))
+    if ((s = gemm_bf16_tn(p->ctx, A[l], B[l], M[l], N[l], Bp, out[l], splits[l],
+                          p->work.as<float>(), st)))
       return s;
   return SPECULA_OK;
 }
@@ -610,18 +593,15 @@ extern "C" int specula_mlp_create(specula_ctx *ctx, int32_t n_in, int32_t n_h1, 
   int s;
   for (int l = 0; l < 3; ++l) {
     const size_t nw = (size_t)p->np[l + 1] * p->np[l], nb = p->np[l + 1];
-    size_t gw = nw;   // the gradient's partials, for every padded batch up to the capacity
-    for (int b = 128; b <= Bp; b += 128)
-      if (b > kDwGroupK) gw = std::max(gw, nw * mlp_splits(p->np[l + 1], p->np[l], b));
     if ((s = p->W[l].alloc(nw * 4)) || (s = p->mW[l].alloc(nw * 4)) || (s = p->vW[l].alloc(nw * 4)) ||
-        (s = p->gW[l].alloc(gw * 4)) || (s = p->Wb[l].alloc(nw * 2)) || (l > 0 && (s = p->WbT[l].alloc(nw * 2))) ||
+        (s = p->gW[l].alloc(nw * 4)) || (s = p->Wb[l].alloc(nw * 2)) || (l > 0 && (s = p->WbT[l].alloc(nw * 2))) ||
         (s = p->b[l].alloc(nb * 4)) || (s = p->mb[l].alloc(nb * 4)) || (s = p->vb[l].alloc(nb * 4)) ||
         (s = p->gb[l].alloc(nb * 4)))
       return s;
     SPECULA_CK(cudaMemset(p->W[l].p, 0, nw * 4));
     SPECULA_CK(cudaMemset(p->mW[l].p, 0, nw * 4));
     SPECULA_CK(cudaMemset(p->vW[l].p, 0, nw * 4));
-    SPECULA_CK(cudaMemset(p->gW[l].p, 0, gw * 4));
+    SPECULA_CK(cudaMemset(p->gW[l].p, 0, nw * 4));
     SPECULA_CK(cudaMemset(p->b[l].p, 0, nb * 4));
     SPECULA_CK(cudaMemset(p->mb[l].p, 0, nb * 4));
     SPECULA_CK(cudaMemset(p->vb[l].p, 0, nb * 4));
@@ -638,13 +618,17 @@ extern "C" int specula_mlp_create(specula_ctx *ctx, int32_t n_in, int32_t n_h1, 
       (s = p->dZb[0].alloc((size_t)Bp * h1 * 2)) || (s = p->dZb[1].alloc((size_t)Bp * h2 * 2)) ||
       (s = p->dZbT[0].alloc((size_t)Bp * h1 * 2)) || (s = p->dZbT[1].alloc((size_t)Bp * h2 * 2)))
     return s;
-  // split-K workspace: the largest of the forward and input-gradient GEMMs, for every
-  // padded batch up to the capacity
+  // split-K workspace: the largest of a step's GEMMs that use it, for every padded
+  // batch up to the capacity
   size_t wf = 1;
   for (int b = 128; b <= Bp; b += 128) {
-    const int shapes[5][3] = {{b, h1, in}, {b, h2, h1}, {b, o, h2}, {b, h2, o}, {b, h1, h2}};
-    for (auto &sh : shapes)
+    const int shapes[8][3] = {{b, h1, in}, {b, h2, h1}, {b, o, h2},  {b, h2, o},
+                              {b, h1, h2}, {h1, in, b}, {h2, h1, b}, {o, h2, b}};
+    // (the last three, the weight gradients, only beyond kDwGroupK)
+    for (int i = 0; i < (b > kDwGroupK ? 8 : 5); ++i) {
+      const auto &sh = shapes[i];
       wf = std::max(wf, (size_t)mlp_splits(sh[0], sh[1], sh[2]) * sh[0] * sh[1]);
+    }
   }
   p->work_floats = wf;
   if ((s = p->work.alloc(wf * 4))) return s;
@@ -711,15 +695,7 @@ extern "C" int specula_mlp_get_layer(specula_mlp *p, int32_t layer, float *W_hos
 extern "C" int specula_mlp_get_grad(specula_mlp *p, int32_t layer, float *dW_host,
                                     float *db_host) {
   if (!p || layer < 0 || layer > 2 || !dW_host || !db_host) return SPECULA_EINVAL;
-  if (p->gsplits[layer] == 1) return copy_out(p, layer, p->gW[layer], p->gb[layer], dW_host, db_host);
-  SPECULA_CK(cudaSetDevice(p->ctx->device));
-  SPECULA_CK(cudaDeviceSynchronize());
-  const size_t n = (size_t)p->np[layer + 1] * p->np[layer];
-  DevBuf g;
-  int s = g.alloc(n * 4);
-  if (!s)
-    s = gemm_split_reduce(p->ctx, p->gW[layer].as<float>(), p->gsplits[layer], n, g.as<float>(), 0);
-  return s ? s : copy_out(p, layer, g, p->gb[layer], dW_host, db_host);
+  return copy_out(p, layer, p->gW[layer], p->gb[layer], dW_host, db_host);
 }
 
 extern "C" int specula_mlp_forward(specula_mlp *p, const float *X_dev, int32_t batch,
@@ -835,8 +811,7 @@ extern "C" int specula_mlp_adam(specula_mlp *p, float lr, float b1, float b2, fl
     const int R = p->np[l + 1], C = p->np[l];
     A.L[l] = AdamLayer{p->W[l].as<float>(),  p->mW[l].as<float>(), p->vW[l].as<float>(),
                        p->b[l].as<float>(),  p->mb[l].as<float>(), p->vb[l].as<float>(),
-                       Partials{p->gW[l].as<float>(), p->gsplits[l], (size_t)R * C},
-                       p->gb[l].as<float>(),
+                       p->gW[l].as<float>(), p->gb[l].as<float>(),
                        p->Wb[l].as<__nv_bfloat16>(), p->WbT[l].as<__nv_bfloat16>(), R, C};
     A.first[l + 1] = A.first[l] + (R / TT) * (C / kAdamC);
     A.bias_first[l + 1] = A.bias_first[l] + (R + TT * 8 - 1) / (TT * 8);
