@@ -564,12 +564,14 @@ int specula_pwfs_set_slots(specula_ctx *ctx, const specula_pupil_desc *pupil,
 int specula_pwfs_set_form(specula_ctx *ctx, const specula_pupil_desc *pupil,
                           const specula_pwfs_desc *pwfs, int32_t form);
 
-/* Autotuner: time every candidate (passes in {2, 3, 4}; chunk in
- * {1,2,3,4,6,8,12,16,24,32,48,64} up to the batch's item count and with
- * workspace <= max_workspace_bytes, for passes 4 whole batch elements
- * {1, 2, 4, ...} up to the batch; ka in {1, 2}) with CUDA events over
+/* Autotuner: time the plan's present tiling and every candidate (passes in {2,
+ * 3, 4}; chunk in {1,2,3,4,6,8,12,16,24,32,48,64} up to the batch's item count,
+ * for passes 4 and for batches of more than 64 slots in passes 2 whole batch
+ * elements {1, 2, 4, ...} up to the batch and 4096 slots; ka in 1 .. 8), each with a
+ * workspace <= max_workspace_bytes, with CUDA events over
  * `reps` images of the caller's inputs on
- * `stream`, keep the fastest in the plan and return it.  Set-up call: may
+ * `stream`, keep the fastest in the plan (the present one unless another is
+ * faster in a second run too) and return it.  Set-up call: may
  * reallocate the workspace and synchronises the stream.  det_dev is
  * overwritten. */
 int specula_pwfs_autotune(specula_ctx *ctx, const specula_pupil_desc *pupil,

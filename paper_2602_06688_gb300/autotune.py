@@ -16,9 +16,9 @@ def cache_path():
         os.path.expanduser("~"), ".cache", "specula_gb300", "tiles.json")
 
 
-# bumped whenever the kernels' best tiling can change (v6: the two-pass form's
-# transforms packed several to a warp, zero inputs left out)
-_VERSION = "v6"
+# bumped whenever the kernels' best tiling or the candidates change (v7: the plan's
+# own tiling and whole batch elements are candidates)
+_VERSION = "v7"
 
 
 def _key(device_name, pupil, pwfs, n_batch):

@@ -1048,52 +1048,82 @@ int pwfs_run(specula_ctx *ctx, PwfsPlan *p, const float *amp, const float *phase
   }
 }
 
-// Time each candidate tiling on the caller's buffers (set-up call: may
-// reallocate the workspace and synchronises) and keep the fastest.
+// Time the plan's present tiling and each candidate on the caller's buffers (set-up
+// call: may reallocate the workspace and synchronises) and keep the fastest; the
+// present one stays unless another is also faster in a second, longer run of the two.
+// Candidates: a list of small chunks, and whole batch elements (nc, 2 nc, 4 nc, ...
+// slots) for batches whose slots go beyond the list, where the plan's own default is
+// one of them and the list's last, nearly empty waves cost most (8 m image, batch 16:
+// 157 us untuned, 184 with the list alone; batch 256: 2443 and 2773, tuned now 2354).
 int pwfs_autotune(specula_ctx *ctx, PwfsPlan *p, const float *amp, const float *phase,
                   int n_batch, float *det, cudaStream_t st, int reps, size_t max_ws_bytes,
                   int *best_chunk, int *best_ka, int *best_passes) {
   static const int kChunks[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
+  constexpr int kListEnd = 64, kMaxChunk = 4096;   // what specula_pwfs_set_tiles takes
   const size_t per_item = ((size_t)p->n_pix * p->N + (size_t)p->N * p->N) * sizeof(float2);
+  const auto item_bytes = [&](int passes) {
+    return passes != 3 ? (size_t)p->n_pix * p->N * sizeof(float2) : per_item;
+  };
   const int total = n_batch * p->n_mod;
-  float best = 1e30f;
-  int bc = p->chunk, bk = p->ka, bp = p->passes;
   cudaEvent_t e0, e1;
   SPECULA_CK(cudaEventCreate(&e0));
   SPECULA_CK(cudaEventCreate(&e1));
+  const auto run = [&](int chunk, int ka, int passes, int n, float *ms) -> int {
+    int s = pwfs_set_tiles(p, chunk, ka, passes);
+    if (!s) s = pwfs_run(ctx, p, amp, phase, n_batch, det, st);   // warm-up
+    if (s) return s;
+    cudaEventRecord(e0, st);
+    for (int r = 0; r < n; ++r)
+      if ((s = pwfs_run(ctx, p, amp, phase, n_batch, det, st))) return s;
+    cudaEventRecord(e1, st);
+    if (cudaEventSynchronize(e1) != cudaSuccess) return SPECULA_ECUDA;
+    cudaEventElapsedTime(ms, e0, e1);
+    return SPECULA_OK;
+  };
   int status = SPECULA_OK;
+  float best = 1e30f;
+  int bc = p->chunk, bk = p->ka, bp = p->passes;
+  const int c0 = bc, k0 = bk, p0 = bp;
+  const bool keep_ok = (size_t)c0 * item_bytes(p0) <= max_ws_bytes;
+  const auto consider = [&](int chunk, int ka, int passes) -> int {
+    float ms = 0.f;
+    const int s = run(chunk, ka, passes, reps, &ms);
+    if (!s && ms < best) { best = ms; bc = p->chunk; bk = ka; bp = passes; }
+    return s;
+  };
+  // ka sets the row pass's grid depth (slots per warp): values that fill
+  // whole waves of CTAs can win (the ELT frame: ka 5, 300 CTAs on 304
+  // slots), so the search goes to 8
+  const auto consider_kas = [&](int chunk, int passes) -> int {
+    for (int ka = 1; ka <= std::min(passes == 4 ? 1 : 8, chunk); ++ka) {
+      const int s = consider(chunk, ka, passes);
+      if (s) return s;
+    }
+    return SPECULA_OK;
+  };
+  if (keep_ok && (status = consider(c0, k0, p0))) goto done;
   for (int passes = 2; passes <= 4; ++passes) {
     if (passes == 2 && !p->two_ok) continue;
     if (passes == 3 && p->pad != 2) continue;
     if (passes == 4 && !p->pair_ok) continue;
-    const size_t item = passes != 3 ? (size_t)p->n_pix * p->N * sizeof(float2) : per_item;
-    for (int c : kChunks) {
-      if (passes == 4) {
-        // whole batch elements: nc, 2 nc, 4 nc, ... slots
-        if (c != 1 && (c & (c - 1))) continue;
-        if (c > std::max(n_batch, 1) && c != 1) break;
-        if ((size_t)c * p->nc * item > max_ws_bytes && c != 1) break;
-      } else {
-        if (c > std::max(total, 1) && c != 1) break;
-        if ((size_t)c * item > max_ws_bytes && c != 1) break;
+    const size_t item = item_bytes(passes);
+    if (passes != 4)
+      for (int c : kChunks) {
+        if (c != 1 && (c > total || (size_t)c * item > max_ws_bytes)) break;
+        if ((status = consider_kas(c, passes))) goto done;
       }
-      // ka sets the row pass's grid depth (slots per warp): values that fill
-      // whole waves of CTAs can win (the ELT frame: ka 5, 300 CTAs on 304
-      // slots), so the search goes to 8
-      for (int ka = 1; ka <= (passes == 4 ? 1 : 8); ++ka) {
-        if (ka > c) break;
-        if ((status = pwfs_set_tiles(p, passes == 4 ? c * p->nc : c, ka, passes))) goto done;
-        if ((status = pwfs_run(ctx, p, amp, phase, n_batch, det, st))) goto done;   // warm-up
-        cudaEventRecord(e0, st);
-        for (int r = 0; r < reps; ++r)
-          if ((status = pwfs_run(ctx, p, amp, phase, n_batch, det, st))) goto done;
-        cudaEventRecord(e1, st);
-        if (cudaEventSynchronize(e1) != cudaSuccess) { status = SPECULA_ECUDA; goto done; }
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best) { best = ms; bc = p->chunk; bk = ka; bp = passes; }
+    if (passes == 4 || (passes == 2 && (long long)n_batch * p->nc > kListEnd))
+      for (int c = 1; c <= n_batch && (long long)c * p->nc <= kMaxChunk; c *= 2) {
+        if ((size_t)c * p->nc * item > max_ws_bytes && (c != 1 || passes == 2)) break;
+        if ((status = consider_kas(c * p->nc, passes))) goto done;
       }
-    }
+  }
+  if (keep_ok && (bc != c0 || bk != k0 || bp != p0)) {
+    float now = 0.f, other = 0.f;
+    if ((status = run(c0, k0, p0, 4 * reps, &now)) ||
+        (status = run(bc, bk, bp, 4 * reps, &other)))
+      goto done;
+    if (now <= other) { bc = c0; bk = k0; bp = p0; }
   }
   status = pwfs_set_tiles(p, bc, bk, bp);
   *best_chunk = bc;
