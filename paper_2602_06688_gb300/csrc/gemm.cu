@@ -623,14 +623,19 @@ static int gemm_split_reduce(specula_ctx *ctx, const float *part, int splits, si
   return SPECULA_OK;
 }
 
-// Whether a product runs on CTA pairs: enough 256 x 256 x kb items for every pair
-// (below that the single CTAs' finer tiles fill the SMs better), no more than an
-// eighth of the rows padding, and K long enough that loading bounds it: 4096 x
-// 4096 at 16 K blocks takes 37.5 us either way, 2048 x 4000 at 209 139 against 169.
+// Whether a product runs on CTA pairs: K long enough that loading bounds it (4096 x
+// 4096 at 16 K blocks takes 37.5 us either way), no more than an eighth of the rows
+// padding, and the pairs' waves shorter in all.  A K block of a tile takes 512
+// clocks on a pair and 768 on a single CTA (k_gemm_pair), so a second wave with few tiles
+// in it costs more than the pairs give: 1152 x 4096 is 144 tiles, one wave of single
+// CTAs, or 80 pair tiles, two waves of 76 (K = 4096: 26.1 against 45.3 us); 2048 x 4000
+// at 209 blocks takes 139 us on pairs against 169.
 static bool gemm_pairs(int M, int tiles_n, int splits, int kb_per_split, int sms) {
   const int tiles_m = (M + GBM - 1) / GBM;
-  return (tiles_m % 2 == 0 || tiles_m >= 8) && kb_per_split >= 16 &&
-         (long long)(tiles_m + 1) / 2 * tiles_n * splits >= sms / 2;
+  const long long cols = (long long)tiles_n * splits;
+  const auto waves = [](long long items, int slots) { return (items + slots - 1) / slots; };
+  return sms >= 2 && (tiles_m % 2 == 0 || tiles_m >= 8) && kb_per_split >= 16 &&
+         512 * waves((tiles_m + 1) / 2 * cols, sms / 2) < 768 * waves(tiles_m * cols, sms);
 }
 
 template <bool TF32, int BN>
