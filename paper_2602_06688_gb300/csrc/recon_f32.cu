@@ -1,11 +1,15 @@
 // Float32 modal reconstructor products: modes[b] = R slopes[b] (Modalrec /
 // Recmat, App. A, Tabs. 3-4), for one slope vector and for batches.
 //
-// Two kernels, each a fixed order of float32 additions (bit-reproducible):
-//   one vector  k_mvm_f32_split  one row of R per CTA
-//   batches     k_mvm_f32_tile   64 rows x 8-64 vectors per CTA, both staged in
-//                                shared memory, K split over a cluster
-// Both read R from HBM once per 64 vectors.  Up to about 20 vectors that read
+// Three kernels, each a fixed order of float32 additions (bit-reproducible):
+//   one vector   k_mvm_f32_split  one row of R per CTA
+//   2-4 vectors  k_mvm_f32_rows   two rows of R per CTA or per warp (and 5-8 vectors
+//                                 where R has few rows)
+//   batches      k_mvm_f32_tile   64 rows x 8-64 vectors per CTA, both staged in
+//                                 shared memory, K split over a cluster
+// Which one, and its tile, follow the batch and the sizes, so the last bits of a
+// frame's modes depend on the batch it is in.
+// All read R from HBM once per 64 vectors.  Up to about 20 vectors that read
 // is the bound (a product takes 2 flops per vector and 4 bytes of R), beyond
 // it the FP32 pipes are.  Measured, against one warp per row and four vectors
 // per pass over R: 4000 x 13344 on 8 vectors 120.8 -> 51.3 us (4.2 TB/s of R),
@@ -100,6 +104,97 @@ __global__ void __launch_bounds__(kSplitWarps * 32) k_mvm_f32_split(
     for (int w = 0; w < kSplitWarps; ++w) v += s_w[w];
     m[row] = v;
   }
+}
+
+// Up to NB slope vectors, two rows of R per WPR warps, each warp a contiguous segment
+// of both: every load of the slopes serves two rows, and there is nothing to stage or
+// to wait for, so a product is as short as its longest warp (the tiles below: at
+// least 4 us).  WPR = 1, a row per warp, where a warp's UL loads take a whole row
+// (kShortRow); else 4.  Before (the tiles) / now, 2 and 4 vectors: 64 x 512 4.5 / 1.9,
+// 4.6 / 2.3 us; 4000 x 200 4.0 / 1.9, 4.0 / 2.3; 500 x 2512 5.5 / 3.5, 5.6 / 4.3;
+// 4000 x 13344 49.6 / 36.6, 49.5 / 44.6.
+constexpr int kRowsUnroll = 4;
+template <int V> constexpr int kShortRow = 32 * kRowsUnroll * V;
+template <int V, int NB, int WPR>
+__global__ void __launch_bounds__(kSplitWarps * 32) k_mvm_f32_rows(
+    const float *__restrict__ R, const float *__restrict__ s, float *__restrict__ m, int n_modes,
+    int n_slopes, int nb) {
+  pdl_wait();
+  using T = typename VecOf<V>::T;
+  constexpr int ROWS = 2, UL = kRowsUnroll;
+  __shared__ float s_w[kSplitWarps][ROWS * NB];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row0 = (blockIdx.x * (kSplitWarps / WPR) + warp / WPR) * ROWS;
+  const T *r4[ROWS], *s4[NB];
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i)
+    r4[i] = reinterpret_cast<const T *>(R + (size_t)min(row0 + i, n_modes - 1) * n_slopes);
+#pragma unroll
+  for (int q = 0; q < NB; ++q)   // vectors past the batch repeat its last
+    s4[q] = reinterpret_cast<const T *>(s + (size_t)min(q, nb - 1) * n_slopes);
+  const int n4 = n_slopes / V;
+  const int seg = (n4 + WPR - 1) / WPR;
+  const int lo = warp % WPR * seg, hi = min(n4, lo + seg);
+  float acc[ROWS][NB];
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+    for (int q = 0; q < NB; ++q) acc[i][q] = 0.f;
+  for (int j0 = lo + lane; j0 < hi; j0 += UL * 32) {
+    T a[UL][ROWS];
+#pragma unroll
+    for (int u = 0; u < UL; ++u)
+#pragma unroll
+      for (int i = 0; i < ROWS; ++i)
+        a[u][i] = (j0 + 32 * u < hi) ? ld_stream(r4[i] + j0 + 32 * u) : T{};
+#pragma unroll
+    for (int u = 0; u < UL; ++u) {
+      const int j = j0 + 32 * u;
+      if (j < hi) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+          const T x = __ldg(s4[q] + j);
+#pragma unroll
+          for (int i = 0; i < ROWS; ++i) acc[i][q] += dotv(a[u][i], x);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const float v = warp_sum_f(acc[i][q]);
+      if constexpr (WPR == 1) {
+        if (lane == 0 && q < nb && row0 + i < n_modes) m[(size_t)q * n_modes + row0 + i] = v;
+      } else {
+        if (lane == 0) s_w[warp][q * ROWS + i] = v;
+      }
+    }
+  if constexpr (WPR > 1) {
+    static_assert(WPR == kSplitWarps, "the CTA's warps share its rows");
+    __syncthreads();
+    const int i = threadIdx.x % ROWS, q = threadIdx.x / ROWS;
+    if (q < min(NB, nb) && row0 + i < n_modes) {
+      float v = 0.f;
+#pragma unroll
+      for (int w = 0; w < kSplitWarps; ++w) v += s_w[w][threadIdx.x];
+      m[(size_t)q * n_modes + row0 + i] = v;
+    }
+  }
+}
+
+template <int V, int NB>
+static int launch_rows(specula_ctx *ctx, const float *R, const float *s, float *m, int n_modes,
+                       int n_slopes, int nb, cudaStream_t st) {
+  if (n_slopes <= kShortRow<V>)
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_RECON, st, (k_mvm_f32_rows<V, NB, 1>),
+                       (n_modes + 2 * kSplitWarps - 1) / (2 * kSplitWarps), kSplitWarps * 32, 0, R,
+                       s, m, n_modes, n_slopes, nb);
+  else
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_RECON, st, (k_mvm_f32_rows<V, NB, kSplitWarps>),
+                       (n_modes + 1) / 2, kSplitWarps * 32, 0, R, s, m, n_modes, n_slopes, nb);
+  return SPECULA_OK;
 }
 
 // Batches: C[b][row] over tiles of 64 rows x 8-64 vectors, 256 threads.  Both
@@ -287,18 +382,25 @@ static int launch_tile(specula_ctx *ctx, const float *R, const float *s, float *
 template <int V>
 static int run_v(specula_ctx *ctx, const float *R, const float *s, float *m, int n_modes,
                  int n_slopes, int nb, cudaStream_t st) {
-  if (nb == 1)
+  if (nb == 1) {
     SPECULA_LAUNCH_PDL(ctx, SPECULA_K_RECON, st, (k_mvm_f32_split<V>), n_modes, kSplitWarps * 32,
                        0, R, s, m, n_modes, n_slopes);
-  else if (nb <= 8)
-    return launch_tile<4, 2, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
-  else if (nb <= 16)
-    return launch_tile<4, 4, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
-  else if (nb <= 32)
-    return launch_tile<8, 4, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
-  else
-    return launch_tile<8, 8, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
-  return SPECULA_OK;
+    return SPECULA_OK;
+  }
+  if (nb == 2) return launch_rows<V, 2>(ctx, R, s, m, n_modes, n_slopes, nb, st);
+  // (single floats: four vectors' loads for two of R cost more than staging does, 500 x
+  // 2511 on 4 vectors 8.8 us against the tiles' 6.4)
+  if (nb <= 4 && (V > 1 || n_slopes <= kShortRow<V>))
+    return launch_rows<V, 4>(ctx, R, s, m, n_modes, n_slopes, nb, st);
+  // 5-8 vectors: the rows where R is too short to give the SMs tiles, up to 16 of them
+  // (8 vectors, rows / tiles: 64 x 512 1.7 / 4.6 us, 500 x 2512 3.9 / 5.6, 1000 x 5000
+  // 8.2 / 12.1; 2000 x 6672 19.9 / 16.2, 4000 x 512 7.2 / 5.6)
+  if (nb <= 8 && n_modes <= 16 * kTm && V == 4)
+    return launch_rows<V, 8>(ctx, R, s, m, n_modes, n_slopes, nb, st);
+  if (nb <= 8) return launch_tile<4, 2, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
+  if (nb <= 16) return launch_tile<4, 4, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
+  if (nb <= 32) return launch_tile<8, 4, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
+  return launch_tile<8, 8, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
 }
 
 int recon_f32_run(specula_ctx *ctx, const float *R, const float *s, float *m, int n_modes,
