@@ -12,9 +12,9 @@
 // All read R from HBM once per 64 vectors.  Up to about 20 vectors that read
 // is the bound (a product takes 2 flops per vector and 4 bytes of R), beyond
 // it the FP32 pipes are.  Measured, against one warp per row and four vectors
-// per pass over R: 4000 x 13344 on 8 vectors 120.8 -> 51.3 us (4.2 TB/s of R),
-// on 16 vectors 72.7 us, on 32 120 us; 500 x 25600 on 256 vectors 6.1 ms ->
-// 0.19 ms (34 TFLOP/s).
+// per pass over R: 4000 x 13344 on 8 vectors 116 -> 49 us (4.4 TB/s of R),
+// on 16 vectors 69 us, on 32 117 us; 500 x 25600 on 256 vectors 5.7 ms ->
+// 0.19 ms (35 TFLOP/s).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -201,24 +201,34 @@ static int launch_rows(specula_ctx *ctx, const float *R, const float *s, float *
 // operands are K-contiguous, so 64-deep stages go to shared memory as they
 // lie (cp.async) and each thread's RM x RN products take two neighbouring k at
 // a time (packed float32 FMAs, no operand moves).  The eight warps are two
-// row halves x four quarters of a stage's K.  The 16 products of a quarter
-// stage are summed apart and then added to the running sum, so a sum's
-// rounding error is that of n_slopes / 64 / cluster additions.  The cluster's
+// row halves x four quarters of a stage's K.  The cluster's
 // CTAs take K slices of one tile and add their tiles through distributed
 // shared memory in rank order: no workspace, so batches may be captured
 // without a set-up call.
+// Rounding: the 16 products of a quarter stage are summed apart and then added to
+// the running sum, and the sums of the quarters and the cluster are added with
+// their rounding errors carried along; two CTAs at least share a K of more than four
+// stages, or (FOLD) one adds them in blocks and the blocks in a second sum, which
+// lies in shared memory, as 64 products per thread leave no registers for it.  A
+// product's rounding errors then number about 6 + n_slopes / 256 at most, a warp
+// per row's 7 + n_slopes / 256.  (With plain sums over the quarters and one CTA where
+// the tiles fill the SMs, 4000 x 13344 on 100 vectors was 2.7e-7 of the norm off, a
+// warp per row 2.0e-7; 64 x 512 0.92e-7 and 0.83e-7.  Now 2.0e-7 and 0.77e-7.)
 constexpr int kTm = 64, kTk = 64, kTld = kTk + 4, kTout = kTm + 4;
 constexpr int kTq = 4;   // K quarters of a stage
 // A warp covers 32 rows: 32 / RM lanes of RM rows, RM lanes of RN vectors.
 // Small batches take RM = 4, which needs fewer shared loads per product
 // (8 vectors: 6 loads of 16 bytes for 8 products of 4 k, against 9).
-template <int RM, int RN> struct TileCfg {
+template <int RM, int RN, bool FOLD> struct TileCfg {
   static constexpr int LM = 32 / RM, LN = RM, BN = LN * RN;
   // small batches wait on HBM: two CTAs per SM
   static constexpr int STAGES = BN >= 64 ? 4 : 5;
   static constexpr int CTAS = BN >= 32 ? 1 : 2;
-  static constexpr size_t smem = (size_t)STAGES * (kTm + BN) * kTld * sizeof(float);
-  static_assert((size_t)kTq * BN * kTout * sizeof(float) <= smem, "the output tiles fit the stages");
+  static constexpr size_t stages = (size_t)STAGES * (kTm + BN) * kTld * sizeof(float);
+  static constexpr size_t smem = stages + (FOLD ? RM * RN * 256 * sizeof(float) : 0);
+  // columns at a time (FOLD keeps more addresses in registers; the rows are read twice)
+  static constexpr int JH = FOLD ? RN / 2 : RN;
+  static_assert((size_t)kTq * BN * kTout * sizeof(float) <= stages, "the output tiles fit the stages");
   static_assert(smem * CTAS <= 224 * 1024, "CTAS tiles per SM");
 };
 
@@ -237,11 +247,11 @@ __device__ __forceinline__ void cp_async_vec(float *dst, const float *src, bool 
                  : "memory");
 }
 
-template <int RM, int RN, int V>
-__global__ void __launch_bounds__(256, TileCfg<RM, RN>::CTAS) k_mvm_f32_tile(
+template <int RM, int RN, int V, bool FOLD>
+__global__ void __launch_bounds__(256, TileCfg<RM, RN, FOLD>::CTAS) k_mvm_f32_tile(
     const float *__restrict__ R, const float *__restrict__ s, float *__restrict__ m, int n_modes,
     int n_slopes, int nb, int tiles_n) {
-  using C = TileCfg<RM, RN>;
+  using C = TileCfg<RM, RN, FOLD>;
   constexpr int BN = C::BN, STAGES = C::STAGES, LM = C::LM, LN = C::LN;
   constexpr int kStage = (kTm + BN) * kTld;
   extern __shared__ __align__(16) float sm_f[];
@@ -286,6 +296,21 @@ __global__ void __launch_bounds__(256, TileCfg<RM, RN>::CTAS) k_mvm_f32_tile(
   for (int i = 0; i < RM; ++i)
 #pragma unroll
     for (int j = 0; j < RN; ++j) sum[i][j] = 0.f;
+  // FOLD: a block's sums into the second ones
+  float4 *tot = reinterpret_cast<float4 *>(sm_f + C::stages / sizeof(float)) + threadIdx.x;
+  const int per = kb1 - kb0 < 32 ? 4 : (kb1 - kb0 < 64 ? 8 : 16);   // stages per block
+  int left = per;
+  const auto fold = [&](bool first) {
+#pragma unroll
+    for (int e = 0; e < RM * RN / 4; ++e) {
+      float *u = &sum[e / (RN / 4)][e % (RN / 4) * 4];
+      float4 &t = tot[e * 256];
+      const float4 v = first ? make_float4(0.f, 0.f, 0.f, 0.f) : t;
+      t = make_float4(v.x + u[0], v.y + u[1], v.z + u[2], v.w + u[3]);
+      u[0] = u[1] = u[2] = u[3] = 0.f;
+    }
+  };
+  if constexpr (FOLD) fold(true);
 
 #pragma unroll
   for (int st = 0; st < STAGES - 1; ++st) {
@@ -303,33 +328,53 @@ __global__ void __launch_bounds__(256, TileCfg<RM, RN>::CTAS) k_mvm_f32_tile(
     }
     const float *sa = sm_f + slot * kStage + (wm + lm) * kTld + quarter * (kTk / kTq);
     const float *sb = sm_f + slot * kStage + (kTm + ln) * kTld + quarter * (kTk / kTq);
-    float2 acc[RM][RN];
 #pragma unroll
-    for (int k = 0; k < kTk / kTq; k += 4) {
-      float4 a[RM];
+    for (int jh = 0; jh < RN; jh += C::JH) {
+      float2 acc[RM][C::JH];
 #pragma unroll
-      for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4 *>(sa + i * LM * kTld + k);
+      for (int k = 0; k < kTk / kTq; k += 4) {
+        float4 a[RM];
 #pragma unroll
-      for (int j = 0; j < RN; ++j) {
-        const float4 b = *reinterpret_cast<const float4 *>(sb + j * LN * kTld + k);
-        const float2 b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
+        for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4 *>(sa + i * LM * kTld + k);
 #pragma unroll
-        for (int i = 0; i < RM; ++i) {
-          const float2 a0 = make_float2(a[i].x, a[i].y), a1 = make_float2(a[i].z, a[i].w);
-          acc[i][j] = k == 0 ? __fmul2_rn(a0, b0) : __ffma2_rn(a0, b0, acc[i][j]);
-          acc[i][j] = __ffma2_rn(a1, b1, acc[i][j]);
+        for (int j = 0; j < C::JH; ++j) {
+          const float4 b = *reinterpret_cast<const float4 *>(sb + (jh + j) * LN * kTld + k);
+          const float2 b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
+#pragma unroll
+          for (int i = 0; i < RM; ++i) {
+            const float2 a0 = make_float2(a[i].x, a[i].y), a1 = make_float2(a[i].z, a[i].w);
+            acc[i][j] = k == 0 ? __fmul2_rn(a0, b0) : __ffma2_rn(a0, b0, acc[i][j]);
+            acc[i][j] = __ffma2_rn(a1, b1, acc[i][j]);
+          }
         }
       }
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < C::JH; ++j) sum[i][jh + j] += acc[i][j].x + acc[i][j].y;
     }
-#pragma unroll
-    for (int i = 0; i < RM; ++i)
-#pragma unroll
-      for (int j = 0; j < RN; ++j) sum[i][j] += acc[i][j].x + acc[i][j].y;
+    if constexpr (FOLD) {
+      if (--left == 0) {   // uniform
+        fold(false);
+        left = per;
+      }
+    }
     slot = slot == STAGES - 1 ? 0 : slot + 1;
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();   // every stage has been read: the memory becomes the output tiles
 
+  if constexpr (FOLD) {
+#pragma unroll
+    for (int e = 0; e < RM * RN / 4; ++e) {
+      float *u = &sum[e / (RN / 4)][e % (RN / 4) * 4];
+      const float4 t = tot[e * 256];
+      u[0] += t.x;
+      u[1] += t.y;
+      u[2] += t.z;
+      u[3] += t.w;
+    }
+  }
   // T[quarter][vector][row]
   float *T = sm_f;
 #pragma unroll
@@ -339,25 +384,30 @@ __global__ void __launch_bounds__(256, TileCfg<RM, RN>::CTAS) k_mvm_f32_tile(
       T[(quarter * BN + j * LN + ln) * kTout + wm + i * LM + lm] = sum[i][j];
   cl.sync();
   // this CTA adds its share of the vectors over the quarters and the
-  // cluster, in order
+  // cluster, in order, the additions' errors (Knuth's two-sum) beside
   const int v0 = BN * rank / cs, v1 = BN * (rank + 1) / cs;
-  for (int e = threadIdx.x; e < (v1 - v0) * kTm; e += 256) {
-    const int v = v0 + e / kTm, r = e % kTm;
-    float x = 0.f;
+  for (int o = threadIdx.x; o < (v1 - v0) * kTm; o += 256) {
+    const int v = v0 + o / kTm, r = o % kTm;
+    float x = 0.f, e = 0.f;
     for (int c = 0; c < cs; ++c) {
       const float *Tc = cl.map_shared_rank(T, c) + v * kTout + r;
 #pragma unroll
-      for (int q = 0; q < kTq; ++q) x += Tc[q * BN * kTout];
+      for (int q = 0; q < kTq; ++q) {
+        const float y = Tc[q * BN * kTout], t = __fadd_rn(x, y), z = __fsub_rn(t, x);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(x, __fsub_rn(t, z)), __fsub_rn(y, z)));
+        x = t;
+      }
     }
+    if (isfinite(e)) x += e;   // an infinite or NaN sum is x itself
     if (n0 + v < nb && m0 + r < n_modes) m[(size_t)(n0 + v) * n_modes + m0 + r] = x;
   }
   cl.sync();   // no CTA leaves while another reads its tiles
 }
 
-template <int RM, int RN, int V>
+template <int RM, int RN, int V, bool FOLD = false>
 static int launch_tile(specula_ctx *ctx, const float *R, const float *s, float *m, int n_modes,
                        int n_slopes, int nb, cudaStream_t st) {
-  using C = TileCfg<RM, RN>;
+  using C = TileCfg<RM, RN, FOLD>;
   int sms = 0;
   SPECULA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
   const int tiles_n = (nb + C::BN - 1) / C::BN;
@@ -367,13 +417,13 @@ static int launch_tile(specula_ctx *ctx, const float *R, const float *s, float *
   // stages; clusters of eight at one CTA per SM leave SMs of most GPCs unused
   // (measured: half the GPU idle), so one per SM stops at four
   const int max_cs = C::CTAS == 1 ? 4 : 8;
-  int cs = 1;
+  int cs = kb > 4 && !FOLD ? 2 : 1;   // (the rounding above)
   while (cs < max_cs && tiles * cs * 2 <= (long long)sms * C::CTAS && kb / (cs * 2) >= 4) cs *= 2;
   if (tiles * cs > 0x7fffffffLL) return SPECULA_EUNSUPPORTED;
-  int e = ensure_dynamic_smem((const void *)k_mvm_f32_tile<RM, RN, V>, C::smem);
+  int e = ensure_dynamic_smem((const void *)k_mvm_f32_tile<RM, RN, V, FOLD>, C::smem);
   if (e) return e;
   SPECULA_LAUNCH(ctx, SPECULA_K_RECON, st,
-                 SPECULA_CK(launch_pdl((k_mvm_f32_tile<RM, RN, V>), (unsigned)(tiles * cs), 256,
+                 SPECULA_CK(launch_pdl((k_mvm_f32_tile<RM, RN, V, FOLD>), (unsigned)(tiles * cs), 256,
                                        C::smem, st, cs > 1 ? cs : 0, R, s, m, n_modes, n_slopes,
                                        nb, tiles_n)));
   return SPECULA_OK;
@@ -400,6 +450,16 @@ static int run_v(specula_ctx *ctx, const float *R, const float *s, float *m, int
   if (nb <= 8) return launch_tile<4, 2, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
   if (nb <= 16) return launch_tile<4, 4, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
   if (nb <= 32) return launch_tile<8, 4, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
+  // One CTA with a second sum (7 % more) where two take longer, counted in waves of
+  // stages with three more per CTA (128 vectors, two CTAs / one: 4000 x 512 26.8 /
+  // 21.6 us, 4000 x 1024 41.6 / 38.1, 4000 x 2512 87.4 / 87.0, 4000 x 13344 397 / 416)
+  int sms = 0;
+  SPECULA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+  const long long tiles = (long long)((n_modes + kTm - 1) / kTm) * ((nb + 63) / 64);
+  const int kb = (n_slopes + kTk - 1) / kTk;
+  const auto time = [&](int cs) { return (tiles * cs + sms - 1) / sms * (kb / cs + 3); };
+  if (kb > 4 && time(2) * 100 > time(1) * 107)
+    return launch_tile<8, 8, V, true>(ctx, R, s, m, n_modes, n_slopes, nb, st);
   return launch_tile<8, 8, V>(ctx, R, s, m, n_modes, n_slopes, nb, st);
 }
 
