@@ -19,52 +19,80 @@ constexpr int kDmUnroll = 8;
 constexpr int kDmMaxCluster = 8;
 constexpr int kLoopThreads = 256;
 
-template <int V> struct DmVec;
-template <> struct DmVec<4> { using T = float4; };
-template <> struct DmVec<1> { using T = float; };
 __device__ __forceinline__ void dm_axpy(float4 &a, float c, float4 v) {
   a.x += c * v.x;
   a.y += c * v.y;
   a.z += c * v.z;
   a.w += c * v.w;
 }
-__device__ __forceinline__ void dm_axpy(float &a, float c, float v) { a += c * v; }
+
+// Four pixels per lane of a tile of 4 LT: neighbours by one 16-byte access (VEC) or LT
+// apart by four of 4 bytes.
+template <bool VEC, int LT> struct DmPixels {
+  int i[4];
+  __device__ DmPixels(int tile, int ln, int n) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) i[k] = tile * 4 * LT + (VEC ? 4 * ln : ln + LT * k);
+  }
+  // (pixels past the grid repeat the last, or the last four)
+  __device__ __forceinline__ float4 load(const float *row, int n) const {
+    if constexpr (VEC)
+      return __ldg(reinterpret_cast<const float4 *>(row + min(i[0], n - 4)));
+    else
+      return make_float4(__ldg(row + min(i[0], n - 1)), __ldg(row + min(i[1], n - 1)),
+                         __ldg(row + min(i[2], n - 1)), __ldg(row + min(i[3], n - 1)));
+  }
+  __device__ __forceinline__ void store(float *phase, int n, float4 v) const {
+    if constexpr (VEC) {
+      if (i[0] < n) *reinterpret_cast<float4 *>(phase + i[0]) = v;
+    } else {
+      if (i[0] < n) phase[i[0]] = v.x;
+      if (i[1] < n) phase[i[1]] = v.y;
+      if (i[2] < n) phase[i[2]] = v.z;
+      if (i[3] < n) phase[i[3]] = v.w;
+    }
+  }
+};
 
 // phase[p] = sum over j of cmd[j] B[j][p].  Bound by reading B once: one
 // thread per pixel over all modes kept 5 KB in flight per SM (500 modes of
-// 160^2 pixels: 33 us for 51 MB).  A CTA of eight warps takes LT V pixels (V
-// = 4 floats per lane where the size and alignment allow, else 1), the modes
+// 160^2 pixels: 33 us for 51 MB).  A CTA of eight warps takes 4 LT pixels, the modes
 // split over the warps, over 32 / LT parts of a warp and, on small pupils, over a
 // cluster of CTAs; eight rows' loads in flight per lane.  Each part adds its
 // modes in order, then the parts' and the CTAs' sums are added in order.
-template <int V, int LT>
+template <bool VEC, int LT>
 __global__ void __launch_bounds__(kDmWarps * 32, 4) k_dm_shape(const float *__restrict__ B,
                                                             const float *__restrict__ cmd,
                                                             float *__restrict__ phase,
                                                             int n_modes, int n_pix2) {
-  using T = typename DmVec<V>::T;
-  __shared__ T s_p[kDmWarps][32];
+  __shared__ float4 s_p[kDmWarps][32];
   pdl_wait();
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nv = n_pix2 / V;
   constexpr int SUB = 32 / LT, NP = kDmWarps * SUB;   // parts of the modes per CTA
   const int ln = lane % LT;
-  const int p = blockIdx.x / cs * LT + ln;
+  const DmPixels<VEC, LT> px(blockIdx.x / cs, ln, n_pix2);
   const int part = rank * NP + warp * SUB + lane / LT, parts = cs * NP;
   int j = (int)((long long)n_modes * part / parts);
   const int j1 = (int)((long long)n_modes * (part + 1) / parts);
-  const T *b = reinterpret_cast<const T *>(B) + min(p, nv - 1);
-  T acc = T{};
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   for (; j + kDmUnroll <= j1; j += kDmUnroll) {
-    T v[kDmUnroll];
+    float4 v[kDmUnroll];
 #pragma unroll
-    for (int u = 0; u < kDmUnroll; ++u) v[u] = __ldg(b + (size_t)(j + u) * nv);
+    for (int u = 0; u < kDmUnroll; ++u) v[u] = px.load(B + (size_t)(j + u) * n_pix2, n_pix2);
 #pragma unroll
     for (int u = 0; u < kDmUnroll; ++u) dm_axpy(acc, __ldg(cmd + j + u), v[u]);
   }
-  for (; j < j1; ++j) dm_axpy(acc, __ldg(cmd + j), __ldg(b + (size_t)j * nv));
+  if (j < j1) {   // the rest's loads in flight together too
+    float4 v[kDmUnroll];
+#pragma unroll
+    for (int u = 0; u < kDmUnroll; ++u)
+      if (j + u < j1) v[u] = px.load(B + (size_t)(j + u) * n_pix2, n_pix2);
+#pragma unroll
+    for (int u = 0; u < kDmUnroll; ++u)
+      if (j + u < j1) dm_axpy(acc, __ldg(cmd + j + u), v[u]);
+  }
   s_p[warp][lane] = acc;
   __syncthreads();
   if (warp == 0) {
@@ -80,7 +108,42 @@ __global__ void __launch_bounds__(kDmWarps * 32, 4) k_dm_shape(const float *__re
     }
     cl.sync();   // no CTA leaves before its sums are read
   }
-  if (rank == 0 && warp == 0 && lane < LT && p < nv) reinterpret_cast<T *>(phase)[p] = acc;
+  if (rank == 0 && warp == 0 && lane < LT) px.store(phase, n_pix2, acc);
+}
+
+// The same for few modes: a warp takes 128 pixels and every mode, eight modes' loads in
+// flight, and adds the sums of the same eight parts in the same order, so the result
+// is k_dm_shape's to the last bit; up to eight modes one chain, as parts of one
+// product round twice.
+template <bool VEC>
+__global__ void __launch_bounds__(kDmWarps * 32) k_dm_few(const float *__restrict__ B,
+                                                          const float *__restrict__ cmd,
+                                                          float *__restrict__ phase, int n_modes,
+                                                          int n_pix2) {
+  pdl_wait();
+  const DmPixels<VEC, 32> px(blockIdx.x * kDmWarps + (threadIdx.x >> 5), threadIdx.x & 31, n_pix2);
+  const int parts = n_modes <= kDmUnroll ? 1 : kDmWarps;
+  float4 sum = make_float4(0.f, 0.f, 0.f, 0.f), acc = sum;
+  int part = 1, next = n_modes / parts;   // modes below `next` are in the part so far
+  for (int j = 0; j < n_modes; j += kDmUnroll) {
+    float4 v[kDmUnroll];
+#pragma unroll
+    for (int u = 0; u < kDmUnroll; ++u)
+      if (j + u < n_modes) v[u] = px.load(B + (size_t)(j + u) * n_pix2, n_pix2);
+#pragma unroll
+    for (int u = 0; u < kDmUnroll; ++u)
+      if (j + u < n_modes) {
+        if (j + u == next) {
+          dm_axpy(sum, 1.f, acc);
+          acc = make_float4(0.f, 0.f, 0.f, 0.f);
+          ++part;
+          next = n_modes * part / parts;
+        }
+        dm_axpy(acc, __ldg(cmd + j + u), v[u]);
+      }
+  }
+  dm_axpy(sum, 1.f, acc);
+  px.store(phase, n_pix2, sum);
 }
 
 // residual = atm - dm over the grid, and its statistics: float64 sums over
@@ -205,8 +268,16 @@ extern "C" int specula_dm_shape(specula_ctx *ctx, int32_t n_modes, int32_t n_pix
   // over a cluster until there are, while every part keeps a full unroll of
   // modes.  (Narrow tiles before clusters, whose CTAs share SMs while others stand
   // idle; with the shorter butterflies of the residual, 8 m step 64.9 -> 62.3 us.)
-  const int px = v4 ? 4 : 1;
-  const auto tiles_of = [&](int lt) { return (n_pix2 / px + lt - 1) / lt; };
+  // k_dm_few up to eight modes, and below four modes per warp where a warp per 128
+  // pixels still gives every SM a CTA (400^2 pixels: 12 modes 4.0 -> 3.1 us, 20 modes
+  // 6.2 -> 5.0; 50 modes 8.6 against 9.8).
+  const auto tiles_of = [&](int lt) { return (int)((n_pix2 + 4LL * lt - 1) / (4 * lt)); };
+  const int few = (tiles_of(32) + kDmWarps - 1) / kDmWarps;
+  if (n_modes <= kDmUnroll || (n_modes < 4 * kDmWarps && few >= sms)) {
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_LOOP, st, (v4 ? k_dm_few<true> : k_dm_few<false>), few,
+                       kDmWarps * 32, 0, basis_dev, cmd_dev, phase_dev, n_modes, n_pix2);
+    return SPECULA_OK;
+  }
   int lt = 32;
   while (v4 && lt > 8 && tiles_of(lt) < 2 * sms &&
          n_modes / (kDmWarps * (64 / lt)) >= kDmUnroll)
@@ -219,8 +290,9 @@ extern "C" int specula_dm_shape(specula_ctx *ctx, int32_t n_modes, int32_t n_pix
   const unsigned grid = (unsigned)tiles * cs;
   const int cluster = cs > 1 ? cs : 0;
   void (*fn)(const float *, const float *, float *, int, int) =
-      !v4 ? k_dm_shape<1, 32>
-          : (lt == 32 ? k_dm_shape<4, 32> : (lt == 16 ? k_dm_shape<4, 16> : k_dm_shape<4, 8>));
+      !v4 ? k_dm_shape<false, 32>
+          : (lt == 32 ? k_dm_shape<true, 32>
+                      : (lt == 16 ? k_dm_shape<true, 16> : k_dm_shape<true, 8>));
   SPECULA_LAUNCH(ctx, SPECULA_K_LOOP, st,
                  SPECULA_CK(launch_pdl(fn, grid, kDmWarps * 32, 0, st, cluster, basis_dev, cmd_dev,
                                        phase_dev, n_modes, n_pix2)));
