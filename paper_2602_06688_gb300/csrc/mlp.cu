@@ -30,8 +30,14 @@ constexpr int TT = 32;   // transpose tile
 // Thread rows of a tile kernel: one element per thread.  The training step's
 // kernels cover 256 rows by about 1000 columns, so the time is that of a few
 // rounds of loads; four elements per thread were four times the rounds
-// (gelu' of 256 x 1024 from 16 partials: 13.8 us).
-constexpr int TY = 32;
+// (gelu' of 256 x 1024 from 16 partials: 13.8 us).  Matrices of more than four waves
+// of such blocks take eight rows, four elements per thread (tile_rows): their time is
+// that of the blocks (4096 x 2560 inputs: 41 us with 32 rows, 28 with 8; bias and GELU of
+// 4096 x 1024: 26, 23).
+constexpr int TY = 32, TYL = 8;
+static int tile_rows(int R, int C, int sms) {
+  return (long long)(R / TT) * (C / TT) > 8LL * sms ? TYL : TY;
+}
 
 __device__ __forceinline__ float gelu_f(float z) {
   return 0.5f * z * (1.0f + erff(z * (float)M_SQRT1_2));
@@ -41,16 +47,16 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
   return 0.5f * (1.0f + erff(z * (float)M_SQRT1_2)) + z * expf(-0.5f * z * z) * inv_sqrt_2pi;
 }
 
-// Tiled writer of a bf16 matrix and, where outT is given, its transpose.  Block (32, TY), grid
+// Tiled writer of a bf16 matrix and, where outT is given, its transpose.  Block (32, RY), grid
 // (C/32, R/32); the value function is evaluated once per element.
-template <class F>
+template <int RY, class F>
 __device__ __forceinline__ void tile_bf16_pair(int R, int C, __nv_bfloat16 *out,
                                                __nv_bfloat16 *outT, F value) {
   __shared__ __nv_bfloat16 tile[TT][TT + 2];
   const int c0 = blockIdx.x * TT, r0 = blockIdx.y * TT;
 #pragma unroll
-  for (int k = 0; k < TT / TY; ++k) {
-    const int dr = threadIdx.y + TY * k, r = r0 + dr, c = c0 + threadIdx.x;
+  for (int k = 0; k < TT / RY; ++k) {
+    const int dr = threadIdx.y + RY * k, r = r0 + dr, c = c0 + threadIdx.x;
     __nv_bfloat16 v = __float2bfloat16_rn(0.f);
     if (r < R && c < C) {
       v = __float2bfloat16_rn(value(r, c));
@@ -61,17 +67,19 @@ __device__ __forceinline__ void tile_bf16_pair(int R, int C, __nv_bfloat16 *out,
   if (!outT) return;   // the whole launch
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < TT / TY; ++k) {
-    const int dc = threadIdx.y + TY * k, c = c0 + dc, r = r0 + threadIdx.x;
+  for (int k = 0; k < TT / RY; ++k) {
+    const int dc = threadIdx.y + RY * k, c = c0 + dc, r = r0 + threadIdx.x;
     if (r < R && c < C) outT[(size_t)c * R + r] = tile[threadIdx.x][dc];
   }
 }
 
 // X [B][n_in] float -> Xb [Bp][in_pad] and XbT [in_pad][Bp] (zero pads)
-__global__ void __launch_bounds__(TT * TY) k_pack_input(const float *__restrict__ X, int B, int n_in, int Bp, int in_pad,
-                             __nv_bfloat16 *Xb, __nv_bfloat16 *XbT) {
+template <int RY>
+__global__ void __launch_bounds__(TT * RY) k_pack_input(const float *__restrict__ X, int B,
+                                                       int n_in, int Bp, int in_pad,
+                                                       __nv_bfloat16 *Xb, __nv_bfloat16 *XbT) {
   pdl_wait();
-  tile_bf16_pair(Bp, in_pad, Xb, XbT, [&](int r, int c) {
+  tile_bf16_pair<RY>(Bp, in_pad, Xb, XbT, [&](int r, int c) {
     return (r < B && c < n_in) ? X[(size_t)r * n_in + c] : 0.f;
   });
 }
@@ -107,12 +115,13 @@ __device__ __forceinline__ float partial_sum(const Partials &P, size_t e) {
 }
 
 // Z = sum of partials + bias; H = gelu(Z) and its transpose in bf16
-__global__ void __launch_bounds__(TT * TY) k_bias_gelu(const Partials P,
+template <int RY>
+__global__ void __launch_bounds__(TT * RY) k_bias_gelu(const Partials P,
                                                       const float *__restrict__ bias,
                                                       float *__restrict__ Z, int R, int C,
                                                       __nv_bfloat16 *H, __nv_bfloat16 *HT) {
   pdl_wait();
-  tile_bf16_pair(R, C, H, HT, [&](int r, int c) {
+  tile_bf16_pair<RY>(R, C, H, HT, [&](int r, int c) {
     const size_t e = (size_t)r * C + c;
     const float z = partial_sum(P, e) + bias[c];
     Z[e] = z;
@@ -135,12 +144,13 @@ __global__ void __launch_bounds__(256) k_output(const Partials P, const float *_
 }
 
 // dA = (sum of partials) gelu'(Z); bf16 dZ and its transpose
-__global__ void __launch_bounds__(TT * TY) k_gelu_back(const Partials P,
+template <int RY>
+__global__ void __launch_bounds__(TT * RY) k_gelu_back(const Partials P,
                                                       const float *__restrict__ Z, float *dA,
                                                       int R, int C, __nv_bfloat16 *dZb,
                                                       __nv_bfloat16 *dZbT) {
   pdl_wait();
-  tile_bf16_pair(R, C, dZb, dZbT, [&](int r, int c) {
+  tile_bf16_pair<RY>(R, C, dZb, dZbT, [&](int r, int c) {
     const size_t e = (size_t)r * C + c;
     const float d = partial_sum(P, e) * gelu_grad_f(Z[e]);
     dA[e] = d;
@@ -165,7 +175,7 @@ __global__ void __launch_bounds__(TT * TY) k_loss_grad(
   pdl_wait();
   __shared__ float s_sq[2][TY];
   float sq = 0.f;
-  tile_bf16_pair(Bp, out_pad, dYb, dYbT, [&](int r, int c) {
+  tile_bf16_pair<TY>(Bp, out_pad, dYb, dYbT, [&](int r, int c) {
     float d = 0.f;
     if (r < B && c < n_out) d = Y[(size_t)r * out_pad + c] - T[(size_t)r * n_out + c];
     sq += d * d;
@@ -287,7 +297,7 @@ __global__ void __launch_bounds__(TT * 8) k_adam(const AdamArgs A, float lr_t, f
 
 __global__ void __launch_bounds__(TT * TY) k_cast_w(const float *__restrict__ W, int R, int C, __nv_bfloat16 *Wb,
                          __nv_bfloat16 *WbT) {
-  tile_bf16_pair(R, C, Wb, WbT, [&](int r, int c) { return W[(size_t)r * C + c]; });
+  tile_bf16_pair<TY>(R, C, Wb, WbT, [&](int r, int c) { return W[(size_t)r * C + c]; });
 }
 
 // column mean and standard deviation of X [R][C] (float64 sums, rows in order)
@@ -706,18 +716,21 @@ extern "C" int specula_mlp_forward(specula_mlp *p, const float *X_dev, int32_t b
   cudaStream_t st = (cudaStream_t)stream;
   specula_ctx *ctx = p->ctx;
   const int in = p->np[0], h1 = p->np[1], h2 = p->np[2], o = p->np[3];
-  const dim3 tb(TT, TY);
-  int s;
-  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_pack_input, dim3(in / TT, Bp / TT), tb, 0, X_dev,
-                     batch, p->n[0], Bp, in, p->Xb.as<__nv_bfloat16>(),
-                     p->XbT.as<__nv_bfloat16>());
+  int sms = 0, s;
+  SPECULA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+  int ry = tile_rows(Bp, in, sms);
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, (ry == TY ? k_pack_input<TY> : k_pack_input<TYL>),
+                     dim3(in / TT, Bp / TT), dim3(TT, ry), 0, X_dev, batch, p->n[0], Bp, in,
+                     p->Xb.as<__nv_bfloat16>(), p->XbT.as<__nv_bfloat16>());
   const void *Hin = p->Xb.p;
   Partials P;
   for (int l = 0; l < 2; ++l) {
     const int K = p->np[l], N = p->np[l + 1];
     if ((s = mlp_gemm(p, Hin, p->Wb[l].p, Bp, N, K, &P, st))) return s;
-    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_bias_gelu, dim3(N / TT, Bp / TT), tb, 0, P,
-                       p->b[l].as<float>(), p->Z[l].as<float>(), Bp, N,
+    ry = tile_rows(Bp, N, sms);
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, (ry == TY ? k_bias_gelu<TY> : k_bias_gelu<TYL>),
+                       dim3(N / TT, Bp / TT), dim3(TT, ry), 0, P, p->b[l].as<float>(),
+                       p->Z[l].as<float>(), Bp, N,
                        p->H[l].as<__nv_bfloat16>(), p->HT[l].as<__nv_bfloat16>());
     Hin = p->H[l].p;
   }
@@ -774,11 +787,11 @@ extern "C" int specula_mlp_backward(specula_mlp *p, const float *T_dev, int32_t 
   cudaStream_t st = (cudaStream_t)stream;
   specula_ctx *ctx = p->ctx;
   const int h1 = p->np[1], h2 = p->np[2], o = p->np[3];
-  const dim3 tb(TT, TY);
   const float scale = 2.0f / ((float)batch * (float)p->n[3]);
   const dim3 gl(o / TT, Bp / TT);
-  int s;
-  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_loss_grad, gl, tb, 0, p->Y.as<float>(), T_dev,
+  int sms = 0, s;
+  SPECULA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+  SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_loss_grad, gl, dim3(TT, TY), 0, p->Y.as<float>(), T_dev,
                      batch, p->n[3], Bp, o, scale, p->dYf.as<float>(), p->dYb.as<__nv_bfloat16>(),
                      p->dYbT.as<__nv_bfloat16>(), p->done.as<unsigned>(), p->part.as<float>(),
                      1.0f / ((float)batch * (float)p->n[3]),
@@ -787,7 +800,9 @@ extern "C" int specula_mlp_backward(specula_mlp *p, const float *T_dev, int32_t 
   if ((s = mlp_gemm(p, p->dYb.p, p->WbT[2].p, Bp, h2, o, &P, st))) return s;
   for (int l = 1; l >= 0; --l) {
     const int N = p->np[l + 1];
-    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, k_gelu_back, dim3(N / TT, Bp / TT), tb, 0, P,
+    const int ry = tile_rows(Bp, N, sms);
+    SPECULA_LAUNCH_PDL(ctx, SPECULA_K_MLP, st, (ry == TY ? k_gelu_back<TY> : k_gelu_back<TYL>),
+                       dim3(N / TT, Bp / TT), dim3(TT, ry), 0, P,
                        p->Z[l].as<float>(), p->dA[l].as<float>(), Bp, N,
                        p->dZb[l].as<__nv_bfloat16>(), p->dZbT[l].as<__nv_bfloat16>());
     if (l == 1)
