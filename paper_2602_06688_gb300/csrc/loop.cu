@@ -199,30 +199,37 @@ __global__ void __launch_bounds__(kLoopThreads) k_loop_residual(
     a[4] += w * (double)sv;
   }
   loop_block_sum(a, s_p);
-  if (threadIdx.x < 5) {
+  // thread q < 5: the warps' sums of value q
+  const auto warps_sum = [&]() {
     double v = 0.0;
-    for (int w = 0; w < kLoopThreads / 32; ++w) v += s_p[threadIdx.x][w];
-    __stcg(part + (size_t)blockIdx.x * 5 + threadIdx.x, v);
+    if (threadIdx.x < 5)
+      for (int w = 0; w < kLoopThreads / 32; ++w) v += s_p[threadIdx.x][w];
+    return v;
+  };
+  double v = warps_sum();
+  if (gridDim.x > 1) {
+    if (threadIdx.x < 5) {
+      __stcg(part + (size_t)blockIdx.x * 5 + threadIdx.x, v);
+      __threadfence();
+    }
+    __syncthreads();
+    // atomicInc wraps to zero on the last CTA: ready for the next launch
+    if (threadIdx.x == 0) s_last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
     __threadfence();
+#pragma unroll
+    for (int q = 0; q < 5; ++q) a[q] = 0.0;
+    for (int b = threadIdx.x; b < gridDim.x; b += blockDim.x)
+#pragma unroll
+      for (int q = 0; q < 5; ++q) a[q] += __ldcg(part + (size_t)b * 5 + q);
+    loop_block_sum(a, s_p);
+    v = warps_sum();
   }
-  __syncthreads();
-  // atomicInc wraps to zero on the last CTA: ready for the next launch
-  if (threadIdx.x == 0) s_last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
+  if (threadIdx.x >= 32) return;
 #pragma unroll
-  for (int q = 0; q < 5; ++q) a[q] = 0.0;
-  for (int b = threadIdx.x; b < gridDim.x; b += blockDim.x)
-#pragma unroll
-    for (int q = 0; q < 5; ++q) a[q] += __ldcg(part + (size_t)b * 5 + q);
-  loop_block_sum(a, s_p);
+  for (int q = 0; q < 5; ++q) a[q] = __shfl_sync(0xffffffffu, v, q);
   if (threadIdx.x != 0) return;
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    a[q] = 0.0;
-    for (int w = 0; w < kLoopThreads / 32; ++w) a[q] += s_p[q][w];
-  }
   if (!(a[0] > 0.0)) {
     stats[0] = 0.0;
     stats[1] = 0.0;
