@@ -30,8 +30,12 @@ def _stream(stream):
     import torch
     if stream is None:
         # the current stream's handle without the Stream object that
-        # torch.cuda.current_stream() builds (3 us of a call's 9)
-        return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        # torch.cuda.current_stream() builds (3 us of a call's 9); the call is not
+        # one of torch's public ones, so the public one stands in for it
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return C.c_void_p(raw(torch.cuda.current_device()))
     if isinstance(stream, int):
         return C.c_void_p(stream)
     return C.c_void_p(stream.cuda_stream)
