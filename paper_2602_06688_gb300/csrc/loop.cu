@@ -266,7 +266,7 @@ extern "C" int specula_dm_shape(specula_ctx *ctx, int32_t n_modes, int32_t n_pix
                                 void *stream) {
   if (!ctx || !basis_dev || !cmd_dev || !phase_dev) return SPECULA_EINVAL;
   if (n_modes < 1 || n_pix2 < 1) return SPECULA_EINVAL;
-  if (n_modes > 12288) return SPECULA_EUNSUPPORTED;
+  if (n_modes > 12288) return SPECULA_EUNSUPPORTED;   // the documented limit
   cudaStream_t st = (cudaStream_t)stream;
   const bool v4 = n_pix2 % 4 == 0 && (((uintptr_t)basis_dev | (uintptr_t)phase_dev) % 16) == 0;
   int sms = 0;

@@ -1113,7 +1113,7 @@ namespace {
 // the task's cost late here).
 //
 // Groups are tasks of one kind and sensor; tasks of a group go in list order.
-// At most `mvm_cap` CTAs take reconstructor tasks while others are left: a
+// At most `mvm_cap` CTAs take reconstructor tasks at a time: a
 // third of the slots draws half the HBM rate while the rest keep computing (a
 // 39 m frame with a half instead: 247 us against 242).  The order before this,
 // sensor after sensor with the pyramids last, left their chains of passes and
@@ -1134,11 +1134,8 @@ bool schedule_tasks(std::vector<MwGroup> &groups, int n_ctr, int workers, int mv
   };
   std::priority_queue<Ev> q;
   std::vector<int> done(n_ctr, 0);
-  size_t left = 0, left_other = 0;
-  for (auto &g : groups) {
-    left += g.t.size();
-    if (!g.t.empty() && g.t[0].type != MT_MVM) left_other += g.t.size();
-  }
+  size_t left = 0;
+  for (auto &g : groups) left += g.t.size();
   int idle = workers, mvm = 0;
   double now = 0.;
   while (left) {
@@ -1149,12 +1146,11 @@ bool schedule_tasks(std::vector<MwGroup> &groups, int n_ctr, int workers, int mv
         if (g.head == g.t.size()) continue;
         const MwTask &t = g.t[g.head];
         const bool is_mvm = t.type == MT_MVM;
-        if (is_mvm && left_other && mvm >= mvm_cap) continue;
+        if (is_mvm && mvm >= mvm_cap) continue;
         if (t.wait_ctr >= 0 && done[t.wait_ctr] < t.wait_val) continue;
         out.push_back(t);
         g.head++;
         left--;
-        if (!is_mvm) left_other--;
         idle--;
         mvm += is_mvm;
         q.push({now + g.cost, -1, is_mvm});

@@ -950,7 +950,7 @@ bool pwfs_split_for(int N, int *N1, int *N2) {
     case 320: *N1 = 20; *N2 = 16; return true;
     case 660: *N1 = 30; *N2 = 22; return true;   // 22 = 2 x 11, prime-factor form
     case 960: *N1 = 30; *N2 = 32; return true;
-    case 1600: *N1 = 32; *N2 = 50; return true;   // wide: 50 = 2 x 25 in two lane strides
+    case 1600: *N1 = 32; *N2 = 50; return true;   // no kernel's: the two-pass form takes 40 x 40
     default: return false;
   }
 }
@@ -1246,8 +1246,10 @@ int pwfs_plan_build(specula_ctx *ctx, const specula_pupil_desc *pupil,
   if ((s = p->gx.upload(gx.data(), gx.size() * sizeof(float2)))) return s;
   if ((s = p->gy.upload(gy.data(), gy.size() * sizeof(float2)))) return s;
   if ((s = p->mask.upload(mk.data(), mk.size() * sizeof(float2)))) return s;
-  if ((s = p->twA.upload(ta.data(), ta.size() * sizeof(float2)))) return s;
-  if ((s = p->twB.upload(tb.data(), tb.size() * sizeof(float2)))) return s;
+  if (p->blockA) {   // the three-pass form's split (and the shifted form's)
+    if ((s = p->twA.upload(ta.data(), ta.size() * sizeof(float2)))) return s;
+    if ((s = p->twB.upload(tb.data(), tb.size() * sizeof(float2)))) return s;
+  }
   std::vector<float2> pa, pb;
   pwfs_host_twiddles(N, p->M1, p->M2, &pa, &pb);
   if ((s = p->tpA.upload(pa.data(), pa.size() * sizeof(float2)))) return s;

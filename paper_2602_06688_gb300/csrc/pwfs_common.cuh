@@ -21,7 +21,7 @@ template <int N1_, int N2_> struct Split {
   // general-offset loads only (the plan refuses pad 2 for them)
   // N2 > 32: the two-pass kernels only, which have their own split
   static constexpr bool WIDE = N2_ > 32;
-  static_assert(N1_ <= 32 && N2_ <= 64, "N1 lanes per warp; N2 in at most two lane strides");
+  static_assert(N1_ <= 32 && N2_ <= 64, "N1 lanes per warp; N2 <= 32 where a kernel runs it");
   static_assert(2 * XB >= N, "a vector's exchange buffer must hold N floats");
 };
 

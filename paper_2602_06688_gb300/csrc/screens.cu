@@ -113,9 +113,10 @@ __global__ void k_screen_final(const double2 *__restrict__ T, const double2 *__r
 // after exact integer range reduction and short polynomials (the table-driven
 // method of Tang, ACM TOMS 16, 378, 1990, for the logarithm; addition theorems
 // for sine and cosine; Goldschmidt's iteration for the square root), about 39
-// float64 operations per pair where log, sqrt and sincospi took about twice
-// that (16.8 million pairs and their transforms: 2.79 -> 1.63 ms).  Largest errors
-// on the CPU over 6 million arguments: radius 1.7e-16 relative, angle 2.1e-16.
+// float64 operations per pair where log, sqrt and sincospi take about twice
+// that.  Largest errors on the CPU over 6 million arguments: radius 1.7e-16
+// relative, angle 2.1e-16; a normal's, against 113-bit arithmetic over half a million,
+// 3.6e-16 of the radius (7.3e-16 with log, cos and sin of the rounded angle).
 constexpr int kLogFirst = 90, kLogCount = 91;   // j = 90 .. 180
 // c = 128 / j rounded, and 2 ln c and 2 n ln 2 as multiples of 2^-40, whose sums
 // are exact, with their remainders
@@ -280,9 +281,6 @@ __global__ void k_rng_complex(uint64_t seed, int sample0, int stream_id, long lo
 // pass 2 (k_screen_cols) transforms the columns, adds the subharmonics and
 // rounds to float32 once.
 
-// Radix-4 Stockham pass of an M = 2^LOGM point inverse DFT (sign +), thread t
-// of M/4, in place in buf with the values held in registers between the two
-// barriers.  L: length transformed so far.  All threads of the CTA call it.
 __device__ __forceinline__ double2 dmul(double2 a, double2 w) {
   return make_double2(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
 }
@@ -302,7 +300,9 @@ __device__ __forceinline__ void dft4(cpair (&x)[4]) {   // natural order, sign +
   x[3] = cpair{fp_add(b.re, e.im), fp_sub(b.im, e.re)};
 }
 
-// M-point inverse DFT of one vector by M/4 threads.  load(i): input i of the
+// M = 2^LOGM point inverse DFT (sign +) of one vector by M/4 threads: radix-4 Stockham
+// passes in place in buf, the values in registers between a pass's two barriers.  All
+// threads of the CTA call it.  load(i): input i of the
 // first pass, called before the first barrier; store(i, v): output i, called
 // after the last barrier (every load and exchange of the CTA is done).  tw[m]
 // = exp(2 pi i m / M).  Odd LOGM ends with a radix-2 pass.
