@@ -486,7 +486,13 @@ int specula_atmo_extract_noalloc(int32_t n_layers, const specula_layer_desc *lay
 /* Build (or reuse) the tables and workspace of a pyramid geometry: modulation
  * tilt tables, pyramid-mask tables and FFT twiddles, computed in float64 on
  * the host and rounded once to float32.  May allocate.  Supported FFT sides
- * N = pad * n_pix: 64, 128, 240, 320, 660, 960, 1600. */
+ * N = pad * n_pix: 64, 128, 240, 320, 660, 960, 1600.
+ * The workspace serves any batch.  In the two-pass form its largest part is at
+ * most 100 MB (or one slot's n_pix N complex): whole batch elements of n_mod / 2 +
+ * 1 slots, up to 32, or equal parts of one; then a float32 partial detector per
+ * modulation point and a complex field for each of those elements and one more.
+ * The 8 m pupil (160 px, 24 points) takes 118 MB, for 19 elements at a time.  It is
+ * the plan's until the context is destroyed; larger tiles (below) make it larger. */
 int specula_pwfs_plan(specula_ctx *ctx, const specula_pupil_desc *pupil,
                       const specula_pwfs_desc *pwfs);
 
@@ -691,7 +697,10 @@ int specula_slopes(specula_ctx *ctx, const specula_slopec_desc *slopec,
 /* Modal reconstruction (Modalrec): modes[b] = R slopes[b] for n_batch slope
  * vectors of n_slopes floats; modes_dev: n_batch * n_modes floats.
  * Accumulation in float32 for every precision.  FP32 runs on the CUDA
- * cores at every batch.  BF16 and BF16X2 (n_slopes a multiple of 8, 16-byte
+ * cores at every batch; which kernel, and so the order of a sum, follows
+ * n_batch, the sizes, the alignment and the number of SMs: the last bits of a
+ * vector's modes can differ from one batch size to another, and are the same
+ * in every call of one.  BF16 and BF16X2 (n_slopes a multiple of 8, 16-byte
  * aligned operands) run on the CUDA cores below 32 vectors; from 32 on, the
  * slopes are split into bfloat16 halves xh + xl in a context-owned
  * workspace and one tensor-core GEMM forms xh Rh^T + xh Rl^T + xl Rh^T
@@ -850,8 +859,8 @@ int specula_mlp_forward(specula_mlp *mlp, const float *X_dev, int32_t batch, flo
                         void *stream);
 /* Inference only (keeps no state for backward): Y_dev = the network applied
  * to X_dev.  For batch <= 4 each layer streams its bf16 weight rows once
- * against the float32 inputs (one warp per output, float32 accumulation and
- * activations): the way to run the network inside a frame.  Larger batches
+ * against the float32 inputs (float32 accumulation and activations): the way
+ * to run the network inside a frame.  Larger batches
  * run as specula_mlp_forward (whose tensor-core GEMMs take bf16 activations,
  * so results differ at the bf16 level).  Per-frame call: enqueues only. */
 int specula_mlp_infer(specula_mlp *mlp, const float *X_dev, int32_t batch, float *Y_dev,
@@ -955,9 +964,10 @@ int specula_rebin(specula_ctx *ctx, const float *in_dev, int32_t n_in, int32_t n
  *   c_k = (1 - leak) c_{k-1} + gain m            (specula_loop_integrate)
  * All sums run in a fixed order: a loop is bit-reproducible. */
 
-/* phase_dev[p] = sum over j (in order) of cmd_dev[j] basis_dev[j][p]:
- * basis n_modes x n_pix2 row-major floats (zero outside the pupil), cmd
- * n_modes floats, phase n_pix2 floats (radians at the sensor wavelength).
+/* phase_dev[p] = sum over j of cmd_dev[j] basis_dev[j][p], parts of the modes
+ * each in order and then their sums in order (how many parts follows the sizes,
+ * the alignment and the number of SMs; one up to 8 modes): basis n_modes x n_pix2
+ * row-major floats (zero outside the pupil), cmd n_modes floats, phase n_pix2 floats (radians at the sensor wavelength).
  * n_modes <= 12288 (SPECULA_EUNSUPPORTED above). */
 int specula_dm_shape(specula_ctx *ctx, int32_t n_modes, int32_t n_pix2, const float *basis_dev,
                      const float *cmd_dev, float *phase_dev, void *stream);
