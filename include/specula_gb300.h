@@ -967,7 +967,8 @@ int specula_rebin(specula_ctx *ctx, const float *in_dev, int32_t n_in, int32_t n
 /* phase_dev[p] = sum over j of cmd_dev[j] basis_dev[j][p], parts of the modes
  * each in order and then their sums in order (how many parts follows the sizes,
  * the alignment and the number of SMs; one up to 8 modes): basis n_modes x n_pix2
- * row-major floats (zero outside the pupil), cmd n_modes floats, phase n_pix2 floats (radians at the sensor wavelength).
+ * row-major floats (zero outside the pupil), cmd n_modes floats, phase n_pix2
+ * floats (radians at the sensor wavelength).
  * n_modes <= 12288 (SPECULA_EUNSUPPORTED above). */
 int specula_dm_shape(specula_ctx *ctx, int32_t n_modes, int32_t n_pix2, const float *basis_dev,
                      const float *cmd_dev, float *phase_dev, void *stream);

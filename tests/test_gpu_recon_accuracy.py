@@ -55,3 +55,23 @@ def test_error_of_batches(nm, ns):
                 e_ref += float((_warp_per_row(torch, Rr, sv[v:v + 4]) - exact[v:v + 4]).square().sum())
         assert e <= 1.05 ** 2 * e_ref, (nb, (e / e_ref) ** 0.5)
     close_checked(sp, ctx)
+
+
+@pytest.mark.parametrize("nm,ns,nb", [(4000, 513, 100), (4000, 514, 100), (3990, 1022, 65),
+                                      (4000, 321, 128), (2500, 516, 200)])
+def test_second_sums_of_odd_sizes(nm, ns, nb):
+    """Loads of one and two floats, K tails and ragged tiles where one CTA keeps a
+    second sum; the bound of tests/test_gpu_recon_f32.py."""
+    torch = need_gpu()
+    sp = load_pkg()
+    ctx = sp.Context(0)
+    g = torch.Generator(device="cuda").manual_seed(nm + ns)
+    R = torch.randn(nm, ns, generator=g, device="cuda")
+    s = torch.randn(nb, ns, generator=g, device="cuda")
+    out = torch.full((nb * nm + 64,), 7.0, device="cuda")
+    sp.specula_recon(ctx, sp.recon_desc(nm, ns, sp.PREC_FP32, R), s, out)
+    err = (out[:nb * nm].view(nb, nm).double() - s.double() @ R.double().T).abs()
+    depth = 40 + -(-ns // 64)
+    assert bool((err <= depth * 2.0 ** -24 * (s.double().abs() @ R.double().abs().T)).all())
+    assert bool((out[nb * nm:] == 7.0).all())
+    close_checked(sp, ctx)
